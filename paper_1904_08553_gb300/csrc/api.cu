@@ -404,7 +404,7 @@ int dcd_destroy(dcd_ctx* c) {
     c->ins.reset(); c->del.reset(); c->dsc.reset(); c->iota.reset(); c->rset_nx.reset();
     c->feat_X.reset(); c->feat_y.reset(); c->feat_v.reset(); c->level0.reset();
     c->gs.reset(); c->goff_d.reset(); c->gid.reset();
-    c->in_prev.reset(); c->in_next.reset();
+    c->in_prev.reset(); c->in_next.reset(); c->kdeg[0].reset(); c->kdeg[1].reset();
     c->kc_mat.reset(); c->kc_mat_nx.reset(); c->kc_idx.reset(); c->kc_idx_nx.reset();
     c->kc_lab.reset(); c->kc_lab_nx.reset(); c->h0.reset(); c->h0_ccid.reset();
     if (c->mem.arena) cudaFreeAsync(c->mem.arena, c->stream);
@@ -500,12 +500,17 @@ static std::vector<BinPlan> candidate_plans() {
   return out;
 }
 
+// Per graph: sum_i e_{i->C(i)} and 2m, kept for the next merge.
+__global__ void save_in(const GraphState* __restrict__ gs, int G, int64_t* __restrict__ out) {
+  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
+    out[g] = gs[g].in_cur;
+    out[G + g] = gs[g].m2;
+  }
+}
+
 // Times one local-move evaluation of every vertex of the current graph under
 // the current labels for each candidate plan and keeps the fastest.  Every
 // plan gives the same proposals; only the time differs.
-__global__ void save_in(const GraphState* __restrict__ gs, int G, int64_t* __restrict__ out) {
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) out[g] = gs[g].in_cur;
-}
 
 int autotune_impl(dcd_ctx* c, int32_t reps, float* best_ms) {
   if (c->t == 0 || reps < 1) return DCD_ESTATE;
@@ -561,7 +566,7 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
   // per-graph state after the merge (2m, sum e_{i->C(i)} under C_{t-1}): a
   // second run from the same state starts from this copy
   std::vector<GraphState> gs0(c->hgs, c->hgs + c->G);
-  const int64_t nnz_new = c->hscratch[8];
+  const int64_t nnz_new = c->hscratch[8], npairs = c->hsc->npairs;
   Csr<int32_t> g{n, nnz_new, c->rp[nxt].get(), c->col[nxt].get(), c->w[nxt].get()};
 
   // ---- R_t ----
@@ -590,15 +595,15 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
       DCD_TRY(pre.alloc(&c->mem, n));
       DCD_TRY_CUDA(cudaMemsetAsync(pre.get(), 0xff, n * sizeof(int32_t), s));  // -1: none
     }
-    DCD_TRY(community_sums(c, n, src_labels, mo.k.get(), a.get(), size.get()));
-    DCD_TRY(screen_batch(c, g, src_labels, mo.k.get(), a.get(), mo, rds.get(), size.get(),
+    DCD_TRY(community_sums(c, n, src_labels, mo.k->get(), a.get(), size.get()));
+    DCD_TRY(screen_batch(c, g, src_labels, mo.k->get(), a.get(), mo, rds.get(), size.get(),
                          use_pre ? pre.get() : nullptr));
     DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 9, &d->r_size, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     DCD_TRY_CUDA(cudaStreamSynchronize(s));
     r_screen = c->hscratch[9];
   }
   if (learned || collect) {
-    DCD_TRY(screen_features(c, g, src_labels, mo.k.get(), a.get(), size.get(), mo, rds.get(), &lp));
+    DCD_TRY(screen_features(c, g, src_labels, mo.k->get(), a.get(), size.get(), mo, rds.get(), &lp));
     c->feat_has_y = false;
   }
   if (mode == DCD_MODE_DELTA) {
@@ -638,15 +643,16 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
     c->n1.pkey = mo.pkey.get();
     c->n1.pdelta = mo.pdelta.get();
     c->n1.P = mo.npairs;
+    c->n1.distinct = npairs;
     c->n1.cprev = c->labels.get();
   }
   DCD_TRY(c->labels_nx.ensure(&c->mem, n));
   if (collect) DCD_TRY(c->level0.ensure(&c->mem, n));
   // the screening's community sums are those of C_{t-1} on G_t, the start of level 0
   if (c->cfg.alg == DCD_ALG_SLM)
-    DCD_TRY(run_slm(c, g, L0.get(), active, mo.k, c->labels_nx.get(), st));
+    DCD_TRY(run_slm(c, g, L0.get(), active, *mo.k, c->labels_nx.get(), st));
   else
-    DCD_TRY(run_louvain(c, g, L0.get(), active, mo.k, c->labels_nx.get(), st,
+    DCD_TRY(run_louvain(c, g, L0.get(), active, *mo.k, c->labels_nx.get(), st,
                         collect ? c->level0.get() : nullptr, per_graph, a.n ? a.get() : nullptr,
                         size.n ? size.get() : nullptr, pre.n ? pre.get() : nullptr));
   if (collect) DCD_TRY(screen_labels(c, src_labels, c->level0.get()));
@@ -661,7 +667,7 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
     DCD_TRY_CUDA(cudaMemcpyAsync(L0b.get(), src_labels, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
     memcpy(c->hgs, gs0.data(), c->G * sizeof(GraphState));
     DCD_TRY_CUDA(cudaMemcpyAsync(c->gs.get(), c->hgs, c->G * sizeof(GraphState), cudaMemcpyHostToDevice, s));
-    DCD_TRY(run_louvain(c, g, L0b.get(), rds.get(), mo.k, lab2.get(), &st2));
+    DCD_TRY(run_louvain(c, g, L0b.get(), rds.get(), *mo.k, lab2.get(), &st2));
     st->q_screen = st2.q;
     if (st->q < st2.q - 1e-3) {
       const double ql = st->q;
@@ -683,24 +689,21 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
     st->coarse0_entries = c->n1.entries;
   }
 
-  // sum_i e_{i->C(i)} of C_t on G_t, kept for the next merge: Louvain's
-  // tracked value, except after a judged learned step (its device state then
-  // holds the second run) and after SLM (which does not track it)
+  // sum_i e_{i->C(i)} of C_t on G_t and 2m, kept for the next merge; the
+  // former is Louvain's tracked value, except after a judged learned step (its
+  // device state then holds the second run) and after SLM (which does not
+  // track it)
   const bool keep_in = c->cfg.alg == DCD_ALG_LOUVAIN && !(learned && c->judge);
-  if (keep_in) {
-    DCD_TRY(c->in_next.ensure(&c->mem, c->G));
-    ::dcd::count_launch(), save_in<<<cdiv(c->G, 128), 128, 0, s>>>(c->gs.get(), c->G, c->in_next.get());
-    DCD_LAUNCH_CHECK();
-  }
+  DCD_TRY(c->in_next.ensure(&c->mem, 2 * (size_t)c->G));
+  ::dcd::count_launch(), save_in<<<cdiv(c->G, 128), 128, 0, s>>>(c->gs.get(), c->G, c->in_next.get());
+  DCD_LAUNCH_CHECK();
 
   if (finish) DCD_TRY(finish(c, user));
 
   // ---- commit ----
-  if (keep_in) {
-    std::swap(c->in_prev.p, c->in_next.p);
-    std::swap(c->in_prev.n, c->in_next.n);
-    std::swap(c->in_prev.mem, c->in_next.mem);
-  }
+  std::swap(c->in_prev.p, c->in_next.p);
+  std::swap(c->in_prev.n, c->in_next.n);
+  std::swap(c->in_prev.mem, c->in_next.mem);
   c->in_valid = keep_in;
   if (c->kc_nx_ready) {
     std::swap(c->kc_mat.p, c->kc_mat_nx.p);
@@ -759,6 +762,7 @@ int dcd_reserve(dcd_ctx* c, int64_t nnz, int64_t records) {
   DCD_TRY(c->rp[nxt].ensure(&c->mem, c->n + 1));
   DCD_TRY(c->col[nxt].ensure(&c->mem, nnz));
   DCD_TRY(c->w[nxt].ensure(&c->mem, nnz));
+  DCD_TRY(c->kdeg[nxt].ensure(&c->mem, c->n));
   DCD_TRY(grow_keep(&c->mem, c->ins, (size_t)records, (size_t)c->n_ins, c->stream));
   DCD_TRY(grow_keep(&c->mem, c->del, (size_t)records, (size_t)c->n_del, c->stream));
   DCD_TRY(c->mem.reserve(step_bytes(c, nnz, 2 * records)));

@@ -23,7 +23,7 @@ constexpr uint8_t kPairIns = 1, kPairDel = 2, kPairPresent = 4;
 
 // pool[v] = R_t[v] | (v has a pair) | (v is a neighbour of a vertex with a pair)
 __global__ void pool_mark(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                          const int64_t* __restrict__ pair_ptr, const uint8_t* __restrict__ rds,
+                          const int32_t* __restrict__ pair_ptr, const uint8_t* __restrict__ rds,
                           uint8_t* __restrict__ pool) {
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t u = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; u < n; u += nw) {
@@ -36,8 +36,8 @@ __global__ void pool_mark(int64_t n, const int64_t* __restrict__ rp, const int32
 
 __global__ void assemble(int64_t m, const int32_t* __restrict__ list, const int64_t* __restrict__ rp,
                          const int64_t* __restrict__ k, const int32_t* __restrict__ L, const int64_t* __restrict__ a,
-                         const int32_t* __restrict__ size, const int64_t* __restrict__ pair_ptr,
-                         const uint8_t* __restrict__ pflag, const int64_t* __restrict__ pw,
+                         const int32_t* __restrict__ size, const int32_t* __restrict__ pair_ptr,
+                         const uint8_t* __restrict__ pflag, const int32_t* __restrict__ pw,
                          const int64_t* __restrict__ eC, const int64_t* __restrict__ eB,
                          const int32_t* __restrict__ dB, const double* __restrict__ sB,
                          const uint8_t* __restrict__ rds, int64_t m2, float* __restrict__ X) {

@@ -1855,7 +1855,7 @@ __global__ void n1_load(const unsigned long long* __restrict__ K, int64_t cells,
 
 // The batch: pair (u, v) adds its weight change to cell (C(u), C(v)).
 template <typename VT>
-__global__ void n1_pairs(const uint64_t* __restrict__ pkey, const int64_t* __restrict__ pdelta, int64_t P,
+__global__ void n1_pairs(const uint64_t* __restrict__ pkey, const int32_t* __restrict__ pdelta, int64_t P,
                          const int32_t* __restrict__ cprev, const int32_t* __restrict__ kidx, int64_t nk,
                          VT* __restrict__ D, uint32_t* __restrict__ bad) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -2165,7 +2165,7 @@ int coarsen_dense(dcd_ctx* c, const Csr<W>& g, const int32_t* ccid, int64_t nc, 
   const int64_t U = c->hscratch[0];
   if (level0) {
     c->n1.used = delta;
-    c->n1.entries = delta ? c->n1.P + c->hscratch[1] : m0;
+    c->n1.entries = delta ? c->n1.distinct + c->hscratch[1] : m0;
     c->n1.h0_ready = keep;
     tracef("level-0 coarse graph: %s, %lld entries read, %lld communities", delta ? "delta rule" : "every entry",
            (long long)c->n1.entries, (long long)nc);

@@ -1,12 +1,18 @@
-// merge.cu -- Delta_t into G_t: batch records, radix sort by (source, sink),
-// distinct pairs, and a tiled merge of the CSR with the pairs that also produces
-// the weighted degrees d_w (Sec. III-A), 2m and sum_i e_{i->C(i)} under the
-// inherited labels.
+// merge.cu -- Delta_t into G_t: batch records sorted by (source, sink), their
+// effect on G_{t-1}, and a tiled merge of the CSR with the pairs.  The
+// weighted degrees d_w (Sec. III-A), 2m and sum_i e_{i->C(i)} of G_t follow
+// from their values on G_{t-1} and the batch's weight changes.
 //
 // The changes are stored as ordered pairs (i,j) and (j,i) (Sec. III-E).  The
 // paper only adds edges; the reading for deletions is: every delete of the
 // step acts first and removes the whole edge, then every insert adds its
 // weight (a new edge or a larger multiplicity).
+//
+// Records.  A record is one 64-bit word, sink << 32 | weight (0: a delete),
+// in its source's segment.  Records of one (source, sink) stay next to each
+// other as null pairs (no flag, no weight change) behind which the last one
+// stands for all; so the pairs of source u are [off[u], off[u+1]) with no
+// compaction, and nothing has to be counted on the host before the merge.
 #include "prims.cuh"
 #include "state.cuh"
 
@@ -16,6 +22,10 @@ namespace {
 
 constexpr uint8_t kPairIns = 1, kPairDel = 2, kPairPresent = 4, kPairAdded = 8, kPairRemoved = 16;
 
+__device__ __forceinline__ bool record_ok(const dcd_edge& e, int64_t n, bool is_ins) {
+  return e.u >= 0 && e.v >= 0 && e.u < n && e.v < n && e.u != e.v && (!is_ins || e.w > 0);
+}
+
 __global__ void validate_records(const dcd_edge* __restrict__ ins, int64_t n_ins,
                                  const dcd_edge* __restrict__ del, int64_t n_del, int64_t n,
                                  uint32_t* __restrict__ err) {
@@ -23,483 +33,618 @@ __global__ void validate_records(const dcd_edge* __restrict__ ins, int64_t n_ins
   bool bad = false;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot;
        i += (int64_t)gridDim.x * blockDim.x) {
-    dcd_edge e = i < n_ins ? ins[i] : del[i - n_ins];
-    bad |= e.u < 0 || e.v < 0 || e.u >= n || e.v >= n || e.u == e.v || (i < n_ins && e.w <= 0);
+    const dcd_edge e = i < n_ins ? ins[i] : del[i - n_ins];
+    bad |= !record_ok(e, n, i < n_ins);
   }
   if (__any_sync(0xffffffffu, bad) && lane_id() == 0) atomicOr(err, kErrBadRecord);
 }
 
-// Record r: inserts first (2i, 2i+1 = both orientations of insert i), then
-// deletes.  key = source << 32 | sink, value = r.
-__global__ void make_records(const dcd_edge* __restrict__ ins, int64_t n_ins, const dcd_edge* __restrict__ del,
-                             int64_t n_del, uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
-  int64_t tot = n_ins + n_del;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    dcd_edge e = i < n_ins ? ins[i] : del[i - n_ins];
-    uint64_t a = (uint64_t)(uint32_t)e.u, b = (uint64_t)(uint32_t)e.v;
-    keys[2 * i] = a << 32 | b;
-    keys[2 * i + 1] = b << 32 | a;
-    vals[2 * i] = (uint32_t)(2 * i);
-    vals[2 * i + 1] = (uint32_t)(2 * i + 1);
-  }
-}
-
-// Records sorted by source with a counting sort, then each source's segment
-// by sink with a rank sort (a record's place = the records of its segment
-// with a smaller key, or an equal key and a smaller index).  Used when no
-// source holds more than kRankSortMax records (the rank sort costs the square
-// of a segment); otherwise the batch takes the LSD radix sort.
-constexpr int64_t kRankSortMax = 4096;
-
+// Records per source, and each record's place in its source's segment (the
+// atomic's return value, so the scatter needs no atomic of its own).  Batches
+// staged from device memory are first checked here: a bad record is reported
+// and takes no place.
 __global__ void rec_count(const dcd_edge* __restrict__ ins, int64_t n_ins, const dcd_edge* __restrict__ del,
-                          int64_t n_del, int32_t* __restrict__ cnt) {
+                          int64_t n_del, int64_t n, int32_t* __restrict__ cnt, int2* __restrict__ rank,
+                          uint32_t* __restrict__ err) {
   const int64_t tot = n_ins + n_del;
+  bool bad = false;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot; i += (int64_t)gridDim.x * blockDim.x) {
     const dcd_edge e = i < n_ins ? ins[i] : del[i - n_ins];
-    atomicAdd(&cnt[e.u], 1);
-    atomicAdd(&cnt[e.v], 1);
+    if (!record_ok(e, n, i < n_ins)) {
+      bad = true;
+      continue;
+    }
+    int2 r;
+    r.x = atomicAdd(&cnt[e.u], 1);
+    r.y = atomicAdd(&cnt[e.v], 1);
+    rank[i] = r;
   }
-}
-
-__global__ void rec_maxseg(const int32_t* __restrict__ cnt, int64_t n, int32_t* __restrict__ mx) {
-  int32_t m = 0;
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
-    m = cnt[v] > m ? cnt[v] : m;
-  m = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)m);
-  if (lane_id() == 0 && m) atomicMax(mx, m);
+  if (bad) atomicOr(err, kErrBadRecord);
 }
 
 __global__ void rec_scatter(const dcd_edge* __restrict__ ins, int64_t n_ins, const dcd_edge* __restrict__ del,
-                            int64_t n_del, const int32_t* __restrict__ off, int32_t* __restrict__ cur,
-                            uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+                            int64_t n_del, int64_t n, const int32_t* __restrict__ off, const int2* __restrict__ rank,
+                            uint64_t* __restrict__ rec) {
   const int64_t tot = n_ins + n_del;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot; i += (int64_t)gridDim.x * blockDim.x) {
     const dcd_edge e = i < n_ins ? ins[i] : del[i - n_ins];
-    const uint64_t a = (uint64_t)(uint32_t)e.u, b = (uint64_t)(uint32_t)e.v;
-    const int32_t pa = off[e.u] + atomicAdd(&cur[e.u], 1);
-    keys[pa] = a << 32 | b;
-    vals[pa] = (uint32_t)(2 * i);
-    const int32_t pb = off[e.v] + atomicAdd(&cur[e.v], 1);
-    keys[pb] = b << 32 | a;
-    vals[pb] = (uint32_t)(2 * i + 1);
+    if (!record_ok(e, n, i < n_ins)) continue;
+    const int2 r = rank[i];
+    const uint64_t w = i < n_ins ? (uint32_t)e.w : 0u;
+    rec[off[e.u] + r.x] = (uint64_t)(uint32_t)e.v << 32 | w;
+    rec[off[e.v] + r.y] = (uint64_t)(uint32_t)e.u << 32 | w;
   }
 }
 
-// Segments longer than kRankSmall are sorted by rec_bitonic instead (a CTA
-// each, a bitonic network in shared memory).
-constexpr int kRankSmall = 64;
+// ---- pairs and their effect on G_{t-1} ----
 
-__global__ void rec_rank(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin, int64_t R,
-                         const int32_t* __restrict__ off, uint64_t* __restrict__ kout, uint32_t* __restrict__ vout) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < R; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint64_t k = kin[i];
-    const int32_t src = (int32_t)(k >> 32);
-    const int64_t a = off[src], b = off[src + 1];
-    if (b - a > kRankSmall) continue;
-    int64_t r = 0;
-    for (int64_t j = a; j < b; j++) {
-      const uint64_t kj = kin[j];
-      r += (kj < k || (kj == k && j < i)) ? 1 : 0;
+struct PairView {
+  const int32_t* off;  // n + 1: records (pairs) of source u are [off[u], off[u+1])
+  const int64_t* rp;   // G_{t-1}
+  const int32_t* col;
+  const int32_t* w;
+  const int32_t* lab0;  // C_{t-1} when sum e_{i->C(i)} is tracked, else NULL
+  const int32_t* gid;
+  uint64_t* pkey;   // source << 32 | sink
+  int32_t* pw;      // summed insert weight
+  uint8_t* pflag;
+  int32_t* pdelta;  // weight in G_t minus weight in G_{t-1}
+  int64_t* epos;    // first entry of G_{t-1} not before the pair (CSR order)
+  int32_t* net;     // +1 adds an entry, -1 removes one
+  GraphState* gs;   // m2 and in_cur receive the changes
+  int64_t* npairs;  // distinct pairs
+  uint32_t* err;
+};
+
+// What one record contributes to the sums of its CTA.
+struct PairSum {
+  long long m2 = 0, in = 0;
+  int heads = 0;
+};
+
+// Pair (u, v) at place p: W the summed insert weight, e its place in row u
+// (first entry with sink >= v), head: the record that stands for its pair.
+__device__ __forceinline__ int32_t put_pair(const PairView& o, int64_t p, int32_t u, int32_t v, int64_t W, bool isins,
+                                            bool isdel, bool head, int64_t e, bool present, PairSum& acc) {
+  uint8_t f = 0;
+  int64_t dlt = 0;
+  int32_t net = 0;
+  if (head) {
+    // deletes remove the whole edge first, then inserts add their weight
+    const int64_t w_old = present ? (int64_t)o.w[e] : 0;
+    const int64_t w_new = (present && !isdel ? w_old : 0) + W;
+    if (isins && w_new > INT32_MAX) atomicOr(o.err, kErrOverflow);
+    const bool add = isins && !present, rem = !isins && isdel && present;
+    dlt = w_new - w_old;
+    net = add ? 1 : rem ? -1 : 0;
+    f = (isins ? kPairIns : 0) | (isdel ? kPairDel : 0) | (present ? kPairPresent : 0) | (add ? kPairAdded : 0) |
+        (rem ? kPairRemoved : 0);
+    acc.m2 += dlt;
+    if (o.lab0 && dlt != 0 && o.lab0[u] == o.lab0[v]) acc.in += dlt;
+    acc.heads++;
+  }
+  o.pkey[p] = (uint64_t)(uint32_t)u << 32 | (uint32_t)v;
+  o.pw[p] = (int32_t)W;
+  o.pflag[p] = f;
+  o.pdelta[p] = (int32_t)dlt;
+  o.epos[p] = e;
+  o.net[p] = net;
+  return (int32_t)dlt;
+}
+
+// First entry of [lo, hi) with a[x] >= v.
+template <typename I>
+__device__ __forceinline__ I lower_bound_col(const int32_t* a, I lo, I hi, int32_t v) {
+  while (lo < hi) {
+    const I mid = (lo + hi) >> 1;
+    if (a[mid] < v) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
+// The CTA's sums into the graph's (every thread of the CTA calls it).  uni:
+// all records of the CTA belong to graph g.
+template <int NT>
+__device__ __forceinline__ void pair_sums_out(const PairView& o, int g, const PairSum& acc) {
+  __shared__ unsigned long long red[3][NT / 32];
+  const unsigned long long m2 = warp_sum((unsigned long long)acc.m2), in = warp_sum((unsigned long long)acc.in);
+  const unsigned heads = __reduce_add_sync(0xffffffffu, (unsigned)acc.heads);
+  const int wid = threadIdx.x >> 5;
+  if (lane_id() == 0) {
+    red[0][wid] = m2;
+    red[1][wid] = in;
+    red[2][wid] = heads;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long a = 0, b = 0, h = 0;
+    for (int x = 0; x < NT / 32; x++) {
+      a += red[0][x];
+      b += red[1][x];
+      h += red[2][x];
     }
-    kout[a + r] = k;
-    vout[a + r] = vin[i];
+    if (a) atomicAdd((unsigned long long*)&o.gs[g].m2, a);
+    if (b) atomicAdd((unsigned long long*)&o.gs[g].in_cur, b);
+    if (h) atomicAdd((unsigned long long*)o.npairs, h);
+  }
+  __syncthreads();
+}
+
+// A record's sums straight into its graph's (CTAs whose sources belong to
+// several graphs).
+__device__ __forceinline__ void pair_sums_add(const PairView& o, int g, PairSum& acc) {
+  if (acc.m2) atomicAdd((unsigned long long*)&o.gs[g].m2, (unsigned long long)acc.m2);
+  if (acc.in) atomicAdd((unsigned long long*)&o.gs[g].in_cur, (unsigned long long)acc.in);
+  acc.m2 = acc.in = 0;
+}
+
+// Segments of at most kSegSmall records are ranked by pair_tile; of at most
+// kSegMid by a CTA each in shared memory (rank); of at most kSegLarge by a
+// CTA each with a bitonic network; longer ones by a CTA's radix sort in
+// global memory.
+constexpr int kSegSmall = 64, kSegMid = 512, kSegLarge = 4096;
+
+// A CTA takes kPairSrc consecutive sources: their records (a counting sort
+// put them next to each other) and, when the batch is dense enough to pay for
+// it, the columns of their rows are staged in shared memory with coalesced
+// loads; a thread then ranks one record in its segment, sums the weights of
+// equal sinks, and looks its sink up in the row.  The row search is what
+// bounds this step: in global memory each of its 5-8 probes costs a sector a
+// lane, in shared memory a few cycles.  12.4 M records on 73 M entries: 556 us
+// for rank, sums, search and degrees, where separate kernels for them took
+// 196 (rank) + 175 (sums) + 683 us (search).  Sources without records only get
+// their k.
+constexpr int kPairSrc = 64;
+constexpr int kPairThreads = 128;
+constexpr int kPairRecs = 1280;
+constexpr int kPairCols = 3072;
+
+__global__ void __launch_bounds__(kPairThreads) pair_tile(PairView o, int64_t n, const uint64_t* __restrict__ rec,
+                                                          const int64_t* __restrict__ k_old,
+                                                          int64_t* __restrict__ k_new, int32_t* __restrict__ big,
+                                                          int32_t* __restrict__ big_cnt) {
+  __shared__ uint64_t s_rec[kPairRecs];
+  __shared__ int32_t s_col[kPairCols];
+  __shared__ int32_t s_off[kPairSrc + 1];
+  __shared__ int64_t s_rp[kPairSrc + 1];
+  __shared__ unsigned long long s_dk[kPairSrc];
+  const int tid = threadIdx.x;
+  const int64_t v0 = (int64_t)blockIdx.x * kPairSrc;
+  const int ns = (int)(n - v0 < kPairSrc ? n - v0 : kPairSrc);
+  for (int x = tid; x <= ns; x += kPairThreads) s_off[x] = o.off[v0 + x];
+  if (tid < kPairSrc) s_dk[tid] = 0;
+  __syncthreads();
+  const int32_t r0 = s_off[0];
+  const int nrec = s_off[ns] - r0;
+  if (nrec > 0) {
+    for (int x = tid; x <= ns; x += kPairThreads) s_rp[x] = o.rp[v0 + x];
+    __syncthreads();
+    const int64_t c0 = s_rp[0], ncol = s_rp[ns] - c0;
+    const bool srec = nrec <= kPairRecs;
+    // a search costs a record about log2(row) probes of a sector each;
+    // staging costs an eighth of a sector an entry
+    const bool scol = ncol <= kPairCols && ncol <= 32 * (int64_t)nrec;
+    if (srec)
+      for (int x = tid; x < nrec; x += kPairThreads) s_rec[x] = rec[r0 + x];
+    if (scol)
+      for (int x = tid; x < (int)ncol; x += kPairThreads) s_col[x] = ld_stream(o.col + c0 + x);
+    if (tid < ns) {  // longer segments: a CTA each, later
+      const int len = s_off[tid + 1] - s_off[tid];
+      if (len > kSegSmall) {
+        const int c = len <= kSegMid ? 0 : len <= kSegLarge ? 1 : 2;
+        big[(int64_t)c * n + atomicAdd(&big_cnt[c], 1)] = (int32_t)(v0 + tid);
+      }
+    }
+    __syncthreads();
+    const int g0 = graph_of(o.gid, v0);
+    const bool uni = !o.gid || g0 == o.gid[v0 + ns - 1];
+    PairSum acc;
+    for (int x = tid; x < nrec; x += kPairThreads) {
+      int lo = 0, hi = ns - 1;  // last source whose segment starts at or before x
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (s_off[mid] - r0 <= x) lo = mid; else hi = mid - 1;
+      }
+      const int a = s_off[lo] - r0, b = s_off[lo + 1] - r0;
+      if (b - a > kSegSmall) continue;
+      const uint64_t me = srec ? s_rec[x] : rec[r0 + x];
+      const uint32_t v = (uint32_t)(me >> 32);
+      int rank = 0;
+      int64_t W = 0;
+      bool isdel = false, head = true;
+      for (int j = a; j < b; j++) {
+        const uint64_t kj = srec ? s_rec[j] : rec[r0 + j];
+        const bool before = kj < me || (kj == me && j < x);
+        rank += before ? 1 : 0;
+        if ((uint32_t)(kj >> 32) == v) {
+          W += (int64_t)(uint32_t)kj;
+          isdel |= (uint32_t)kj == 0;
+          head &= before || j == x;
+        }
+      }
+      int64_t e;
+      bool present;
+      if (scol) {
+        const int q1 = (int)(s_rp[lo + 1] - c0);
+        const int q = lower_bound_col<int>(s_col, (int)(s_rp[lo] - c0), q1, (int32_t)v);
+        present = q < q1 && s_col[q] == (int32_t)v;
+        e = c0 + q;
+      } else {
+        const int64_t e1 = s_rp[lo + 1];
+        e = lower_bound_col<int64_t>(o.col, s_rp[lo], e1, (int32_t)v);
+        present = e < e1 && o.col[e] == (int32_t)v;
+      }
+      const int32_t u = (int32_t)(v0 + lo);
+      const int32_t d = put_pair(o, (int64_t)r0 + a + rank, u, (int32_t)v, W, W > 0, isdel, head, e, present, acc);
+      if (d) atomicAdd(&s_dk[lo], (unsigned long long)(long long)d);
+      if (!uni) pair_sums_add(o, graph_of(o.gid, u), acc);
+    }
+    __syncthreads();
+    pair_sums_out<kPairThreads>(o, g0, acc);
+  }
+  if (tid < ns) k_new[v0 + tid] = k_old[v0 + tid] + (int64_t)s_dk[tid];
+}
+
+// One pair of a long segment whose sorted neighbourhood the caller knows; the
+// row is searched in global memory.
+__device__ __forceinline__ int32_t put_searched(const PairView& o, int64_t p, int32_t u, uint32_t v, int64_t W,
+                                                bool isdel, bool head, PairSum& acc) {
+  const int64_t e1 = o.rp[u + 1];
+  const int64_t e = lower_bound_col<int64_t>(o.col, o.rp[u], e1, (int32_t)v);
+  const bool present = e < e1 && o.col[e] == (int32_t)v;
+  return put_pair(o, p, u, (int32_t)v, W, W > 0, isdel, head, e, present, acc);
+}
+
+// k and the graph's sums of one long segment.
+template <int NT>
+__device__ __forceinline__ void segment_out(const PairView& o, int32_t u, const PairSum& acc, int64_t* k_new) {
+  const unsigned long long dk = warp_sum((unsigned long long)acc.m2);
+  if (lane_id() == 0 && dk) atomicAdd((unsigned long long*)&k_new[u], dk);
+  pair_sums_out<NT>(o, graph_of(o.gid, u), acc);
+}
+
+// Segments of kSegSmall + 1 .. kSegMid records: a CTA each, ranked in shared
+// memory (every thread reads the same word at the same time).
+constexpr int kMidThreads = 128;
+__global__ void __launch_bounds__(kMidThreads) pair_mid(PairView o, const uint64_t* __restrict__ rec,
+                                                        const int32_t* __restrict__ list,
+                                                        const int32_t* __restrict__ cnt, int64_t* __restrict__ k_new) {
+  __shared__ uint64_t s[kSegMid];
+  const int nl = *cnt, tid = threadIdx.x;
+  for (int i = blockIdx.x; i < nl; i += gridDim.x) {
+    const int32_t u = list[i];
+    const int32_t a = o.off[u];
+    const int len = o.off[u + 1] - a;
+    for (int x = tid; x < len; x += kMidThreads) s[x] = rec[a + x];
+    __syncthreads();
+    PairSum acc;
+    for (int x = tid; x < len; x += kMidThreads) {
+      const uint64_t me = s[x];
+      const uint32_t v = (uint32_t)(me >> 32);
+      int rank = 0;
+      int64_t W = 0;
+      bool isdel = false, head = true;
+      for (int j = 0; j < len; j++) {
+        const uint64_t kj = s[j];
+        const bool before = kj < me || (kj == me && j < x);
+        rank += before ? 1 : 0;
+        if ((uint32_t)(kj >> 32) == v) {
+          W += (int64_t)(uint32_t)kj;
+          isdel |= (uint32_t)kj == 0;
+          head &= before || j == x;
+        }
+      }
+      put_searched(o, (int64_t)a + rank, u, v, W, isdel, head, acc);
+    }
+    segment_out<kMidThreads>(o, u, acc, k_new);
   }
 }
 
-// sources whose segment is longer than kRankSmall
-__global__ void rec_big_list(const int32_t* __restrict__ off, int64_t n, int32_t* __restrict__ list,
-                             int32_t* __restrict__ cnt) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (blockIdx.x * (int64_t)blockDim.x) + (threadIdx.x & ~31); base < n; base += stride) {
-    const int64_t v = base + lane_id();
-    const bool big = v < n && off[v + 1] - off[v] > kRankSmall;
-    const unsigned bal = __ballot_sync(0xffffffffu, big);
-    if (!bal) continue;
-    int32_t slot = 0;
-    if (lane_id() == 0) slot = atomicAdd(cnt, __popc(bal));
-    slot = __shfl_sync(0xffffffffu, slot, 0);
-    if (big) list[slot + __popc(bal & lanemask_lt())] = (int32_t)v;
+// The pairs of a sorted segment s[0 .. len) of source u at place a.
+template <typename P>
+__device__ __forceinline__ void put_sorted(const PairView& o, int32_t u, int64_t a, int len, const P* s, int tid,
+                                           int NT, PairSum& acc) {
+  for (int x = tid; x < len; x += NT) {
+    const uint32_t v = (uint32_t)(s[x] >> 32);
+    const bool head = x + 1 == len || (uint32_t)(s[x + 1] >> 32) != v;
+    int64_t W = 0;
+    bool isdel = false;
+    if (head)
+      for (int j = x; j >= 0 && (uint32_t)(s[j] >> 32) == v; j--) {
+        W += (int64_t)(uint32_t)s[j];
+        isdel |= (uint32_t)s[j] == 0;
+      }
+    put_searched(o, a + x, u, v, W, isdel, head, acc);
   }
 }
 
-// One CTA per long segment (at most kRankSortMax records): a bitonic sort in
-// shared memory, padded to a power of two with the largest key.
-__global__ void __launch_bounds__(1024) rec_bitonic(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-                                                    const int32_t* __restrict__ off, const int32_t* __restrict__ list,
-                                                    const int32_t* __restrict__ cnt, uint64_t* __restrict__ kout,
-                                                    uint32_t* __restrict__ vout) {
-  __shared__ uint64_t sk[kRankSortMax];
-  __shared__ uint32_t sv[kRankSortMax];
-  const int64_t nl = *cnt;
-  for (int64_t i = blockIdx.x; i < nl; i += gridDim.x) {
-    const int32_t v = list[i];
-    const int64_t a = off[v];
-    const int len = (int)(off[v + 1] - a);
+// Segments of kSegMid + 1 .. kSegLarge records: a CTA each, a bitonic network
+// in shared memory, padded to a power of two with the largest key.
+constexpr int kLargeThreads = 512;
+__global__ void __launch_bounds__(kLargeThreads) pair_large(PairView o, const uint64_t* __restrict__ rec,
+                                                            const int32_t* __restrict__ list,
+                                                            const int32_t* __restrict__ cnt,
+                                                            int64_t* __restrict__ k_new) {
+  __shared__ uint64_t s[kSegLarge];
+  const int nl = *cnt, tid = threadIdx.x;
+  for (int i = blockIdx.x; i < nl; i += gridDim.x) {
+    const int32_t u = list[i];
+    const int32_t a = o.off[u];
+    const int len = o.off[u + 1] - a;
     int P = 1;
     while (P < len) P <<= 1;
-    for (int x = threadIdx.x; x < P; x += blockDim.x) {
-      sk[x] = x < len ? kin[a + x] : ~0ull;
-      sv[x] = x < len ? vin[a + x] : 0u;
-    }
+    for (int x = tid; x < P; x += kLargeThreads) s[x] = x < len ? rec[a + x] : ~0ull;
     __syncthreads();
     for (int k = 2; k <= P; k <<= 1)
       for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int x = threadIdx.x; x < P; x += blockDim.x) {
-          const int y = x ^ j;
-          if (y > x) {
-            const bool up = (x & k) == 0;
-            const uint64_t kx = sk[x], ky = sk[y];
-            if ((kx > ky) == up) {
-              sk[x] = ky;
-              sk[y] = kx;
-              const uint32_t t = sv[x];
-              sv[x] = sv[y];
-              sv[y] = t;
-            }
+        for (int q = tid; q < P / 2; q += kLargeThreads) {
+          const int x = ((q & ~(j - 1)) << 1) | (q & (j - 1)), y = x | j;  // the q-th pair at distance j
+          const uint64_t kx = s[x], ky = s[y];
+          if ((kx > ky) == ((x & k) == 0)) {
+            s[x] = ky;
+            s[y] = kx;
           }
         }
         __syncthreads();
       }
-    for (int x = threadIdx.x; x < len; x += blockDim.x) {
-      kout[a + x] = sk[x];
-      vout[a + x] = sv[x];
-    }
-    __syncthreads();
+    PairSum acc;
+    put_sorted(o, u, a, len, s, tid, kLargeThreads, acc);
+    segment_out<kLargeThreads>(o, u, acc, k_new);
   }
 }
 
-__global__ void run_heads(const uint64_t* __restrict__ keys, int64_t R, int32_t* __restrict__ head) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < R; e += (int64_t)gridDim.x * blockDim.x)
-    head[e] = (e == 0 || keys[e] != keys[e - 1]) ? 1 : 0;
-}
-
-// One thread per run of equal keys: sum of insert weights, delete flag.
-__global__ void reduce_pairs(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ vals, int64_t R,
-                             const int32_t* __restrict__ head, const int32_t* __restrict__ pid,
-                             const dcd_edge* __restrict__ ins, int64_t n_ins, uint64_t* __restrict__ pkey,
-                             int64_t* __restrict__ pw, uint8_t* __restrict__ pflag) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < R; e += (int64_t)gridDim.x * blockDim.x) {
-    if (!head[e]) continue;
-    uint64_t k = keys[e];
-    int64_t W = 0;
-    uint8_t f = 0;
-    for (int64_t x = e; x < R && keys[x] == k; x++) {
-      uint32_t r = vals[x];
-      if ((int64_t)r < 2 * n_ins) {
-        W += ins[r >> 1].w;
-        f |= kPairIns;
-      } else {
-        f |= kPairDel;
+// Longer segments: a CTA each, a stable LSD radix sort by sink in global
+// memory (8-bit digits; x and y swap per digit), then as above.
+constexpr int kHugeThreads = 512;
+__global__ void __launch_bounds__(kHugeThreads) pair_huge(PairView o, uint64_t* rec, uint64_t* tmp,
+                                                          const int32_t* __restrict__ list,
+                                                          const int32_t* __restrict__ cnt, int bits,
+                                                          int64_t* __restrict__ k_new) {
+  constexpr int NW = kHugeThreads / 32;
+  __shared__ uint32_t base[256], wcnt[NW][256];
+  const int nl = *cnt, tid = threadIdx.x, wid = tid >> 5;
+  for (int i = blockIdx.x; i < nl; i += gridDim.x) {
+    const int32_t u = list[i];
+    const int32_t a = o.off[u];
+    const int len = o.off[u + 1] - a;
+    uint64_t *x = rec + a, *y = tmp + a;
+    for (int b = 32; b < 32 + bits; b += 8) {
+      if (tid < 256) base[tid] = 0;
+      for (int q = tid; q < NW * 256; q += kHugeThreads) (&wcnt[0][0])[q] = 0;
+      __syncthreads();
+      for (int e = tid; e < len; e += kHugeThreads) atomicAdd(&base[(uint32_t)(x[e] >> b) & 255u], 1u);
+      __syncthreads();
+      if (wid == 0) {  // exclusive scan of the 256 digit counts
+        uint32_t run = 0;
+        for (int q = 0; q < 8; q++) {
+          const uint32_t c = base[q * 32 + lane_id()];
+          const uint32_t inc = warp_incl_scan(c);
+          base[q * 32 + lane_id()] = run + inc - c;
+          run += __shfl_sync(0xffffffffu, inc, 31);
+        }
       }
-    }
-    int32_t p = pid[e];
-    pkey[p] = k;
-    pw[p] = W;
-    pflag[p] = f;
-  }
-}
-
-__device__ __forceinline__ int64_t lower_bound_i32(const int32_t* __restrict__ a, int64_t lo, int64_t hi, int32_t x) {
-  while (lo < hi) {
-    int64_t mid = (lo + hi) >> 1;
-    if (a[mid] < x) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
-// Per pair: was the edge in G_{t-1}; does the merge add or remove a row entry.
-// With lab0 (C_{t-1}) given, also the change the pair makes to
-// sum_i e_{i->C(i)} under C_{t-1}: its new weight minus its old one when both
-// ends share a community, added into in_delta[graph].
-__global__ void pair_status(const uint64_t* __restrict__ pkey, const int64_t* __restrict__ pw,
-                            uint8_t* __restrict__ pflag, int64_t P, const int64_t* __restrict__ rp,
-                            const int32_t* __restrict__ col, const int32_t* __restrict__ w,
-                            int32_t* __restrict__ added, int32_t* __restrict__ removed,
-                            int64_t* __restrict__ src_cnt, uint32_t* __restrict__ err,
-                            const int32_t* __restrict__ lab0, const int32_t* __restrict__ gid,
-                            int64_t* __restrict__ in_delta, int64_t* __restrict__ pdelta) {
-  // warp-uniform trip count: the lanes of a warp sum their in_delta changes
-  // per graph before one lane adds them (most pairs of a step add into the
-  // same word)
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t p0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31u); p0 < P; p0 += stride) {
-    const int64_t p = p0 + lane_id();
-    int64_t dlt = 0;
-    int32_t graph = 0, src = -1;
-    if (p < P) {
-      uint64_t k = pkey[p];
-      int32_t u = (int32_t)(k >> 32), v = (int32_t)(k & 0xffffffffu);
-      int64_t b = rp[u], e = rp[u + 1];
-      int64_t pos = lower_bound_i32(col, b, e, v);
-      bool present = pos < e && col[pos] == v;
-      uint8_t f = pflag[p];
-      bool isins = f & kPairIns, isdel = f & kPairDel;
-      bool add = isins && !present;
-      bool rem = !isins && isdel && present;
-      if (isins) {
-        int64_t nw = (present && !isdel) ? (int64_t)w[pos] + pw[p] : pw[p];
-        if (nw > INT32_MAX) atomicOr(err, kErrOverflow);
+      __syncthreads();
+      for (int e0 = 0; e0 < len; e0 += kHugeThreads) {
+        const int e = e0 + tid;
+        const bool ok = e < len;
+        const uint64_t key = ok ? x[e] : 0;
+        const uint32_t d = ok ? (uint32_t)(key >> b) & 255u : 256u;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const int rk = __popc(peers & lanemask_lt());
+        if (ok && rk == 0) wcnt[wid][d] = __popc(peers);
+        __syncthreads();
+        if (tid < 256) {  // thread t owns digit t: the warps' places, then the next round's base
+          uint32_t run = base[tid];
+          for (int q = 0; q < NW; q++) {
+            const uint32_t c = wcnt[q][tid];
+            wcnt[q][tid] = run;
+            run += c;
+          }
+          base[tid] = run;
+        }
+        __syncthreads();
+        if (ok) y[wcnt[wid][d] + rk] = key;
+        __syncthreads();
+        for (int q = tid; q < NW * 256; q += kHugeThreads) (&wcnt[0][0])[q] = 0;
+        __syncthreads();
       }
-      // deletes remove the whole edge first, then inserts add their weight
-      const int64_t w_old = present ? (int64_t)w[pos] : 0;
-      const int64_t w_new = ((present && !isdel) ? w_old : 0) + (isins ? pw[p] : 0);
-      pdelta[p] = w_new - w_old;
-      if (lab0 && lab0[u] == lab0[v]) {
-        dlt = w_new - w_old;
-        graph = graph_of(gid, u);
-      }
-      f |= (present ? kPairPresent : 0) | (add ? kPairAdded : 0) | (rem ? kPairRemoved : 0);
-      pflag[p] = f;
-      added[p] = add;
-      removed[p] = rem;
-      src = u;
+      uint64_t* t = x;
+      x = y;
+      y = t;
     }
-    {
-      // pairs are sorted by source: one add per run of equal sources
-      const unsigned same = __match_any_sync(0xffffffffu, src);
-      if (src >= 0 && (int)(__ffs(same) - 1) == (int)lane_id())
-        atomicAdd((unsigned long long*)&src_cnt[src], (unsigned long long)__popc(same));
-    }
-    if (lab0) {
-      const unsigned peers = __match_any_sync(0xffffffffu, graph);
-      // two's-complement sum of the peers' changes, 16 bits at a time
-      const unsigned long long x = (unsigned long long)dlt;
-      unsigned long long sum = 0;
-#pragma unroll
-      for (int q = 0; q < 4; q++)
-        sum += (unsigned long long)__reduce_add_sync(peers, (unsigned)(x >> (16 * q)) & 0xffffu) << (16 * q);
-      if (sum != 0 && (int)(__ffs(peers) - 1) == (int)lane_id())
-        atomicAdd((unsigned long long*)&in_delta[graph], sum);
-    }
+    PairSum acc;
+    put_sorted(o, u, a, len, x, tid, kHugeThreads, acc);
+    segment_out<kHugeThreads>(o, u, acc, k_new);
   }
 }
 
-// sum_i e_{i->C(i)} under C_{t-1} on G_t from its value on G_{t-1} (kept by
-// the previous update) and the batch's change.
-__global__ void seed_in(GraphState* __restrict__ gs, int G, const int64_t* __restrict__ in_prev,
-                        const int64_t* __restrict__ in_delta) {
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x)
-    gs[g].in_cur += in_prev[g] + in_delta[g];
+// sum_i e_{i->C(i)} and 2m of G_{t-1} per graph (kept by the previous update:
+// prev[g], prev[G + g]); with_in: the former is tracked through the merge.
+__global__ void seed_sums(GraphState* __restrict__ gs, int G, const int64_t* __restrict__ prev, int with_in) {
+  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
+    gs[g].in_cur += with_in ? prev[g] : 0;
+    gs[g].m2 += prev[G + g];
+  }
+}
+
+// k of a graph whose degrees no update of this context has computed (a
+// loaded checkpoint), and its 2m into *m2.
+__global__ void row_degrees(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ w,
+                            int64_t* __restrict__ k, unsigned long long* __restrict__ m2) {
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  long long tot = 0;
+  for (int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; v < n; v += nw) {
+    long long x = 0;
+    for (int64_t e = rp[v] + lane_id(); e < rp[v + 1]; e += 32) x += w[e];
+    x = warp_sum(x);
+    if (lane_id() == 0) k[v] = x;
+    tot += x;
+  }
+  if (lane_id() == 0 && tot) atomicAdd(m2, (unsigned long long)tot);
+}
+
+// sum_i e_{i->C(i)} under labels L over every entry (when no update kept it:
+// labels set by the caller, a loaded checkpoint).
+__global__ void in_weight(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
+                          const int32_t* __restrict__ w, const int32_t* __restrict__ L,
+                          const int32_t* __restrict__ gid, GraphState* __restrict__ gs) {
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  int cur = 0;
+  unsigned long long acc = 0;
+  for (int64_t u = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; u < n; u += nw) {
+    const int g = graph_of(gid, u);
+    if (g != cur) {
+      acc = warp_sum(acc);
+      if (lane_id() == 0 && acc) atomicAdd((unsigned long long*)&gs[cur].in_cur, acc);
+      acc = 0;
+      cur = g;
+    }
+    const int32_t Lu = L[u];
+    const int64_t e1 = rp[u + 1];
+    for (int64_t e = rp[u] + lane_id(); e < e1; e += 32) {
+      const int32_t x = ld_stream(w + e);
+      if (L[ld_stream(col + e)] == Lu) acc += (unsigned long long)x;
+    }
+  }
+  acc = warp_sum(acc);
+  if (lane_id() == 0 && acc) atomicAdd((unsigned long long*)&gs[cur].in_cur, acc);
 }
 
 // ---- tiled merge ----
 //
-// The merge as one merge of two sorted sequences: the old entries (key =
-// source << 32 | sink, in CSR order) and the pairs (same keys), an entry
-// before a pair of equal key.  With A(q), R(q) the added and removed pairs
-// among the first q, an old entry e lands at e + A(q) - R(q) (q: pairs of
-// smaller key) and an added pair q at i + A(q) - R(q) (i: old entries of
-// smaller key), so rows need not be merged one by one: the merged sequence is
-// cut into tiles of kMergeTile items, a CTA each, whatever rows they cover.
+// The merge as one merge of two sorted sequences: the old entries, in CSR
+// order, and the pairs, where pair q comes before entry epos[q].  Pair q is
+// item q + epos[q] of the merged sequence.  With S(q) the entries added minus
+// removed by the pairs before q, an old entry e lands at e + S over the pairs
+// with epos <= e, and an added pair q at epos[q] + S(q); neither depends on
+// the row, so the sequence is cut into tiles of kMergeTile items whatever
+// rows they cover.
 constexpr int kMergeTile = 2048;
 constexpr int kMergeThreads = 256;
-constexpr int kMergeRows = 1024;  // row starts staged per tile (more: searched in global memory)
+constexpr int kMergeItems = kMergeTile / kMergeThreads;
 
-// Row u's start in the new CSR: rp_o[u] + A(pair_ptr[u]) - R(pair_ptr[u]).
-__global__ void new_rows(const int64_t* __restrict__ rp_o, const int64_t* __restrict__ pair_ptr,
-                         const int32_t* __restrict__ pA, const int32_t* __restrict__ pR, int64_t n,
-                         int64_t* __restrict__ rp_n) {
-  for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u <= n; u += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t p = pair_ptr[u];
-    rp_n[u] = rp_o[u] + pA[p] - pR[p];
-  }
+// Row u's start in the new CSR.
+__global__ void new_rows(const int64_t* __restrict__ rp_o, const int32_t* __restrict__ off,
+                         const int32_t* __restrict__ S, int64_t n, int64_t* __restrict__ rp_n) {
+  for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u <= n; u += (int64_t)gridDim.x * blockDim.x)
+    rp_n[u] = rp_o[u] + S[off[u]];
 }
 
-// Tile t starts at merged item d = t * kMergeTile: se[t] old entries and sq[t]
-// pairs come before it, su[t] is the row of item d.  Rows are found on
-// W(u) = rp_o[u] + pair_ptr[u] (the merged items of rows before u), then
-// the split inside the row by a merge-path search over its sinks.
-__global__ void merge_split(int64_t n, const int64_t* __restrict__ rp_o, const int32_t* __restrict__ col_o,
-                            const int64_t* __restrict__ pp, const uint64_t* __restrict__ pkey, int64_t nt,
-                            int64_t total, int64_t* __restrict__ se, int64_t* __restrict__ sq,
-                            int64_t* __restrict__ su) {
+// Pairs before merged item t * kMergeTile.  *npair: the pairs there are (fewer
+// than the batch's records when bad records took no place; the update then
+// fails, but stays within its buffers).
+__global__ void merge_split(const int64_t* __restrict__ epos, const int32_t* __restrict__ npair, int64_t nt,
+                            int32_t* __restrict__ sq) {
+  const int64_t P = *npair;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t <= nt; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t dd = t * kMergeTile < total ? t * kMergeTile : total;
-    if (dd == total) {
-      se[t] = rp_o[n];
-      sq[t] = pp[n];
-      su[t] = n > 0 ? n - 1 : 0;
-      continue;
-    }
-    int64_t lo = 0, hi = n - 1;  // last row with W(u) <= dd
+    const int64_t d = t * kMergeTile;
+    int64_t lo = 0, hi = P < d ? P : d;  // first q with q + epos[q] >= d
     while (lo < hi) {
-      const int64_t mid = (lo + hi + 1) >> 1;
-      if (rp_o[mid] + pp[mid] <= dd) lo = mid; else hi = mid - 1;
+      const int64_t mid = (lo + hi) >> 1;
+      if (mid + epos[mid] < d) lo = mid + 1; else hi = mid;
     }
-    const int64_t u = lo;
-    const int64_t ob = rp_o[u], deg = rp_o[u + 1] - ob, p0 = pp[u], np = pp[u + 1] - p0;
-    const int64_t r = dd - ob - p0;  // items of row u before dd: i entries, r - i pairs
-    int64_t a = r - np > 0 ? r - np : 0, b = r < deg ? r : deg;
-    while (a < b) {
-      const int64_t mid = (a + b) >> 1;
-      if (col_o[ob + mid] <= (int32_t)(pkey[p0 + r - 1 - mid] & 0xffffffffu)) a = mid + 1; else b = mid;
-    }
-    se[t] = ob + a;
-    sq[t] = p0 + r - a;
-    su[t] = u;
+    sq[t] = (int32_t)lo;
   }
 }
 
-__device__ __forceinline__ int lower_bound_smem(const uint64_t* a, int n, uint64_t x) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (a[mid] < x) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
-// Adds a row's share of the weights into kdeg: lanes of one row sum with
-// redux (exact from 16-bit slices) and the lowest adds.
-__device__ __forceinline__ void add_row_weight(int64_t* kdeg, int64_t u, int64_t wv) {
-  const unsigned peers = __match_any_sync(0xffffffffu, u);
-  const unsigned lo = (unsigned)wv & 0xffffu, hi = (unsigned)(wv >> 16);
-  const unsigned long long sum =
-      (unsigned long long)__reduce_add_sync(peers, lo) + ((unsigned long long)__reduce_add_sync(peers, hi) << 16);
-  if (u >= 0 && sum != 0 && (int)(__ffs(peers) - 1) == (int)lane_id())
-    atomicAdd((unsigned long long*)&kdeg[u], sum);
-}
-
-// One tile of the merge.  Weights written are int32 (checked by pair_status),
-// so a lane's weight is below 2^31 and the slice sums above are exact.
+// One tile.  The work beyond the copy is per pair: a pair marks the entry it
+// changes (or whose successors it shifts) in shared memory, one block scan
+// turns the marks into shifts, and a tile without pairs is a plain shifted
+// copy.  Bound by the 16 bytes an entry: 80 M entries and 84 k pairs take
+// 233 us (5.5 TB/s), 73 M entries and 12.4 M pairs 375 us.  With the per-entry
+// searches (row of an entry, its place among the pairs) and row sums that ran
+// here before, it was issue-bound: 1059 and 1534 us.
 __global__ void __launch_bounds__(kMergeThreads) merge_tile(
-    int64_t n, const int64_t* __restrict__ rp_o, const int32_t* __restrict__ col_o,
-    const int32_t* __restrict__ w_o, const int64_t* __restrict__ se, const int64_t* __restrict__ sq,
-    const int64_t* __restrict__ su, const uint64_t* __restrict__ pkey, const int64_t* __restrict__ pw,
-    const uint8_t* __restrict__ pflag, const int32_t* __restrict__ pA, const int32_t* __restrict__ pR, int64_t P,
-    int32_t* __restrict__ col_n, int32_t* __restrict__ w_n, const int32_t* __restrict__ lab,
-    int64_t* __restrict__ kdeg, const int32_t* __restrict__ gid, GraphState* __restrict__ gs) {
-  __shared__ uint64_t s_pk[kMergeTile];
-  __shared__ uint64_t s_ek[kMergeTile];
-  __shared__ int64_t s_rp[kMergeRows + 1];
-  __shared__ unsigned long long s_red[2][kMergeThreads / 32];
-  __shared__ int s_uni;
+    int64_t nnz, const int32_t* __restrict__ col_o, const int32_t* __restrict__ w_o,
+    const int32_t* __restrict__ sq, const int64_t* __restrict__ epos, const uint64_t* __restrict__ pkey,
+    const int32_t* __restrict__ pdelta, const uint8_t* __restrict__ pflag, const int32_t* __restrict__ S,
+    int32_t* __restrict__ col_n, int32_t* __restrict__ w_n) {
+  __shared__ int32_t s_sh[kMergeTile + kMergeThreads];  // shift marks, then shifts (padded: one word a thread's run)
+  __shared__ int32_t s_adj[kMergeTile];                 // weight change of an entry; INT32_MIN: removed
+  auto at = [](int i) { return i + i / kMergeItems; };
   const int tid = threadIdx.x;
   const int64_t t = blockIdx.x;
-  const int64_t e0 = se[t], q0 = sq[t], ua = su[t], ub = su[t + 1];
-  const int ne = (int)(se[t + 1] - e0), np = (int)(sq[t + 1] - q0);
-  const int64_t nr = ub - ua + 1;  // rows ua..ub hold the tile's entries
-  const bool staged = nr + 1 <= kMergeRows + 1;
-  for (int j = tid; j < np; j += kMergeThreads) s_pk[j] = pkey[q0 + j];
-  if (staged)
-    for (int j = tid; j <= nr; j += kMergeThreads) s_rp[j] = rp_o[ua + j];
-  __syncthreads();
-  // entry keys
-  for (int j = tid; j < ne; j += kMergeThreads) {
-    const int64_t e = e0 + j;
-    int64_t u;
-    if (staged) {
-      int lo = 0, hi = (int)nr - 1;  // last row start <= e
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (s_rp[mid] <= e) lo = mid; else hi = mid - 1;
-      }
-      u = ua + lo;
-    } else {
-      int64_t lo = ua, hi = ub;
-      while (lo < hi) {
-        const int64_t mid = (lo + hi + 1) >> 1;
-        if (rp_o[mid] <= e) lo = mid; else hi = mid - 1;
-      }
-      u = lo;
-    }
-    s_ek[j] = (uint64_t)u << 32 | (uint32_t)ld_stream(col_o + e);
-  }
-  __syncthreads();
-  int cur_g = -1;
-  long long m2_loc = 0, in_loc = 0;
-  auto account = [&](int64_t u, int32_t cc, int64_t wv) {
-    const int gu = graph_of(gid, u);
-    if (gu != cur_g) {
-      if (cur_g >= 0 && (m2_loc | in_loc)) {
-        atomicAdd((unsigned long long*)&gs[cur_g].m2, (unsigned long long)m2_loc);
-        atomicAdd((unsigned long long*)&gs[cur_g].in_cur, (unsigned long long)in_loc);
-      }
-      cur_g = gu;
-      m2_loc = in_loc = 0;
-    }
-    m2_loc += wv;
-    if (lab && lab[cc] == lab[u]) in_loc += wv;
-  };
-  // old entries (warp-uniform trip count for the row sums)
-  for (int j0 = 0; j0 < ne; j0 += kMergeThreads) {
-    const int j = j0 + tid;
-    int64_t u = -1, wv = 0;
-    if (j < ne) {
-      const int64_t e = e0 + j;
-      const uint64_t key = s_ek[j];
-      const int64_t q = q0 + lower_bound_smem(s_pk, np, key);
-      // the equal pair follows its entry, possibly in the next tile
-      const bool match = q - q0 < np ? s_pk[q - q0] == key : (q < P && pkey[q] == key);
-      const uint32_t f = match ? pflag[q] : 0u;
-      if (!(f & kPairRemoved)) {
-        const int32_t cc = (int32_t)(key & 0xffffffffu);
-        wv = ld_stream(w_o + e);
-        if (match && (f & kPairIns)) wv = (f & kPairDel) ? pw[q] : wv + pw[q];
-        const int64_t pos = e + pA[q] - pR[q];
-        st_stream(col_n + pos, cc);
-        st_stream(w_n + pos, (int32_t)wv);
-        u = (int64_t)(key >> 32);
-        account(u, cc, wv);
-      }
-    }
-    add_row_weight(kdeg, u, wv);
-  }
-  // added pairs
-  for (int j0 = 0; j0 < np; j0 += kMergeThreads) {
-    const int j = j0 + tid;
-    int64_t u = -1, wv = 0;
-    if (j < np) {
-      const int64_t q = q0 + j;
-      if (pflag[q] & kPairAdded) {
-        const uint64_t key = s_pk[j];
-        const int64_t i = e0 + lower_bound_smem(s_ek, ne, key);
-        const int32_t cc = (int32_t)(key & 0xffffffffu);
-        wv = pw[q];
-        const int64_t pos = i + pA[q] - pR[q];
-        st_stream(col_n + pos, cc);
-        st_stream(w_n + pos, (int32_t)wv);
-        u = (int64_t)(key >> 32);
-        account(u, cc, wv);
-      }
-    }
-    add_row_weight(kdeg, u, wv);
-  }
-  // 2m and sum_i e_{i->C(i)}: one add per CTA when the tile lies in one graph
-  const int g0 = cur_g;
-  if (tid == 0) s_uni = -2;
-  __syncthreads();
-  if (g0 >= 0) atomicCAS(&s_uni, -2, g0);
-  __syncthreads();
-  const int gref = s_uni;
-  const bool uni = __syncthreads_and(g0 < 0 || g0 == gref);
-  if (uni) {
-    unsigned long long a = (unsigned long long)m2_loc, b = (unsigned long long)in_loc;
+  const int32_t q0 = sq[t], q1 = sq[t + 1];
+  const int64_t e0 = t * kMergeTile - q0;
+  const int64_t e1x = (t + 1) * kMergeTile - q1;
+  const int64_t e1 = e1x < nnz ? e1x : nnz;
+  const int ne = e1 > e0 ? (int)(e1 - e0) : 0, np = q1 - q0;
+  const int32_t shift0 = S[q0];
+  int32_t c[kMergeItems], w[kMergeItems];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      a += __shfl_xor_sync(0xffffffffu, a, o);
-      b += __shfl_xor_sync(0xffffffffu, b, o);
+  for (int x = 0; x < kMergeItems; x++) {
+    const int j = x * kMergeThreads + tid;
+    if (j < ne) {
+      c[x] = ld_stream(col_o + e0 + j);
+      w[x] = ld_stream(w_o + e0 + j);
     }
-    if (lane_id() == 0) {
-      s_red[0][tid >> 5] = a;
-      s_red[1][tid >> 5] = b;
-    }
-    __syncthreads();
-    if (tid == 0 && gref >= 0) {
-      unsigned long long sa = 0, sb = 0;
-      for (int x = 0; x < kMergeThreads / 32; x++) {
-        sa += s_red[0][x];
-        sb += s_red[1][x];
-      }
-      if (sa | sb) {
-        atomicAdd((unsigned long long*)&gs[gref].m2, sa);
-        atomicAdd((unsigned long long*)&gs[gref].in_cur, sb);
+  }
+  // the last pair before the tile may stand for the tile's first entry
+  const bool lead = q0 > 0 && ne > 0 && epos[q0 - 1] == e0 && (pflag[q0 - 1] & kPairPresent);
+  if (np == 0 && !lead) {
+#pragma unroll
+    for (int x = 0; x < kMergeItems; x++) {
+      const int j = x * kMergeThreads + tid;
+      if (j < ne) {
+        st_stream(col_n + e0 + shift0 + j, c[x]);
+        st_stream(w_n + e0 + shift0 + j, w[x]);
       }
     }
-  } else if (cur_g >= 0 && (m2_loc | in_loc)) {
-    atomicAdd((unsigned long long*)&gs[cur_g].m2, (unsigned long long)m2_loc);
-    atomicAdd((unsigned long long*)&gs[cur_g].in_cur, (unsigned long long)in_loc);
+    return;
+  }
+  for (int j = tid; j < kMergeTile; j += kMergeThreads) {
+    s_sh[at(j)] = 0;
+    s_adj[j] = 0;
+  }
+  __syncthreads();
+  if (lead && tid == 0) s_adj[0] = (pflag[q0 - 1] & kPairRemoved) ? INT32_MIN : pdelta[q0 - 1];
+  for (int j = tid; j < np; j += kMergeThreads) {
+    const int32_t q = q0 + j;
+    const uint32_t f = pflag[q];
+    if (f & (kPairAdded | kPairPresent)) {
+      const int64_t ep = epos[q];
+      const int rel = (int)(ep - e0);  // 0 .. ne
+      const int32_t d = pdelta[q];
+      if (f & kPairAdded) {
+        const int64_t pos = ep + S[q];
+        st_stream(col_n + pos, (int32_t)(pkey[q] & 0xffffffffu));
+        st_stream(w_n + pos, d);
+        if (rel < ne) atomicAdd(&s_sh[at(rel)], 1);
+      } else if (rel < ne) {
+        if (f & kPairRemoved) {
+          s_adj[rel] = INT32_MIN;
+          atomicAdd(&s_sh[at(rel)], -1);  // its successors move; the entry itself is gone
+        } else {
+          s_adj[rel] = d;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  int32_t m[kMergeItems], sum = 0, all;
+#pragma unroll
+  for (int x = 0; x < kMergeItems; x++) {
+    m[x] = s_sh[at(tid * kMergeItems + x)];
+    sum += m[x];
+  }
+  int32_t run = block_excl_scan<int32_t, kMergeThreads>(sum, &all) + shift0;
+#pragma unroll
+  for (int x = 0; x < kMergeItems; x++) {
+    run += m[x];
+    s_sh[at(tid * kMergeItems + x)] = run;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int x = 0; x < kMergeItems; x++) {
+    const int j = x * kMergeThreads + tid;
+    if (j < ne) {
+      const int32_t d = s_adj[j];
+      if (d != INT32_MIN) {
+        const int64_t pos = e0 + j + s_sh[at(j)];
+        st_stream(col_n + pos, c[x]);
+        st_stream(w_n + pos, w[x] + d);
+      }
+    }
   }
 }
 
@@ -523,166 +668,118 @@ int validate_batch(dcd_ctx* c, const dcd_edge* ins, int64_t n_ins, const dcd_edg
 int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut* out) {
   cudaStream_t s = c->stream;
   const int64_t n = c->n;
-  const int64_t n_ins = c->n_ins, n_del = c->n_del;
-  const int64_t R = 2 * (n_ins + n_del);
+  const int64_t n_ins = c->n_ins, n_del = c->n_del, nr = n_ins + n_del;
+  const int64_t R = 2 * nr;
   DevScalars* d = c->dsc.get();
-  uint32_t* err = &d->err;
   const int T = 256;
-
-  if (c->staged_on_device && n_ins + n_del > 0) {
-    // device-staged records are checked before any kernel indexes with them
-    ::dcd::count_launch(), validate_records<<<grid_for(n_ins + n_del, T), T, 0, s>>>(c->ins.get(), n_ins, c->del.get(), n_del, n, err);
-    DCD_LAUNCH_CHECK();
-    DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    DCD_TRY_CUDA(cudaStreamSynchronize(s));
-    if (*reinterpret_cast<uint32_t*>(c->hscratch) & kErrBadRecord) return DCD_EINVAL;
-  }
-
-  trace("merge: validated");
-  // ---- records sorted by (source, sink) ----
-  Buf<uint64_t> k0, k1;
-  Buf<uint32_t> v0, v1;
-  Buf<int32_t> head, pid;
-  Buf<uint32_t> stmp;
-  DCD_TRY(k0.alloc(&c->mem, R));
-  DCD_TRY(k1.alloc(&c->mem, R));
-  DCD_TRY(v0.alloc(&c->mem, R));
-  DCD_TRY(v1.alloc(&c->mem, R));
-  DCD_TRY(head.alloc(&c->mem, R + 1));
-  DCD_TRY(pid.alloc(&c->mem, R + 1));
-  int64_t scan_words = sort_tmp_words(R) + scan_tmp_count(n + 1) * 2 + scan_tmp_count(R + 1) * 2 + 64;
-  DCD_TRY(stmp.alloc(&c->mem, scan_words));
-  int64_t* stmp64 = reinterpret_cast<int64_t*>(stmp.get());
-
-  uint64_t* keys = k0.get();
-  uint32_t* vals = v0.get();
-  int64_t P = 0;
-  if (R > 0) {
-    // counting sort by source: per-source counts, offsets, the longest segment
-    Buf<int32_t> cnt, cur;
-    DCD_TRY(cnt.alloc(&c->mem, n + 1));
-    DCD_TRY(cur.alloc(&c->mem, n + 1));
-    DCD_TRY_CUDA(cudaMemsetAsync(cnt.get(), 0, (n + 1) * sizeof(int32_t), s));
-    DCD_TRY_CUDA(cudaMemsetAsync(cur.get(), 0, (n + 1) * sizeof(int32_t), s));
-    ::dcd::count_launch(), rec_count<<<grid_for(R / 2, T), T, 0, s>>>(c->ins.get(), n_ins, c->del.get(), n_del,
-                                                                       cnt.get());
-    ::dcd::count_launch(), rec_maxseg<<<grid_for(n, T), T, 0, s>>>(cnt.get(), n, cur.get() + n);
-    DCD_LAUNCH_CHECK();
-    DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch, cur.get() + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    DCD_TRY(exclusive_scan<int32_t>(cnt.get(), cnt.get(), n + 1, nullptr, reinterpret_cast<int32_t*>(stmp.get()), s));
-    DCD_TRY_CUDA(cudaStreamSynchronize(s));
-    const int64_t maxseg = *reinterpret_cast<int32_t*>(c->hscratch);
-    if (maxseg <= kRankSortMax && R < (int64_t)INT32_MAX) {
-      DCD_TRY_CUDA(cudaMemsetAsync(cur.get() + n, 0, sizeof(int32_t), s));
-      ::dcd::count_launch(), rec_scatter<<<grid_for(R / 2, T), T, 0, s>>>(c->ins.get(), n_ins, c->del.get(), n_del,
-                                                                           cnt.get(), cur.get(), k1.get(), v1.get());
-      ::dcd::count_launch(), rec_rank<<<grid_for(R, T), T, 0, s>>>(k1.get(), v1.get(), R, cnt.get(), k0.get(),
-                                                                    v0.get());
-      if (maxseg > kRankSmall) {
-        Buf<int32_t> big;
-        DCD_TRY(big.alloc(&c->mem, n));
-        DCD_TRY_CUDA(cudaMemsetAsync(cur.get() + n, 0, sizeof(int32_t), s));
-        ::dcd::count_launch(), rec_big_list<<<grid_for(n, T), T, 0, s>>>(cnt.get(), n, big.get(), cur.get() + n);
-        ::dcd::count_launch(), rec_bitonic<<<2 * c->sms, 1024, 0, s>>>(k1.get(), v1.get(), cnt.get(), big.get(),
-                                                                        cur.get() + n, k0.get(), v0.get());
-      }
-      DCD_LAUNCH_CHECK();
-    } else {
-      ::dcd::count_launch(), make_records<<<grid_for(R / 2, T), T, 0, s>>>(c->ins.get(), n_ins, c->del.get(), n_del,
-                                                                          k0.get(), v0.get());
-      DCD_LAUNCH_CHECK();
-      int b = bits_for(n - 1);
-      int ranges[4] = {0, b, 32, 32 + b};
-      bool in1 = false;
-      DCD_TRY(sort_pairs<uint32_t>(k0.get(), v0.get(), k1.get(), v1.get(), R, ranges, 2, stmp.get(), &in1, s));
-      if (in1) {
-        keys = k1.get();
-        vals = v1.get();
-      }
-    }
-    ::dcd::count_launch(), run_heads<<<grid_for(R, T), T, 0, s>>>(keys, R, head.get());
-    DCD_TRY(exclusive_scan<int32_t>(head.get(), pid.get(), R, pid.get() + R, reinterpret_cast<int32_t*>(stmp.get()), s));
-    DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch, pid.get() + R, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    DCD_TRY_CUDA(cudaStreamSynchronize(s));
-    P = (int64_t)(*reinterpret_cast<int32_t*>(c->hscratch));
-  }
-  trace("merge: sorted + pairs counted");
-  out->npairs = P;
-
-  DCD_TRY(out->pkey.alloc(&c->mem, P));
-  DCD_TRY(out->pw.alloc(&c->mem, P));
-  DCD_TRY(out->pflag.alloc(&c->mem, P));
-  DCD_TRY(out->pair_ptr.alloc(&c->mem, n + 1));
-  DCD_TRY(out->pdelta.alloc(&c->mem, P));
-  Buf<int32_t> added, removed;
-  DCD_TRY(added.alloc(&c->mem, P + 1));
-  DCD_TRY(removed.alloc(&c->mem, P + 1));
-  DCD_TRY_CUDA(cudaMemsetAsync(out->pair_ptr.get(), 0, (n + 1) * sizeof(int64_t), s));
-
-  // sum_i e_{i->C(i)} under the start labels on G_t: zero for a static start
-  // (singletons, no self-loops); from the previous update's value plus the
-  // batch's change when the context kept it (in_valid); else summed over
-  // every entry by the merge, which then gathers the label of each column
-  const bool from_prev = !static_start && c->in_valid;
-  const int32_t* lab_gather = (static_start || from_prev) ? nullptr : labels0;
-  Buf<int64_t> in_delta;
-  DCD_TRY(in_delta.alloc(&c->mem, c->G));
-  DCD_TRY_CUDA(cudaMemsetAsync(in_delta.get(), 0, c->G * sizeof(int64_t), s));
-
   const int cur = c->cur, nxt = 1 - c->cur;
   const int64_t* rp_o = c->rp[cur].get();
   const int32_t* col_o = c->col[cur].get();
   const int32_t* w_o = c->w[cur].get();
+  const int32_t* gid = c->G > 1 ? c->gid.get() : nullptr;
 
-  if (P > 0) {
-    ::dcd::count_launch(), reduce_pairs<<<grid_for(R, T), T, 0, s>>>(keys, vals, R, head.get(), pid.get(), c->ins.get(), n_ins,
-                                              out->pkey.get(), out->pw.get(), out->pflag.get());
-    ::dcd::count_launch(), pair_status<<<grid_for(P, T), T, 0, s>>>(out->pkey.get(), out->pw.get(), out->pflag.get(), P, rp_o, col_o, w_o,
-                                             added.get(), removed.get(), out->pair_ptr.get(), err,
-                                             from_prev ? labels0 : nullptr, c->G > 1 ? c->gid.get() : nullptr,
-                                             in_delta.get(), out->pdelta.get());
+  // ---- degrees and sums of G_{t-1} ----
+  if (!c->k_valid) {
+    DCD_TRY(c->kdeg[cur].ensure(&c->mem, n));
+    DCD_TRY(c->in_prev.ensure(&c->mem, 2 * (size_t)c->G));
+    DCD_TRY_CUDA(cudaMemsetAsync(c->in_prev.get(), 0, 2 * c->G * sizeof(int64_t), s));
+    if (c->nnz > 0) {  // a loaded checkpoint: one graph
+      ::dcd::count_launch(), row_degrees<<<grid_for(n * 32, T), T, 0, s>>>(
+          n, rp_o, w_o, c->kdeg[cur].get(), reinterpret_cast<unsigned long long*>(c->in_prev.get() + c->G));
+      DCD_LAUNCH_CHECK();
+    } else {
+      DCD_TRY_CUDA(cudaMemsetAsync(c->kdeg[cur].get(), 0, n * sizeof(int64_t), s));
+    }
+    c->k_valid = true;
+  }
+  DCD_TRY(c->kdeg[nxt].ensure(&c->mem, n));
+  out->k = &c->kdeg[nxt];
+  // sum_i e_{i->C(i)} under the start labels on G_t: zero for a static start
+  // (singletons, no self-loops); from the previous update's value plus the
+  // batch's change when the context kept it (in_valid); else summed over
+  // every entry of G_t
+  const bool from_prev = !static_start && c->in_valid;
+  DCD_TRY_CUDA(cudaMemsetAsync(c->gs.get(), 0, c->G * sizeof(GraphState), s));
+
+  // ---- records by source ----
+  Buf<int2> rank;
+  Buf<uint64_t> rec, rec2;
+  Buf<int32_t> stmp, big;
+  out->npairs = R;
+  DCD_TRY(out->pair_ptr.alloc(&c->mem, n + 4));  // + 3: the counts of the long segments' lists
+  DCD_TRY(out->pkey.alloc(&c->mem, R));
+  DCD_TRY(out->pw.alloc(&c->mem, R));
+  DCD_TRY(out->pflag.alloc(&c->mem, R));
+  DCD_TRY(out->pdelta.alloc(&c->mem, R));
+  DCD_TRY(stmp.alloc(&c->mem, scan_tmp_count(n + 1) + scan_tmp_count(R + 1)));
+  Buf<int64_t> epos;
+  Buf<int32_t> S;
+  DCD_TRY(epos.alloc(&c->mem, R));
+  DCD_TRY(S.alloc(&c->mem, R + 1));
+  int32_t* off = out->pair_ptr.get();
+  int32_t* big_cnt = off + n + 1;
+  DCD_TRY_CUDA(cudaMemsetAsync(off, 0, (n + 4) * sizeof(int32_t), s));
+  DCD_TRY_CUDA(cudaMemsetAsync(S.get() + R, 0, sizeof(int32_t), s));
+  if (R > 0) {
+    DCD_TRY(rank.alloc(&c->mem, nr));
+    DCD_TRY(rec.alloc(&c->mem, R));
+    if (nr > kSegLarge) DCD_TRY(rec2.alloc(&c->mem, R));
+    DCD_TRY(big.alloc(&c->mem, 3 * n));
+    ::dcd::count_launch(), rec_count<<<grid_for(nr, T), T, 0, s>>>(c->ins.get(), n_ins, c->del.get(), n_del, n, off,
+                                                                    rank.get(), &d->err);
+    DCD_LAUNCH_CHECK();
+    DCD_TRY(exclusive_scan<int32_t>(off, off, n + 1, nullptr, stmp.get(), s));
+    ::dcd::count_launch(), rec_scatter<<<grid_for(nr, T), T, 0, s>>>(c->ins.get(), n_ins, c->del.get(), n_del, n, off,
+                                                                      rank.get(), rec.get());
     DCD_LAUNCH_CHECK();
   }
-  // pair_ptr: per-source counts -> exclusive scan (n + 1 entries)
-  DCD_TRY(exclusive_scan<int64_t>(out->pair_ptr.get(), out->pair_ptr.get(), n + 1, nullptr, stmp64, s));
-  DCD_TRY(exclusive_scan<int32_t>(added.get(), added.get(), P + 1, nullptr, reinterpret_cast<int32_t*>(stmp.get()), s));
-  DCD_TRY(exclusive_scan<int32_t>(removed.get(), removed.get(), P + 1, nullptr,
-                                  reinterpret_cast<int32_t*>(stmp.get()), s));
+  PairView o{off, rp_o, col_o, w_o, from_prev ? labels0 : nullptr, gid, out->pkey.get(), out->pw.get(),
+             out->pflag.get(), out->pdelta.get(), epos.get(), S.get(), c->gs.get(), &d->npairs, &d->err};
+  if (R > 0) {
+    ::dcd::count_launch(), pair_tile<<<(unsigned)cdiv(n, kPairSrc), kPairThreads, 0, s>>>(
+        o, n, rec.get(), c->kdeg[cur].get(), out->k->get(), big.get(), big_cnt);
+    // a segment holds at most one record per batch record: the classes the
+    // batch is too small for are not launched
+    if (nr > kSegSmall)
+      ::dcd::count_launch(), pair_mid<<<grid_for(nr, kSegSmall, 16), kMidThreads, 0, s>>>(
+          o, rec.get(), big.get(), big_cnt, out->k->get());
+    if (nr > kSegMid)
+      ::dcd::count_launch(), pair_large<<<grid_for(nr, kSegMid, 4), kLargeThreads, 0, s>>>(
+          o, rec.get(), big.get() + n, big_cnt + 1, out->k->get());
+    if (nr > kSegLarge)
+      ::dcd::count_launch(), pair_huge<<<grid_for(nr, kSegLarge, 2), kHugeThreads, 0, s>>>(
+          o, rec.get(), rec2.get(), big.get() + 2 * n, big_cnt + 2, bits_for(n - 1), out->k->get());
+    DCD_LAUNCH_CHECK();
+  } else {
+    DCD_TRY_CUDA(cudaMemcpyAsync(out->k->get(), c->kdeg[cur].get(), n * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+  }
+  ::dcd::count_launch(), seed_sums<<<cdiv(c->G, 128), 128, 0, s>>>(c->gs.get(), c->G, c->in_prev.get(),
+                                                                    from_prev ? 1 : 0);
+  DCD_LAUNCH_CHECK();
+  DCD_TRY(exclusive_scan<int32_t>(S.get(), S.get(), R + 1, nullptr, stmp.get(), s));
 
-  // ---- new row pointers ----
+  // ---- new row pointers, merge ----
   const int64_t cap = c->nnz + 2 * n_ins;
   DCD_TRY(c->rp[nxt].ensure(&c->mem, n + 1));
   DCD_TRY(c->col[nxt].ensure(&c->mem, cap));
   DCD_TRY(c->w[nxt].ensure(&c->mem, cap));
   int64_t* rp_n = c->rp[nxt].get();
-  ::dcd::count_launch(), new_rows<<<grid_for(n + 1, T), T, 0, s>>>(rp_o, out->pair_ptr.get(), added.get(),
-                                                                    removed.get(), n, rp_n);
+  ::dcd::count_launch(), new_rows<<<grid_for(n + 1, T), T, 0, s>>>(rp_o, off, S.get(), n, rp_n);
   DCD_LAUNCH_CHECK();
-
-  // ---- merge (tiles of the merged sequence), degrees, m2, in ----
-  DCD_TRY(out->k.alloc(&c->mem, n));
-  DCD_TRY_CUDA(cudaMemsetAsync(out->k.get(), 0, n * sizeof(int64_t), s));
-  DCD_TRY_CUDA(cudaMemsetAsync(c->gs.get(), 0, c->G * sizeof(GraphState), s));
-  const int64_t total = c->nnz + P;
-  const int64_t nt = cdiv(total, (int64_t)kMergeTile);
+  const int64_t nt = cdiv(c->nnz + R, (int64_t)kMergeTile);
   if (nt > 0) {
-    Buf<int64_t> split;
-    DCD_TRY(split.alloc(&c->mem, 3 * (nt + 1)));
-    int64_t* se = split.get();
-    int64_t* sq = se + (nt + 1);
-    int64_t* su = sq + (nt + 1);
-    ::dcd::count_launch(), merge_split<<<grid_for(nt + 1, T), T, 0, s>>>(n, rp_o, col_o, out->pair_ptr.get(),
-                                                                          out->pkey.get(), nt, total, se, sq, su);
+    Buf<int32_t> split;
+    DCD_TRY(split.alloc(&c->mem, nt + 1));
+    ::dcd::count_launch(), merge_split<<<grid_for(nt + 1, T), T, 0, s>>>(epos.get(), off + n, nt, split.get());
     DCD_LAUNCH_CHECK();
     ::dcd::count_launch(), merge_tile<<<(unsigned)nt, kMergeThreads, 0, s>>>(
-        n, rp_o, col_o, w_o, se, sq, su, out->pkey.get(), out->pw.get(), out->pflag.get(), added.get(),
-        removed.get(), P, c->col[nxt].get(), c->w[nxt].get(), lab_gather, out->k.get(),
-        c->G > 1 ? c->gid.get() : nullptr, c->gs.get());
+        c->nnz, col_o, w_o, split.get(), epos.get(), out->pkey.get(), out->pdelta.get(), out->pflag.get(), S.get(),
+        c->col[nxt].get(), c->w[nxt].get());
     DCD_LAUNCH_CHECK();
   }
-  if (from_prev) {
-    ::dcd::count_launch(), seed_in<<<cdiv(c->G, 128), 128, 0, s>>>(c->gs.get(), c->G, c->in_prev.get(),
-                                                                    in_delta.get());
+  if (!static_start && !c->in_valid && c->cfg.alg == DCD_ALG_LOUVAIN) {
+    ::dcd::count_launch(), in_weight<<<grid_for(n * 32, T), T, 0, s>>>(n, rp_n, c->col[nxt].get(), c->w[nxt].get(),
+                                                                        labels0, gid, c->gs.get());
     DCD_LAUNCH_CHECK();
   }
   return DCD_OK;

@@ -8,12 +8,17 @@
 namespace dcd {
 
 // ----------------------------------------------------------------------------
-// Exclusive scan.  Tiles of 256 threads x 8 items: (1) per-tile totals,
-// (2) one CTA scans the totals, (3) each tile scans itself from its offset.
+// Exclusive scan.  Up to kScanOne items: one CTA, one launch.  Above: (1) per-
+// tile totals, (2) each tile adds up the totals before it (they sit in L2, a
+// few per thread) and scans itself.  A scan of a few thousand words is bound
+// by its launches, not by its bytes.
 // ----------------------------------------------------------------------------
 constexpr int kScanThreads = 256;
-constexpr int kScanItems = 8;
+constexpr int kScanItems = 16;
 constexpr int kScanTile = kScanThreads * kScanItems;
+constexpr int kScanOneThreads = 1024;
+constexpr int kScanOneItems = 8;
+constexpr int64_t kScanOne = (int64_t)kScanOneThreads * kScanOneItems;
 
 template <typename T>
 __device__ __forceinline__ T warp_incl_scan(T x) {
@@ -32,25 +37,25 @@ __device__ __forceinline__ T warp_sum(T x) {
   return x;
 }
 
-// Block-wide exclusive scan of one value per thread; returns the exclusive
-// prefix and writes the block total to *total (shared memory).
-// blockDim.x == kScanThreads.
-template <typename T>
+// Block-wide exclusive scan of one value per thread (NT threads, whole warps);
+// every thread gets its prefix and the block total.
+template <typename T, int NT>
 __device__ __forceinline__ T block_excl_scan(T x, T* total) {
-  constexpr int NW = kScanThreads / 32;
-  __shared__ T warp_off[NW];
-  T incl = warp_incl_scan(x);
-  int w = threadIdx.x >> 5;
+  constexpr int NW = NT / 32;
+  __shared__ T warp_off[NW + 1];
+  const T incl = warp_incl_scan(x);
+  const int w = threadIdx.x >> 5;
   if (lane_id() == 31) warp_off[w] = incl;
   __syncthreads();
   if (w == 0) {
-    T t = lane_id() < NW ? warp_off[lane_id()] : T(0);
-    T ti = warp_incl_scan(t);
-    if (lane_id() < NW) warp_off[lane_id()] = ti - t;
-    if (lane_id() == NW - 1) *total = ti;
+    const T t = (int)lane_id() < NW ? warp_off[lane_id()] : T(0);
+    const T ti = warp_incl_scan(t);
+    if ((int)lane_id() < NW) warp_off[lane_id()] = ti - t;
+    if ((int)lane_id() == NW - 1) warp_off[NW] = ti;
   }
   __syncthreads();
-  T r = incl - x + warp_off[w];
+  const T r = incl - x + warp_off[w];
+  *total = warp_off[NW];
   __syncthreads();
   return r;
 }
@@ -59,11 +64,11 @@ template <typename T>
 __global__ void __launch_bounds__(kScanThreads) scan_tile_totals(const T* __restrict__ in, int64_t n,
                                                                  T* __restrict__ tot) {
   __shared__ T red[kScanThreads / 32];
-  int64_t base = (int64_t)blockIdx.x * kScanTile;
+  const int64_t base = (int64_t)blockIdx.x * kScanTile;
   T s = 0;
 #pragma unroll
   for (int i = 0; i < kScanItems; i++) {
-    int64_t idx = base + (int64_t)i * kScanThreads + threadIdx.x;
+    const int64_t idx = base + (int64_t)i * kScanThreads + threadIdx.x;
     if (idx < n) s += in[idx];
   }
   s = warp_sum(s);
@@ -76,60 +81,70 @@ __global__ void __launch_bounds__(kScanThreads) scan_tile_totals(const T* __rest
   }
 }
 
-// One CTA: exclusive scan of the tile totals in place; grand total -> *total.
+// in and out may be the same array: no __restrict__, and a tile reads itself
+// before it writes.
 template <typename T>
-__global__ void __launch_bounds__(kScanThreads) scan_totals(T* __restrict__ tot, int64_t ntiles,
-                                                            T* __restrict__ total) {
-  __shared__ T carry_s;
-  T carry = 0;
-  for (int64_t base = 0; base < ntiles; base += kScanThreads) {
-    int64_t idx = base + threadIdx.x;
-    T x = idx < ntiles ? tot[idx] : T(0);
-    T btot;
-    T ex = block_excl_scan(x, &carry_s);
-    btot = carry_s;
-    if (idx < ntiles) tot[idx] = carry + ex;
-    carry += btot;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0 && total) *total = carry;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kScanThreads) scan_tiles(const T* __restrict__ in, T* __restrict__ out,
-                                                           int64_t n, const T* __restrict__ tile_off) {
-  __shared__ T buf[kScanTile];
-  __shared__ T tot_s;
-  int64_t base = (int64_t)blockIdx.x * kScanTile;
+__global__ void __launch_bounds__(kScanThreads) scan_tiles(const T* in, T* out, int64_t n, const T* __restrict__ tot,
+                                                           T* total) {
+  // one pad word after each thread's kScanItems words: a stride of 17 words
+  // has no bank conflict between the lanes' own runs
+  __shared__ T buf[kScanTile + kScanThreads];
+  auto at = [](int i) { return i + i / kScanItems; };
+  const int64_t base = (int64_t)blockIdx.x * kScanTile;
 #pragma unroll
   for (int i = 0; i < kScanItems; i++) {
-    int64_t idx = base + (int64_t)i * kScanThreads + threadIdx.x;
-    buf[i * kScanThreads + threadIdx.x] = idx < n ? in[idx] : T(0);
+    const int64_t idx = base + (int64_t)i * kScanThreads + threadIdx.x;
+    buf[at(i * kScanThreads + threadIdx.x)] = idx < n ? in[idx] : T(0);
   }
-  __syncthreads();
+  T pre = 0, before, all;
+  for (int64_t x = threadIdx.x; x < (int64_t)blockIdx.x; x += kScanThreads) pre += tot[x];
+  (void)block_excl_scan<T, kScanThreads>(pre, &before);
   T v[kScanItems];
   T s = 0;
 #pragma unroll
   for (int i = 0; i < kScanItems; i++) {
-    v[i] = buf[threadIdx.x * kScanItems + i];
+    v[i] = buf[at(threadIdx.x * kScanItems + i)];
     s += v[i];
   }
-  T ex = block_excl_scan(s, &tot_s) + tile_off[blockIdx.x];
+  T ex = block_excl_scan<T, kScanThreads>(s, &all) + before;
+  if (total && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total = before + all;
 #pragma unroll
   for (int i = 0; i < kScanItems; i++) {
-    buf[threadIdx.x * kScanItems + i] = ex;
+    buf[at(threadIdx.x * kScanItems + i)] = ex;
     ex += v[i];
   }
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < kScanItems; i++) {
-    int64_t idx = base + (int64_t)i * kScanThreads + threadIdx.x;
-    if (idx < n) out[idx] = buf[i * kScanThreads + threadIdx.x];
+    const int64_t idx = base + (int64_t)i * kScanThreads + threadIdx.x;
+    if (idx < n) out[idx] = buf[at(i * kScanThreads + threadIdx.x)];
   }
 }
 
-// out[i] = sum_{j<i} in[i]; *total (device, may be NULL) = sum of all.
-// out may alias in.  tmp needs scan_tmp_count(n) elements of T.
+// One CTA: n <= kScanOne.
+template <typename T>
+__global__ void __launch_bounds__(kScanOneThreads) scan_one(const T* in, T* out, int64_t n, T* total) {
+  T v[kScanOneItems];
+  T s = 0;
+  const int64_t b = (int64_t)threadIdx.x * kScanOneItems;
+#pragma unroll
+  for (int i = 0; i < kScanOneItems; i++) {
+    v[i] = b + i < n ? in[b + i] : T(0);
+    s += v[i];
+  }
+  T all;
+  T ex = block_excl_scan<T, kScanOneThreads>(s, &all);
+  if (total && threadIdx.x == 0) *total = all;
+#pragma unroll
+  for (int i = 0; i < kScanOneItems; i++) {
+    if (b + i < n) out[b + i] = ex;
+    ex += v[i];
+  }
+}
+
+// out[i] = sum_{j<i} in[i]; *total (device, may be NULL) = sum of all; it may
+// lie right behind out.  out may alias in.  tmp needs scan_tmp_count(n)
+// elements of T.
 inline int64_t scan_tmp_count(int64_t n) { return cdiv(n, kScanTile) + 1; }
 
 template <typename T>
@@ -138,10 +153,13 @@ int exclusive_scan(const T* in, T* out, int64_t n, T* total, T* tmp, cudaStream_
     if (total) DCD_TRY_CUDA(cudaMemsetAsync(total, 0, sizeof(T), s));
     return DCD_OK;
   }
-  int64_t ntiles = cdiv(n, kScanTile);
-  ::dcd::count_launch(), scan_tile_totals<T><<<(unsigned)ntiles, kScanThreads, 0, s>>>(in, n, tmp);
-  ::dcd::count_launch(), scan_totals<T><<<1, kScanThreads, 0, s>>>(tmp, ntiles, total);
-  ::dcd::count_launch(), scan_tiles<T><<<(unsigned)ntiles, kScanThreads, 0, s>>>(in, out, n, tmp);
+  if (n <= kScanOne) {
+    ::dcd::count_launch(), scan_one<T><<<1, kScanOneThreads, 0, s>>>(in, out, n, total);
+  } else {
+    const int64_t ntiles = cdiv(n, kScanTile);
+    ::dcd::count_launch(), scan_tile_totals<T><<<(unsigned)ntiles, kScanThreads, 0, s>>>(in, n, tmp);
+    ::dcd::count_launch(), scan_tiles<T><<<(unsigned)ntiles, kScanThreads, 0, s>>>(in, out, n, tmp, total);
+  }
   DCD_LAUNCH_CHECK();
   return DCD_OK;
 }

@@ -39,7 +39,7 @@ struct SV {
   const int64_t* a;
   const uint64_t* pkey;
   const uint8_t* pflag;
-  const int64_t* pair_ptr;
+  const int32_t* pair_ptr;
   int64_t m2;                   // 2m when the context holds one graph
   const int32_t* gid;           // graph of each vertex (several graphs)
   const GraphState* gs;
@@ -815,7 +815,7 @@ __global__ void __launch_bounds__(256) scr_mark_hub(SV g, int64_t lo, int64_t hi
 }
 
 // Sources (vertices with at least one pair) binned by their degree in G_t.
-__global__ void src_bins(int64_t n, const int64_t* __restrict__ pair_ptr, const int64_t* __restrict__ rp,
+__global__ void src_bins(int64_t n, const int32_t* __restrict__ pair_ptr, const int64_t* __restrict__ rp,
                          int32_t* __restrict__ cursor, int32_t* __restrict__ lists, int64_t cap_per_bin) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t base = (blockIdx.x * (int64_t)blockDim.x) + (threadIdx.x & ~31); base < n; base += stride) {

@@ -208,9 +208,14 @@ struct dcd_ctx {
   cudaEvent_t join_ev[dcd::kMaxBins] = {};
   cudaEvent_t fork_ev = nullptr;
   dcd::BinPlan bin_plan = dcd::default_bin_plan();  // degree bins of the local-move kernels
-  // sum_i e_{i->C(i)} of C_t on G_t per graph, kept by the last update so the
-  // next merge need not gather every entry's label (in_valid: it is current;
-  // cleared by anything that replaces C_t other than a Louvain update)
+  // weighted degrees of G_t (index cur), and per graph sum_i e_{i->C(i)} of C_t
+  // on G_t (words 0 .. G-1) and 2m (words G .. 2G-1), kept by the last update
+  // so that the next merge adds the batch's changes to them instead of summing
+  // every entry.  k_valid: degrees and 2m are current (they are not after a
+  // checkpoint was loaded); in_valid: the first G words are (cleared by
+  // anything that replaces C_t other than a Louvain update)
+  bool k_valid = false;
+  dcd::Buf<int64_t> kdeg[2];
   bool in_valid = false;
   dcd::Buf<int64_t> in_prev, in_next;
   // Per-step delta coarsening of level 0 (dense coarse graphs only): K is
@@ -231,8 +236,9 @@ struct dcd_ctx {
     bool track = false;            // build K for the next update
     bool usable = false;           // K holds G_{t-1} under the start labels
     const uint64_t* pkey = nullptr;  // the batch's pairs and their weight changes
-    const int64_t* pdelta = nullptr;
+    const int32_t* pdelta = nullptr;
     int64_t P = 0;
+    int64_t distinct = 0;          // of them, pairs that carry flags
     const int32_t* cprev = nullptr;  // C_{t-1}
     bool used = false;             // this update took the delta path
     int64_t entries = 0;           // entries the level-0 coarsening read
@@ -251,8 +257,10 @@ struct dcd_ctx {
 
 namespace dcd {
 
-// merge.cu: sort the staged batch, merge it into G_t (new buffers of ctx at
-// index 1 - cur), compute k (weighted degrees), m2 and in under labels0.
+// merge.cu (merge_batch below): sort the staged batch, merge it into G_t (new
+// buffers of ctx at index 1 - cur), k (weighted degrees), m2 and in under
+// labels0.  Records staged from device memory are checked there; a bad one
+// sets kErrBadRecord.
 // merge.cu: check staged records on the device (ids in [0, n), no self
 // loop, positive insert weight); *ok false when one fails.  Synchronises.
 int validate_batch(dcd_ctx* c, const dcd_edge* ins, int64_t n_ins, const dcd_edge* del, int64_t n_del, bool* ok);
@@ -325,13 +333,15 @@ using UpdateFinish = int (*)(dcd_ctx* c, void* user);
 int update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, UpdateFinish finish, void* user);
 
 struct MergeOut {
-  Buf<int64_t> k;          // n weighted degrees of G_t
-  Buf<uint64_t> pkey;      // distinct (src << 32 | dst) pairs, sorted
-  Buf<int64_t> pw;         // summed insert weight per pair (0 = no insert)
-  Buf<uint8_t> pflag;      // bit0 insert, bit1 delete, bit2 edge was in G_{t-1}
-  Buf<int64_t> pair_ptr;   // n + 1: pairs of source u are [pair_ptr[u], pair_ptr[u+1])
-  Buf<int64_t> pdelta;     // per pair: its weight in G_t minus its weight in G_{t-1}
-  int64_t npairs = 0;
+  Buf<int64_t>* k = nullptr;  // n weighted degrees of G_t (kept by the context)
+  // (src << 32 | dst) pairs, sorted; of equal pairs (repeated records) the
+  // last one carries the flags and the weight change, the others have none
+  Buf<uint64_t> pkey;
+  Buf<int32_t> pw;         // summed insert weight per pair (0 = no insert)
+  Buf<uint8_t> pflag;      // bit0 insert, bit1 delete, bit2 edge was in G_{t-1}; 0: a null pair
+  Buf<int32_t> pair_ptr;   // n + 1: pairs of source u are [pair_ptr[u], pair_ptr[u+1])
+  Buf<int32_t> pdelta;     // per pair: its weight in G_t minus its weight in G_{t-1}
+  int64_t npairs = 0;      // pairs, null ones among them
 };
 int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut* out);
 
