@@ -226,8 +226,8 @@ int dcd_set_mode(dcd_ctx* ctx, int32_t mode);
  * receives its time per evaluation.  Errors: DCD_ESTATE before the first
  * update or for reps < 1, DCD_ENOMEM, DCD_ECUDA. */
 #define DCD_MAX_BINS 12
-#define DCD_LM_SEG16 0   /* <= 16 entries: 8 lanes per vertex, 4 vertices a warp   */
-#define DCD_LM_SEG32 1   /* <= 32: 16 lanes per vertex, 2 vertices a warp          */
+#define DCD_LM_SEG16 0   /* <= 16 entries: 4 lanes read a row, one lane chooses     */
+#define DCD_LM_SEG32 1   /* <= 32: 8 lanes read a row, one lane chooses             */
 #define DCD_LM_SEG64 2   /* <= 64: 16 lanes per vertex, 2 vertices a warp          */
 #define DCD_LM_WARP128 3 /* <= 128: a warp per vertex                              */
 #define DCD_LM_WARP256 4 /* <= 256: a warp per vertex                              */

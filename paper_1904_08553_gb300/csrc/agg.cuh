@@ -94,28 +94,23 @@ __device__ __forceinline__ void warp_argmax(long long& S, int32_t& D) {
   D = (int32_t)dmin;
 }
 
-// Argmax of (S, D) over the SEG-lane segment of the calling lane (mask: that
-// segment's lanes); SEG = 32 is the whole warp.
-template <int SEG>
-__device__ __forceinline__ void seg_argmax(long long& S, int32_t& D, unsigned mask) {
-  const unsigned long long u = (unsigned long long)S ^ 0x8000000000000000ull;
-  const unsigned hi = (unsigned)(u >> 32), lo = (unsigned)u;
-  const unsigned mhi = __reduce_max_sync(mask, hi);
-  const unsigned mlo = __reduce_max_sync(mask, hi == mhi ? lo : 0u);
-  const bool top = hi == mhi && lo == mlo;
-  const unsigned dmin = __reduce_min_sync(mask, top ? (unsigned)D : 0xffffffffu);
-  S = (long long)((((unsigned long long)mhi << 32) | mlo) ^ 0x8000000000000000ull);
-  D = (int32_t)dmin;
-}
-template <int SEG>
-__device__ __forceinline__ void seg_argmax(i128& S, int32_t& D, unsigned) {
+// Argmax of (S, D) over the SEG-lane segment of the calling lane, all lanes of
+// the warp calling.  Below a whole warp it runs on shuffles: a redux over a
+// part of the warp executes once per segment, one after another, where the
+// shuffles take all segments in the same instruction.
+template <int SEG, typename ST>
+__device__ __forceinline__ void seg_argmax(ST& S, int32_t& D) {
+  if constexpr (SEG == 32) {
+    warp_argmax(S, D);
+  } else {
 #pragma unroll
-  for (int o = SEG / 2; o > 0; o >>= 1) {
-    const i128 s2 = shfl_xor_st(S, o);
-    const int32_t d2 = __shfl_xor_sync(0xffffffffu, D, o);
-    if (better(s2, d2, S, D)) {
-      S = s2;
-      D = d2;
+    for (int o = SEG / 2; o > 0; o >>= 1) {
+      const ST s2 = shfl_xor_st(S, o);
+      const int32_t d2 = __shfl_xor_sync(0xffffffffu, D, o);
+      if (better(s2, d2, S, D)) {
+        S = s2;
+        D = d2;
+      }
     }
   }
 }
@@ -252,15 +247,18 @@ __device__ __forceinline__ uint32_t probe_claim(int32_t* keys, uint32_t mask, in
   }
 }
 
-// Sum over the S lanes of the calling lane's segment: 32-bit sums are exact
-// with 64-bit gains (every sum of a vertex's weights is below 2m < 2^31),
-// 64-bit sums with 128-bit gains.
+// Sum over the S lanes of the calling lane's segment, all lanes of the warp
+// calling: 32-bit sums are exact with 64-bit gains (every sum of a vertex's
+// weights is below 2m < 2^31), 64-bit sums with 128-bit gains.
 template <int S>
-__device__ __forceinline__ int64_t seg_total(unsigned x, unsigned smask) {
-  return (int64_t)__reduce_add_sync(smask, x);
+__device__ __forceinline__ int64_t seg_total(unsigned x) {
+  if constexpr (S == 32) return (int64_t)__reduce_add_sync(0xffffffffu, x);
+#pragma unroll
+  for (int o = S / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return (int64_t)x;
 }
 template <int S>
-__device__ __forceinline__ int64_t seg_total(unsigned long long x, unsigned) {
+__device__ __forceinline__ int64_t seg_total(unsigned long long x) {
 #pragma unroll
   for (int o = S / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
   return (int64_t)x;

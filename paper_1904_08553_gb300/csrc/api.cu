@@ -582,6 +582,7 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
   Buf<int64_t> a;
   Buf<int32_t> size;
   LearnedPool lp;
+  EntryLabels nlab;
   // the first level-0 pass of a Delta-screening update reads the state the
   // screening reads (C_{t-1}, its sums on G_t): the screening hands over its
   // proposals for the sources whose rows it sums (one Louvain graph)
@@ -603,7 +604,7 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
     r_screen = c->hscratch[9];
   }
   if (learned || collect) {
-    DCD_TRY(screen_features(c, g, src_labels, mo.k->get(), a.get(), size.get(), mo, rds.get(), &lp));
+    DCD_TRY(screen_features(c, g, src_labels, mo.k->get(), a.get(), size.get(), mo, rds.get(), &nlab, &lp));
     c->feat_has_y = false;
   }
   if (mode == DCD_MODE_DELTA) {
@@ -652,7 +653,7 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
   if (c->cfg.alg == DCD_ALG_SLM)
     DCD_TRY(run_slm(c, g, L0.get(), active, *mo.k, c->labels_nx.get(), st));
   else
-    DCD_TRY(run_louvain(c, g, L0.get(), active, *mo.k, c->labels_nx.get(), st,
+    DCD_TRY(run_louvain(c, g, L0.get(), active, *mo.k, c->labels_nx.get(), st, &nlab,
                         collect ? c->level0.get() : nullptr, per_graph, a.n ? a.get() : nullptr,
                         size.n ? size.get() : nullptr, pre.n ? pre.get() : nullptr));
   if (collect) DCD_TRY(screen_labels(c, src_labels, c->level0.get()));
@@ -667,7 +668,7 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
     DCD_TRY_CUDA(cudaMemcpyAsync(L0b.get(), src_labels, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
     memcpy(c->hgs, gs0.data(), c->G * sizeof(GraphState));
     DCD_TRY_CUDA(cudaMemcpyAsync(c->gs.get(), c->hgs, c->G * sizeof(GraphState), cudaMemcpyHostToDevice, s));
-    DCD_TRY(run_louvain(c, g, L0b.get(), rds.get(), *mo.k, lab2.get(), &st2));
+    DCD_TRY(run_louvain(c, g, L0b.get(), rds.get(), *mo.k, lab2.get(), &st2, &nlab));
     st->q_screen = st2.q;
     if (st->q < st2.q - 1e-3) {
       const double ql = st->q;

@@ -98,7 +98,7 @@ __global__ void move_labels(int64_t m, const int32_t* __restrict__ list, const i
 }  // namespace
 
 int screen_features(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L0, const int64_t* k, const int64_t* a,
-                    const int32_t* size, const MergeOut& mo, const uint8_t* rds, LearnedPool* out) {
+                    const int32_t* size, const MergeOut& mo, const uint8_t* rds, EntryLabels* nlab, LearnedPool* out) {
   cudaStream_t s = c->stream;
   const int64_t n = g.n;
   const int T = 256;
@@ -107,7 +107,7 @@ int screen_features(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L0, const 
   DCD_TRY_CUDA(cudaMemsetAsync(pool.get(), 0, n, s));
   count_launch(), pool_mark<<<grid_for(n * 32, T, 16), T, 0, s>>>(n, g.rp, g.col, mo.pair_ptr.get(), rds, pool.get());
   DCD_LAUNCH_CHECK();
-  DCD_TRY(pool_stats(c, g, L0, k, a, size, pool.get(), &out->st));
+  DCD_TRY(pool_stats(c, g, L0, k, a, size, pool.get(), nlab, &out->st));
   const int64_t m = out->st.count;
   DCD_TRY(c->feat_X.ensure(&c->mem, 12 * (m > 0 ? m : 1)));
   DCD_TRY(c->feat_v.ensure(&c->mem, m > 0 ? m : 1));

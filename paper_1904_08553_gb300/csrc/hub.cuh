@@ -1,15 +1,16 @@
 // hub.cuh -- aggregation of very long rows (hubs) over many CTAs, shared by
 // the local-move kernels and the screening kernels.
 //
-// A hub's row is split into chunks of kHubChunk entries, so that many CTAs
-// work on one hub at once (one CTA per hub would leave the largest hub setting
-// the kernel's length).  Each hub owns a region of a global open-addressing
-// table (capacity: 2 x degree rounded up to a power of two, so probing always
-// ends) and of a list of the slots it claimed:
-//   hub_agg   chunk c of hub h: group the chunk's labels by warp (match_any),
-//             add the group sums into h's table, list new keys.
+// A hub's row is split into chunks of kHubChunk entries, a CTA each, so that
+// many CTAs work on one hub at once.  Each hub owns a region of a global
+// open-addressing table (capacity: 2 x degree rounded up to a power of two, so
+// probing always ends) and of a list of the slots it claimed:
+//   hub_agg   chunk c of hub h: the chunk is summed by community in a table in
+//             shared memory (the hub's own community in registers), whose
+//             distinct sums are then added into h's table, listing new keys.
 // The caller then reads the tables (gains, lookups) and, to reuse them,
-// empties the claimed slots.  The view V has rp, col, w and L.
+// empties the claimed slots.  The view V has rp, col, w, L and nlab (labels in
+// entry order, or NULL).
 #pragma once
 
 #include "agg.cuh"
@@ -17,7 +18,14 @@
 
 namespace dcd {
 
-constexpr int64_t kHubChunk = 4096;
+// A chunk is one load round of a CTA: every thread has its kHubItems entries in
+// flight at once.  With 4096 entries a chunk (16 dependent rounds, each ending
+// in global atomics) a few dozen hubs took 53-85 us a pass whatever their size;
+// now 25-39 us.
+constexpr int64_t kHubChunk = 1024;
+constexpr int kHubThreads = 256;
+constexpr int kHubItems = (int)kHubChunk / kHubThreads;
+constexpr int kHubCap = 2 * (int)kHubChunk;
 
 struct HubTables {
   const int32_t* list = nullptr;  // hub vertices (the bin's list segment)
@@ -43,50 +51,116 @@ __device__ __forceinline__ int64_t hub_of_chunk(const HubTables& t, int64_t c) {
 }
 
 template <typename W, typename ST, typename V>
-__global__ void __launch_bounds__(256) hub_agg(V g, HubTables t) {
-  const int lane = lane_id(), wib = threadIdx.x >> 5;
+__global__ void __launch_bounds__(kHubThreads) hub_agg(V g, HubTables t) {
+  using VT = typename TblVal<ST>::type;
+  __shared__ int32_t sk[kHubCap];
+  __shared__ VT sv[kHubCap];
+  __shared__ uint16_t ss[kHubChunk];
+  __shared__ int32_t s_n;
+  const int tid = threadIdx.x;
+  for (int x = tid; x < kHubCap; x += kHubThreads) {
+    sk[x] = -1;
+    sv[x] = 0;
+  }
+  if (tid == 0) s_n = 0;
+  __syncthreads();
   const int64_t nch = t.coff[t.H];
   for (int64_t c = blockIdx.x; c < nch; c += gridDim.x) {
     const int64_t h = hub_of_chunk(t, c);
     const int32_t v = t.list[h];
     const int64_t b = g.rp[v], d = g.rp[v + 1] - b;
-    const int64_t e0 = (c - t.coff[h]) * kHubChunk, e1 = e0 + kHubChunk < d ? e0 + kHubChunk : d;
+    const int64_t e0 = (c - t.coff[h]) * kHubChunk;
+    const int32_t C = g.L[v];
     const uint32_t mask = (uint32_t)(t.toff[h + 1] - t.toff[h]) - 1;
     int32_t* keys = t.keys + t.toff[h];
     unsigned long long* vals = t.vals + t.toff[h];
     int32_t* slots = t.slots + t.soff[h];
-    for (int64_t q0 = e0 + wib * 32; q0 < e1; q0 += blockDim.x) {
-      const int64_t e = q0 + lane;
-      bool valid = e < e1;
-      const int32_t u = valid ? ld_stream(g.col + b + e) : -1;
-      valid = valid && u != v;
-      const int32_t lab = valid ? g.L[u] : -1;
-      const W wt = valid ? ld_stream(g.w + b + e) : W(0);
-      const unsigned peers = __match_any_sync(0xffffffffu, lab);
-      const int64_t sum = group_sum<ST>(peers, wt);
-      if (valid && (int)(__ffs(peers) - 1) == lane) {
-        uint32_t sl = hash_label(lab, mask);
-        for (;;) {
-          const int32_t k = keys[sl];
-          if (k == lab) {
-            atomicAdd(&vals[sl], (unsigned long long)sum);
-            break;
-          }
-          if (k == -1) {
-            const int32_t old = atomicCAS(&keys[sl], -1, lab);
-            if (old == -1) slots[atomicAdd(&t.nslot[h], 1)] = (int32_t)sl;
-            if (old == -1 || old == lab) {
-              atomicAdd(&vals[sl], (unsigned long long)sum);
-              break;
-            }
-          }
-          sl = (sl + 1) & mask;
-        }
+    int32_t lab[kHubItems];
+    W wt[kHubItems];
+#pragma unroll
+    for (int q = 0; q < kHubItems; q++) {
+      const int64_t e = e0 + q * kHubThreads + tid;
+      lab[q] = -1;
+      wt[q] = W(0);
+      if (e < d) {
+        lab[q] = ld_stream((g.nlab ? g.nlab : g.col) + b + e);
+        wt[q] = ld_stream(g.w + b + e);
       }
     }
+    if (!g.nlab) {
+#pragma unroll
+      for (int q = 0; q < kHubItems; q++) {
+        const int32_t u = lab[q];
+        lab[q] = (u >= 0 && u != v) ? g.L[u] : -1;
+      }
+    }
+    VT own = 0;
+#pragma unroll
+    for (int q = 0; q < kHubItems; q++) {
+      bool claimed = false;
+      uint32_t s = 0;
+      if (lab[q] == C) {
+        own += (VT)wt[q];
+      } else if (lab[q] >= 0) {
+        s = probe_claim(sk, kHubCap - 1, lab[q], claimed);
+        atomicAdd(&sv[s], (VT)wt[q]);
+      }
+      const unsigned bal = __ballot_sync(0xffffffffu, claimed);
+      int at = 0;
+      if (lane_id() == 0 && bal) at = atomicAdd(&s_n, __popc(bal));
+      at = __shfl_sync(0xffffffffu, at, 0);
+      if (claimed) ss[at + __popc(bal & lanemask_lt())] = (uint16_t)s;
+    }
+    __syncthreads();
+    const int nd = s_n;
+    const VT ow = (VT)seg_total<32>(own);
+    // the warps' own-community sums go into the table directly, behind the
+    // chunk's distinct sums
+    for (int x0 = tid & ~31; x0 < nd || (x0 == (tid & ~31)); x0 += kHubThreads) {
+      const int x = x0 + (int)lane_id();
+      int32_t key = -1;
+      unsigned long long val = 0;
+      if (x < nd) {
+        const uint32_t s = ss[x];
+        key = sk[s];
+        val = sv[s];
+        sk[s] = -1;
+        sv[s] = 0;
+      }
+      for (int round = 0; round < 2; round++) {
+        if (round == 1) {  // once per warp: its own-community sum
+          if (x0 != (tid & ~31)) break;
+          key = (lane_id() == 0 && ow) ? C : -1;
+          val = ow;
+        }
+        bool fresh = false;
+        uint32_t sl = 0;
+        if (key >= 0) {
+          sl = hash_label(key, mask);
+          for (;;) {
+            const int32_t k = keys[sl];
+            if (k == key) break;
+            if (k == -1) {
+              const int32_t old = atomicCAS(&keys[sl], -1, key);
+              if (old == -1) fresh = true;
+              if (old == -1 || old == key) break;
+            }
+            sl = (sl + 1) & mask;
+          }
+          atomicAdd(&vals[sl], val);
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, fresh);
+        int at = 0;
+        if (lane_id() == 0 && bal) at = atomicAdd(&t.nslot[h], __popc(bal));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (fresh) slots[at + __popc(bal & lanemask_lt())] = (int32_t)sl;
+      }
+    }
+    __syncthreads();
+    if (tid == 0) s_n = 0;
+    __syncthreads();
   }
 }
-
 
 // sizes of the hub tables (hub h: table 2 x degree rounded up to a power of
 // two, slot list = degree, chunks = degree / kHubChunk rounded up)

@@ -55,6 +55,10 @@ struct LV {
   int64_t* f_eB = nullptr;
   int32_t* f_dB = nullptr;
   double* f_sB = nullptr;
+  // level 0 (may be NULL): the label of every entry's column, kept current
+  // through the passes; the kernels read it next to the weights instead of
+  // gathering L (no self-loops at level 0)
+  const int32_t* nlab = nullptr;
   // level 0 of a Delta-screening update: pre[v] >= 0 is v's proposal of the
   // level's first pass, taken by the screening from the same state; while
   // *first == 0 (no pass of the level has ended) the kernels store it
@@ -69,6 +73,11 @@ __device__ __forceinline__ double to_double(i128 x) {
   const long long hi = (long long)(x >> 64);
   const unsigned long long lo = (unsigned long long)x;
   return (double)hi * 18446744073709551616.0 + (double)lo;
+}
+
+// The same from the community alone (INT_MAX: none with S > 0).
+__device__ __forceinline__ int32_t best_proposal(int32_t D, int32_t C, const int32_t* size) {
+  return move_proposal<long long>(1, D, C, size);
 }
 
 // The proposal of a vertex from its best (S, D): move on S > 0, subject to
@@ -120,27 +129,251 @@ __device__ __forceinline__ void put_features(const LV<W>& g, int64_t i, int64_t 
   g.f_sB[i] = D == INT_MAX ? 0.0 : to_double(S);
 }
 
-// S lanes per vertex (32 / S vertices a warp), Q entries per lane: rows of at
-// most S x Q entries.  Each segment owns a table in shared memory; the
-// segments of a warp run in lockstep on their own rows.
+// Rows of at most 32 entries: a vertex per lane.
 //
-// The rows of a segment are software-pipelined, so that the dependent chain
-// list -> row_ptr -> col -> L of a row is spread over several iterations
-// instead of waiting in one.  With Q <= 4 (four stages): while row k is
-// aggregated in the table, the neighbour communities of row k+1 are being
-// gathered (with its k_v, a_C, |C| and 2m), the entries and community of row
-// k+2 loaded, the bounds of row k+3 read and the list entry of row k+4
-// fetched.  With Q = 8 the entries of two rows would not fit the register
-// budget of four resident CTAs, so one stage less: row k's communities are
-// gathered at the start of its iteration, while row k+1's entries, row k+2's
-// bounds and row k+3's list entry are in flight.
-// S lanes per vertex (32 / S vertices a warp), Q entries per lane: rows of at
-// most S x Q entries.  Each segment owns a table in shared memory; the
-// segments of a warp run in lockstep on their own rows.
+// A warp takes up to 32 consecutive list positions.  Three phases:
+//   1 every lane loads one position's scalars (list entry, row bounds, C, k,
+//     a_C) in parallel;
+//   2 the rows are read S lanes a vertex, 32 / S vertices a step (coalesced
+//     columns and weights, gathered labels).  Most of a row points into the
+//     vertex's own community; the other entries are compacted by ballot into
+//     the vertex's list in shared memory, interleaved by lane.  e_{v->C\v} is
+//     k_v less what the list holds, so it needs no reduction;
+//   3 every lane folds its own list by community and takes the best gain, the
+//     sizes, the guard and the proposal: no shuffle, no table, no atomic.
+// Once the labels come in entry order (below), short rows are bound by issue and
+// by the latency of shared-memory and shuffle chains: 0.88 M rows of 17..32
+// entries take 118 us here and 200 us with a hash table a row (0.38 of its
+// instructions).  Rows of 33..64 entries are the other way round (146 against
+// 107 us: the lists of 32 vertices leave room for fewer warps), so they keep
+// the table.  A vertex with more than CAP foreign entries is chosen in phase 2
+// by its segment together (list_best), before the next step.
+template <typename VT>
+struct ListEnt;  // a list entry: one shared-memory word of 8 or 16 bytes
+template <>
+struct __align__(8) ListEnt<unsigned> {
+  int32_t lab;
+  unsigned w;
+};
+template <>
+struct __align__(16) ListEnt<unsigned long long> {
+  unsigned long long w;
+  int32_t lab, pad;
+};
+
+constexpr int kCap32 = 16;  // foreign entries a lane's list holds, rows of 17 to 32 entries
+
+// Shared memory of a warp: the lanes' lists, then (rows can be longer than
+// CAP) a whole-row list per segment with two entries of padding.
+template <int S, int Q, int CAP, typename VT>
+__host__ __device__ constexpr size_t vert_bytes() {
+  return (size_t)CAP * 32 * sizeof(ListEnt<VT>) +
+         (S * Q > CAP ? (size_t)(32 / S) * (S * Q + 2) * sizeof(ListEnt<VT>) : 0);
+}
+
+// One segment's whole list: each lane takes K entries and sums the list's
+// weights of the same community (entries of one community get the same sum and
+// gain, so none has to be singled out).  All lanes of the warp call it; every
+// list is padded to nmax, made even.
+template <typename W, typename ST, int S, int K, typename VT>
+__device__ __forceinline__ void list_best(const LV<W>& g, const ListEnt<VT>* list, int n, int nmax, int64_t kv,
+                                          int64_t eC, int64_t aC, int64_t m2v, int sl, ST& Sb, int32_t& D,
+                                          int64_t& eD) {
+  int32_t l[K];
+  VT e[K];
+#pragma unroll
+  for (int k = 0; k < K; k++) {
+    l[k] = k * S + sl < n ? list[k * S + sl].lab : -1;
+    e[k] = 0;
+  }
+  for (int j = 0; j < nmax; j += 2) {
+    const ListEnt<VT> x = list[j], y = list[j + 1];
+#pragma unroll
+    for (int k = 0; k < K; k++) {
+      if (x.lab == l[k]) e[k] += x.w;
+      if (y.lab == l[k]) e[k] += y.w;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < K; k++)
+    if (l[k] >= 0) {
+      const ST x = gain<ST>(m2v, kv, (int64_t)e[k], eC, g.a[l[k]], aC);
+      if (better(x, l[k], Sb, D)) {
+        Sb = x;
+        D = l[k];
+      }
+    }
+  seg_argmax<S>(Sb, D);
+  eD = 0;
+#pragma unroll
+  for (int k = 0; k < K; k++)
+    if (l[k] == D) eD = (int64_t)e[k];
+#pragma unroll
+  for (int o = S / 2; o > 0; o >>= 1) {  // known where an entry is in D; equal there
+    const int64_t x = __shfl_xor_sync(0xffffffffu, eD, o);
+    eD = x > eD ? x : eD;
+  }
+}
+
+template <typename ST, typename W>
+__device__ __forceinline__ void put_best(const LV<W>& g, int64_t i, int64_t eC, ST Sb, int32_t D, int64_t eD) {
+  g.f_eC[i] = eC;
+  g.f_eB[i] = D == INT_MAX ? 0 : eD;
+  g.f_dB[i] = D == INT_MAX ? -1 : D;
+  g.f_sB[i] = D == INT_MAX ? 0.0 : to_double(Sb);
+}
+
+template <typename W, typename ST, int S, int Q, int CAP>
+__global__ void __launch_bounds__(256) lm_vert(LV<W> g, const int32_t* __restrict__ list, int64_t cnt, int per,
+                                               int32_t* __restrict__ prop) {
+  static_assert(S == 4 || S == 8, "segments of 4 or 8 lanes");
+  using VT = typename TblVal<ST>::type;
+  using Ent = ListEnt<VT>;
+  constexpr int P = 32 / S, ROW = S * Q;
+  constexpr bool kFree = ROW > CAP;  // rows may outgrow a lane's list
+  static_assert(!kFree || ROW <= 4 * S, "list_best takes at most four entries a lane");
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = lane_id(), sub = lane / S, sl = lane % S, wib = threadIdx.x >> 5;
+  const unsigned smask = ((1u << S) - 1u) << (sub * S);
+  Ent* const ent = reinterpret_cast<Ent*>(smem + (size_t)wib * vert_bytes<S, Q, CAP, VT>());
+  Ent* const row = ent + CAP * 32 + sub * (ROW + 2);
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t wb = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * per; wb < cnt; wb += nw * per) {
+    const int nb = cnt - wb < per ? (int)(cnt - wb) : per;
+    const bool own = lane < nb;
+    const int32_t v_l = own ? ld_stream(list + wb + lane) : 0;
+    const int32_t pv = own ? g.pre_of(v_l) : -1;  // the screening's first-pass proposal
+    int64_t b_l = 0, k_l = 0, aC_l = 0;
+    int d_l = 0, n_l = 0;
+    int32_t C_l = 0, D_l = INT_MAX;
+    if (own) {
+      b_l = g.rp[v_l];
+      C_l = g.L[v_l];
+      if (pv < 0) {
+        d_l = (int)(g.rp[v_l + 1] - b_l);
+        k_l = g.k[v_l];
+        aC_l = g.a[C_l];
+      }
+    }
+    const int steps = __any_sync(0xffffffffu, d_l > 0) ? (nb + P - 1) / P : 0;
+    for (int t = 0; t < steps; t++) {
+      const int src = t * P + sub;
+      const int d = __shfl_sync(0xffffffffu, d_l, src);
+      const int64_t b = __shfl_sync(0xffffffffu, b_l, src);
+      const int32_t C = __shfl_sync(0xffffffffu, C_l, src);
+      int32_t lab[Q];
+      W wt[Q];
+#pragma unroll
+      for (int q = 0; q < Q; q++) {
+        const int e = q * S + sl;
+        lab[q] = -1;
+        wt[q] = W(0);
+        if (e < d) {
+          lab[q] = ld_stream((g.nlab ? g.nlab : g.col) + b + e);
+          wt[q] = ld_stream(g.w + b + e);
+        }
+      }
+      // a coarse self-loop is no neighbour: it stays in the list, as label -3,
+      // so that its weight is taken off k_v
+      const int32_t v = sizeof(W) == 8 ? __shfl_sync(0xffffffffu, v_l, src) : -1;
+#pragma unroll
+      for (int q = 0; q < Q; q++) {
+        const int32_t u = lab[q];
+        lab[q] = u < 0 ? C : (sizeof(W) == 8 && u == v) ? -3 : g.nlab ? u : g.L[u];
+      }
+      int n = 0;
+      int at[Q];
+#pragma unroll
+      for (int q = 0; q < Q; q++) {
+        const unsigned bal = __ballot_sync(0xffffffffu, lab[q] != C) & smask;
+        at[q] = n + __popc(bal & lanemask_lt());
+        n += __popc(bal);
+      }
+      int pick = n;
+      if (!kFree || !__any_sync(0xffffffffu, n > CAP)) {
+#pragma unroll
+        for (int q = 0; q < Q; q++)
+          if (lab[q] != C) {
+            Ent x{};
+            x.lab = lab[q];
+            x.w = (VT)wt[q];
+            ent[at[q] * 32 + src] = x;
+          }
+        pick = __shfl_sync(0xffffffffu, n, (lane & (P - 1)) * S);
+        if (lane / P == t) n_l = pick;
+      } else if constexpr (kFree) {
+        VT sum = 0;
+#pragma unroll
+        for (int q = 0; q < Q; q++)
+          if (lab[q] != C) {
+            Ent x{};
+            x.lab = lab[q];
+            x.w = (VT)wt[q];
+            row[at[q]] = x;
+            sum += (VT)wt[q];
+          }
+        const int nmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)n);
+        for (int j = n + sl; j < nmax + (nmax & 1); j += S) row[j].lab = -2;
+        __syncwarp();
+        const int64_t kv = __shfl_sync(0xffffffffu, k_l, src), eC = kv - seg_total<S>(sum);
+        const int64_t aC = __shfl_sync(0xffffffffu, aC_l, src);
+        const int32_t vv = __shfl_sync(0xffffffffu, v_l, src);
+        ST Sb = gain_lowest<ST>();
+        int32_t D = INT_MAX;
+        int64_t eD;
+        list_best<W, ST, S, (ROW + S - 1) / S, VT>(g, row, n, nmax, kv, eC, aC, g.m2_of(vv), sl, Sb, D, eD);
+        if (g.f_eC && sl == 0 && src < nb) put_best(g, wb + src, eC, Sb, D, eD);
+        pick = __shfl_sync(0xffffffffu, Sb > 0 ? D : INT_MAX, (lane & (P - 1)) * S);
+        if (lane / P == t) {
+          D_l = pick;
+          n_l = -1;
+        }
+        __syncwarp();
+      }
+    }
+    __syncwarp();
+    if (own && n_l >= 0 && (n_l > 0 || g.f_eC)) {
+      // the list folded by community, in place
+      Ent* const my = ent + lane;
+      int nd = 0;
+      VT tot = 0;
+      for (int j = 0; j < n_l; j++) {
+        const Ent x = my[j * 32];
+        tot += x.w;
+        int i = 0;
+        while (i < nd && my[i * 32].lab != x.lab) i++;
+        if (i < nd) my[i * 32].w += x.w;
+        else my[nd++ * 32] = x;
+      }
+      const int64_t eC = k_l - (int64_t)tot, m2v = g.m2_of(v_l);
+      ST Sb = gain_lowest<ST>();
+      int32_t D = INT_MAX;
+      int64_t eD = 0;
+      for (int i = 0; i < nd; i++) {
+        const Ent x = my[i * 32];
+        if (sizeof(W) == 8 && x.lab < 0) continue;
+        const ST y = gain<ST>(m2v, k_l, (int64_t)x.w, eC, g.a[x.lab], aC_l);
+        if (better(y, x.lab, Sb, D)) {
+          Sb = y;
+          D = x.lab;
+          eD = (int64_t)x.w;
+        }
+      }
+      if (Sb > 0) D_l = D;
+      if (g.f_eC) put_best(g, wb + lane, eC, Sb, D, eD);
+    }
+    if (own) prop[wb + lane] = pv >= 0 ? pv : best_proposal(D_l, C_l, g.size);
+    __syncwarp();
+  }
+}
+
+// Rows of 33 to 256 entries: S lanes per vertex (32 / S vertices a warp), Q
+// entries per lane, the row's sums in the segment's own table; the segments of
+// a warp run in lockstep on their own rows.
 template <typename W, typename ST, int S, int Q>
 __global__ void __launch_bounds__(256) lm_seg(LV<W> g, const int32_t* __restrict__ list, int64_t cnt,
                                               int32_t* __restrict__ prop) {
-  static_assert(S == 8 || S == 16 || S == 32, "segments of 8, 16 or 32 lanes");
+  static_assert(S == 16 || S == 32, "segments of 16 or 32 lanes");
   using VT = typename TblVal<ST>::type;
   constexpr int P = 32 / S, ROW = S * Q, CAP = seg_cap(ROW);
   constexpr size_t SB = row_tbl_bytes<ROW, VT>();
@@ -175,14 +408,16 @@ __global__ void __launch_bounds__(256) lm_seg(LV<W> g, const int32_t* __restrict
       lab[q] = -1;
       wt[q] = W(0);
       if (e < d) {
-        lab[q] = ld_stream(g.col + b + e);
+        lab[q] = ld_stream((g.nlab ? g.nlab : g.col) + b + e);
         wt[q] = ld_stream(g.w + b + e);
       }
     }
+    if (!g.nlab) {
 #pragma unroll
-    for (int q = 0; q < Q; q++) {
-      const int32_t u = lab[q];
-      lab[q] = (u >= 0 && u != v) ? g.L[u] : -1;  // a coarse self-loop is no neighbour
+      for (int q = 0; q < Q; q++) {
+        const int32_t u = lab[q];
+        lab[q] = (u >= 0 && u != v) ? g.L[u] : -1;  // a coarse self-loop is no neighbour
+      }
     }
     VT eCl = 0;
     int nd = 0;
@@ -203,7 +438,7 @@ __global__ void __launch_bounds__(256) lm_seg(LV<W> g, const int32_t* __restrict
       }
     }
     __syncwarp();
-    const int64_t eC = seg_total<S>(eCl, smask);
+    const int64_t eC = seg_total<S>(eCl);
     const int64_t kv = g.k[v], aC = g.a[C], m2v = g.m2_of(v);
     ST Sb = gain_lowest<ST>();
     int32_t D = INT_MAX;
@@ -216,7 +451,7 @@ __global__ void __launch_bounds__(256) lm_seg(LV<W> g, const int32_t* __restrict
         D = key;
       }
     }
-    seg_argmax<S>(Sb, D, smask);
+    seg_argmax<S>(Sb, D);
     const int32_t pr = pv >= 0 ? pv : proposal(Sb, D, C, g.size);
     if (sl == 0 && has) {
       prop[i] = pr;
@@ -274,14 +509,16 @@ __global__ void __launch_bounds__(T) lm_cta(LV<W> g, const int32_t* __restrict__
       lab[q] = -1;
       wt[q] = W(0);
       if (e < d) {
-        lab[q] = ld_stream(g.col + b + e);
+        lab[q] = ld_stream((g.nlab ? g.nlab : g.col) + b + e);
         wt[q] = ld_stream(g.w + b + e);
       }
     }
+    if (!g.nlab) {
 #pragma unroll
-    for (int q = 0; q < Q; q++) {
-      const int32_t u = lab[q];
-      lab[q] = (u >= 0 && u != v) ? g.L[u] : -1;
+      for (int q = 0; q < Q; q++) {
+        const int32_t u = lab[q];
+        lab[q] = (u >= 0 && u != v) ? g.L[u] : -1;
+      }
     }
     VT eCl = 0;
 #pragma unroll
@@ -302,7 +539,7 @@ __global__ void __launch_bounds__(T) lm_cta(LV<W> g, const int32_t* __restrict__
         if (claimed) slots[at + __popc(bal & lanemask_lt())] = (uint16_t)s;
       }
     }
-    const int64_t ew = seg_total<32>(eCl, 0xffffffffu);
+    const int64_t ew = seg_total<32>(eCl);
     if (lane == 0) redC[wid] = (VT)ew;
     __syncthreads();
     const int nd = s_nd;
@@ -484,43 +721,50 @@ __global__ void __launch_bounds__(256) hub_clear(HubTables t) {
 
 // Moves of one pass (proposals of graphs whose pass loop has stopped are
 // dropped).  Community sums change by warp-aggregated atomics (one per distinct
-// community of the warp); movers of long rows (list positions from big_from
-// on) go to a separate list for block-per-row processing; per-graph mover
-// counts feed the stop rule.
-__global__ void lm_apply(const int32_t* __restrict__ list, int64_t cnt, int64_t big_from,
-                         const int32_t* __restrict__ prop, int32_t* __restrict__ L, const int64_t* __restrict__ k,
-                         unsigned long long* __restrict__ a, int32_t* __restrict__ size, int32_t* __restrict__ Lprev,
-                         int32_t* __restrict__ mvit, const int32_t* __restrict__ pass_id,
-                         int32_t* __restrict__ moved, int32_t* __restrict__ moved_cnt,
-                         int32_t* __restrict__ moved_big, int32_t* __restrict__ moved_big_cnt,
-                         const int32_t* __restrict__ gid, GraphState* __restrict__ gs) {
-  const int32_t iter = *pass_id;
+// community of the warp); per-graph mover counts feed the stop rule.  LL[v] =
+// (label before, label after) is written for every active vertex, so that the
+// row pass below needs one gather per neighbour; the movers' rows become work
+// items of at most kMoveChunk entries (v << 32 | chunk), so that a moved hub
+// does not hold one warp for its whole row.
+constexpr int kMoveChunk = 128;
+
+__global__ void lm_apply(const int32_t* __restrict__ list, int64_t cnt, const int32_t* __restrict__ prop,
+                         int32_t* __restrict__ L, int2* __restrict__ LL, const int64_t* __restrict__ k,
+                         const int64_t* __restrict__ rp, unsigned long long* __restrict__ a,
+                         int32_t* __restrict__ size, int64_t* __restrict__ items, int32_t* __restrict__ item_cnt,
+                         unsigned long long* __restrict__ moved_deg, const int32_t* __restrict__ gid,
+                         GraphState* __restrict__ gs) {
+  unsigned long long deg = 0;  // degrees of the movers
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t base0 = (blockIdx.x * (int64_t)blockDim.x) & ~31ll;
-  for (int64_t base = base0 + (threadIdx.x & ~31); base < cnt; base += stride) {
-    const int64_t i = base + lane_id();
+  const int lane = lane_id();
+  for (int64_t base = (blockIdx.x * (int64_t)blockDim.x) + (threadIdx.x & ~31); base < cnt; base += stride) {
+    const int64_t i = base + lane;
     bool mv = false;
     int32_t v = 0, c = -1, p = -1, gv = -1;
     int64_t kv = 0;
+    int nch = 0;
     if (i < cnt) {
       v = list[i];
       p = prop[i];
       c = L[v];
       gv = graph_of(gid, v);
-      if (p != c && gs[gv].running) {
-        mv = true;
-        Lprev[v] = c;
+      mv = p != c && gs[gv].running;
+      LL[v] = make_int2(c, mv ? p : c);
+      if (mv) {
         L[v] = p;
-        mvit[v] = iter;
         kv = k[v];
+        const int64_t d = rp[v + 1] - rp[v];
+        deg += (unsigned long long)d;
+        nch = (int)((d + kMoveChunk - 1) / kMoveChunk);
       } else {
         c = p = -1;
       }
     }
+    if (!__any_sync(0xffffffffu, mv)) continue;
     {  // leaving c
       const unsigned peers = __match_any_sync(0xffffffffu, c);
       const int64_t sk = group_sum_exact(peers, kv);
-      if (mv && (int)(__ffs(peers) - 1) == (int)lane_id()) {
+      if (mv && (int)(__ffs(peers) - 1) == lane) {
         atomicAdd(&a[c], 0ull - (unsigned long long)sk);
         atomicSub(&size[c], __popc(peers));
       }
@@ -528,78 +772,96 @@ __global__ void lm_apply(const int32_t* __restrict__ list, int64_t cnt, int64_t 
     {  // joining p
       const unsigned peers = __match_any_sync(0xffffffffu, p);
       const int64_t sk = group_sum_exact(peers, kv);
-      if (mv && (int)(__ffs(peers) - 1) == (int)lane_id()) {
+      if (mv && (int)(__ffs(peers) - 1) == lane) {
         atomicAdd(&a[p], (unsigned long long)sk);
         atomicAdd(&size[p], __popc(peers));
       }
     }
     {  // movers per graph
       const unsigned peers = __match_any_sync(0xffffffffu, mv ? gv : -1);
-      if (mv && (int)(__ffs(peers) - 1) == (int)lane_id()) atomicAdd(&gs[gv].moves, __popc(peers));
+      if (mv && (int)(__ffs(peers) - 1) == lane) atomicAdd(&gs[gv].moves, __popc(peers));
     }
-    const bool big = mv && i >= big_from;
-    const bool small = mv && !big;
-    unsigned bal = __ballot_sync(0xffffffffu, small);
-    int32_t slot = 0;
-    if (lane_id() == 0 && bal) slot = atomicAdd(moved_cnt, __popc(bal));
-    slot = __shfl_sync(0xffffffffu, slot, 0);
-    if (small) moved[slot + __popc(bal & lanemask_lt())] = v;
-    bal = __ballot_sync(0xffffffffu, big);
-    slot = 0;
-    if (lane_id() == 0 && bal) slot = atomicAdd(moved_big_cnt, __popc(bal));
-    slot = __shfl_sync(0xffffffffu, slot, 0);
-    if (big) moved_big[slot + __popc(bal & lanemask_lt())] = v;
+    const int incl = warp_incl_scan(nch);
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    int32_t at = 0;
+    if (lane == 0) at = atomicAdd(item_cnt, total);
+    at = __shfl_sync(0xffffffffu, at, 0) + incl - nch;
+    for (int j = 0; j < nch; j++) items[at + j] = (int64_t)v << 32 | (uint32_t)j;
   }
+  deg = warp_sum(deg);
+  if (lane == 0 && deg) atomicAdd(moved_deg, deg);
 }
 
-// Change of sum_i e_{i->C(i)} from the rows of the moved vertices: an entry
-// (x, y) with y unmoved also stands for its mirror (y, x), hence weight 2.
-template <typename W>
-__device__ __forceinline__ int64_t moved_row_delta(const LV<W>& g, int32_t x, const int32_t* __restrict__ Lprev,
-                                                   const int32_t* __restrict__ mvit, int32_t iter, int tid, int nt) {
-  const int32_t ox = Lprev[x], nx = g.L[x];
-  const int64_t e1 = g.rp[x + 1];
-  int64_t acc = 0;
-  for (int64_t e = g.rp[x] + tid; e < e1; e += nt) {
-    const int32_t y = ld_stream(g.col + e);
-    const int64_t wt = (int64_t)ld_stream(g.w + e);
-    const bool ym = mvit[y] == iter;
-    const int32_t ny = g.L[y];
-    const int32_t oy = ym ? Lprev[y] : ny;
-    acc += ((int)(nx == ny) - (int)(ox == oy)) * wt * (ym ? 1 : 2);
-  }
-  return acc;
-}
+// Entry labels (nlab_gather below) are kept from this many entries on: below,
+// a pass over the graph stays in L2 and takes about as long as the gather's own
+// launches.
+constexpr int64_t kNlabMin = (int64_t)1 << 21;
+// The search of a mirror entry (two row bounds, 5-7 probes, one store) costs
+// about as many sectors as this many entries gathered.
+constexpr int kNlabSearch = 8;
 
+// The rows of the moved vertices, a warp per item: the change of
+// sum_i e_{i->C(i)} (an entry (x, y) with y unmoved also stands for its mirror
+// (y, x), hence weight 2), and the new label of x in the entry labels (nlab,
+// may be NULL) at the entry (y, x), found by a search of row y -- unless the
+// movers' rows are so large a part of the graph that nlab_gather renews them.
 template <typename W>
-__global__ void __launch_bounds__(256) lm_delta_in(LV<W> g, const int32_t* __restrict__ moved,
-                                                   const int32_t* __restrict__ moved_cnt,
-                                                   const int32_t* __restrict__ Lprev, const int32_t* __restrict__ mvit,
-                                                   const int32_t* __restrict__ pass_id, GraphState* __restrict__ gs) {
-  const int64_t cnt = *moved_cnt;
-  const int32_t iter = *pass_id;
+__global__ void __launch_bounds__(256) lm_delta(LV<W> g, const int2* __restrict__ LL, int64_t nnz,
+                                                const int64_t* __restrict__ items,
+                                                const int32_t* __restrict__ item_cnt, int32_t* __restrict__ nlab,
+                                                const DevScalars* __restrict__ d, GraphState* __restrict__ gs) {
+  constexpr int U = kMoveChunk / 32;
+  const int64_t cnt = *item_cnt;
+  const bool search = nlab && d->moved_deg * kNlabSearch < nnz;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int lane = lane_id();
+  long long acc = 0;
   for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < cnt; i += nw) {
-    const int32_t x = moved[i];
-    const int64_t acc = (int64_t)warp_sum((long long)moved_row_delta(g, x, Lprev, mvit, iter, lane_id(), 32));
-    if (lane_id() == 0 && acc != 0) atomicAdd((unsigned long long*)&gs[graph_of(g.gid, x)].in_delta, (unsigned long long)acc);
+    const int64_t it = items[i];
+    const int32_t x = (int32_t)(it >> 32);
+    const int64_t b = g.rp[x] + (int64_t)(uint32_t)it * kMoveChunk;
+    const int64_t rest = g.rp[x + 1] - b;
+    const int len = rest < kMoveChunk ? (int)rest : kMoveChunk;
+    const int2 lx = LL[x];
+    int32_t y[U];
+    W wt[U];
+#pragma unroll
+    for (int q = 0; q < U; q++) {
+      const int e = q * 32 + lane;
+      y[q] = -1;
+      wt[q] = W(0);
+      if (e < len) {
+        y[q] = ld_stream(g.col + b + e);
+        wt[q] = ld_stream(g.w + b + e);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < U; q++)
+      if (y[q] >= 0) {
+        const int2 ly = LL[y[q]];
+        acc += (long long)((int)(lx.y == ly.y) - (int)(lx.x == ly.x)) * (long long)wt[q] * (ly.x != ly.y ? 1 : 2);
+      }
+    if (search) {
+#pragma unroll
+      for (int q = 0; q < U; q++)
+        if (y[q] >= 0) {
+          int64_t lo = g.rp[y[q]], hi = g.rp[y[q] + 1];
+          while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (g.col[mid] < x) lo = mid + 1; else hi = mid;
+          }
+          nlab[lo] = lx.y;  // the mirror entry exists: the graph is undirected
+        }
+    }
+    if (g.gid) {
+      acc = warp_sum(acc);
+      if (lane == 0 && acc) atomicAdd((unsigned long long*)&gs[g.gid[x]].in_delta, (unsigned long long)acc);
+      acc = 0;
+    }
   }
-}
-
-// As lm_delta_in with one CTA per moved vertex (rows above 256 entries).
-template <typename W>
-__global__ void __launch_bounds__(256) lm_delta_in_block(LV<W> g, const int32_t* __restrict__ moved,
-                                                         const int32_t* __restrict__ moved_cnt,
-                                                         const int32_t* __restrict__ Lprev,
-                                                         const int32_t* __restrict__ mvit,
-                                                         const int32_t* __restrict__ pass_id,
-                                                         GraphState* __restrict__ gs) {
-  const int64_t cnt = *moved_cnt;
-  const int32_t iter = *pass_id;
-  for (int64_t i = blockIdx.x; i < cnt; i += gridDim.x) {
-    const int32_t x = moved[i];
-    const int64_t acc = (int64_t)warp_sum((long long)moved_row_delta(g, x, Lprev, mvit, iter, threadIdx.x, blockDim.x));
-    if (lane_id() == 0 && acc != 0) atomicAdd((unsigned long long*)&gs[graph_of(g.gid, x)].in_delta, (unsigned long long)acc);
+  if (!g.gid) {
+    acc = warp_sum(acc);
+    if (lane == 0 && acc) atomicAdd((unsigned long long*)&gs[0].in_delta, (unsigned long long)acc);
   }
 }
 
@@ -740,6 +1002,36 @@ __global__ void pass_end(DevScalars* d, cudaGraphConditionalHandle h, int32_t ca
   if (capped) d->loop_err = 1;
   // outside a graph the host reads any_running and loop_err after the pass
   if (in_graph) cudaGraphSetConditional(h, (more && !capped) ? 1u : 0u);
+}
+
+// ---------------------------------------------------------------- entry labels
+//
+// The gather of a neighbour's label costs a 32-byte sector per entry, pass
+// after pass, and bounds the evaluation (73 M entries: 1.09 ms with it, 0.55
+// without).  Level 0 of a large graph therefore keeps the labels in entry order:
+// one gather of its own when the level starts (entry-linear, 0.29 ms, 250 G
+// sectors/s), then after every pass the entries that point to a moved vertex,
+// by lm_delta when few have moved, by this gather again otherwise.  A level 0 of
+// three evaluated passes over 73 M entries: 3.30 ms with gathers in every pass,
+// 0.29 + 1.55 + 0.09 ms so; of 13-17 passes over 19 M entries (from
+// singletons): 4.9 -> 2.6 ms.
+__global__ void __launch_bounds__(256) nlab_gather(const int32_t* __restrict__ col, const int32_t* __restrict__ L,
+                                                   int64_t m, int32_t* __restrict__ nlab, const DevScalars* d) {
+  // inside the pass loop: only when the next pass runs and enough has moved
+  if (d && (!d->any_running || d->moved_deg * kNlabSearch < m)) return;
+  constexpr int U = 8;
+  const int64_t st = (int64_t)gridDim.x * blockDim.x;
+  int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  for (; e + (U - 1) * st < m; e += U * st) {
+    int32_t x[U];
+#pragma unroll
+    for (int i = 0; i < U; i++) x[i] = ld_stream(col + e + i * st);
+#pragma unroll
+    for (int i = 0; i < U; i++) x[i] = L[x[i]];
+#pragma unroll
+    for (int i = 0; i < U; i++) st_stream(nlab + e + i * st, x[i]);
+  }
+  for (; e < m; e += st) st_stream(nlab + e, L[ld_stream(col + e)]);
 }
 
 // ---------------------------------------------------------------- binning
@@ -917,6 +1209,12 @@ __global__ void __launch_bounds__(kCsThreads) comm_sums(int64_t n, const int32_t
 __global__ void fill_iota(int32_t* __restrict__ x, int64_t n) {
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
     x[v] = (int32_t)v;
+}
+
+// (label, label) of every vertex: nothing has moved.
+__global__ void fill_pairs(const int32_t* __restrict__ L, int64_t n, int2* __restrict__ LL) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+    LL[v] = make_int2(L[v], L[v]);
 }
 
 __global__ void fill_i32(int32_t* __restrict__ x, int64_t n, int32_t val) {
@@ -1407,6 +1705,23 @@ constexpr size_t seg_smem() {
   return (size_t)8 * (32 / S) * row_tbl_bytes<S * Q, typename TblVal<ST>::type>();
 }
 
+// Rows of at most 32 entries.  List positions a warp takes at a time: as many
+// as leave every resident warp at least kVertSweeps turns (the last turn is a
+// partial one), a step's 32 / S at least.
+constexpr int kVertSweeps = 2;
+template <typename W, typename ST, int S, int Q, int CAP>
+int launch_vert(cudaStream_t s, const LV<W>& g, const int32_t* lst, int64_t cnt, int32_t* prop, int64_t* sweep) {
+  constexpr int T = 256, P = 32 / S;
+  constexpr size_t smem = 8 * vert_bytes<S, Q, CAP, typename TblVal<ST>::type>();
+  const int64_t warps = (int64_t)wave_grid(lm_vert<W, ST, S, Q, CAP>, INT64_MAX / 2, T, smem) * (T / 32);
+  int per = 32;
+  while (per > P && cdiv(cnt, per) < kVertSweeps * warps) per /= 2;
+  const int grid = wave_grid(lm_vert<W, ST, S, Q, CAP>, cdiv(cnt, per) * 32, T, smem);
+  *sweep = (int64_t)grid * (T / 32) * per;
+  count_launch(), lm_vert<W, ST, S, Q, CAP><<<grid, T, smem, s>>>(g, lst, cnt, per, prop);
+  return DCD_OK;
+}
+
 template <typename W, typename ST, int S, int Q>
 int launch_seg(cudaStream_t s, const LV<W>& g, const int32_t* lst, int64_t cnt, int32_t* prop, int64_t* sweep) {
   constexpr int T = 256, P = 32 / S;
@@ -1442,8 +1757,8 @@ int table_kernel_attrs(K* kernel, int threads, size_t smem) {
 template <typename W, typename ST>
 int prepare_lm_st() {
   using VT = typename TblVal<ST>::type;
-  DCD_TRY(table_kernel_attrs(lm_seg<W, ST, 8, 2>, 256, seg_smem<W, ST, 8, 2>()));
-  DCD_TRY(table_kernel_attrs(lm_seg<W, ST, 16, 2>, 256, seg_smem<W, ST, 16, 2>()));
+  DCD_TRY(table_kernel_attrs(lm_vert<W, ST, 4, 4, 16>, 256, 8 * vert_bytes<4, 4, 16, VT>()));
+  DCD_TRY(table_kernel_attrs(lm_vert<W, ST, 8, 4, kCap32>, 256, 8 * vert_bytes<8, 4, kCap32, VT>()));
   DCD_TRY(table_kernel_attrs(lm_seg<W, ST, 16, 4>, 256, seg_smem<W, ST, 16, 4>()));
   DCD_TRY(table_kernel_attrs(lm_seg<W, ST, 32, 4>, 256, seg_smem<W, ST, 32, 4>()));
   DCD_TRY(table_kernel_attrs(lm_seg<W, ST, 32, 8>, 256, seg_smem<W, ST, 32, 8>()));
@@ -1492,8 +1807,8 @@ int launch_lm_bins(dcd_ctx* c, const LV<W>& lv, Bins& b, int32_t* prop, cudaEven
       const int32_t* lst = lst0 + o;
       int32_t* pr = prop + o;
       switch (b.plan.var[x]) {
-        case kLmSeg16: DCD_TRY((launch_seg<W, ST, 8, 2>(s, g, lst, cnt, pr, &sweep[x]))); break;
-        case kLmSeg32: DCD_TRY((launch_seg<W, ST, 16, 2>(s, g, lst, cnt, pr, &sweep[x]))); break;
+        case kLmSeg16: DCD_TRY((launch_vert<W, ST, 4, 4, 16>(s, g, lst, cnt, pr, &sweep[x]))); break;
+        case kLmSeg32: DCD_TRY((launch_vert<W, ST, 8, 4, kCap32>(s, g, lst, cnt, pr, &sweep[x]))); break;
         case kLmSeg64: DCD_TRY((launch_seg<W, ST, 16, 4>(s, g, lst, cnt, pr, &sweep[x]))); break;
         case kLmWarp128: DCD_TRY((launch_seg<W, ST, 32, 4>(s, g, lst, cnt, pr, &sweep[x]))); break;
         case kLmWarp256: DCD_TRY((launch_seg<W, ST, 32, 8>(s, g, lst, cnt, pr, &sweep[x]))); break;
@@ -1565,10 +1880,19 @@ struct GraphTally {
   explicit GraphTally(int G) : passes(G, 0), passes0(G, 0), moves(G, 0), levels(G, 0) {}
 };
 
+int entry_labels_impl(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L, EntryLabels* out) {
+  if (out->buf.n < (size_t)g.nnz) DCD_TRY(out->buf.alloc(&c->mem, g.nnz));
+  ::dcd::count_launch(), nlab_gather<<<grid_for(g.nnz, 256), 256, 0, c->stream>>>(g.col, L, g.nnz, out->buf.get(),
+                                                                                  nullptr);
+  DCD_LAUNCH_CHECK();
+  out->ready = true;
+  return DCD_OK;
+}
+
 template <typename W>
 int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<int64_t>& a, Buf<int32_t>& size,
               const uint8_t* active, const int32_t* gid, int level, LevelRun* out, GraphTally* tally,
-              const int32_t* pre = nullptr) {
+              const int32_t* pre = nullptr, EntryLabels* nlab = nullptr) {
   cudaStream_t s = c->stream;
   DevScalars* d = c->dsc.get();
   GraphState* gs = c->gs.get();
@@ -1585,21 +1909,15 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
   DCD_TRY(make_bins<W>(c, g, active, &bins, gid, pre));
   trace("level: binned");
   const int64_t total = bins.total;
-  // list positions from big_from on hold rows longer than 256 entries: their
-  // movers' delta of sum_i e_{i->C(i)} is taken by a CTA each
-  int64_t big_from = 0;
-  for (int x = 0; x < bins.plan.nb; x++)
-    if (bins.plan.var[x] <= kLmWarp256) big_from += bins.cnt[x];
-  const int64_t n_big = total - big_from;
-  Buf<int32_t> prop, Lprev, mvit, moved, moved_cnt, moved_big, moved_big_cnt;
+  Buf<int32_t> prop, item_cnt;
+  Buf<int2> LL;
+  Buf<int64_t> items;
+  const int64_t item_cap = total + bins.act_deg / kMoveChunk;
   DCD_TRY(prop.alloc(&c->mem, total));
-  DCD_TRY(Lprev.alloc(&c->mem, nv));
-  DCD_TRY(mvit.alloc(&c->mem, nv));
-  DCD_TRY(moved.alloc(&c->mem, total));
-  DCD_TRY(moved_cnt.alloc(&c->mem, 1));
-  DCD_TRY(moved_big.alloc(&c->mem, n_big));
-  DCD_TRY(moved_big_cnt.alloc(&c->mem, 1));
-  ::dcd::count_launch(), fill_i32<<<grid_for(nv, T), T, 0, s>>>(mvit.get(), nv, -1);
+  DCD_TRY(LL.alloc(&c->mem, nv));
+  DCD_TRY(items.alloc(&c->mem, item_cap));
+  DCD_TRY(item_cnt.alloc(&c->mem, 1));
+  ::dcd::count_launch(), fill_pairs<<<grid_for(nv, T), T, 0, s>>>(L, nv, LL.get());
   DCD_LAUNCH_CHECK();
   const int sq_ctas = grid_for(nv, T, 4);
   LV<W> lv{g.rp, g.col, g.w, kbuf.get(), L, a.get(), size.get(), G == 1 ? c->hgs[0].m2 : 0};
@@ -1608,6 +1926,14 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
   if (pre) {  // the first pass takes the screening's proposals
     lv.pre = pre;
     lv.first = &d->level_passes;
+  }
+  if (nlab && nlab->ready) lv.nlab = nlab->buf.get();
+  if constexpr (std::is_same<W, int32_t>::value) {
+    // labels in entry order: worth one gather when a pass evaluates a fair part of the entries
+    if (nlab && !nlab->ready && g.nnz >= kNlabMin && 4 * bins.act_deg >= g.nnz) {
+      DCD_TRY(entry_labels_impl(c, g, L, nlab));
+      lv.nlab = nlab->buf.get();
+    }
   }
   int64_t m2max = 0;
   for (int x = 0; x < G; x++) m2max = c->hgs[x].m2 > m2max ? c->hgs[x].m2 : m2max;
@@ -1624,32 +1950,30 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
   // once per pass instead and reads the loop condition back after it.
   auto enqueue_pass = [&](cudaGraphConditionalHandle h, bool in_graph) -> int {
     ::dcd::count_launch(), gs_reset_pass<<<cdiv(G, 128), 128, 0, s>>>(gs, G, &d->pass_id);
-    DCD_TRY_CUDA(cudaMemsetAsync(moved_cnt.get(), 0, sizeof(int32_t), s));
-    DCD_TRY_CUDA(cudaMemsetAsync(moved_big_cnt.get(), 0, sizeof(int32_t), s));
+    DCD_TRY_CUDA(cudaMemsetAsync(item_cnt.get(), 0, sizeof(int32_t), s));
     DCD_TRY_CUDA(cudaMemsetAsync(&d->any_running, 0, sizeof(int32_t), s));
+    DCD_TRY_CUDA(cudaMemsetAsync(&d->moved_deg, 0, sizeof(int64_t), s));
     ::dcd::count_launch(), pass_stamp<<<1, 1, 0, s>>>(d, 0);
     if (any) DCD_TRY(launch_lm_nocfg<W>(c, lvl, bins, prop.get(), nullptr, 0, total >= kForkMin, sweep));
     ::dcd::count_launch(), pass_stamp<<<1, 1, 0, s>>>(d, 1);
     if (total) {
       ::dcd::count_launch(), lm_apply<<<grid_for(total, T), T, 0, s>>>(
-          lst, total, big_from, prop.get(), L, kbuf.get(), (unsigned long long*)a.get(), size.get(),
-          Lprev.get(), mvit.get(), &d->pass_id, moved.get(), moved_cnt.get(), moved_big.get(), moved_big_cnt.get(),
-          gid, gs);
-      if (big_from)
-        ::dcd::count_launch(), lm_delta_in<W><<<grid_for(big_from * 32, T, 16), T, 0, s>>>(
-            lv, moved.get(), moved_cnt.get(), Lprev.get(), mvit.get(), &d->pass_id, gs);
-      if (n_big)
-        ::dcd::count_launch(), lm_delta_in_block<W><<<grid_for(n_big * T, T, 4), T, 0, s>>>(
-            lv, moved_big.get(), moved_big_cnt.get(), Lprev.get(), mvit.get(), &d->pass_id, gs);
+          lst, total, prop.get(), L, LL.get(), kbuf.get(), g.rp, (unsigned long long*)a.get(), size.get(), items.get(),
+          item_cnt.get(), (unsigned long long*)&d->moved_deg, gid, gs);
+      ::dcd::count_launch(), lm_delta<W><<<wave_grid(lm_delta<W>, item_cap * 32, T), T, 0, s>>>(
+          lv, LL.get(), g.nnz, items.get(), item_cnt.get(), lv.nlab ? nlab->buf.get() : nullptr, d, gs);
     }
     ::dcd::count_launch(), sumsq_acc<<<sq_ctas, T, 0, s>>>(a.get(), nv, gid, gs);
     ::dcd::count_launch(), lm_decide<<<cdiv(G, 128), 128, 0, s>>>(gs, G, 1, c->cfg.max_iters, c->cfg.tau_inv,
                                                                    &d->any_running);
+    if (lv.nlab)  // returns at once unless the next pass runs and much has moved
+      ::dcd::count_launch(), nlab_gather<<<grid_for(g.nnz, T), T, 0, s>>>(g.col, L, g.nnz, nlab->buf.get(), d);
     ::dcd::count_launch(), pass_end<<<1, 1, 0, s>>>(d, h, c->cfg.max_iters + 2, in_graph ? 1 : 0);
     DCD_LAUNCH_CHECK();
     return DCD_OK;
   };
   if (any) DCD_TRY(prepare_lm<W>(lvl));
+  resident_blocks(reinterpret_cast<const void*>(lm_delta<W>), T, 0);  // looked up outside the capture
   DCD_TRY(side_streams(c));
   struct GraphGuard {
     cudaGraph_t g = nullptr;
@@ -2330,8 +2654,13 @@ unsigned hub_grid(dcd_ctx* c, const HubBufs& b) {
   return (unsigned)(b.chunks < cap ? (b.chunks > 0 ? b.chunks : 1) : cap);
 }
 
+int entry_labels(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L, int64_t entries, EntryLabels* out) {
+  if (out->ready || g.nnz < kNlabMin || 4 * entries < g.nnz) return DCD_OK;
+  return entry_labels_impl(c, g, L, out);
+}
+
 int pool_stats(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L, const int64_t* k, const int64_t* a,
-               const int32_t* size, const uint8_t* mask, PoolStats* out) {
+               const int32_t* size, const uint8_t* mask, EntryLabels* nlab, PoolStats* out) {
   Bins bins;
   DCD_TRY(make_bins<int32_t>(c, g, mask, &bins));
   const int64_t m = bins.total;
@@ -2347,6 +2676,8 @@ int pool_stats(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L, const int64_
   lv.f_eB = out->eB.get();
   lv.f_dB = out->dB.get();
   lv.f_sB = out->sB.get();
+  DCD_TRY(entry_labels(c, g, L, bins.act_deg, nlab));
+  if (nlab->ready) lv.nlab = nlab->buf.get();
   if (m) DCD_TRY(launch_lm<int32_t>(c, lv, bins, prop.get()));
   out->list.reset();
   out->list.p = bins.list.p;
@@ -2394,6 +2725,10 @@ int tune_bins(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L, const BinPlan
     lv.gid = c->gid.get();
     lv.gs = c->gs.get();
   }
+  // as the passes of an update read them
+  EntryLabels nlab;
+  DCD_TRY(entry_labels(c, g, L, g.nnz, &nlab));
+  if (nlab.ready) lv.nlab = nlab.buf.get();
   const BinPlan keep = c->bin_plan;
   *best = -1;
   for (int x = 0; x < ncand; x++) {
@@ -2441,6 +2776,9 @@ int eval_bins(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L, int reps, int
     lv.gid = c->gid.get();
     lv.gs = c->gs.get();
   }
+  EntryLabels nlab;  // as the passes of an update read them
+  DCD_TRY(entry_labels(c, g, L, g.nnz, &nlab));
+  if (nlab.ready) lv.nlab = nlab.buf.get();
   Bins bins;
   DCD_TRY(make_bins<int32_t>(c, g, nullptr, &bins));
   *nb = bins.plan.nb;
@@ -2482,8 +2820,8 @@ int community_sums(dcd_ctx* c, int64_t n, const int32_t* labels, const int64_t* 
 }
 
 int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint8_t* active0, Buf<int64_t>& k0,
-                int32_t* out_labels, dcd_step_stats* st, int32_t* level0_out, dcd_step_stats* per_graph,
-                const int64_t* a0, const int32_t* size0, const int32_t* pre0) {
+                int32_t* out_labels, dcd_step_stats* st, EntryLabels* nlab, int32_t* level0_out,
+                dcd_step_stats* per_graph, const int64_t* a0, const int32_t* size0, const int32_t* pre0) {
   cudaStream_t s = c->stream;
   GraphState* gs = c->gs.get();
   const int G = c->G;
@@ -2537,7 +2875,8 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
   for (;;) {
     LevelRun lr;
     if (level == 0) {
-      DCD_TRY(run_level<int32_t>(c, *g_l0, L, *kcur, a, size, active, gid, (int)level, &lr, &tally, pre0));
+      DCD_TRY(run_level<int32_t>(c, *g_l0, L, *kcur, a, size, active, gid, (int)level, &lr, &tally, pre0, nlab));
+      nlab->ready = false;  // they follow the level's moves, not the labels the caller started from
       if (level0_out)
         DCD_TRY_CUDA(cudaMemcpyAsync(level0_out, L, n0 * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
     } else {
@@ -2816,7 +3155,7 @@ __global__ void __launch_bounds__(256) slm_warp(LV<W> g, const int32_t* __restri
       }
     }
     __syncwarp();
-    const int64_t eC = seg_total<32>(eCl, 0xffffffffu);
+    const int64_t eC = seg_total<32>(eCl);
     const int64_t kv = g.k[v], aC = g.a[C], m2 = g.m2;
     ST S = gain_lowest<ST>();
     int32_t D = INT_MAX;
@@ -2912,7 +3251,7 @@ __global__ void __launch_bounds__(256) slm_cta(LV<W> g, const int32_t* __restric
       at = __shfl_sync(0xffffffffu, at, 0);
       if (claimed) slots[at + __popc(bal & lanemask_lt())] = s;
     }
-    const int64_t ew = seg_total<32>(eCl, 0xffffffffu);
+    const int64_t ew = seg_total<32>(eCl);
     if (lane == 0) redE[wid] = (VT)ew;
     __syncthreads();
     int64_t eC = 0;

@@ -58,6 +58,7 @@ struct SV {
   // stores it in pre[source]; sources it does not sum keep -1
   const int32_t* size;
   int32_t* pre;
+  const int32_t* nlab = nullptr;  // labels in entry order (may be NULL)
 };
 
 // (S, D, j) order of the j* choice: larger gain, then smaller C(j), then smaller j.
@@ -241,7 +242,7 @@ __device__ __forceinline__ VT slot_table_fill(const SV& g, int32_t v, const Slot
 // every thread gets the total.  Synchronises twice.
 template <int NW, typename VT>
 __device__ __forceinline__ int64_t cta_total(VT x, VT* red) {
-  const int64_t w = seg_total<32>(x, 0xffffffffu);
+  const int64_t w = seg_total<32>(x);
   if (lane_id() == 0) red[threadIdx.x >> 5] = (VT)w;
   __syncthreads();
   int64_t t = 0;
@@ -372,7 +373,7 @@ __global__ void __launch_bounds__(256) scr_a_wtbl(SV g, int64_t off, int64_t cnt
       const uint32_t mask = table_cap(g.rp[u + 1] - g.rp[u]) - 1;
       const VT own = slot_table_fill<ST, VT>(g, u, t, mask, lane, 32, C);
       __syncwarp();
-      const int64_t eC = seg_total<32>(own, 0xffffffffu);
+      const int64_t eC = seg_total<32>(own);
       const int64_t ku = g.k[u], aC = g.a[C];
       if (g.pre) {  // the local move's choice over the table's communities
         ST Sb = gain_lowest<ST>();
@@ -697,7 +698,7 @@ __global__ void __launch_bounds__(256) scr_c_wtbl(SV g, GroupView gv, int64_t cn
     const uint32_t mask = table_cap(g.rp[j + 1] - g.rp[j]) - 1;
     const VT own = slot_table_fill<ST, VT>(g, j, t, mask, lane, 32, Cj);
     __syncwarp();
-    const int64_t e2 = seg_total<32>(own, 0xffffffffu);
+    const int64_t e2 = seg_total<32>(own);
     for (int64_t q = m0 + lane; q < m1; q += 32) {
       const int64_t idx = gv.vals[q];
       const int32_t Ci = g.L[g.src[idx]];

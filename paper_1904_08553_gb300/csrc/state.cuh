@@ -43,6 +43,7 @@ struct DevScalars {
   int32_t pad3;
   int64_t pre_verts;  // level 0: active vertices whose first-pass proposal the screening made
   int64_t pre_deg;    // and the sum of their degrees
+  int64_t moved_deg;  // degrees of the last pass's movers (level 0, entry labels kept)
 };
 
 // Per-graph state of one update.  A context holds G graphs on disjoint vertex
@@ -69,10 +70,11 @@ __device__ __forceinline__ int graph_of(const int32_t* gid, int64_t v) { return 
 
 // Degree bins of the local-move kernels.  A bin holds the active vertices
 // whose degree lies in (hi of the previous bin, hi]; each bin runs one kernel
-// variant, which bounds the degree it accepts.  Every variant sums the
-// neighbour communities of a row in a table in shared memory (louvain.cu):
-//   kLmSeg16     1..16     8 lanes a vertex (4 vertices a warp), 2 entries a lane
-//   kLmSeg32     ..32      16 lanes a vertex (2 vertices a warp), 2 entries a lane
+// variant, which bounds the degree it accepts.  The variants up to 32 entries
+// fold a row's foreign entries in a list per lane, the others sum the
+// neighbour communities in a table in shared memory (louvain.cu):
+//   kLmSeg16     1..16     4 lanes read a row (8 rows at a time), a lane chooses
+//   kLmSeg32     ..32      8 lanes read a row (4 rows at a time), a lane chooses
 //   kLmSeg64     ..64      16 lanes a vertex (2 vertices a warp), 4 entries a lane
 //   kLmWarp128   ..128     one warp a vertex, 4 entries a lane
 //   kLmWarp256   ..256     one warp a vertex, 8 entries a lane
@@ -332,6 +334,16 @@ struct SideBySide {
 using UpdateFinish = int (*)(dcd_ctx* c, void* user);
 int update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, UpdateFinish finish, void* user);
 
+// The label of every entry's column (level 0), from one gather per update;
+// ready: it holds the labels the update starts from.
+struct EntryLabels {
+  Buf<int32_t> buf;
+  bool ready = false;
+};
+// louvain.cu: gather them when the graph is large and a pass over `entries`
+// entries is a fair part of it.
+int entry_labels(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L, int64_t entries, EntryLabels* out);
+
 struct MergeOut {
   Buf<int64_t>* k = nullptr;  // n weighted degrees of G_t (kept by the context)
   // (src << 32 | dst) pairs, sorted; of equal pairs (repeated records) the
@@ -358,8 +370,8 @@ int screen_batch(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* labels0, cons
 // Writes canonical labels to out_labels and fills stats.
 // a0 / size0 (may be NULL): community sums of labels0, when the caller has them.
 int run_louvain(dcd_ctx* c, const Csr<int32_t>& g, int32_t* labels0, const uint8_t* active0,
-                Buf<int64_t>& k, int32_t* out_labels, dcd_step_stats* st, int32_t* level0_out = nullptr,
-                dcd_step_stats* per_graph = nullptr, const int64_t* a0 = nullptr, const int32_t* size0 = nullptr,
+                Buf<int64_t>& k, int32_t* out_labels, dcd_step_stats* st, EntryLabels* nlab,
+                int32_t* level0_out = nullptr, dcd_step_stats* per_graph = nullptr, const int64_t* a0 = nullptr, const int32_t* size0 = nullptr,
                 const int32_t* pre0 = nullptr);
 
 // louvain.cu: multi-level smart local moving (dSLM) from level-0 labels and
@@ -378,14 +390,14 @@ struct PoolStats {
   int64_t count = 0;
 };
 int pool_stats(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L, const int64_t* k, const int64_t* a,
-               const int32_t* size, const uint8_t* mask, PoolStats* out);
+               const int32_t* size, const uint8_t* mask, EntryLabels* nlab, PoolStats* out);
 
 // features.cu: the learned screen's pool, features, R'_t and move labels.
 struct LearnedPool {
   PoolStats st;
 };
 int screen_features(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L0, const int64_t* k, const int64_t* a,
-                    const int32_t* size, const MergeOut& mo, const uint8_t* rds, LearnedPool* out);
+                    const int32_t* size, const MergeOut& mo, const uint8_t* rds, EntryLabels* nlab, LearnedPool* out);
 int learned_rset_build(dcd_ctx* c, const LearnedPool& lp, const uint8_t* rds, const float* p, uint8_t* r,
                        int64_t* r_size);
 int screen_labels(dcd_ctx* c, const int32_t* before, const int32_t* after);
