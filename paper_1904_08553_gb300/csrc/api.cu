@@ -553,6 +553,11 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
   MergeOut mo;
   DCD_TRY(merge_batch(c, src_labels, mode == DCD_MODE_STATIC, &mo));
   const int nxt = 1 - c->cur;
+  const bool learned = mode == DCD_MODE_LEARNED;
+  const bool collect = c->collect && !first;
+  const bool screen = mode == DCD_MODE_DELTA || learned || collect;
+  SourceBins sb;
+  if (screen) DCD_TRY(source_counts(c, c->rp[nxt].get(), mo.pair_ptr.get(), &sb));
   DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 8, c->rp[nxt].get() + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   DCD_TRY_CUDA(cudaMemcpyAsync(c->hsc, d, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
   DCD_TRY_CUDA(cudaMemcpyAsync(c->hgs, c->gs.get(), c->G * sizeof(GraphState), cudaMemcpyDeviceToHost, s));
@@ -574,8 +579,6 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
   DCD_TRY(rnew.ensure(&c->mem, n));
   const uint8_t* active = nullptr;
   int64_t r_size = n, r_screen = -1;
-  const bool learned = mode == DCD_MODE_LEARNED;
-  const bool collect = c->collect && !first;
   if (learned && !c->mlp) return DCD_ESTATE;
   DCD_TRY_CUDA(cudaEventRecord(c->ev[9], s));
   Buf<uint8_t> rds;  // R_t of Delta-screening
@@ -588,7 +591,14 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
   // proposals for the sources whose rows it sums (one Louvain graph)
   Buf<int32_t> pre;
   const bool use_pre = mode == DCD_MODE_DELTA && !collect && c->G == 1 && c->cfg.alg == DCD_ALG_LOUVAIN;
-  if (mode == DCD_MODE_DELTA || learned || collect) {
+  if (screen) {
+    for (int x = 0; x < sb.plan.nb; x++) {
+      sb.cnt[x] = c->hsc->bcnt[x];
+      sb.total += sb.cnt[x];
+      sb.deg += c->hsc->bdeg[x];
+    }
+    // the sources' rows are read by the screening, most rows again by the passes
+    DCD_TRY(entry_labels(c, g, src_labels, sb.deg, &nlab));
     DCD_TRY(a.alloc(&c->mem, n));
     DCD_TRY(size.alloc(&c->mem, n));
     DCD_TRY(rds.alloc(&c->mem, n));
@@ -597,11 +607,8 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
       DCD_TRY_CUDA(cudaMemsetAsync(pre.get(), 0xff, n * sizeof(int32_t), s));  // -1: none
     }
     DCD_TRY(community_sums(c, n, src_labels, mo.k->get(), a.get(), size.get()));
-    DCD_TRY(screen_batch(c, g, src_labels, mo.k->get(), a.get(), mo, rds.get(), size.get(),
-                         use_pre ? pre.get() : nullptr));
-    DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 9, &d->r_size, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    DCD_TRY_CUDA(cudaStreamSynchronize(s));
-    r_screen = c->hscratch[9];
+    DCD_TRY(screen_batch(c, g, src_labels, mo.k->get(), a.get(), mo, sb, nlab.ready ? nlab.buf.get() : nullptr,
+                         rds.get(), size.get(), use_pre ? pre.get() : nullptr));
   }
   if (learned || collect) {
     DCD_TRY(screen_features(c, g, src_labels, mo.k->get(), a.get(), size.get(), mo, rds.get(), &nlab, &lp));
@@ -609,7 +616,6 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
   }
   if (mode == DCD_MODE_DELTA) {
     DCD_TRY_CUDA(cudaMemcpyAsync(rnew.get(), rds.get(), n, cudaMemcpyDeviceToDevice, s));
-    r_size = r_screen;
     active = rnew.get();
   } else if (learned) {
     Buf<float> p;
@@ -657,6 +663,10 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
                         collect ? c->level0.get() : nullptr, per_graph, a.n ? a.get() : nullptr,
                         size.n ? size.get() : nullptr, pre.n ? pre.get() : nullptr));
   if (collect) DCD_TRY(screen_labels(c, src_labels, c->level0.get()));
+  if (screen) {  // the scalars were read back with the passes' results
+    r_screen = c->hsc->r_screen;
+    if (mode == DCD_MODE_DELTA) r_size = r_screen;
+  }
   if (learned && c->judge && st) {
     // the judge: plain Delta-screening from the same state; keep it when the
     // learned set loses more than 1e-3 of modularity

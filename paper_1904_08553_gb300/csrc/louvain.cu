@@ -27,8 +27,10 @@
 #include <vector>
 
 #include "agg.cuh"
+#include "bins.cuh"
 #include "hub.cuh"
 #include "prims.cuh"
+#include "rows.cuh"
 #include "state.cuh"
 
 namespace dcd {
@@ -106,19 +108,6 @@ __device__ __forceinline__ int32_t proposal(ST S, int32_t D, int32_t C, const in
 // most half of it is ever in use and every probe sequence ends at the key or
 // at an empty slot.
 
-__host__ __device__ constexpr int seg_cap(int row) {
-  int c = 32;
-  while (c < 2 * row) c <<= 1;
-  return c;
-}
-
-// Shared memory of one row table: keys (int32), sums (VT), the claimed-slot
-// list (one uint16 per row entry); a multiple of 16 bytes.
-template <int ROW, typename VT>
-__host__ __device__ constexpr size_t row_tbl_bytes() {
-  return ((size_t)seg_cap(ROW) * (4 + sizeof(VT)) + (size_t)ROW * 2 + 15) / 16 * 16;
-}
-
 // The learned screen's per-row statistics (see LV).
 template <typename W, typename ST, typename VT>
 __device__ __forceinline__ void put_features(const LV<W>& g, int64_t i, int64_t eC, const int32_t* keys,
@@ -148,73 +137,6 @@ __device__ __forceinline__ void put_features(const LV<W>& g, int64_t i, int64_t 
 // 107 us: the lists of 32 vertices leave room for fewer warps), so they keep
 // the table.  A vertex with more than CAP foreign entries is chosen in phase 2
 // by its segment together (list_best), before the next step.
-template <typename VT>
-struct ListEnt;  // a list entry: one shared-memory word of 8 or 16 bytes
-template <>
-struct __align__(8) ListEnt<unsigned> {
-  int32_t lab;
-  unsigned w;
-};
-template <>
-struct __align__(16) ListEnt<unsigned long long> {
-  unsigned long long w;
-  int32_t lab, pad;
-};
-
-constexpr int kCap32 = 16;  // foreign entries a lane's list holds, rows of 17 to 32 entries
-
-// Shared memory of a warp: the lanes' lists, then (rows can be longer than
-// CAP) a whole-row list per segment with two entries of padding.
-template <int S, int Q, int CAP, typename VT>
-__host__ __device__ constexpr size_t vert_bytes() {
-  return (size_t)CAP * 32 * sizeof(ListEnt<VT>) +
-         (S * Q > CAP ? (size_t)(32 / S) * (S * Q + 2) * sizeof(ListEnt<VT>) : 0);
-}
-
-// One segment's whole list: each lane takes K entries and sums the list's
-// weights of the same community (entries of one community get the same sum and
-// gain, so none has to be singled out).  All lanes of the warp call it; every
-// list is padded to nmax, made even.
-template <typename W, typename ST, int S, int K, typename VT>
-__device__ __forceinline__ void list_best(const LV<W>& g, const ListEnt<VT>* list, int n, int nmax, int64_t kv,
-                                          int64_t eC, int64_t aC, int64_t m2v, int sl, ST& Sb, int32_t& D,
-                                          int64_t& eD) {
-  int32_t l[K];
-  VT e[K];
-#pragma unroll
-  for (int k = 0; k < K; k++) {
-    l[k] = k * S + sl < n ? list[k * S + sl].lab : -1;
-    e[k] = 0;
-  }
-  for (int j = 0; j < nmax; j += 2) {
-    const ListEnt<VT> x = list[j], y = list[j + 1];
-#pragma unroll
-    for (int k = 0; k < K; k++) {
-      if (x.lab == l[k]) e[k] += x.w;
-      if (y.lab == l[k]) e[k] += y.w;
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < K; k++)
-    if (l[k] >= 0) {
-      const ST x = gain<ST>(m2v, kv, (int64_t)e[k], eC, g.a[l[k]], aC);
-      if (better(x, l[k], Sb, D)) {
-        Sb = x;
-        D = l[k];
-      }
-    }
-  seg_argmax<S>(Sb, D);
-  eD = 0;
-#pragma unroll
-  for (int k = 0; k < K; k++)
-    if (l[k] == D) eD = (int64_t)e[k];
-#pragma unroll
-  for (int o = S / 2; o > 0; o >>= 1) {  // known where an entry is in D; equal there
-    const int64_t x = __shfl_xor_sync(0xffffffffu, eD, o);
-    eD = x > eD ? x : eD;
-  }
-}
-
 template <typename ST, typename W>
 __device__ __forceinline__ void put_best(const LV<W>& g, int64_t i, int64_t eC, ST Sb, int32_t D, int64_t eD) {
   g.f_eC[i] = eC;
@@ -321,7 +243,7 @@ __global__ void __launch_bounds__(256) lm_vert(LV<W> g, const int32_t* __restric
         ST Sb = gain_lowest<ST>();
         int32_t D = INT_MAX;
         int64_t eD;
-        list_best<W, ST, S, (ROW + S - 1) / S, VT>(g, row, n, nmax, kv, eC, aC, g.m2_of(vv), sl, Sb, D, eD);
+        list_best<LV<W>, ST, S, (ROW + S - 1) / S, VT>(g, row, n, nmax, kv, eC, aC, g.m2_of(vv), sl, Sb, D, eD);
         if (g.f_eC && sl == 0 && src < nb) put_best(g, wb + src, eC, Sb, D, eD);
         pick = __shfl_sync(0xffffffffu, Sb > 0 ? D : INT_MAX, (lane & (P - 1)) * S);
         if (lane / P == t) {
@@ -1034,176 +956,72 @@ __global__ void __launch_bounds__(256) nlab_gather(const int32_t* __restrict__ c
   for (; e < m; e += st) st_stream(nlab + e, L[ld_stream(col + e)]);
 }
 
-// ---------------------------------------------------------------- binning
-
-// Active vertices per degree bin, their degree sums and largest degree.  The
-// lanes of a warp are grouped by bin (match_any); each group's leader updates
-// the warp's own counters (leaders hold distinct bins, so no two update one
-// counter), and the warps' counters meet in shared memory, then in global
-// memory, once per CTA.
-__global__ void __launch_bounds__(256) bin_count(const int64_t* __restrict__ rp, int64_t n,
-                                                 const uint8_t* __restrict__ active, DevScalars* d,
-                                                 const int32_t* __restrict__ gid,
-                                                 const GraphState* __restrict__ gs, BinPlan plan,
-                                                 const int32_t* __restrict__ pre) {
-  constexpr int NW = 256 / 32;
-  __shared__ unsigned long long wc[NW][kMaxBins], wdb[NW][kMaxBins];
-  __shared__ long long wmax[NW][kMaxBins];
-  const int lane = lane_id(), wid = threadIdx.x >> 5;
-  for (int b = lane; b < kMaxBins; b += 32) {
-    wc[wid][b] = 0;
-    wdb[wid][b] = 0;
-    wmax[wid][b] = 0;
-  }
-  __syncwarp();
-  unsigned long long deg_sum = 0, act = 0, pre_deg = 0, pre_cnt = 0;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (blockIdx.x * (int64_t)blockDim.x) + (threadIdx.x & ~31); base < n; base += stride) {
-    const int64_t v = base + lane;
-    bool ok = v < n && (!active || active[v]) && (!gid || gs[gid[v]].running);
-    const int64_t deg = ok ? rp[v + 1] - rp[v] : 0;
-    deg_sum += (unsigned long long)deg;
-    act += ok ? 1 : 0;
-    // a first-pass proposal from the screening, which the table kernels take
-    // (the hub kernels evaluate their rows all the same)
-    if (pre && deg > 0 && pre[v] >= 0 && plan.var[bin_of(plan, deg)] != kLmHub) {
-      pre_deg += (unsigned long long)deg;
-      pre_cnt += 1;
-    }
-    const int bin = (ok && deg > 0) ? bin_of(plan, deg) : -1;
-    const unsigned peers = __match_any_sync(0xffffffffu, bin);
-    const int64_t ds = group_sum_exact(peers, deg);
-    const unsigned mx = __reduce_max_sync(peers, (unsigned)deg);
-    if (bin >= 0 && (int)(__ffs(peers) - 1) == lane) {
-      wc[wid][bin] += __popc(peers);
-      wdb[wid][bin] += (unsigned long long)ds;
-      if ((long long)mx > wmax[wid][bin]) wmax[wid][bin] = (long long)mx;
-    }
-    __syncwarp();
-  }
-  deg_sum = warp_sum(deg_sum);
-  act = warp_sum(act);
-  if (pre) {
-    pre_deg = warp_sum(pre_deg);
-    pre_cnt = warp_sum(pre_cnt);
-    if (lane == 0 && pre_cnt) {
-      atomicAdd((unsigned long long*)&d->pre_deg, pre_deg);
-      atomicAdd((unsigned long long*)&d->pre_verts, pre_cnt);
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < plan.nb) {
-    const int b = threadIdx.x;
-    unsigned long long c = 0, db = 0;
-    long long mx = 0;
-    for (int x = 0; x < NW; x++) {
-      c += wc[x][b];
-      db += wdb[x][b];
-      mx = wmax[x][b] > mx ? wmax[x][b] : mx;
-    }
-    if (c) {
-      atomicAdd((unsigned long long*)&d->bcnt[b], c);
-      atomicAdd((unsigned long long*)&d->bdeg[b], db);
-      atomicMax((long long*)&d->bmax[b], mx);
-    }
-  }
-  if (lane == 0 && act) {
-    atomicAdd((unsigned long long*)&d->act_deg, deg_sum);
-    atomicAdd((unsigned long long*)&d->ncomm, act);
-  }
-}
-
-__global__ void bin_scatter(const int64_t* __restrict__ rp, int64_t n, const uint8_t* __restrict__ active,
-                            const DevScalars* __restrict__ d, int32_t* __restrict__ cursor,
-                            int32_t* __restrict__ list, const int32_t* __restrict__ gid,
-                            const GraphState* __restrict__ gs, BinPlan plan) {
-  __shared__ int32_t off[kMaxBins];
-  if (threadIdx.x == 0) {
-    int64_t o = 0;
-    for (int b = 0; b < plan.nb; b++) {
-      off[b] = (int32_t)o;
-      o += d->bcnt[b];
-    }
-  }
-  __syncthreads();
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t base0 = (blockIdx.x * (int64_t)blockDim.x) + (threadIdx.x & ~31);
-  for (int64_t base = base0; base < n; base += stride) {
-    const int64_t v = base + lane_id();
-    int bin = -1;
-    if (v < n && (!active || active[v]) && (!gid || gs[gid[v]].running)) {
-      const int64_t deg = rp[v + 1] - rp[v];
-      if (deg > 0) bin = bin_of(plan, deg);
-    }
-    for (int b = 0; b < plan.nb; b++) {
-      const unsigned bal = __ballot_sync(0xffffffffu, bin == b);
-      if (!bal) continue;
-      int32_t slot = 0;
-      if (lane_id() == 0) slot = atomicAdd(&cursor[b], __popc(bal));
-      slot = __shfl_sync(0xffffffffu, slot, 0);
-      if (bin == b) list[off[b] + slot + __popc(bal & lanemask_lt())] = (int32_t)v;
-    }
-  }
-}
-
 // ---------------------------------------------------------------- sums
 
-// a_C and |C| of every label: each warp groups its 32 vertices by label,
-// each CTA adds the group sums into a shared table (labels of a CTA repeat
-// heavily when communities are large), and the table goes to global memory
-// once per CTA; labels that find no slot within a few probes go there
-// directly.
+// a_C and |C| of every label: a CTA adds its vertices into a shared table
+// (labels of a CTA repeat when communities are large), which goes to global
+// memory once per CTA; labels that find no slot within a few probes go there
+// directly.  VT: 32-bit sums when 2m < 2^32 bounds every one of them; shared
+// memory adds those natively, 64-bit sums by a compare-and-swap loop (2 M
+// vertices: 22 us, 123 with 64-bit sums and a warp match first).
 constexpr int kCsSlots = 2048;
 constexpr int kCsThreads = 1024;
 
+template <typename VT>
 __global__ void __launch_bounds__(kCsThreads) comm_sums(int64_t n, const int32_t* __restrict__ L,
                                                         const int64_t* __restrict__ k,
                                                         unsigned long long* __restrict__ a, int32_t* __restrict__ size) {
   __shared__ int32_t tk[kCsSlots];
   __shared__ int32_t tc[kCsSlots];
-  __shared__ unsigned long long tv[kCsSlots];
+  __shared__ VT tv[kCsSlots];
   for (int x = threadIdx.x; x < kCsSlots; x += blockDim.x) {
     tk[x] = -1;
     tc[x] = 0;
     tv[x] = 0;
   }
   __syncthreads();
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (blockIdx.x * (int64_t)blockDim.x) + (threadIdx.x & ~31); base < n; base += stride) {
-    const int64_t v = base + lane_id();
-    const int32_t c = v < n ? L[v] : -1;
-    const int64_t kv = v < n ? k[v] : 0;
-    const unsigned peers = __match_any_sync(0xffffffffu, c);
-    const int64_t sk = group_sum_exact(peers, kv);
-    if (c >= 0 && (int)(__ffs(peers) - 1) == (int)lane_id()) {
-      uint32_t sl = hash_label(c, kCsSlots - 1);
-      bool done = false;
-      for (int probe = 0; probe < 8 && !done; probe++) {
-        const int32_t key = tk[sl];
-        if (key == c) {
-          done = true;
-        } else if (key == -1) {
-          const int32_t old = atomicCAS(&tk[sl], -1, c);
-          done = old == -1 || old == c;
-        }
-        if (done) {
-          atomicAdd(&tv[sl], (unsigned long long)sk);
-          atomicAdd(&tc[sl], __popc(peers));
-        }
-        sl = (sl + 1) & (kCsSlots - 1);
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t c = L[v];
+    const int64_t kv = k[v];
+    uint32_t sl = hash_label(c, kCsSlots - 1);
+    bool done = false;
+    for (int probe = 0; probe < 8 && !done; probe++) {
+      const int32_t key = tk[sl];
+      if (key == c) {
+        done = true;
+      } else if (key == -1) {
+        const int32_t old = atomicCAS(&tk[sl], -1, c);
+        done = old == -1 || old == c;
       }
-      if (!done) {
-        atomicAdd(&a[c], (unsigned long long)sk);
-        atomicAdd(&size[c], __popc(peers));
-      }
+      if (!done) sl = (sl + 1) & (kCsSlots - 1);
+    }
+    if (done) {
+      atomicAdd(&tv[sl], (VT)kv);
+      atomicAdd(&tc[sl], 1);
+    } else {
+      atomicAdd(&a[c], (unsigned long long)kv);
+      atomicAdd(&size[c], 1);
     }
   }
   __syncthreads();
   for (int x = threadIdx.x; x < kCsSlots; x += blockDim.x)
     if (tk[x] >= 0) {
-      atomicAdd(&a[tk[x]], tv[x]);
+      atomicAdd(&a[tk[x]], (unsigned long long)tv[x]);
       atomicAdd(&size[tk[x]], tc[x]);
     }
+}
+
+// a and size are zero; m2max bounds the sum of k over any community.
+int launch_comm_sums(dcd_ctx* c, int64_t n, const int32_t* L, const int64_t* k, int64_t m2max, int64_t* a,
+                     int32_t* size) {
+  const int grid = grid_for(n, kCsThreads, 2);
+  unsigned long long* ua = (unsigned long long*)a;
+  if (m2max < ((int64_t)1 << 32))
+    ::dcd::count_launch(), comm_sums<unsigned><<<grid, kCsThreads, 0, c->stream>>>(n, L, k, ua, size);
+  else
+    ::dcd::count_launch(), comm_sums<unsigned long long><<<grid, kCsThreads, 0, c->stream>>>(n, L, k, ua, size);
+  DCD_LAUNCH_CHECK();
+  return DCD_OK;
 }
 
 __global__ void fill_iota(int32_t* __restrict__ x, int64_t n) {
@@ -1667,7 +1485,8 @@ int make_bins(dcd_ctx* c, const Csr<W>& g, const uint8_t* active, Bins* b, const
   DCD_TRY_CUDA(cudaMemsetAsync(&d->act_deg, 0, 2 * sizeof(int64_t), s));  // act_deg, ncomm
   DCD_TRY_CUDA(cudaMemsetAsync(&d->bcnt[0], 0, 3 * kMaxBins * sizeof(int64_t), s));  // bcnt, bdeg, bmax
   DCD_TRY_CUDA(cudaMemsetAsync(&d->pre_verts, 0, 2 * sizeof(int64_t), s));           // pre_verts, pre_deg
-  ::dcd::count_launch(), bin_count<<<grid_for(nv, T), T, 0, s>>>(g.rp, nv, active, d, gid, c->gs.get(), plan, pre);
+  ::dcd::count_launch(), bin_count<<<grid_for(nv, T), T, 0, s>>>(g.rp, nv, WantActive{active, gid, c->gs.get()}, d, plan,
+                                                                    pre);
   DCD_LAUNCH_CHECK();
   DCD_TRY_CUDA(cudaMemcpyAsync(c->hsc, d, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
   DCD_TRY_CUDA(cudaStreamSynchronize(s));
@@ -1689,8 +1508,8 @@ int make_bins(dcd_ctx* c, const Csr<W>& g, const uint8_t* active, Bins* b, const
   DCD_TRY(cursor.alloc(&c->mem, kMaxBins));
   DCD_TRY_CUDA(cudaMemsetAsync(cursor.get(), 0, kMaxBins * sizeof(int32_t), s));
   if (b->total > 0) {
-    ::dcd::count_launch(), bin_scatter<<<grid_for(nv, T), T, 0, s>>>(g.rp, nv, active, d, cursor.get(),
-                                                                       b->list.get(), gid, c->gs.get(), plan);
+    ::dcd::count_launch(), bin_scatter<<<bin_scatter_grid(nv), kBinThreads, 0, s>>>(
+        g.rp, nv, WantActive{active, gid, c->gs.get()}, d, cursor.get(), b->list.get(), plan);
     DCD_LAUNCH_CHECK();
   }
   // tables of the hub bin: a region per hub, sized by its degree
@@ -2813,10 +2632,9 @@ int community_sums(dcd_ctx* c, int64_t n, const int32_t* labels, const int64_t* 
   cudaStream_t s = c->stream;
   DCD_TRY_CUDA(cudaMemsetAsync(a, 0, n * sizeof(int64_t), s));
   DCD_TRY_CUDA(cudaMemsetAsync(size, 0, n * sizeof(int32_t), s));
-  ::dcd::count_launch(), comm_sums<<<grid_for(n, kCsThreads, 2), kCsThreads, 0, s>>>(n, labels, k,
-                                                                                   (unsigned long long*)a, size);
-  DCD_LAUNCH_CHECK();
-  return DCD_OK;
+  int64_t m2max = 0;
+  for (int x = 0; x < c->G; x++) m2max = c->hgs[x].m2 > m2max ? c->hgs[x].m2 : m2max;
+  return launch_comm_sums(c, n, labels, k, m2max, a, size);
 }
 
 int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint8_t* active0, Buf<int64_t>& k0,
@@ -3403,10 +3221,7 @@ struct SlmLevel {
   int sums(const int32_t* L) {
     DCD_TRY_CUDA(cudaMemsetAsync(a.get(), 0, g.n * sizeof(int64_t), c->stream));
     DCD_TRY_CUDA(cudaMemsetAsync(size.get(), 0, g.n * sizeof(int32_t), c->stream));
-    ::dcd::count_launch(), comm_sums<<<grid_for(g.n, kCsThreads, 2), kCsThreads, 0, c->stream>>>(
-        g.n, L, k, (unsigned long long*)a.get(), size.get());
-    DCD_LAUNCH_CHECK();
-    return DCD_OK;
+    return launch_comm_sums(c, g.n, L, k, m2, a.get(), size.get());
   }
 
   // N = m2 * in - sum a^2 of labels L (Eq. 1 scaled by m2^2), exact
@@ -3445,7 +3260,7 @@ struct SlmLevel {
     plan.hi[1] = INT64_MAX;
     DCD_TRY_CUDA(cudaMemsetAsync(&d->act_deg, 0, 2 * sizeof(int64_t), s));
     DCD_TRY_CUDA(cudaMemsetAsync(&d->bcnt[0], 0, 3 * kMaxBins * sizeof(int64_t), s));
-    ::dcd::count_launch(), bin_count<<<grid_for(n, T), T, 0, s>>>(g.rp, n, active, d, nullptr, nullptr, plan,
+    ::dcd::count_launch(), bin_count<<<grid_for(n, T), T, 0, s>>>(g.rp, n, WantActive{active, nullptr, nullptr}, d, plan,
                                                                    nullptr);
     DCD_LAUNCH_CHECK();
     DCD_TRY_CUDA(cudaMemcpyAsync(c->hsc, d, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
@@ -3457,8 +3272,8 @@ struct SlmLevel {
     DCD_TRY(cursor.alloc(&c->mem, kMaxBins));
     DCD_TRY_CUDA(cudaMemsetAsync(cursor.get(), 0, kMaxBins * sizeof(int32_t), s));
     if (total)
-      ::dcd::count_launch(), bin_scatter<<<grid_for(n, T), T, 0, s>>>(g.rp, n, active, d, cursor.get(), list.get(),
-                                                                       nullptr, nullptr, plan);
+      ::dcd::count_launch(), bin_scatter<<<bin_scatter_grid(n), kBinThreads, 0, s>>>(
+          g.rp, n, WantActive{active, nullptr, nullptr}, d, cursor.get(), list.get(), plan);
     // CTA tables in global memory for the long rows
     using VT = typename TblVal<ST>::type;
     const uint32_t tcap = cnt1 ? table_cap(maxd1) : 64;

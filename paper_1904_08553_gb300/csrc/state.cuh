@@ -43,6 +43,12 @@ struct DevScalars {
   int32_t pad3;
   int64_t pre_verts;  // level 0: active vertices whose first-pass proposal the screening made
   int64_t pre_deg;    // and the sum of their degrees
+  // screening: |R_t|, degrees and row chunks of the sources whose neighbourhood
+  // is marked, vertices whose rows are still to be read (cleared together)
+  int64_t r_screen;
+  int64_t gamma_deg;
+  int64_t gamma_items;
+  int64_t rest_cnt;
   int64_t moved_deg;  // degrees of the last pass's movers (level 0, entry labels kept)
 };
 
@@ -132,15 +138,6 @@ inline BinPlan default_bin_plan() {
   }
   return p;
 }
-
-// The screening kernels' source bins: 1..32 a warp, 33..256 a warp with a
-// shared table, 257..4096 a CTA with a shared table, larger: hub tables in
-// global memory (hub.cuh).
-constexpr int kBinWarpMax = 32;
-constexpr int kBinMidMax = 256;
-constexpr int kBinLargeMax = 4096;
-constexpr int kMidCap = 512;     // table_cap(kBinMidMax)
-constexpr int kLargeCap = 8192;  // table_cap(kBinLargeMax)
 
 }  // namespace dcd
 
@@ -357,13 +354,24 @@ struct MergeOut {
 };
 int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut* out);
 
-// screen.cu: Algorithm 2 plus the deletion rule -> rset (n bytes).
-// size and pre may be NULL; with pre, the first local-move pass's proposal of
-// every source whose row phase A sums is written to pre[source] (others -1;
-// the caller fills pre with -1).
-int screen_batch(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* labels0, const int64_t* k,
-                 const int64_t* a, const MergeOut& mo, uint8_t* rset, const int32_t* size = nullptr,
-                 int32_t* pre = nullptr);
+// The batch's sources (vertices with pairs) by degree in G_t.
+struct SourceBins {
+  BinPlan plan;
+  int64_t cnt[kMaxBins] = {};
+  int64_t total = 0, deg = 0;  // sources with entries, and the sum of their degrees
+};
+// screen.cu: the counts, into the context's device scalars (no synchronisation;
+// the caller reads bcnt and bdeg back with the merge's results).
+int source_counts(dcd_ctx* c, const int64_t* rp, const int32_t* pair_ptr, SourceBins* sb);
+
+// screen.cu: Algorithm 2 plus the deletion rule -> rset (n bytes); |R_t| into
+// the device scalar r_screen (no synchronisation).
+// nlab (labels0 in entry order), size and pre may be NULL; with pre, the first
+// local-move pass's proposal of every source whose row phase A sums is written
+// to pre[source] (others -1; the caller fills pre with -1).
+int screen_batch(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* labels0, const int64_t* k, const int64_t* a,
+                 const MergeOut& mo, const SourceBins& sb, const int32_t* nlab, uint8_t* rset,
+                 const int32_t* size = nullptr, int32_t* pre = nullptr);
 
 // louvain.cu: Algorithm 1 from level-0 labels (modified in place into the
 // level-0 result), level-0 active flags (NULL = all), k and m2 of G_t.
