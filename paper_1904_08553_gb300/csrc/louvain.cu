@@ -1047,12 +1047,55 @@ __global__ void mark_used(int64_t n, const int32_t* __restrict__ L, int32_t* __r
     if (!used[L[v]]) used[L[v]] = 1;  // a read first: most labels are already marked
 }
 
-// The same flags from the tracked community sizes: label x is used iff
-// |x| > 0.  A coalesced pass over the labels, where mark_used writes a few
-// hundred hot addresses from every vertex when communities are large.
-__global__ void used_from_size(int64_t n, const int32_t* __restrict__ size, int32_t* __restrict__ used) {
-  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x)
-    used[x] = size[x] > 0 ? 1 : 0;
+// Labels in use of a level, from the tracked community sizes and sums (a
+// coalesced pass over the labels).  A community with a_C = 0 holds only
+// vertices without entries: nothing above this level can change it, so only
+// the others become vertices of the next level (ids 0 .. nz - 1, in label
+// order); the communities without entries are numbered behind them.  R-MAT 22
+// has 1.8 M communities, 700 of them with entries: its coarse graph is dense
+// and follows the delta rule (0.5-0.9 ms), where the sort of every entry's key
+// took 4.8.  Packed for one scan: low word the former, high word the latter.
+__global__ void label_flags(int64_t n, const int32_t* __restrict__ size, const int64_t* __restrict__ a,
+                            int64_t* __restrict__ f) {
+  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x <= n; x += (int64_t)gridDim.x * blockDim.x)
+    f[x] = (x < n && size[x] > 0) ? (a[x] != 0 ? 1 : (int64_t)1 << 32) : 0;
+}
+
+// cid[x]: the id of label x (-1: not in use), from the scanned flags (f[n]:
+// the totals).  Per graph the labels in use, those without entries among them,
+// and the graph of every next-level vertex.
+__global__ void label_ids(int64_t n, const int32_t* __restrict__ size, const int64_t* __restrict__ a,
+                          const int64_t* __restrict__ f, const int32_t* __restrict__ gid, int32_t* __restrict__ cid,
+                          GraphState* __restrict__ gs, int32_t* __restrict__ gid_next) {
+  const int32_t nz = (int32_t)f[n];
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  int cur = -1;
+  unsigned long long used_sum = 0, iso_sum = 0;
+  for (int64_t base = (blockIdx.x * (int64_t)blockDim.x) + (threadIdx.x & ~31); base < n; base += stride) {
+    const int64_t x = base + lane_id();
+    const bool used = x < n && size[x] > 0, iso = used && a[x] == 0;
+    if (x < n) {
+      const int64_t p = f[x];
+      cid[x] = !used ? -1 : iso ? nz + (int32_t)(p >> 32) : (int32_t)p;
+      if (used && !iso && gid_next) gid_next[(int32_t)p] = gid[x];
+    }
+    if (!gid) {  // one graph: counted once per warp at the end
+      used_sum += __popc(__ballot_sync(0xffffffffu, used));
+      iso_sum += __popc(__ballot_sync(0xffffffffu, iso));
+      cur = 0;
+      continue;
+    }
+    const int g = used ? gid[x] : -1;
+    const unsigned peers = __match_any_sync(0xffffffffu, g), isos = __ballot_sync(0xffffffffu, iso);
+    if (used && (int)(__ffs(peers) - 1) == (int)lane_id()) {
+      atomicAdd((unsigned long long*)&gs[g].nc, (unsigned long long)__popc(peers));
+      if (peers & isos) atomicAdd((unsigned long long*)&gs[g].iso, (unsigned long long)__popc(peers & isos));
+    }
+  }
+  if (cur == 0 && lane_id() == 0) {
+    if (used_sum) atomicAdd((unsigned long long*)&gs[0].nc, used_sum);
+    if (iso_sum) atomicAdd((unsigned long long*)&gs[0].iso, iso_sum);
+  }
 }
 
 // Row of entry e for the entry-linear walks below: a warp walks a range of
@@ -1398,6 +1441,34 @@ __global__ void coarse_k(int64_t n, const int32_t* __restrict__ cid, const int64
     if (cid[c + 1] != cid[c]) kc[cid[c]] = a[c];
 }
 
+// Start of the next level from label_ids' numbering: k = a of the community,
+// singletons (labels 0 .. nz - 1, a = k, |C| = 1).
+__global__ void level_start(int64_t n, int64_t nz, const int32_t* __restrict__ cid, const int64_t* __restrict__ a,
+                            int64_t* __restrict__ kc, int32_t* __restrict__ Lc) {
+  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t x = cid[c];
+    if (x >= 0 && x < nz) kc[x] = a[c];
+    if (c < nz) Lc[c] = (int32_t)c;
+  }
+}
+__global__ void level_sums(int64_t nz, const int64_t* __restrict__ kc, int64_t* __restrict__ a,
+                           int32_t* __restrict__ size) {
+  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < nz; c += (int64_t)gridDim.x * blockDim.x) {
+    a[c] = kc[c];
+    size[c] = 1;
+  }
+}
+
+// Vertex of the next level (of nz) of every original vertex; values from nv on
+// name the communities without entries, which stay behind the level's own.
+__global__ void compose_ids(int64_t n0, int64_t nv, int64_t nz, int32_t* __restrict__ comp,
+                            const int32_t* __restrict__ L, const int32_t* __restrict__ cid) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n0; v += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t x = comp[v];
+    comp[v] = x < nv ? cid[L[x]] : (int32_t)(x - nv + nz);
+  }
+}
+
 __global__ void compose(int64_t n0, int32_t* __restrict__ comp, const int32_t* __restrict__ L,
                         const int32_t* __restrict__ cid) {
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n0; v += (int64_t)gridDim.x * blockDim.x)
@@ -1406,12 +1477,17 @@ __global__ void compose(int64_t n0, int32_t* __restrict__ comp, const int32_t* _
 
 // ---------------------------------------------------------------- finish
 
-__global__ void final_min(int64_t n0, const int32_t* __restrict__ comp, const int32_t* __restrict__ L,
+// The label of level vertex x; a community without entries (x >= nv) is its own.
+__device__ __forceinline__ int32_t level_label(const int32_t* __restrict__ L, int64_t nv, int32_t x) {
+  return x < nv ? L[x] : x;
+}
+
+__global__ void final_min(int64_t n0, int64_t nv, const int32_t* __restrict__ comp, const int32_t* __restrict__ L,
                           int32_t* __restrict__ minid) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t base = (blockIdx.x * (int64_t)blockDim.x) + (threadIdx.x & ~31); base < n0; base += stride) {
     const int64_t v = base + lane_id();
-    const int32_t c = v < n0 ? L[comp[v]] : -1;
+    const int32_t c = v < n0 ? level_label(L, nv, comp[v]) : -1;
     const unsigned peers = __match_any_sync(0xffffffffu, c);
     const unsigned mn = __reduce_min_sync(peers, v < n0 ? (unsigned)v : 0xffffffffu);
     // labels of large communities repeat across the grid: read first, and
@@ -1423,7 +1499,7 @@ __global__ void final_min(int64_t n0, const int32_t* __restrict__ comp, const in
 
 // Canonical labels (smallest member id, a vertex id of the context) and the
 // number of communities per graph.
-__global__ void final_labels(int64_t n0, const int32_t* __restrict__ comp, const int32_t* __restrict__ L,
+__global__ void final_labels(int64_t n0, int64_t nv, const int32_t* __restrict__ comp, const int32_t* __restrict__ L,
                              const int32_t* __restrict__ minid, int32_t* __restrict__ out,
                              const int32_t* __restrict__ gid, GraphState* __restrict__ gs) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -1432,7 +1508,7 @@ __global__ void final_labels(int64_t n0, const int32_t* __restrict__ comp, const
     int g = -1;
     bool head = false;
     if (v < n0) {
-      const int32_t x = minid[L[comp[v]]];
+      const int32_t x = minid[level_label(L, nv, comp[v])];
       head = x == (int32_t)v;
       g = graph_of(gid, v);
       out[v] = x;
@@ -1904,7 +1980,7 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
 // Compaction of one level: returns nc; fills the coarse graph when nc < n.
 template <typename W>
 int used_labels(dcd_ctx* c, const Csr<W>& g, const int32_t* L, Buf<int32_t>& cid, int64_t* nc,
-                const int32_t* gid, Buf<int32_t>* gid_next, const int32_t* size = nullptr) {
+                const int32_t* gid, Buf<int32_t>* gid_next) {
   cudaStream_t s = c->stream;
   const int T = 256;
   const int64_t nv = g.n;
@@ -1912,8 +1988,7 @@ int used_labels(dcd_ctx* c, const Csr<W>& g, const int32_t* L, Buf<int32_t>& cid
   Buf<int32_t> tmp;
   DCD_TRY(tmp.alloc(&c->mem, scan_tmp_count(nv + 1)));
   DCD_TRY_CUDA(cudaMemsetAsync(cid.get(), 0, (nv + 1) * sizeof(int32_t), s));
-  if (size) ::dcd::count_launch(), used_from_size<<<grid_for(nv, T), T, 0, s>>>(nv, size, cid.get());
-  else ::dcd::count_launch(), mark_used<<<grid_for(nv, T), T, 0, s>>>(nv, L, cid.get());
+  ::dcd::count_launch(), mark_used<<<grid_for(nv, T), T, 0, s>>>(nv, L, cid.get());
   DCD_LAUNCH_CHECK();
   DCD_TRY(exclusive_scan<int32_t>(cid.get(), cid.get(), nv + 1, nullptr, tmp.get(), s));
   ::dcd::count_launch(), gs_reset_nc<<<cdiv(c->G, 128), 128, 0, s>>>(c->gs.get(), c->G);
@@ -1926,6 +2001,33 @@ int used_labels(dcd_ctx* c, const Csr<W>& g, const int32_t* L, Buf<int32_t>& cid
   DCD_LAUNCH_CHECK();
   DCD_TRY_CUDA(cudaMemcpyAsync(c->hgs, c->gs.get(), c->G * sizeof(GraphState), cudaMemcpyDeviceToHost, s));
   DCD_TRY_CUDA(cudaStreamSynchronize(s));
+  return DCD_OK;
+}
+
+// The same for a Louvain level, whose community sizes and sums are tracked:
+// ids by label_ids, nz vertices of the next level; per-graph counts in hgs.
+int level_labels(dcd_ctx* c, int64_t nv, const int32_t* size, const int64_t* a, Buf<int32_t>& cid, int64_t* nz,
+                 const int32_t* gid, Buf<int32_t>* gid_next) {
+  cudaStream_t s = c->stream;
+  const int T = 256;
+  Buf<int64_t> f, tmp;
+  DCD_TRY(cid.alloc(&c->mem, nv));
+  DCD_TRY(f.alloc(&c->mem, nv + 1));
+  DCD_TRY(tmp.alloc(&c->mem, scan_tmp_count(nv + 1)));
+  if (gid_next) DCD_TRY(gid_next->alloc(&c->mem, nv));
+  ::dcd::count_launch(), gs_reset_nc<<<cdiv(c->G, 128), 128, 0, s>>>(c->gs.get(), c->G);
+  ::dcd::count_launch(), label_flags<<<grid_for(nv + 1, T), T, 0, s>>>(nv, size, a, f.get());
+  DCD_LAUNCH_CHECK();
+  DCD_TRY(exclusive_scan<int64_t>(f.get(), f.get(), nv + 1, nullptr, tmp.get(), s));
+  ::dcd::count_launch(), label_ids<<<grid_for(nv, T), T, 0, s>>>(nv, size, a, f.get(), gid, cid.get(), c->gs.get(),
+                                                                 gid_next ? gid_next->get() : nullptr);
+  DCD_LAUNCH_CHECK();
+  DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch, f.get() + nv, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 1, &c->dsc.get()->n1_new, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  DCD_TRY_CUDA(cudaMemcpyAsync(c->hgs, c->gs.get(), c->G * sizeof(GraphState), cudaMemcpyDeviceToHost, s));
+  DCD_TRY_CUDA(cudaStreamSynchronize(s));
+  *nz = (int64_t)(int32_t)c->hscratch[0];
+  c->n1.fresh = (int64_t)(int32_t)c->hscratch[1];
   return DCD_OK;
 }
 
@@ -1990,10 +2092,30 @@ __device__ __forceinline__ void cell_add(VT* D, long long cell, long long x) {
   if (cell >= 0 && sum != VT(0) && (int)(__ffs(peers) - 1) == (int)lane_id()) atomicAdd(&D[cell], sum);
 }
 
+// K (nk0 x nk0) into the upper left of D (nk x nk); the rest is zero.
 template <typename VT>
-__global__ void n1_load(const unsigned long long* __restrict__ K, int64_t cells, VT* __restrict__ D) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < cells; i += (int64_t)gridDim.x * blockDim.x)
-    D[i] = (VT)K[i];
+__global__ void n1_load(const unsigned long long* __restrict__ K, int64_t nk0, int64_t nk, VT* __restrict__ D) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nk * nk; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = i / nk, x = i % nk;
+    D[i] = (r < nk0 && x < nk0) ? (VT)K[r * nk0 + x] : VT(0);
+  }
+}
+
+// Rows for the communities of C_{t-1} that had no entries in G_{t-1} (so none
+// in K) and get some from the batch: the first pair to name one numbers it.
+__global__ void n1_new_labels(const uint64_t* __restrict__ pkey, const int32_t* __restrict__ pdelta, int64_t P,
+                              const int32_t* __restrict__ cprev, int64_t nk0, int32_t* __restrict__ kidx,
+                              int32_t* __restrict__ klab, int64_t most, int32_t* __restrict__ cnt) {
+  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < P; p += (int64_t)gridDim.x * blockDim.x) {
+    if (pdelta[p] == 0) continue;
+    const int32_t l = cprev[(int32_t)(pkey[p] >> 32)];  // both ends of an edge come as sources
+    if (kidx[l] != -1 || atomicCAS(&kidx[l], -1, -2) != -1) continue;
+    const int64_t x = nk0 + atomicAdd(cnt, 1);
+    if (x < most) {
+      kidx[l] = (int32_t)x;
+      klab[x] = l;
+    }
+  }
 }
 
 // The batch: pair (u, v) adds its weight change to cell (C(u), C(v)).
@@ -2115,34 +2237,36 @@ __global__ void n1_compact(const VT* __restrict__ D, int64_t nk, const int32_t* 
 
 // K for the next update, from this update's level-0 matrix H (nc0 x nc0):
 // F(i) = the final label of level-1 vertex i (any member's), then the cells
-// of H folded onto the final communities in label order.  A final label is
-// its community's smallest member, so label v is in use exactly when
-// fin[v] == v.  The members of a level-1 vertex share one final label: each
-// CTA keeps the first it sees per level-1 vertex in shared memory (nc0 <=
-// 4096 entries) and writes those once, so the few hundred cells of F are not
-// written by every vertex.
+// of H folded onto the final communities with entries, in any order.  The
+// members of a level-1 vertex share one final label: each CTA keeps the first
+// it sees per level-1 vertex in shared memory (nc0 <= 4096 entries) and writes
+// those once, so the few hundred cells of F are not written by every vertex.
 __global__ void n1_final_of(int64_t n, int64_t nc0, const int32_t* __restrict__ ccid,
-                            const int32_t* __restrict__ fin, int32_t* __restrict__ F, int32_t* __restrict__ used) {
+                            const int32_t* __restrict__ fin, int32_t* __restrict__ F) {
   extern __shared__ int32_t fs[];
   for (int64_t i = threadIdx.x; i < nc0; i += blockDim.x) fs[i] = -1;
   __syncthreads();
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t f = fin[v];
-    used[v] = f == (int32_t)v ? 1 : 0;
     const int32_t c = ccid[v];
-    if (fs[c] < 0) fs[c] = f;  // every writer of fs[c] writes the same value
+    // (a vertex of a community without entries has no level-1 vertex)
+    if (c < nc0 && fs[c] < 0) fs[c] = fin[v];  // every writer of fs[c] writes the same value
   }
   __syncthreads();
   for (int64_t i = threadIdx.x; i < nc0; i += blockDim.x)
     if (fs[i] >= 0 && F[i] != fs[i]) F[i] = fs[i];
 }
 
-__global__ void n1_index(int64_t n, const int32_t* __restrict__ used, const int32_t* __restrict__ idx,
-                         int32_t* __restrict__ kidx, int32_t* __restrict__ klab) {
-  for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n; l += (int64_t)gridDim.x * blockDim.x) {
-    const bool u = used[l] != 0;
-    kidx[l] = u ? idx[l] : -1;
-    if (u) klab[idx[l]] = (int32_t)l;
+// Rows of K: the distinct labels of F (at most nk), numbered as they come.
+__global__ void n1_index(int64_t nc0, const int32_t* __restrict__ F, int64_t nk, int32_t* __restrict__ kidx,
+                         int32_t* __restrict__ klab, int32_t* __restrict__ cnt) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nc0; i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t l = F[i];
+    if (kidx[l] != -1 || atomicCAS(&kidx[l], -1, -2) != -1) continue;
+    const int32_t x = atomicAdd(cnt, 1);
+    if (x < nk) {
+      kidx[l] = x;
+      klab[x] = l;
+    }
   }
 }
 
@@ -2165,7 +2289,8 @@ int n1_build(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L0, const int32_t
              unsigned long long* entries, bool* ok) {
   cudaStream_t s = c->stream;
   const int T = 256;
-  const int64_t nk = c->kc_n;
+  const int64_t nk0 = c->kc_n, nk = nk0 + c->n1.fresh;
+  const int32_t *kidx = c->n1.kidx, *klab = c->n1.klab;
   Buf<VT> D;
   Buf<int64_t> items;
   Buf<int32_t> cnt;
@@ -2176,16 +2301,16 @@ int n1_build(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L0, const int32_t
   DCD_TRY(bad.alloc(&c->mem, 1));
   DCD_TRY_CUDA(cudaMemsetAsync(cnt.get(), 0, sizeof(int32_t), s));
   DCD_TRY_CUDA(cudaMemsetAsync(bad.get(), 0, sizeof(uint32_t), s));
-  ::dcd::count_launch(), n1_load<VT><<<grid_for(nk * nk, T), T, 0, s>>>(c->kc_mat.get(), nk * nk, D.get());
+  ::dcd::count_launch(), n1_load<VT><<<grid_for(nk * nk, T), T, 0, s>>>(c->kc_mat.get(), nk0, nk, D.get());
   if (c->n1.P > 0)
     ::dcd::count_launch(), n1_pairs<VT><<<grid_for(c->n1.P, T), T, 0, s>>>(
-        c->n1.pkey, c->n1.pdelta, c->n1.P, c->n1.cprev, c->kc_idx.get(), nk, D.get(), bad.get());
+        c->n1.pkey, c->n1.pdelta, c->n1.P, c->n1.cprev, kidx, nk, D.get(), bad.get());
   ::dcd::count_launch(), n1_movers_list<<<grid_for(g.n, T), T, 0, s>>>(g.n, L0, c->n1.cprev, g.rp, items.get(),
                                                                         cnt.get(), entries);
   ::dcd::count_launch(), n1_movers<VT><<<wave_grid(n1_movers<VT>, g.n * 32, T), T, 0, s>>>(
-      items.get(), cnt.get(), g.rp, g.col, g.w, L0, c->n1.cprev, c->kc_idx.get(), nk, D.get(), bad.get());
-  ::dcd::count_launch(), n1_compact<VT><<<grid_for(nk * nk, T), T, 0, s>>>(D.get(), nk, c->kc_lab.get(), cid, L0,
-                                                                            nc, H, bad.get());
+      items.get(), cnt.get(), g.rp, g.col, g.w, L0, c->n1.cprev, kidx, nk, D.get(), bad.get());
+  ::dcd::count_launch(), n1_compact<VT><<<grid_for(nk * nk, T), T, 0, s>>>(D.get(), nk, klab, cid, L0, nc, H,
+                                                                            bad.get());
   DCD_LAUNCH_CHECK();
   DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 2, bad.get(), sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
   DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 3, cnt.get(), sizeof(int32_t), cudaMemcpyDeviceToHost, s));
@@ -2196,49 +2321,70 @@ int n1_build(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L0, const int32_t
   return DCD_OK;
 }
 
-// K of this update's final labels (into the *_nx buffers; taken at commit).
+// The index of K for this update (before level 0's labels are numbered): a copy
+// of the kept one, extended by the batch's new communities; their number comes
+// back with the labels' (c->n1.fresh).
+int n1_extend(dcd_ctx* c, Buf<int32_t>& kidx, Buf<int32_t>& klab) {
+  c->n1.fresh = 0;
+  c->n1.kidx = c->n1.klab = nullptr;
+  if (!c->n1.usable) return DCD_OK;
+  cudaStream_t s = c->stream;
+  const int T = 256;
+  const int64_t n = c->n;
+  int32_t* cnt = reinterpret_cast<int32_t*>(&c->dsc.get()->n1_new);
+  DCD_TRY(kidx.alloc(&c->mem, n));
+  DCD_TRY(klab.alloc(&c->mem, kDenseNc));
+  c->n1.kidx = kidx.get();
+  c->n1.klab = klab.get();
+  DCD_TRY_CUDA(cudaMemcpyAsync(kidx.get(), c->kc_idx.get(), n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+  DCD_TRY_CUDA(cudaMemcpyAsync(klab.get(), c->kc_lab.get(), c->kc_n * sizeof(int32_t), cudaMemcpyDeviceToDevice,
+                               s));
+  DCD_TRY_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int64_t), s));
+  if (c->n1.P > 0) {
+    ::dcd::count_launch(), n1_new_labels<<<grid_for(c->n1.P, T), T, 0, s>>>(
+        c->n1.pkey, c->n1.pdelta, c->n1.P, c->n1.cprev, c->kc_n, kidx.get(), klab.get(), kDenseNc, cnt);
+    DCD_LAUNCH_CHECK();
+  }
+  return DCD_OK;
+}
+
+// K of this update's final labels (into the *_nx buffers; taken at commit);
+// nk: the communities with entries.
 template <typename VT>
-int n1_keep_t(dcd_ctx* c, int64_t n, const int32_t* fin) {
+int n1_keep_t(dcd_ctx* c, int64_t n, const int32_t* fin, int64_t nk) {
   cudaStream_t s = c->stream;
   const int T = 256;
   const int64_t nc0 = c->n1.h0_nc;
-  Buf<int32_t> F, used, idx;
-  Buf<int32_t> stmp;
+  if (nk > kDenseNc || nk < 0) return DCD_OK;  // cannot happen (nk <= nc0); kept out of K's size bound
+  Buf<int32_t> F, cnt;
   DCD_TRY(F.alloc(&c->mem, nc0 > 0 ? nc0 : 1));
-  DCD_TRY(used.alloc(&c->mem, n + 1));
-  DCD_TRY(idx.alloc(&c->mem, n + 1));
-  DCD_TRY(stmp.alloc(&c->mem, scan_tmp_count(n + 1) + 1));
-  DCD_TRY_CUDA(cudaMemsetAsync(used.get() + n, 0, sizeof(int32_t), s));
-  {
-    const int64_t blocks = cdiv(n, (int64_t)T);
-    const int grid = (int)(blocks < 4 * c->sms ? blocks : 4 * c->sms);
-    ::dcd::count_launch(), n1_final_of<<<grid > 0 ? grid : 1, T, nc0 * sizeof(int32_t), s>>>(
-        n, nc0, c->h0_ccid.get(), fin, F.get(), used.get());
-  }
-  DCD_LAUNCH_CHECK();
-  DCD_TRY(exclusive_scan<int32_t>(used.get(), idx.get(), n + 1, nullptr, stmp.get(), s));
-  DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch, idx.get() + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  DCD_TRY_CUDA(cudaStreamSynchronize(s));
-  const int64_t nk = *reinterpret_cast<int32_t*>(c->hscratch);
-  if (nk > kDenseNc) return DCD_OK;  // cannot happen (nk <= nc0); kept out of K's size bound
+  DCD_TRY(cnt.alloc(&c->mem, 1));
   DCD_TRY(c->kc_idx_nx.ensure(&c->mem, n));
   DCD_TRY(c->kc_lab_nx.ensure(&c->mem, nk > 0 ? nk : 1));
   DCD_TRY(c->kc_mat_nx.ensure(&c->mem, nk * nk > 0 ? nk * nk : 1));
+  DCD_TRY_CUDA(cudaMemsetAsync(c->kc_idx_nx.get(), 0xff, n * sizeof(int32_t), s));
   DCD_TRY_CUDA(cudaMemsetAsync(c->kc_mat_nx.get(), 0, nk * nk * sizeof(unsigned long long), s));
-  ::dcd::count_launch(), n1_index<<<grid_for(n, T), T, 0, s>>>(n, used.get(), idx.get(), c->kc_idx_nx.get(),
-                                                                c->kc_lab_nx.get());
-  ::dcd::count_launch(), n1_fold<VT><<<grid_for(nc0 * nc0, T), T, 0, s>>>(
-      reinterpret_cast<const VT*>(c->h0.get()), nc0, F.get(), c->kc_idx_nx.get(), nk, c->kc_mat_nx.get());
-  DCD_LAUNCH_CHECK();
+  DCD_TRY_CUDA(cudaMemsetAsync(cnt.get(), 0, sizeof(int32_t), s));
+  if (nc0 > 0) {
+    const int64_t blocks = cdiv(n, (int64_t)T);
+    const int grid = (int)(blocks < 4 * c->sms ? blocks : 4 * c->sms);
+    ::dcd::count_launch(), n1_final_of<<<grid > 0 ? grid : 1, T, nc0 * sizeof(int32_t), s>>>(
+        n, nc0, c->h0_ccid.get(), fin, F.get());
+    ::dcd::count_launch(), n1_index<<<grid_for(nc0, T), T, 0, s>>>(nc0, F.get(), nk, c->kc_idx_nx.get(),
+                                                                   c->kc_lab_nx.get(), cnt.get());
+    ::dcd::count_launch(), n1_fold<VT><<<grid_for(nc0 * nc0, T), T, 0, s>>>(
+        reinterpret_cast<const VT*>(c->h0.get()), nc0, F.get(), c->kc_idx_nx.get(), nk, c->kc_mat_nx.get());
+    DCD_LAUNCH_CHECK();
+  }
   c->kc_n_nx = nk;
   c->kc_nx_ready = true;
   return DCD_OK;
 }
 
-int n1_keep(dcd_ctx* c, int64_t n, const int32_t* fin) {
+int n1_keep(dcd_ctx* c, int64_t n, const int32_t* fin, int64_t nk) {
   c->kc_nx_ready = false;
   if (!c->n1.track || !c->n1.h0_ready) return DCD_OK;
-  return c->n1.h0_wide ? n1_keep_t<unsigned long long>(c, n, fin) : n1_keep_t<unsigned>(c, n, fin);
+  return c->n1.h0_wide ? n1_keep_t<unsigned long long>(c, n, fin, nk) : n1_keep_t<unsigned>(c, n, fin, nk);
 }
 
 // Dense coarsening (nc <= kDenseNc): matrix, emit, count, scan, write.
@@ -2269,7 +2415,7 @@ int coarsen_dense(dcd_ctx* c, const Csr<W>& g, const int32_t* ccid, int64_t nc, 
   DCD_TRY_CUDA(cudaMemsetAsync(ent.get(), 0, sizeof(unsigned long long), s));
   bool delta = false;
   if constexpr (std::is_same<W, int32_t>::value) {
-    if (level0 && c->n1.usable && c->kc_valid) {
+    if (level0 && c->n1.usable && c->kc_valid && c->kc_n + c->n1.fresh <= kDenseNc) {
       bool ok = false;
       DCD_TRY(n1_build<VT>(c, g, L, cid, nc, dense, ent.get(), &ok));
       delta = ok;
@@ -2667,6 +2813,7 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
   // per-graph host state of the level loop
   std::vector<int64_t> nv(G);
   std::vector<i128> N_start(G);
+  std::vector<int64_t> iso_live(G, 0);  // communities without entries of the graphs whose levels go on
   for (int x = 0; x < G; x++) nv[x] = c->goff[x + 1] - c->goff[x];
   GraphTally tally(G);
 
@@ -2689,6 +2836,8 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
   const uint8_t* active = active0;
   const int32_t* gid = gid0;
   int64_t nvu = n0;  // vertices of the union at this level
+  Buf<int32_t> n1_kidx, n1_klab;  // level-0 delta coarsening: K's index, extended
+  int64_t iso = 0;   // communities without entries at the end of level 0
 
   for (;;) {
     LevelRun lr;
@@ -2714,7 +2863,12 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
       verts0_pre = lr.verts_pre;
     }
     edges_total += lr.edges;
-    verts_total += lr.verts;
+    // the statistics count the communities without entries as vertices of
+    // every coarse level (of the graphs that were still running)
+    int64_t iso_running = 0;
+    if (level > 0)
+      for (int x = 0; x < G; x++) iso_running += iso_live[x];
+    verts_total += lr.verts + iso_running * lr.passes;
     for (int x = 0; x < 4; x++) {
       ms_bin[x] += lr.ms_bin[x];
       edges_bin[x] += lr.edges_bin[x];
@@ -2728,9 +2882,8 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
     int64_t nc = 0;
     const int nx = which ^ 1;
     Buf<int32_t>* gnext = G > 1 ? &gidc[nx] : nullptr;
-    // the level's tracked sizes give the used labels
-    if (level == 0) DCD_TRY(used_labels<int32_t>(c, *g_l0, L, cid, &nc, gid, gnext, size.get()));
-    else DCD_TRY(used_labels<int64_t>(c, *g_lc, L, cid, &nc, gid, gnext, size.get()));
+    if (level == 0 && G == 1) DCD_TRY(n1_extend(c, n1_kidx, n1_klab));
+    DCD_TRY(level_labels(c, nvu, size.get(), a.get(), cid, &nc, gid, gnext));
     trace("level: labels counted");
     level++;
     // level stop per graph: nothing merged, or (from the second level on) a
@@ -2747,7 +2900,11 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
       else
         all_done = false;
       N_start[x] = N_end;
-      nv[x] = X.nc;
+      nv[x] = level == 1 ? X.nc - X.iso : X.nc;  // communities without entries stay behind
+    }
+    for (int x = 0; x < G; x++) {
+      if (level == 1) iso += c->hgs[x].iso;
+      iso_live[x] = c->hgs[x].done ? 0 : c->hgs[x].iso;
     }
     if (all_done) {
       DCD_TRY_CUDA(cudaEventRecord(c->ev[6], s));
@@ -2764,13 +2921,11 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
     else DCD_TRY(coarsen<int64_t>(c, *g_lc, L, cid.get(), nc, &cg[nx]));
     DCD_TRY(kc[nx].alloc(&c->mem, nc));
     DCD_TRY(Lc[nx].alloc(&c->mem, nc));
-    ::dcd::count_launch(), coarse_k<<<grid_for(nvu, T), T, 0, s>>>(nvu, cid.get(), a.get(), kc[nx].get());
-    ::dcd::count_launch(), compose<<<grid_for(n0, T), T, 0, s>>>(n0, comp.get(), L, cid.get());
-    ::dcd::count_launch(), fill_iota<<<grid_for(nc, T), T, 0, s>>>(Lc[nx].get(), nc);
-    DCD_LAUNCH_CHECK();
-    // next level starts from singletons: a = k, |C| = 1; in and sum a^2 carry over
-    DCD_TRY_CUDA(cudaMemcpyAsync(a.get(), kc[nx].get(), nc * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-    ::dcd::count_launch(), fill_i32<<<grid_for(nc, T), T, 0, s>>>(size.get(), nc, 1);
+    ::dcd::count_launch(), compose_ids<<<grid_for(n0, T), T, 0, s>>>(n0, nvu, nc, comp.get(), L, cid.get());
+    // next level starts from singletons; in and sum a^2 carry over
+    ::dcd::count_launch(), level_start<<<grid_for(nvu, T), T, 0, s>>>(nvu, nc, cid.get(), a.get(), kc[nx].get(),
+                                                                      Lc[nx].get());
+    ::dcd::count_launch(), level_sums<<<grid_for(nc, T), T, 0, s>>>(nc, kc[nx].get(), a.get(), size.get());
     DCD_LAUNCH_CHECK();
     DCD_TRY_CUDA(cudaEventRecord(c->ev[6], s));
     DCD_TRY_CUDA(cudaEventSynchronize(c->ev[6]));
@@ -2798,18 +2953,18 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
   DCD_TRY_CUDA(cudaEventRecord(c->ev[7], s));
   {
     Buf<int32_t> minid;
-    DCD_TRY(minid.alloc(&c->mem, nvu));
-    ::dcd::count_launch(), fill_i32<<<grid_for(nvu, T), T, 0, s>>>(minid.get(), nvu, INT32_MAX);
-    ::dcd::count_launch(), final_min<<<grid_for(n0, T), T, 0, s>>>(n0, comp.get(), L, minid.get());
+    DCD_TRY(minid.alloc(&c->mem, nvu + iso));
+    ::dcd::count_launch(), fill_i32<<<grid_for(nvu + iso, T), T, 0, s>>>(minid.get(), nvu + iso, INT32_MAX);
+    ::dcd::count_launch(), final_min<<<grid_for(n0, T), T, 0, s>>>(n0, nvu, comp.get(), L, minid.get());
     ::dcd::count_launch(), gs_reset_nc<<<cdiv(G, 128), 128, 0, s>>>(gs, G);
-    ::dcd::count_launch(), final_labels<<<grid_for(n0, T), T, 0, s>>>(n0, comp.get(), L, minid.get(), out_labels,
-                                                                       gid0, gs);
+    ::dcd::count_launch(), final_labels<<<grid_for(n0, T), T, 0, s>>>(n0, nvu, comp.get(), L, minid.get(),
+                                                                       out_labels, gid0, gs);
     DCD_LAUNCH_CHECK();
     DCD_TRY_CUDA(cudaEventRecord(c->ev[8], s));
     DCD_TRY_CUDA(cudaMemcpyAsync(c->hgs, gs, G * sizeof(GraphState), cudaMemcpyDeviceToHost, s));
     DCD_TRY_CUDA(cudaStreamSynchronize(s));
   }
-  if (G == 1) DCD_TRY(n1_keep(c, n0, out_labels));
+  if (G == 1) DCD_TRY(n1_keep(c, n0, out_labels, c->hgs[0].ncomm - iso));
   float tf = 0.f;
   cudaEventElapsedTime(&tf, c->ev[7], c->ev[8]);
   auto fill = [&](dcd_step_stats* o, int x) {
@@ -3477,9 +3632,9 @@ int run_slm(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint8_t*
     Buf<int32_t> mid;
     DCD_TRY(mid.alloc(&c->mem, nv));
     ::dcd::count_launch(), fill_i32<<<grid_for(nv, T), T, 0, s>>>(mid.get(), nv, INT32_MAX);
-    ::dcd::count_launch(), final_min<<<grid_for(n0, T), T, 0, s>>>(n0, comp.get(), Lcur, mid.get());
+    ::dcd::count_launch(), final_min<<<grid_for(n0, T), T, 0, s>>>(n0, nv, comp.get(), Lcur, mid.get());
     ::dcd::count_launch(), gs_reset_nc<<<1, 128, 0, s>>>(c->gs.get(), 1);
-    ::dcd::count_launch(), final_labels<<<grid_for(n0, T), T, 0, s>>>(n0, comp.get(), Lcur, mid.get(), out_labels,
+    ::dcd::count_launch(), final_labels<<<grid_for(n0, T), T, 0, s>>>(n0, nv, comp.get(), Lcur, mid.get(), out_labels,
                                                                        nullptr, c->gs.get());
     DCD_LAUNCH_CHECK();
     DCD_TRY_CUDA(cudaEventRecord(c->ev[8], s));

@@ -49,6 +49,7 @@ struct DevScalars {
   int64_t gamma_deg;
   int64_t gamma_items;
   int64_t rest_cnt;
+  int64_t n1_new;  // communities K gets a row for in this update
   int64_t moved_deg;  // degrees of the last pass's movers (level 0, entry labels kept)
 };
 
@@ -70,6 +71,7 @@ struct GraphState {
   int32_t running;     // the graph's pass loop at this level goes on
   int32_t passes;      // passes at this level
   int32_t done;        // the graph's levels are over
+  int64_t iso;         // labels in use at the end of level 0 whose community has no entries (a_C = 0)
 };
 
 __device__ __forceinline__ int graph_of(const int32_t* gid, int64_t v) { return gid ? gid[v] : 0; }
@@ -219,8 +221,8 @@ struct dcd_ctx {
   dcd::Buf<int64_t> in_prev, in_next;
   // Per-step delta coarsening of level 0 (dense coarse graphs only): K is
   // the coarse graph of G_t under C_t (the last committed labels) as a dense
-  // kc_n x kc_n matrix over the communities of C_t in label order; kc_idx maps
-  // a label to its row (-1: no community); kc_lab is the inverse.  The next
+  // kc_n x kc_n matrix over the communities of C_t with entries, in any order;
+  // kc_idx maps a label to its row (-1: none); kc_lab is the inverse.  The next
   // update builds its level-0 coarse graph from K, the batch's weight changes
   // and the rows of the vertices that changed community at level 0, instead
   // of from every entry of G_{t+1}.  The *_nx copies are built during an
@@ -238,12 +240,14 @@ struct dcd_ctx {
     const int32_t* pdelta = nullptr;
     int64_t P = 0;
     int64_t distinct = 0;          // of them, pairs that carry flags
+    int64_t fresh = 0;             // communities that K has no row for and the batch gives entries
     const int32_t* cprev = nullptr;  // C_{t-1}
     bool used = false;             // this update took the delta path
     int64_t entries = 0;           // entries the level-0 coarsening read
     bool h0_ready = false;         // h0 holds this update's level-0 matrix
     int64_t h0_nc = 0;
     bool h0_wide = false;          // 64-bit cells
+    const int32_t *kidx = nullptr, *klab = nullptr;  // K's index extended by the fresh communities (this run's)
   } n1;
   dcd::Buf<unsigned char> h0;      // level-0 dense coarse matrix of this update
   dcd::Buf<int32_t> h0_ccid;       // level-1 vertex of every vertex
