@@ -5,15 +5,19 @@
 // accumulators.  A warp owns 16 rows: layer-1 and layer-2 accumulator tiles
 // are turned into the next product's A fragments in registers (bias, ReLU,
 // BF16 pack).  Training adds the backward pass in the same kernel: the
-// activation gradients stay in registers, the weight gradients of a CTA's 64
-// rows are formed with mma from shared-memory tiles, and per-CTA partial
-// gradients are reduced in a fixed order (deterministic), then Adam updates
-// the FP32 master weights and refreshes the BF16 copies.
+// activation gradients stay in registers, the weight gradients of a CTA's rows
+// are formed 64 rows at a time with mma from shared-memory tiles and stay in
+// registers until its rows are done, and the CTAs' partial gradients are
+// reduced in a fixed order (deterministic), then Adam updates the FP32 master
+// weights and refreshes the BF16 copies.  A training run is one cooperative
+// kernel over all its mini-batches: a step is a few microseconds of work, so
+// four launches a step were most of its time.
 #include <cuda_bf16.h>
 
 #include <cmath>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -70,28 +74,41 @@ __global__ void prepare(const float* __restrict__ P, __nv_bfloat16* __restrict__
   }
 }
 
-struct Smem {
-  __nv_bfloat16 w1t[64 * 16];
-  __nv_bfloat16 w2[64 * 64];
-  __nv_bfloat16 w2t[64 * 64];
+// Row strides in shared memory (elements): a fragment load reads 8 rows at 4
+// consecutive words each, which these strides spread over all 32 banks (the
+// natural 64 and 16 put all rows, or every other one, on the same four).
+constexpr int SH = 72, SX = 24;
+
+struct __align__(16) Smem {
+  __nv_bfloat16 w1t[64 * SX];
+  __nv_bfloat16 w2t[64 * SH];
   float w3f[64];
-  __nv_bfloat16 w3[64];
   float b1[64], b2[64];
+  float b3;
 };
 
-__device__ __forceinline__ void load_weights(Smem& s, const Weights& W) {
-  for (int i = threadIdx.x; i < 64 * 64; i += blockDim.x) {
-    s.w2[i] = W.w2[i];
-    s.w2t[i] = W.w2t[i];
-    if (i < 64 * 16) s.w1t[i] = W.w1t[i];
-    if (i < 64) {
-      s.w3[i] = W.w3[i];
-      s.w3f[i] = __bfloat162float(W.w3[i]);
-      s.b1[i] = W.P[OFF_B1 + i];
-      s.b2[i] = W.P[OFF_B2 + i];
-    }
+// Rows of `cols` BF16 words (a multiple of 8) into padded rows, 16 bytes a
+// load, around L1: another CTA of the same kernel may have written them.
+__device__ __forceinline__ void load_rows(__nv_bfloat16* dst, int stride, const __nv_bfloat16* src, int rows, int cols) {
+  const int per = cols / 8;
+  for (int i = threadIdx.x; i < rows * per; i += blockDim.x) {
+    const uint4 v = __ldcg(reinterpret_cast<const uint4*>(src) + i);
+    *reinterpret_cast<uint4*>(dst + (i / per) * stride + (i % per) * 8) = v;
   }
-  __syncthreads();
+}
+
+// The caller synchronises.
+__device__ __forceinline__ void load_weights(Smem& s, const Weights& W) {
+  load_rows(s.w2t, SH, W.w2t, 64, 64);
+  load_rows(s.w1t, SX, W.w1t, 64, 16);
+  if (threadIdx.x < 64) {
+    const int i = threadIdx.x;
+    const unsigned short w3 = __ldcg(reinterpret_cast<const unsigned short*>(W.w3) + i);
+    s.w3f[i] = __uint_as_float((uint32_t)w3 << 16);
+    s.b1[i] = __ldcg(W.P + OFF_B1 + i);
+    s.b2[i] = __ldcg(W.P + OFF_B2 + i);
+    if (i == 0) s.b3 = __ldcg(W.P + OFF_B3);
+  }
 }
 
 // Forward of one 16-row tile.  Outputs: the X fragment, the layer-1
@@ -103,20 +120,24 @@ struct Fwd {
   float z0, z1;  // logits of rows g and g + 8
 };
 
-__device__ __forceinline__ void forward_tile(const Smem& s, const float* __restrict__ X, int64_t r0, int64_t n,
-                                             float b3, Fwd& f) {
+__device__ __forceinline__ void load_x(const float* __restrict__ X, int64_t r0, int64_t n, uint32_t (&xa)[4]) {
   const int lane = lane_id(), g = lane >> 2, t = lane & 3;
   const int64_t ra = r0 + g, rb = r0 + g + 8;
   auto xv = [&](int64_t r, int c) -> float { return (r < n && c < NF) ? X[r * NF + c] : 0.f; };
-  f.xa[0] = pack_bf16(xv(ra, 2 * t), xv(ra, 2 * t + 1));
-  f.xa[1] = pack_bf16(xv(rb, 2 * t), xv(rb, 2 * t + 1));
-  f.xa[2] = pack_bf16(xv(ra, 2 * t + 8), xv(ra, 2 * t + 9));
-  f.xa[3] = pack_bf16(xv(rb, 2 * t + 8), xv(rb, 2 * t + 9));
+  xa[0] = pack_bf16(xv(ra, 2 * t), xv(ra, 2 * t + 1));
+  xa[1] = pack_bf16(xv(rb, 2 * t), xv(rb, 2 * t + 1));
+  xa[2] = pack_bf16(xv(ra, 2 * t + 8), xv(ra, 2 * t + 9));
+  xa[3] = pack_bf16(xv(rb, 2 * t + 8), xv(rb, 2 * t + 9));
+}
+
+// f.xa holds the tile's rows.
+__device__ __forceinline__ void forward_tile(const Smem& s, float b3, Fwd& f) {
+  const int lane = lane_id(), g = lane >> 2, t = lane & 3;
   float c1[8][4];
 #pragma unroll
   for (int j = 0; j < 8; j++) {
     c1[j][0] = c1[j][1] = c1[j][2] = c1[j][3] = 0.f;
-    const __nv_bfloat16* col = s.w1t + (8 * j + g) * 16;
+    const __nv_bfloat16* col = s.w1t + (8 * j + g) * SX;
     mma16816(c1[j], f.xa, ld_pair(col + 2 * t), ld_pair(col + 2 * t + 8));
   }
 #pragma unroll
@@ -137,7 +158,7 @@ __device__ __forceinline__ void forward_tile(const Smem& s, const float* __restr
   for (int kk = 0; kk < 4; kk++)
 #pragma unroll
     for (int j = 0; j < 8; j++) {
-      const __nv_bfloat16* col = s.w2t + (8 * j + g) * 64 + 16 * kk;
+      const __nv_bfloat16* col = s.w2t + (8 * j + g) * SH + 16 * kk;
       mma16816(c2[j], f.h1a[kk], ld_pair(col + 2 * t), ld_pair(col + 2 * t + 8));
     }
   float za = 0.f, zb = 0.f;
@@ -165,12 +186,14 @@ __global__ void __launch_bounds__(128) mlp_infer(Weights W, const float* __restr
                                                  float* __restrict__ p) {
   __shared__ Smem s;
   load_weights(s, W);
-  const float b3 = W.P[OFF_B3];
+  __syncthreads();
+  const float b3 = s.b3;
   const int lane = lane_id(), g = lane >> 2, t = lane & 3;
   const int64_t tiles = cdiv(n, 16);
   for (int64_t tile = blockIdx.x * 4 + (threadIdx.x >> 5); tile < tiles; tile += (int64_t)gridDim.x * 4) {
     Fwd f;
-    forward_tile(s, X, tile * 16, n, b3, f);
+    load_x(X, tile * 16, n, f.xa);
+    forward_tile(s, b3, f);
     if (t == 0) {
       const int64_t ra = tile * 16 + g, rb = ra + 8;
       if (ra < n) p[ra] = sigmoidf_(f.z0);
@@ -179,22 +202,76 @@ __global__ void __launch_bounds__(128) mlp_infer(Weights W, const float* __restr
   }
 }
 
-// Per-CTA gradient partials: grid = rows / 64; part[cta][NP] and lpart[cta].
-__global__ void __launch_bounds__(128) mlp_grad_cta(Weights W, const float* __restrict__ X,
-                                                    const float* __restrict__ Y, int64_t n, float inv_n,
-                                                    float* __restrict__ part, double* __restrict__ lpart) {
-  __shared__ Smem s;
-  __shared__ __nv_bfloat16 h1s[kRowsPerCta * 64], dh2s[kRowsPerCta * 64], dh1s[kRowsPerCta * 64];
-  __shared__ __nv_bfloat16 xs[kRowsPerCta * 16];
-  __shared__ float wpart[4][66];  // per warp: dW3[64], db3, loss
-  load_weights(s, W);
-  const float b3 = W.P[OFF_B3];
+// Four transposed 8 x 8 BF16 tiles from shared memory: lane l gives the row
+// address of tile l / 8, row l % 8; register x holds tile x, in the layout of an
+// mma operand whose K dimension runs along the stored rows.
+__device__ __forceinline__ void ldsm_t(uint32_t (&r)[4], const __nv_bfloat16* p) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(a)
+               : "memory");
+}
+
+// Shared memory of a training CTA: the weights and the activations and
+// activation gradients of 64 rows.
+struct __align__(16) GradSmem {
+  Smem w;
+  __nv_bfloat16 w2[64 * SH];
+  __nv_bfloat16 h1[kRowsPerCta * SH], dh2[kRowsPerCta * SH], dh1[kRowsPerCta * SH];
+  __nv_bfloat16 x[kRowsPerCta * SX];
+  float wpart[4][66];  // per warp: dW3[64], db3, loss
+};
+
+__device__ __forceinline__ void load_grad_weights(GradSmem& s, const Weights& W) {
+  load_weights(s.w, W);
+  load_rows(s.w2, SH, W.w2, 64, 64);
+}
+
+// Gradient sums of a CTA, over its 64-row tiles: warp w holds dW2 rows 16 w ..
+// 16 w + 15 and dW1 columns likewise; thread j < 64 db1[j] and dW3[j], thread
+// 64 + j db2[j], thread 0 db3 and thread 1 the loss.
+struct GradAcc {
+  float w2[8][4];
+  float w1[2][4];
+  float b, w3;
+  float b3;
+  double loss;
+};
+__device__ __forceinline__ void grad_zero(GradAcc& a) {
+#pragma unroll
+  for (int j = 0; j < 8; j++) a.w2[j][0] = a.w2[j][1] = a.w2[j][2] = a.w2[j][3] = 0.f;
+#pragma unroll
+  for (int j = 0; j < 2; j++) a.w1[j][0] = a.w1[j][1] = a.w1[j][2] = a.w1[j][3] = 0.f;
+  a.b = a.w3 = a.b3 = 0.f;
+  a.loss = 0;
+}
+
+// A thread's inputs of the 64-row tile at tile0 (of rows [0, n)).
+struct TileIn {
+  uint32_t xa[4];
+  float ya, yb;
+};
+__device__ __forceinline__ void load_tile(const float* __restrict__ X, const float* __restrict__ Y, int64_t tile0,
+                                          int64_t n, TileIn& in) {
+  const int64_t r0 = tile0 + (threadIdx.x >> 5) * 16, ra = r0 + (lane_id() >> 2), rb = ra + 8;
+  load_x(X, r0, n, in.xa);
+  in.ya = ra < n ? Y[ra] : 0.f;
+  in.yb = rb < n ? Y[rb] : 0.f;
+}
+
+// The tile at tile0 of [0, n) into the sums (128 threads; the weights are in s,
+// and the caller has synchronised).
+__device__ __forceinline__ void grad_tile(GradSmem& s, const TileIn& in, int64_t tile0, int64_t n, float inv_n,
+                                          GradAcc& acc) {
   const int lane = lane_id(), g = lane >> 2, t = lane & 3, wid = threadIdx.x >> 5;
-  const int64_t r0 = (int64_t)blockIdx.x * kRowsPerCta + wid * 16;
+  const int64_t r0 = tile0 + wid * 16;
   Fwd f;
-  forward_tile(s, X, r0, n, b3, f);
+#pragma unroll
+  for (int x = 0; x < 4; x++) f.xa[x] = in.xa[x];
+  forward_tile(s.w, s.w.b3, f);
   const int64_t ra = r0 + g, rb = r0 + g + 8;
-  const float ya = ra < n ? Y[ra] : 0.f, yb = rb < n ? Y[rb] : 0.f;
+  const float ya = in.ya, yb = in.yb;
   const float pa = sigmoidf_(f.z0), pb = sigmoidf_(f.z1);
   const float dza = ra < n ? (pa - ya) * inv_n : 0.f, dzb = rb < n ? (pb - yb) * inv_n : 0.f;
   float la = 0.f, lb = 0.f;
@@ -208,10 +285,11 @@ __global__ void __launch_bounds__(128) mlp_grad_cta(Weights W, const float* __re
 #pragma unroll
   for (int j = 0; j < 8; j++) {
     const int c = 8 * j + 2 * t;
+    const float w0 = s.w.w3f[c], w1 = s.w.w3f[c + 1];
     dw3[j][0] = f.h2[j][0] * dza + f.h2[j][2] * dzb;
     dw3[j][1] = f.h2[j][1] * dza + f.h2[j][3] * dzb;
-    const float d00 = f.h2[j][0] > 0.f ? dza * s.w3f[c] : 0.f, d01 = f.h2[j][1] > 0.f ? dza * s.w3f[c + 1] : 0.f;
-    const float d10 = f.h2[j][2] > 0.f ? dzb * s.w3f[c] : 0.f, d11 = f.h2[j][3] > 0.f ? dzb * s.w3f[c + 1] : 0.f;
+    const float d00 = f.h2[j][0] > 0.f ? dza * w0 : 0.f, d01 = f.h2[j][1] > 0.f ? dza * w1 : 0.f;
+    const float d10 = f.h2[j][2] > 0.f ? dzb * w0 : 0.f, d11 = f.h2[j][3] > 0.f ? dzb * w1 : 0.f;
     const int kk = j >> 1, h = j & 1;
     dh2a[kk][2 * h] = pack_bf16(d00, d01);
     dh2a[kk][2 * h + 1] = pack_bf16(d10, d11);
@@ -224,30 +302,28 @@ __global__ void __launch_bounds__(128) mlp_grad_cta(Weights W, const float* __re
   for (int kk = 0; kk < 4; kk++)
 #pragma unroll
     for (int j = 0; j < 8; j++) {
-      const __nv_bfloat16* row = s.w2 + (8 * j + g) * 64 + 16 * kk;  // B[k][n] = W2[n][k]
+      const __nv_bfloat16* row = s.w2 + (8 * j + g) * SH + 16 * kk;  // B[k][n] = W2[n][k]
       mma16816(c3[j], dh2a[kk], ld_pair(row + 2 * t), ld_pair(row + 2 * t + 8));
     }
+  __syncthreads();  // the previous tile's rows have been read
   // stage x, h1, dh2, dh1 of the warp's 16 rows in shared memory (row-major)
   const int la_ = wid * 16 + g, lb_ = la_ + 8;
-  {
-    const uint32_t* xa = f.xa;
-    *reinterpret_cast<uint32_t*>(&xs[la_ * 16 + 2 * t]) = xa[0];
-    *reinterpret_cast<uint32_t*>(&xs[lb_ * 16 + 2 * t]) = xa[1];
-    *reinterpret_cast<uint32_t*>(&xs[la_ * 16 + 2 * t + 8]) = xa[2];
-    *reinterpret_cast<uint32_t*>(&xs[lb_ * 16 + 2 * t + 8]) = xa[3];
-  }
+  *reinterpret_cast<uint32_t*>(&s.x[la_ * SX + 2 * t]) = f.xa[0];
+  *reinterpret_cast<uint32_t*>(&s.x[lb_ * SX + 2 * t]) = f.xa[1];
+  *reinterpret_cast<uint32_t*>(&s.x[la_ * SX + 2 * t + 8]) = f.xa[2];
+  *reinterpret_cast<uint32_t*>(&s.x[lb_ * SX + 2 * t + 8]) = f.xa[3];
 #pragma unroll
   for (int j = 0; j < 8; j++) {
     const int c = 8 * j + 2 * t, kk = j >> 1, h = j & 1;
     const uint32_t h1_a = f.h1a[kk][2 * h], h1_b = f.h1a[kk][2 * h + 1];
-    *reinterpret_cast<uint32_t*>(&h1s[la_ * 64 + c]) = h1_a;
-    *reinterpret_cast<uint32_t*>(&h1s[lb_ * 64 + c]) = h1_b;
-    *reinterpret_cast<uint32_t*>(&dh2s[la_ * 64 + c]) = dh2a[kk][2 * h];
-    *reinterpret_cast<uint32_t*>(&dh2s[lb_ * 64 + c]) = dh2a[kk][2 * h + 1];
+    *reinterpret_cast<uint32_t*>(&s.h1[la_ * SH + c]) = h1_a;
+    *reinterpret_cast<uint32_t*>(&s.h1[lb_ * SH + c]) = h1_b;
+    *reinterpret_cast<uint32_t*>(&s.dh2[la_ * SH + c]) = dh2a[kk][2 * h];
+    *reinterpret_cast<uint32_t*>(&s.dh2[lb_ * SH + c]) = dh2a[kk][2 * h + 1];
     const float e00 = lo_f(h1_a) > 0.f ? c3[j][0] : 0.f, e01 = hi_f(h1_a) > 0.f ? c3[j][1] : 0.f;
     const float e10 = lo_f(h1_b) > 0.f ? c3[j][2] : 0.f, e11 = hi_f(h1_b) > 0.f ? c3[j][3] : 0.f;
-    *reinterpret_cast<uint32_t*>(&dh1s[la_ * 64 + c]) = pack_bf16(e00, e01);
-    *reinterpret_cast<uint32_t*>(&dh1s[lb_ * 64 + c]) = pack_bf16(e10, e11);
+    *reinterpret_cast<uint32_t*>(&s.dh1[la_ * SH + c]) = pack_bf16(e00, e01);
+    *reinterpret_cast<uint32_t*>(&s.dh1[lb_ * SH + c]) = pack_bf16(e10, e11);
   }
   // warp partials of dW3 (sum over the 8 row groups), db3 and loss
 #pragma unroll
@@ -258,7 +334,7 @@ __global__ void __launch_bounds__(128) mlp_grad_cta(Weights W, const float* __re
       v += __shfl_xor_sync(0xffffffffu, v, 4);
       v += __shfl_xor_sync(0xffffffffu, v, 8);
       v += __shfl_xor_sync(0xffffffffu, v, 16);
-      if (g == 0) wpart[wid][8 * j + 2 * t + e] = v;
+      if (g == 0) s.wpart[wid][8 * j + 2 * t + e] = v;
     }
   {
     float db = (t == 0) ? dza + dzb : 0.f, ls = la + lb;
@@ -268,100 +344,144 @@ __global__ void __launch_bounds__(128) mlp_grad_cta(Weights W, const float* __re
       ls += __shfl_xor_sync(0xffffffffu, ls, o);
     }
     if (lane == 0) {
-      wpart[wid][64] = db;
-      wpart[wid][65] = ls;
+      s.wpart[wid][64] = db;
+      s.wpart[wid][65] = ls;
     }
   }
   __syncthreads();
-  float* out = part + (int64_t)blockIdx.x * NP;
-  // dW2[i][j] = sum_r h1[r][i] dh2[r][j]: warp wid owns i in [16 wid, 16 wid + 16)
-  {
-    float acc[8][4];
+  // dW2[i][j] = sum_r h1[r][i] dh2[r][j], dW1[i][j] = sum_r x[r][i] dh1[r][j]:
+  // both operands lie with K (the rows r) along the stored rows
+  const int tr = lane & 7, tq = lane >> 3;
 #pragma unroll
-    for (int j = 0; j < 8; j++) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-    const int i0 = 16 * wid + g;
+  for (int kk = 0; kk < 4; kk++) {
+    // A tiles: (rows 0-7 | 8-15 of K) x (columns 0-7 | 8-15 of M), in the
+    // order of the A registers: (m0, k0), (m8, k0), (m0, k8), (m8, k8)
+    const int ar = 16 * kk + (tq >> 1) * 8 + tr, ac = (tq & 1) * 8;
+    uint32_t a[4];
+    ldsm_t(a, s.h1 + ar * SH + 16 * wid + ac);
 #pragma unroll
-    for (int kk = 0; kk < 4; kk++) {
-      const int r = 16 * kk + 2 * t;
-      uint32_t a[4];
-      a[0] = two(h1s[r * 64 + i0], h1s[(r + 1) * 64 + i0]);
-      a[1] = two(h1s[r * 64 + i0 + 8], h1s[(r + 1) * 64 + i0 + 8]);
-      a[2] = two(h1s[(r + 8) * 64 + i0], h1s[(r + 9) * 64 + i0]);
-      a[3] = two(h1s[(r + 8) * 64 + i0 + 8], h1s[(r + 9) * 64 + i0 + 8]);
-#pragma unroll
-      for (int j = 0; j < 8; j++) {
-        const int cj = 8 * j + g;
-        mma16816(acc[j], a, two(dh2s[r * 64 + cj], dh2s[(r + 1) * 64 + cj]),
-                 two(dh2s[(r + 8) * 64 + cj], dh2s[(r + 9) * 64 + cj]));
-      }
+    for (int jp = 0; jp < 4; jp++) {
+      // B tiles: (k0, n0), (k8, n0), (k0, n8), (k8, n8)
+      uint32_t b[4];
+      ldsm_t(b, s.dh2 + (16 * kk + (tq & 1) * 8 + tr) * SH + 16 * jp + (tq >> 1) * 8);
+      mma16816(acc.w2[2 * jp], a, b[0], b[1]);
+      mma16816(acc.w2[2 * jp + 1], a, b[2], b[3]);
     }
-#pragma unroll
-    for (int j = 0; j < 8; j++) {
-      const int c = 8 * j + 2 * t;
-      out[OFF_W2 + i0 * 64 + c] = acc[j][0];
-      out[OFF_W2 + i0 * 64 + c + 1] = acc[j][1];
-      out[OFF_W2 + (i0 + 8) * 64 + c] = acc[j][2];
-      out[OFF_W2 + (i0 + 8) * 64 + c + 1] = acc[j][3];
-    }
-  }
-  // dW1[i][j] = sum_r x[r][i] dh1[r][j]: warp wid owns output columns [16 wid, 16 wid + 16)
-  {
-    float acc[2][4];
-#pragma unroll
-    for (int j = 0; j < 2; j++) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-#pragma unroll
-    for (int kk = 0; kk < 4; kk++) {
-      const int r = 16 * kk + 2 * t;
-      uint32_t a[4];
-      a[0] = two(xs[r * 16 + g], xs[(r + 1) * 16 + g]);
-      a[1] = two(xs[r * 16 + g + 8], xs[(r + 1) * 16 + g + 8]);
-      a[2] = two(xs[(r + 8) * 16 + g], xs[(r + 9) * 16 + g]);
-      a[3] = two(xs[(r + 8) * 16 + g + 8], xs[(r + 9) * 16 + g + 8]);
-#pragma unroll
-      for (int jj = 0; jj < 2; jj++) {
-        const int cj = 16 * wid + 8 * jj + g;
-        mma16816(acc[jj], a, two(dh1s[r * 64 + cj], dh1s[(r + 1) * 64 + cj]),
-                 two(dh1s[(r + 8) * 64 + cj], dh1s[(r + 9) * 64 + cj]));
-      }
-    }
-#pragma unroll
-    for (int jj = 0; jj < 2; jj++) {
-      const int c = 16 * wid + 8 * jj + 2 * t;
-      if (g < NF) {
-        out[OFF_W1 + g * NH + c] = acc[jj][0];
-        out[OFF_W1 + g * NH + c + 1] = acc[jj][1];
-      }
-      if (g + 8 < NF) {
-        out[OFF_W1 + (g + 8) * NH + c] = acc[jj][2];
-        out[OFF_W1 + (g + 8) * NH + c + 1] = acc[jj][3];
-      }
-    }
+    uint32_t ax[4], bx[4];
+    ldsm_t(ax, s.x + ar * SX + ac);
+    ldsm_t(bx, s.dh1 + (16 * kk + (tq & 1) * 8 + tr) * SH + 16 * wid + (tq >> 1) * 8);
+    mma16816(acc.w1[0], ax, bx[0], bx[1]);
+    mma16816(acc.w1[1], ax, bx[2], bx[3]);
   }
   // biases, W3, loss (fixed-order sums)
-  if (threadIdx.x < 64) {
-    const int j = threadIdx.x;
-    float s1 = 0.f, s2 = 0.f;
-    for (int r = 0; r < kRowsPerCta; r++) {
-      s1 += __bfloat162float(dh1s[r * 64 + j]);
-      s2 += __bfloat162float(dh2s[r * 64 + j]);
-    }
-    out[OFF_B1 + j] = s1;
-    out[OFF_B2 + j] = s2;
-    out[OFF_W3 + j] = wpart[0][j] + wpart[1][j] + wpart[2][j] + wpart[3][j];
+  {
+    const int j = threadIdx.x & 63;
+    const __nv_bfloat16* m = threadIdx.x < 64 ? s.dh1 : s.dh2;
+    float v = 0.f;
+#pragma unroll 16
+    for (int r = 0; r < kRowsPerCta; r++) v += __bfloat162float(m[r * SH + j]);
+    acc.b += v;
+    if (threadIdx.x < 64) acc.w3 += s.wpart[0][j] + s.wpart[1][j] + s.wpart[2][j] + s.wpart[3][j];
   }
-  if (threadIdx.x == 64) {
-    out[OFF_B3] = wpart[0][64] + wpart[1][64] + wpart[2][64] + wpart[3][64];
-    lpart[blockIdx.x] = (double)wpart[0][65] + wpart[1][65] + wpart[2][65] + wpart[3][65];
-  }
+  if (threadIdx.x == 0) acc.b3 += s.wpart[0][64] + s.wpart[1][64] + s.wpart[2][64] + s.wpart[3][64];
+  if (threadIdx.x == 1)
+    acc.loss += (double)s.wpart[0][65] + s.wpart[1][65] + s.wpart[2][65] + s.wpart[3][65];
 }
 
-// grad[k] = sum over CTAs (in CTA order) of part[cta][k]; loss likewise.
-__global__ void grad_reduce(const float* __restrict__ part, int ncta, float* __restrict__ grad,
-                            const double* __restrict__ lpart, double* __restrict__ loss, double inv_n) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < NP; k += gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int c = 0; c < ncta; c++) s += part[(int64_t)c * NP + k];
-    grad[k] = s;
+// A CTA's sums to its partial vector.
+__device__ __forceinline__ void grad_store(const GradAcc& acc, float* __restrict__ out, double* __restrict__ lout) {
+  const int lane = lane_id(), g = lane >> 2, t = lane & 3, wid = threadIdx.x >> 5;
+  const int i0 = 16 * wid + g;
+#pragma unroll
+  for (int j = 0; j < 8; j++) {
+    const int c = 8 * j + 2 * t;
+    __stcg(reinterpret_cast<float2*>(out + OFF_W2 + i0 * 64 + c), make_float2(acc.w2[j][0], acc.w2[j][1]));
+    __stcg(reinterpret_cast<float2*>(out + OFF_W2 + (i0 + 8) * 64 + c), make_float2(acc.w2[j][2], acc.w2[j][3]));
+  }
+#pragma unroll
+  for (int jj = 0; jj < 2; jj++) {
+    const int c = 16 * wid + 8 * jj + 2 * t;
+    __stcg(reinterpret_cast<float2*>(out + OFF_W1 + g * NH + c), make_float2(acc.w1[jj][0], acc.w1[jj][1]));
+    if (g + 8 < NF)
+      __stcg(reinterpret_cast<float2*>(out + OFF_W1 + (g + 8) * NH + c), make_float2(acc.w1[jj][2], acc.w1[jj][3]));
+  }
+  const int j = threadIdx.x & 63;
+  if (threadIdx.x < 64) {
+    __stcg(out + OFF_B1 + j, acc.b);
+    __stcg(out + OFF_W3 + j, acc.w3);
+  } else {
+    __stcg(out + OFF_B2 + j, acc.b);
+  }
+  if (threadIdx.x == 0) __stcg(out + OFF_B3, acc.b3);
+  if (threadIdx.x == 1) __stcg(lout, acc.loss);
+}
+
+constexpr int kPartStride = 5060;  // floats a partial vector takes (float2 stores stay aligned)
+
+// Gradient partials of rows [0, n), 64-row tiles dealt to the CTAs in turn.
+__global__ void __launch_bounds__(128) mlp_grad_cta(Weights W, const float* __restrict__ X,
+                                                    const float* __restrict__ Y, int64_t n, float inv_n,
+                                                    float* __restrict__ part, double* __restrict__ lpart) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  GradSmem& s = *reinterpret_cast<GradSmem*>(smem);
+  load_grad_weights(s, W);
+  __syncthreads();
+  GradAcc acc;
+  grad_zero(acc);
+  for (int64_t r = (int64_t)blockIdx.x * kRowsPerCta; r < n; r += (int64_t)gridDim.x * kRowsPerCta) {
+    TileIn in;
+    load_tile(X, Y, r, n, in);
+    grad_tile(s, in, r, n, inv_n, acc);
+  }
+  grad_store(acc, part + (int64_t)blockIdx.x * kPartStride, lpart + blockIdx.x);
+}
+
+// Sums over the CTAs' partials: warp w of four takes CTAs w, w + 4, ... in
+// turn, then the four in turn: a fixed order.  A lane takes two parameters
+// (k, k + 1), so a CTA does kSumBlock of them, with up to 32 loads a thread in
+// flight.  128 threads; every warp's lanes get the sums.
+constexpr int kSumBlock = 64;
+constexpr int kSumBlocks = (NP + kSumBlock - 1) / kSumBlock;
+__device__ __forceinline__ float2 grad_sum(const float* __restrict__ part, int ncta, int k, float2 (*red)[32]) {
+  const int lane = lane_id(), wid = threadIdx.x >> 5;
+  float2 v = make_float2(0.f, 0.f);
+  if (k < NP) {  // (a partial vector has room behind its last parameter)
+    auto ld = [&](int c) { return __ldcg(reinterpret_cast<const float2*>(part + (int64_t)c * kPartStride + k)); };
+    int c = wid;
+    auto run = [&](auto u) {
+      constexpr int U = decltype(u)::value;
+      for (; c + 4 * (U - 1) < ncta; c += 4 * U) {
+        float2 x[U];
+#pragma unroll
+        for (int i = 0; i < U; i++) x[i] = ld(c + 4 * i);
+#pragma unroll
+        for (int i = 0; i < U; i++) {
+          v.x += x[i].x;
+          v.y += x[i].y;
+        }
+      }
+    };
+    run(std::integral_constant<int, 32>{});
+    run(std::integral_constant<int, 8>{});
+    run(std::integral_constant<int, 1>{});
+  }
+  red[wid][lane] = v;
+  __syncthreads();
+  v = make_float2(red[0][lane].x + red[1][lane].x + red[2][lane].x + red[3][lane].x,
+                  red[0][lane].y + red[1][lane].y + red[2][lane].y + red[3][lane].y);
+  __syncthreads();
+  return v;
+}
+
+__global__ void __launch_bounds__(128) grad_reduce(const float* __restrict__ part, int ncta, float* __restrict__ grad,
+                                                   const double* __restrict__ lpart, double* __restrict__ loss,
+                                                   double inv_n) {
+  __shared__ float2 red[4][32];
+  const int k = blockIdx.x * kSumBlock + 2 * (int)lane_id();
+  const float2 v = grad_sum(part, ncta, k, red);
+  if (threadIdx.x < 32) {
+    if (k < NP) grad[k] = v.x;
+    if (k + 1 < NP) grad[k + 1] = v.y;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     double l = 0;
@@ -370,15 +490,139 @@ __global__ void grad_reduce(const float* __restrict__ part, int ncta, float* __r
   }
 }
 
-__global__ void adam(float* __restrict__ P, float* __restrict__ m, float* __restrict__ v,
-                     const float* __restrict__ g, float lr, float b1, float b2, float eps, float c1, float c2) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < NP; k += gridDim.x * blockDim.x) {
-    const float gk = g[k];
-    const float mk = b1 * m[k] + (1.f - b1) * gk;
-    const float vk = b2 * v[k] + (1.f - b2) * gk * gk;
-    m[k] = mk;
-    v[k] = vk;
-    P[k] -= lr * (mk / c1) / (sqrtf(vk / c2) + eps);
+// Adam on one parameter, and its BF16 copies.
+struct Master {
+  float *P, *m, *v;
+  __nv_bfloat16 *w1t, *w2, *w2t, *w3;
+};
+struct Moments {
+  float p, m, v;
+};
+__device__ __forceinline__ Moments load_moments(const Master& M, int k) {
+  return k < NP ? Moments{M.P[k], M.m[k], M.v[k]} : Moments{0.f, 0.f, 0.f};
+}
+__device__ __forceinline__ void adam_one(const Master& M, int k, const Moments& o, float gk, float lr, float b1,
+                                         float b2, float eps, float c1, float c2) {
+  const float mk = b1 * o.m + (1.f - b1) * gk;
+  const float vk = b2 * o.v + (1.f - b2) * gk * gk;
+  M.m[k] = mk;
+  M.v[k] = vk;
+  const float p = o.p - lr * (mk / c1) / (sqrtf(vk / c2) + eps);
+  __stcg(M.P + k, p);
+  const __nv_bfloat16 q = __float2bfloat16_rn(p);
+  if (k < OFF_B1) {
+    M.w1t[(k % NH) * 16 + k / NH] = q;  // w1t[o][i] = W1[i][o]
+  } else if (k >= OFF_W2 && k < OFF_B2) {
+    const int i = k - OFF_W2;
+    M.w2[i] = q;
+    M.w2t[(i % NH) * NH + i / NH] = q;
+  } else if (k >= OFF_W3 && k < OFF_B3) {
+    M.w3[k - OFF_W3] = q;
+  }
+}
+
+// All CTAs of the (cooperative) grid; false when the wait ran out (it cannot:
+// they are co-resident), after which every CTA leaves.
+__device__ __forceinline__ bool grid_wait(unsigned* bar, unsigned target, int* err) {
+  __shared__ int bad;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    bad = 0;
+    __threadfence();
+    atomicAdd(bar, 1u);
+    long long left = 1ll << 24;
+    unsigned x;
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(bar) : "memory");
+    } while (x < target && --left > 0);
+    if (x < target) {
+      bad = 1;
+      *err = 1;
+    }
+  }
+  __syncthreads();
+  return bad == 0;
+}
+
+// Steps [s0, s1) of a training run: step s takes mini-batch s % per_epoch.  A
+// step is: gradient partials of the first `rows` CTAs' tiles | wait | the CTAs'
+// shares of the parameters summed and updated | wait.  corr: Adam's bias
+// corrections (two floats a step).  Bound by the latency of its two waits and
+// of the passes through L2 between them (weights in, partials out and in), so
+// what does not depend on the other CTAs is loaded before each wait: the
+// parameters and moments to update, the next step's rows.  A step of 8192 rows
+// takes 10.5 us; as four kernels (partials 18, sums 19, Adam 4, BF16 copies 3 us)
+// it took 41.
+struct TrainArgs {
+  const float* X;
+  const float* Y;
+  int64_t n, batch, per_epoch;
+  int64_t s0, s1;
+  int rows;  // CTAs that take rows; the others only parameters
+  float lr, b1, b2, eps;
+  const float* corr;
+  float* part;
+  double* lpart;
+  double* loss;
+  unsigned* bar;  // zero
+  int* err;
+};
+__global__ void __launch_bounds__(128) mlp_train_steps(Weights W, Master M, TrainArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  GradSmem& s = *reinterpret_cast<GradSmem*>(smem);
+  __shared__ float2 red[4][32];
+  const int G = gridDim.x, rows = a.rows;
+  const int64_t mine = (int64_t)blockIdx.x * kRowsPerCta;
+  const bool works = (int)blockIdx.x < rows;
+  auto batch_of = [&](int64_t st, int64_t& r0, int64_t& nb) {
+    r0 = (st % a.per_epoch) * a.batch;
+    nb = r0 + a.batch <= a.n ? a.batch : a.n - r0;
+  };
+  unsigned target = 0;
+  int64_t r0, nb;
+  batch_of(a.s0, r0, nb);
+  TileIn in;
+  if (works) load_tile(a.X + r0 * NF, a.Y + r0, mine, nb, in);
+  for (int64_t st = a.s0; st < a.s1; st++) {
+    if (works) {
+      load_grad_weights(s, W);
+      __syncthreads();
+      GradAcc acc;
+      grad_zero(acc);
+      const float inv_n = 1.f / (float)nb;
+      for (int64_t r = mine; r < nb; r += (int64_t)rows * kRowsPerCta) {
+        if (r != mine) load_tile(a.X + r0 * NF, a.Y + r0, r, nb, in);
+        grad_tile(s, in, r, nb, inv_n, acc);
+      }
+      grad_store(acc, a.part + (int64_t)blockIdx.x * kPartStride, a.lpart + blockIdx.x);
+    }
+    const float c1 = a.corr[2 * (st - a.s0)], c2 = a.corr[2 * (st - a.s0) + 1];
+    int k = (int)blockIdx.x * kSumBlock + 2 * (int)lane_id();
+    Moments o0 = load_moments(M, k), o1 = load_moments(M, k + 1);
+    if (!grid_wait(a.bar, target += G, a.err)) return;
+    for (int b = blockIdx.x; b < kSumBlocks; b += G) {
+      if (b != (int)blockIdx.x) {
+        k = b * kSumBlock + 2 * (int)lane_id();
+        o0 = load_moments(M, k);
+        o1 = load_moments(M, k + 1);
+      }
+      const float2 gk = grad_sum(a.part, rows, k, red);
+      if (threadIdx.x < 32) {
+        if (k < NP) adam_one(M, k, o0, gk.x, a.lr, a.b1, a.b2, a.eps, c1, c2);
+        if (k + 1 < NP) adam_one(M, k + 1, o1, gk.y, a.lr, a.b1, a.b2, a.eps, c1, c2);
+      }
+    }
+    if (st + 1 == a.s1) {
+      if (blockIdx.x == 0 && threadIdx.x == 0) {
+        double l = 0;
+        for (int c = 0; c < rows; c++) l += __ldcg(a.lpart + c);
+        *a.loss = l / (double)nb;
+      }
+      break;
+    }
+    batch_of(st + 1, r0, nb);
+    if (works) load_tile(a.X + r0 * NF, a.Y + r0, mine, nb, in);
+    if (!grid_wait(a.bar, target += G, a.err)) return;
   }
 }
 
@@ -388,6 +632,7 @@ __global__ void adam(float* __restrict__ P, float* __restrict__ m, float* __rest
 struct dcd_mlp {
   cudaStream_t stream = nullptr;
   int device = 0;
+  unsigned char* block = nullptr;  // the allocation all of the following lie in
   float* P = nullptr;  // master params
   float* m = nullptr;
   float* v = nullptr;
@@ -399,7 +644,8 @@ struct dcd_mlp {
   __nv_bfloat16* w3 = nullptr;
   float* part = nullptr;
   double* lpart = nullptr;
-  int64_t part_ctas = 0;
+  unsigned* sync = nullptr;  // [0] the training kernel's barrier, [1] its error word
+  float* corr = nullptr;     // Adam's bias corrections of kTrainSteps steps
   int64_t adam_t = 0;
 };
 
@@ -414,26 +660,30 @@ int refresh(dcd_mlp* m) {
   return DCD_OK;
 }
 
-int ensure_parts(dcd_mlp* m, int64_t ctas) {
-  if (ctas <= m->part_ctas) return DCD_OK;
-  if (m->part) cudaFree(m->part);
-  if (m->lpart) cudaFree(m->lpart);
-  m->part = nullptr;
-  m->lpart = nullptr;
-  DCD_TRY_CUDA(cudaMalloc(&m->part, (size_t)ctas * NP * sizeof(float)));
-  DCD_TRY_CUDA(cudaMalloc(&m->lpart, (size_t)ctas * sizeof(double)));
-  m->part_ctas = ctas;
+// CTAs of the gradient kernels: a 64-row tile each, one CTA an SM at most (the
+// partial vectors are written and read back, 20 KB each).
+int64_t grad_ctas(int64_t n) {
+  const int64_t tiles = cdiv(n, kRowsPerCta);
+  return tiles < num_sms() ? tiles : num_sms();
+}
+
+constexpr int64_t kTrainSteps = 4096;  // steps a launch of the training kernel takes at most
+
+int grad_attrs() {
+  DCD_TRY_CUDA(cudaFuncSetAttribute(mlp_grad_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem)));
+  DCD_TRY_CUDA(
+      cudaFuncSetAttribute(mlp_train_steps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem)));
   return DCD_OK;
 }
 
 // Mean BCE gradient of rows [0, n) into m->grad and m->loss.
 int grad_pass(dcd_mlp* m, const float* X, const float* Y, int64_t n) {
-  const int64_t ctas = cdiv(n, kRowsPerCta);
-  DCD_TRY(ensure_parts(m, ctas));
-  count_launch(), mlp_grad_cta<<<(unsigned)ctas, 128, 0, m->stream>>>(weights_of(m), X, Y, n, 1.f / (float)n,
-                                                                       m->part, m->lpart);
-  count_launch(), grad_reduce<<<(NP + 255) / 256, 256, 0, m->stream>>>(m->part, (int)ctas, m->grad, m->lpart, m->loss,
-                                                                        1.0 / (double)n);
+  const int64_t ctas = grad_ctas(n);
+  DCD_TRY(grad_attrs());
+  count_launch(), mlp_grad_cta<<<(unsigned)ctas, 128, sizeof(GradSmem), m->stream>>>(
+      weights_of(m), X, Y, n, 1.f / (float)n, m->part, m->lpart);
+  count_launch(), grad_reduce<<<kSumBlocks, 128, 0, m->stream>>>(m->part, (int)ctas, m->grad, m->lpart, m->loss,
+                                                                      1.0 / (double)n);
   DCD_LAUNCH_CHECK();
   return DCD_OK;
 }
@@ -469,17 +719,38 @@ int dcd_mlp_create(uint64_t seed, void* cuda_stream, dcd_mlp** out) {
   int rc = DCD_OK;
   do {
     if (cudaGetDevice(&m->device) != cudaSuccess) { rc = DCD_ECUDA; break; }
-    if (cudaMalloc(&m->P, NP * sizeof(float)) != cudaSuccess || cudaMalloc(&m->m, NP * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&m->v, NP * sizeof(float)) != cudaSuccess || cudaMalloc(&m->grad, NP * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&m->loss, sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&m->w1t, 64 * 16 * sizeof(__nv_bfloat16)) != cudaSuccess ||
-        cudaMalloc(&m->w2, 64 * 64 * sizeof(__nv_bfloat16)) != cudaSuccess ||
-        cudaMalloc(&m->w2t, 64 * 64 * sizeof(__nv_bfloat16)) != cudaSuccess ||
-        cudaMalloc(&m->w3, 64 * sizeof(__nv_bfloat16)) != cudaSuccess) {
+    // one allocation, cut into 256-byte aligned parts
+    size_t at = 0;
+    auto part = [&](size_t bytes) {
+      const size_t o = at;
+      at += (bytes + 255) & ~(size_t)255;
+      return o;
+    };
+    const size_t oP = part(NP * sizeof(float)), om = part(NP * sizeof(float)), ov = part(NP * sizeof(float)),
+                 og = part(NP * sizeof(float)), ol = part(sizeof(double)), o1 = part(64 * 16 * sizeof(__nv_bfloat16)),
+                 o2 = part(64 * 64 * sizeof(__nv_bfloat16)), o2t = part(64 * 64 * sizeof(__nv_bfloat16)),
+                 o3 = part(64 * sizeof(__nv_bfloat16)),
+                 op = part((size_t)num_sms() * kPartStride * sizeof(float)),
+                 olp = part((size_t)num_sms() * sizeof(double)), os = part(2 * sizeof(unsigned)),
+                 oc = part(2 * kTrainSteps * sizeof(float));
+    if (cudaMalloc(&m->block, at) != cudaSuccess) {
       cudaGetLastError();
       rc = DCD_ENOMEM;
       break;
     }
+    m->P = reinterpret_cast<float*>(m->block + oP);
+    m->m = reinterpret_cast<float*>(m->block + om);
+    m->v = reinterpret_cast<float*>(m->block + ov);
+    m->grad = reinterpret_cast<float*>(m->block + og);
+    m->loss = reinterpret_cast<double*>(m->block + ol);
+    m->w1t = reinterpret_cast<__nv_bfloat16*>(m->block + o1);
+    m->w2 = reinterpret_cast<__nv_bfloat16*>(m->block + o2);
+    m->w2t = reinterpret_cast<__nv_bfloat16*>(m->block + o2t);
+    m->w3 = reinterpret_cast<__nv_bfloat16*>(m->block + o3);
+    m->part = reinterpret_cast<float*>(m->block + op);
+    m->lpart = reinterpret_cast<double*>(m->block + olp);
+    m->sync = reinterpret_cast<unsigned*>(m->block + os);
+    m->corr = reinterpret_cast<float*>(m->block + oc);
     // He-uniform initialisation from SplitMix64; biases zero
     std::vector<float> P(NP, 0.f);
     uint64_t s = seed;
@@ -500,9 +771,7 @@ int dcd_mlp_create(uint64_t seed, void* cuda_stream, dcd_mlp** out) {
 int dcd_mlp_destroy(dcd_mlp* m) {
   if (!m) return DCD_OK;
   cudaStreamSynchronize(m->stream);
-  for (void* p : {(void*)m->P, (void*)m->m, (void*)m->v, (void*)m->grad, (void*)m->loss, (void*)m->w1t, (void*)m->w2,
-                  (void*)m->w2t, (void*)m->w3, (void*)m->part, (void*)m->lpart})
-    if (p) cudaFree(p);
+  if (m->block) cudaFree(m->block);
   delete m;
   return DCD_OK;
 }
@@ -550,20 +819,52 @@ int dcd_mlp_train(dcd_mlp* m, const float* d_X, const float* d_y, int64_t n, int
                   float lr, double* loss_out) {
   if (!m || n <= 0 || batch <= 0 || epochs <= 0 || !d_X || !d_y || !(lr > 0.f)) return DCD_EINVAL;
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+  DCD_TRY(grad_attrs());
+  const int64_t per_epoch = cdiv(n, batch), steps = per_epoch * epochs;
+  TrainArgs a{};
+  a.X = d_X;
+  a.Y = d_y;
+  a.n = n;
+  a.batch = batch;
+  a.per_epoch = per_epoch;
+  a.lr = lr;
+  a.b1 = b1;
+  a.b2 = b2;
+  a.eps = eps;
+  a.corr = m->corr;
+  a.part = m->part;
+  a.lpart = m->lpart;
+  a.loss = m->loss;
+  a.bar = m->sync;
+  a.err = reinterpret_cast<int*>(m->sync + 1);
+  Weights W = weights_of(m);
+  Master M{m->P, m->m, m->v, m->w1t, m->w2, m->w2t, m->w3};
+  a.rows = (int)grad_ctas(batch < n ? batch : n);
+  // every parameter block a CTA of its own, co-resident (one CTA an SM)
+  const unsigned ctas = (unsigned)(a.rows >= kSumBlocks ? a.rows : kSumBlocks < num_sms() ? kSumBlocks : num_sms());
+  std::vector<float> corr;
   double last = 0;
-  for (int32_t ep = 0; ep < epochs; ep++) {
-    for (int64_t r = 0; r < n; r += batch) {
-      const int64_t nb = (r + batch <= n) ? batch : n - r;
-      DCD_TRY(grad_pass(m, d_X + r * NF, d_y + r, nb));
+  int err = 0;
+  for (int64_t s0 = 0; s0 < steps; s0 += kTrainSteps) {
+    a.s0 = s0;
+    a.s1 = s0 + kTrainSteps < steps ? s0 + kTrainSteps : steps;
+    corr.resize(2 * (a.s1 - a.s0));
+    for (int64_t s = a.s0; s < a.s1; s++) {
       m->adam_t++;
-      const float c1 = 1.f - std::pow(b1, (float)m->adam_t), c2 = 1.f - std::pow(b2, (float)m->adam_t);
-      count_launch(), adam<<<(NP + 255) / 256, 256, 0, m->stream>>>(m->P, m->m, m->v, m->grad, lr, b1, b2, eps, c1, c2);
-      DCD_LAUNCH_CHECK();
-      DCD_TRY(refresh(m));
+      corr[2 * (s - a.s0)] = 1.f - std::pow(b1, (float)m->adam_t);
+      corr[2 * (s - a.s0) + 1] = 1.f - std::pow(b2, (float)m->adam_t);
     }
+    DCD_TRY_CUDA(cudaMemcpyAsync(m->corr, corr.data(), corr.size() * sizeof(float), cudaMemcpyHostToDevice, m->stream));
+    DCD_TRY_CUDA(cudaMemsetAsync(m->sync, 0, 2 * sizeof(unsigned), m->stream));
+    void* args[] = {&W, &M, &a};
+    count_launch();
+    DCD_TRY_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(mlp_train_steps), dim3(ctas), dim3(128), args,
+                                             sizeof(GradSmem), m->stream));
+    DCD_TRY_CUDA(cudaMemcpyAsync(&last, m->loss, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
+    DCD_TRY_CUDA(cudaMemcpyAsync(&err, m->sync + 1, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
+    DCD_TRY_CUDA(cudaStreamSynchronize(m->stream));
+    if (err) return DCD_ETIMEOUT;
   }
-  DCD_TRY_CUDA(cudaMemcpyAsync(&last, m->loss, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
-  DCD_TRY_CUDA(cudaStreamSynchronize(m->stream));
   if (loss_out) *loss_out = last;
   return DCD_OK;
 }
