@@ -38,34 +38,107 @@ __global__ void na_clear(unsigned long long* s, int64_t n) {
 }
 
 // Per row u: d_w(u), the intra-community weight of the row, and a_C += d_w(u).
-__global__ void na_rows(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                        const int32_t* __restrict__ w, const int32_t* __restrict__ L, unsigned long long* s) {
-  unsigned long long* tail = s + kNoAllocWords - kNoAllocTail;
-  unsigned long long m2 = 0, in = 0;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t u = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; u < n; u += nw) {
-    const int32_t Lu = L[u];
-    const bool ok = Lu >= 0 && Lu < n;
-    unsigned long long ks = 0, is = 0;
-    for (int64_t e = rp[u] + lane_id(); e < rp[u + 1]; e += 32) {
-      const int32_t y = col[e];
-      const unsigned long long wv = (unsigned long long)(int64_t)w[e];
+//
+// Bound by the gather of a label per entry, a 32-byte sector each (a bare gather
+// of as many runs at 250 G sectors/s).  A CTA takes 256 consecutive rows: bounds
+// and labels coalesced, then 8 lanes a row (4 rows a warp step) with 8 entries a
+// lane in flight, and rows above kNaLong entries by the whole CTA: 255 us for
+// 1 M rows and 42 M entries (16 or 32 lanes a row: 275-330).  A warp a row, one
+// entry a lane in flight, took 635 us.
+constexpr int kNaThreads = 256, kNaGroup = 8, kNaUnroll = 8, kNaLong = 512;
+
+// Entries [e0, e1) of a row with label Lu by `step` threads, kNaUnroll at once.
+__device__ __forceinline__ void na_entries(int64_t e0, int64_t e1, int step, int64_t n, const int32_t* __restrict__ col,
+                                           const int32_t* __restrict__ w, const int32_t* __restrict__ L, int32_t Lu,
+                                           unsigned long long& ks, unsigned long long& is, bool& bad) {
+  for (int64_t e = e0; e < e1; e += (int64_t)step * kNaUnroll) {
+    int32_t y[kNaUnroll], x[kNaUnroll];
+#pragma unroll
+    for (int i = 0; i < kNaUnroll; i++) {
+      const int64_t f = e + (int64_t)i * step;
+      y[i] = 0;
+      x[i] = 0;
+      if (f < e1) {
+        y[i] = ld_stream(col + f);
+        x[i] = ld_stream(w + f);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kNaUnroll; i++) {
+      const bool ok = y[i] >= 0 && y[i] < n;
+      bad |= !ok;
+      const unsigned long long wv = (unsigned long long)(int64_t)x[i];
       ks += wv;
-      if (y >= 0 && y < n && L[y] == Lu) is += wv;
-      if (y < 0 || y >= n) tail[4] = 1;
+      if (ok && L[y[i]] == Lu) is += wv;  // (a lane past the row adds a weight of 0)
     }
-    ks = warp_sum(ks);
-    is = warp_sum(is);
-    if (lane_id() == 0) {
-      if (ok) atomicAdd(&s[Lu], ks);
-      else tail[4] = 1;
-    }
-    m2 += ks;
-    in += is;
   }
-  if (lane_id() == 0) {
-    atomicAdd(&tail[0], m2);
-    atomicAdd(&tail[1], in);
+}
+
+__global__ void __launch_bounds__(kNaThreads) na_rows(int64_t n, const int64_t* __restrict__ rp,
+                                                      const int32_t* __restrict__ col, const int32_t* __restrict__ w,
+                                                      const int32_t* __restrict__ L, unsigned long long* s) {
+  __shared__ int32_t s_long[kNaThreads];
+  __shared__ int s_nlong;
+  __shared__ unsigned long long red[2][kNaThreads / 32];
+  unsigned long long* tail = s + kNoAllocWords - kNoAllocTail;
+  const int tid = threadIdx.x, lane = lane_id(), grp = lane / kNaGroup, gl = lane % kNaGroup;
+  unsigned long long m2 = 0, in = 0;
+  bool bad = false;
+  for (int64_t u0 = (int64_t)blockIdx.x * kNaThreads; u0 < n; u0 += (int64_t)gridDim.x * kNaThreads) {
+    if (tid == 0) s_nlong = 0;
+    __syncthreads();
+    const int64_t u = u0 + tid;
+    int64_t b = 0, e = 0;
+    int32_t Lu = 0;
+    if (u < n) {
+      b = rp[u];
+      e = rp[u + 1];
+      Lu = L[u];
+      if (Lu < 0 || Lu >= n) bad = true;
+      if (e - b > kNaLong) {
+        s_long[atomicAdd(&s_nlong, 1)] = tid;
+        e = b;
+      }
+    }
+    unsigned long long ks_l = 0;
+    for (int t = 0; t < kNaGroup; t++) {  // the warp's rows, four at a time
+      const int src = t * (32 / kNaGroup) + grp;
+      const int64_t rb = __shfl_sync(0xffffffffu, b, src), re = __shfl_sync(0xffffffffu, e, src);
+      const int32_t rl = __shfl_sync(0xffffffffu, Lu, src);
+      unsigned long long ks = 0, is = 0;
+      na_entries(rb + gl, re, kNaGroup, n, col, w, L, rl, ks, is, bad);
+      in += is;
+#pragma unroll
+      for (int o = kNaGroup / 2; o > 0; o >>= 1) ks += __shfl_xor_sync(0xffffffffu, ks, o);
+      const unsigned long long mine = __shfl_sync(0xffffffffu, ks, (lane & (32 / kNaGroup - 1)) * kNaGroup);
+      if (lane / (32 / kNaGroup) == t) ks_l = mine;
+    }
+    if (ks_l && Lu >= 0 && Lu < n) atomicAdd(&s[Lu], ks_l);
+    m2 += ks_l;
+    __syncthreads();
+    for (int i = 0; i < s_nlong; i++) {
+      const int64_t v = u0 + s_long[i];
+      const int32_t vl = L[v];
+      unsigned long long ks = 0;
+      na_entries(rp[v] + tid, rp[v + 1], kNaThreads, n, col, w, L, vl, ks, in, bad);
+      m2 += ks;
+      ks = warp_sum(ks);
+      if (lane == 0 && ks && vl >= 0 && vl < n) atomicAdd(&s[vl], ks);
+    }
+    __syncthreads();
+  }
+  if (bad) tail[4] = 1;
+  m2 = warp_sum(m2);
+  in = warp_sum(in);
+  if (lane == 0) {
+    red[0][tid >> 5] = m2;
+    red[1][tid >> 5] = in;
+  }
+  __syncthreads();
+  if (tid < 2) {
+    unsigned long long t = 0;
+    for (int x = 0; x < kNaThreads / 32; x++) t += red[tid][x];
+    if (t) atomicAdd(&tail[tid], t);
   }
 }
 
@@ -95,13 +168,29 @@ __global__ void na_sumsq(int64_t n, unsigned long long* s) {
   }
 }
 
-__global__ void na_final(int64_t n, unsigned long long* s) {
-  unsigned long long* tail = s + kNoAllocWords - kNoAllocTail;
-  unsigned __int128 sq = 0;
-  for (int b = 0; b < kNoAllocCtas; b++) sq += ((unsigned __int128)s[n + 2 * b + 1] << 64) | s[n + 2 * b];
-  const __int128 N = (__int128)(long long)tail[0] * (__int128)(long long)tail[1] - (__int128)sq;
-  tail[2] = (unsigned long long)N;
-  tail[3] = (unsigned long long)((unsigned __int128)N >> 64);
+// One CTA of kNoAllocCtas threads: the partials of the sum of squares in a
+// tree (integers: any order gives the same total), then N.
+__global__ void __launch_bounds__(kNoAllocCtas) na_final(int64_t n, unsigned long long* s) {
+  __shared__ unsigned long long lo_s[kNoAllocCtas], hi_s[kNoAllocCtas];
+  const int b = threadIdx.x;
+  lo_s[b] = s[n + 2 * b];
+  hi_s[b] = s[n + 2 * b + 1];
+  __syncthreads();
+  for (int o = kNoAllocCtas / 2; o > 0; o >>= 1) {
+    if (b < o) {
+      const unsigned long long x = lo_s[b], y = x + lo_s[b + o];
+      lo_s[b] = y;
+      hi_s[b] += hi_s[b + o] + (y < x ? 1ull : 0ull);
+    }
+    __syncthreads();
+  }
+  if (b == 0) {
+    unsigned long long* tail = s + kNoAllocWords - kNoAllocTail;
+    const unsigned __int128 sq = ((unsigned __int128)hi_s[0] << 64) | lo_s[0];
+    const __int128 N = (__int128)(long long)tail[0] * (__int128)(long long)tail[1] - (__int128)sq;
+    tail[2] = (unsigned long long)N;
+    tail[3] = (unsigned long long)((unsigned __int128)N >> 64);
+  }
 }
 
 // Device address of the scratch array on the current device.  Looked up on
@@ -130,9 +219,9 @@ extern "C" int dcd_modularity_noalloc(int64_t n, const int64_t* d_row_ptr, const
   DCD_TRY(scratch_for_current_device(&sc));
   const int T = 256;
   count_launch(), na_clear<<<grid_for(n, T), T, 0, s>>>(sc, n);
-  count_launch(), na_rows<<<grid_for(n * 32, T), T, 0, s>>>(n, d_row_ptr, d_col, d_w, d_labels, sc);
+  count_launch(), na_rows<<<grid_for(n, kNaThreads), kNaThreads, 0, s>>>(n, d_row_ptr, d_col, d_w, d_labels, sc);
   count_launch(), na_sumsq<<<kNoAllocCtas, T, 0, s>>>(n, sc);
-  count_launch(), na_final<<<1, 1, 0, s>>>(n, sc);
+  count_launch(), na_final<<<1, kNoAllocCtas, 0, s>>>(n, sc);
   DCD_LAUNCH_CHECK();
   unsigned long long tail[kNoAllocTail];
   DCD_TRY_CUDA(cudaMemcpyAsync(tail, sc + kNoAllocWords - kNoAllocTail, sizeof(tail), cudaMemcpyDeviceToHost, s));
