@@ -270,4 +270,26 @@ __host__ __device__ __forceinline__ uint32_t table_cap(int64_t deg) {
   return c;
 }
 
+// ---- 128-bit sums and the stop rule ----
+__device__ __forceinline__ void add128(unsigned long long* lo, unsigned long long* hi, unsigned __int128 v) {
+  const unsigned long long vlo = (unsigned long long)v, vhi = (unsigned long long)(v >> 64);
+  if (!(vlo | vhi)) return;
+  const unsigned long long old = atomicAdd(lo, vlo);
+  const unsigned long long carry = (old + vlo < old) ? 1ull : 0ull;
+  if (vhi + carry) atomicAdd(hi, vhi + carry);
+}
+
+__device__ __forceinline__ bool below_tau(i128 gain, i128 base, int64_t tau_inv) {
+  const i128 y = base < 0 ? -base : base;
+  return gain <= y / (i128)tau_inv;
+}
+
+__device__ __forceinline__ i128 ld128(const int64_t* lo) {
+  return (i128)(((unsigned __int128)(unsigned long long)lo[1] << 64) | (unsigned long long)lo[0]);
+}
+__device__ __forceinline__ void st128(int64_t* lo, i128 x) {
+  lo[0] = (int64_t)(unsigned long long)x;
+  lo[1] = (int64_t)(unsigned long long)((unsigned __int128)x >> 64);
+}
+
 }  // namespace dcd

@@ -787,14 +787,6 @@ __global__ void __launch_bounds__(256) lm_delta(LV<W> g, const int2* __restrict_
   }
 }
 
-__device__ __forceinline__ void add128(unsigned long long* lo, unsigned long long* hi, unsigned __int128 v) {
-  const unsigned long long vlo = (unsigned long long)v, vhi = (unsigned long long)(v >> 64);
-  if (!(vlo | vhi)) return;
-  const unsigned long long old = atomicAdd(lo, vlo);
-  const unsigned long long carry = (old + vlo < old) ? 1ull : 0ull;
-  if (vhi + carry) atomicAdd(hi, vhi + carry);
-}
-
 // sum over labels of a^2 per graph, unsigned 128-bit: every contribution is
 // added with a carry into the high word, so the total is exact in any order.
 // One graph: a CTA reduction then one addition per CTA; several graphs: one
@@ -835,19 +827,6 @@ __global__ void __launch_bounds__(256) sumsq_acc(const int64_t* __restrict__ a, 
     for (int w = 0; w < 8; w++) t += ((unsigned __int128)shi[w] << 64) | slo[w];
     add128(&gs[0].sq_lo, &gs[0].sq_hi, t);
   }
-}
-
-__device__ __forceinline__ bool below_tau(i128 gain, i128 base, int64_t tau_inv) {
-  const i128 y = base < 0 ? -base : base;
-  return gain <= y / (i128)tau_inv;
-}
-
-__device__ __forceinline__ i128 ld128(const int64_t* lo) {
-  return (i128)(((unsigned __int128)(unsigned long long)lo[1] << 64) | (unsigned long long)lo[0]);
-}
-__device__ __forceinline__ void st128(int64_t* lo, i128 x) {
-  lo[0] = (int64_t)(unsigned long long)x;
-  lo[1] = (int64_t)(unsigned long long)((unsigned __int128)x >> 64);
 }
 
 // Per-pass accumulators back to zero (one thread per graph).
@@ -1295,10 +1274,10 @@ __global__ void __launch_bounds__(kEmitThreads) emit_dense(int64_t n, int64_t m,
                                                            const int32_t* __restrict__ col,
                                                            const W* __restrict__ w,
                                                            const int32_t* __restrict__ ccid, uint32_t nc,
+                                                           const uint32_t* __restrict__ rowbase, uint32_t cells,
                                                            int64_t per_warp, VT* __restrict__ dense) {
   extern __shared__ __align__(16) unsigned char smem[];
   VT* local = reinterpret_cast<VT*>(smem);
-  const uint32_t cells = nc * nc;
   if (SMEM) {
     for (uint32_t x = threadIdx.x; x < cells; x += blockDim.x) local[x] = 0;
     __syncthreads();
@@ -1316,7 +1295,8 @@ __global__ void __launch_bounds__(kEmitThreads) emit_dense(int64_t n, int64_t m,
       uint32_t key = 0xffffffffu;
       W wt = W(0);
       if (valid) {
-        key = (uint32_t)ccid[row] * nc + (uint32_t)ccid[col[e]];
+        const uint32_t cr = (uint32_t)ccid[row];
+        key = (rowbase ? rowbase[cr] : cr * nc) + (uint32_t)ccid[col[e]];
         wt = w[e];
       }
       const unsigned peers = __match_any_sync(0xffffffffu, key);
@@ -2387,62 +2367,198 @@ int n1_keep(dcd_ctx* c, int64_t n, const int32_t* fin, int64_t nk) {
   return c->n1.h0_wide ? n1_keep_t<unsigned long long>(c, n, fin, nk) : n1_keep_t<unsigned>(c, n, fin, nk);
 }
 
-// Dense coarsening (nc <= kDenseNc): matrix, emit, count, scan, write.
+// Block layout of the level-0 coarse graphs of several graphs: the matrix of
+// graph g starts at cell co[g], has nz_g rows and columns, and its communities
+// are ids cb[g] .. cb[g + 1] - 1; cell (a, b) is rowbase[a] + b (modulo 2^32,
+// as all cell arithmetic here).
+struct DenseBlocks {
+  int64_t cells = 0;
+  std::vector<int64_t> co, cb;
+  Buf<uint32_t> rowbase;
+};
+
+__global__ void fill_rowbase(const int64_t* __restrict__ co, const int64_t* __restrict__ cb, int G,
+                             uint32_t* __restrict__ rowbase) {
+  for (int g = blockIdx.x; g < G; g += gridDim.x) {
+    const int64_t b = cb[g], nz = cb[g + 1] - b;
+    for (int64_t r = threadIdx.x; r < nz; r += blockDim.x) rowbase[b + r] = (uint32_t)(co[g] + r * nz - b);
+  }
+}
+
+// The dense coarse matrix (cells in all; blocks NULL: one nc x nc matrix) of the
+// sums of every entry, or of level 0 by the delta rule.  The level-0 matrix of
+// one graph is kept for the next update's delta rule.
 template <typename W, typename VT>
-int coarsen_dense(dcd_ctx* c, const Csr<W>& g, const int32_t* ccid, int64_t nc, CoarseGraph* out, bool level0,
-                  const int32_t* L, const int32_t* cid) {
+int dense_matrix(dcd_ctx* c, const Csr<W>& g, const int32_t* ccid, int64_t nc, const DenseBlocks* blocks, bool level0,
+                 const int32_t* L, const int32_t* cid, Buf<VT>& dense_local, Buf<unsigned long long>& ent,
+                 VT** dense_out, bool* delta_out) {
   cudaStream_t s = c->stream;
-  const int T = 256;
-  const int64_t m0 = g.nnz;
-  Buf<VT> dense_local;
-  Buf<int64_t> stmp;
-  Buf<unsigned long long> ent;
+  const int64_t m0 = g.nnz, cells = blocks ? blocks->cells : nc * nc;
   VT* dense = nullptr;
-  // level 0 keeps its matrix for the next update's delta coarsening
   const bool keep = level0 && c->n1.track;
   if (keep) {
-    DCD_TRY(c->h0.ensure(&c->mem, (size_t)nc * nc * sizeof(VT) + 16));
+    DCD_TRY(c->h0.ensure(&c->mem, (size_t)cells * sizeof(VT) + 16));
     dense = reinterpret_cast<VT*>(c->h0.get());
     c->n1.h0_nc = nc;
     c->n1.h0_wide = sizeof(VT) == 8;
   } else {
-    DCD_TRY(dense_local.alloc(&c->mem, nc * nc));
+    DCD_TRY(dense_local.alloc(&c->mem, cells));
     dense = dense_local.get();
   }
-  DCD_TRY(stmp.alloc(&c->mem, scan_tmp_count(nc + 1) + 1));
   DCD_TRY(ent.alloc(&c->mem, 1));
-  DCD_TRY_CUDA(cudaMemsetAsync(dense, 0, nc * nc * sizeof(VT), s));
+  DCD_TRY_CUDA(cudaMemsetAsync(dense, 0, cells * sizeof(VT), s));
   DCD_TRY_CUDA(cudaMemsetAsync(ent.get(), 0, sizeof(unsigned long long), s));
   bool delta = false;
   if constexpr (std::is_same<W, int32_t>::value) {
-    if (level0 && c->n1.usable && c->kc_valid && c->kc_n + c->n1.fresh <= kDenseNc) {
+    if (level0 && !blocks && c->n1.usable && c->kc_valid && c->kc_n + c->n1.fresh <= kDenseNc) {
       bool ok = false;
       DCD_TRY(n1_build<VT>(c, g, L, cid, nc, dense, ent.get(), &ok));
       delta = ok;
       if (!ok) {  // rebuild from every entry
-        DCD_TRY_CUDA(cudaMemsetAsync(dense, 0, nc * nc * sizeof(VT), s));
+        DCD_TRY_CUDA(cudaMemsetAsync(dense, 0, cells * sizeof(VT), s));
         DCD_TRY_CUDA(cudaMemsetAsync(ent.get(), 0, sizeof(unsigned long long), s));
       }
     }
   }
   if (!delta && m0 > 0) {
+    const uint32_t* rb = blocks ? blocks->rowbase.get() : nullptr;
     // a CTA copy of the matrix when it fits in shared memory (two CTAs an SM)
-    const size_t msm = (size_t)nc * nc * sizeof(VT);
+    const size_t msm = (size_t)cells * sizeof(VT);
     if (msm <= kDenseSmem) {
       DCD_TRY_CUDA(cudaFuncSetAttribute(emit_dense<W, VT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)kDenseSmem));
       const int grid = wave_grid(emit_dense<W, VT, true>, cdiv(m0, 32) * 32, kEmitThreads, msm);
       const int64_t per_warp = cdiv(cdiv(m0, (int64_t)grid * (kEmitThreads / 32)), 32) * 32;
       ::dcd::count_launch(), emit_dense<W, VT, true><<<grid, kEmitThreads, msm, s>>>(
-          g.n, m0, g.rp, g.col, g.w, ccid, (uint32_t)nc, per_warp, dense);
+          g.n, m0, g.rp, g.col, g.w, ccid, (uint32_t)nc, rb, (uint32_t)cells, per_warp, dense);
     } else {
       const int grid = wave_grid(emit_dense<W, VT, false>, cdiv(m0, 32) * 32, kEmitThreads);
       const int64_t per_warp = cdiv(cdiv(m0, (int64_t)grid * (kEmitThreads / 32)), 32) * 32;
       ::dcd::count_launch(), emit_dense<W, VT, false><<<grid, kEmitThreads, 0, s>>>(
-          g.n, m0, g.rp, g.col, g.w, ccid, (uint32_t)nc, per_warp, dense);
+          g.n, m0, g.rp, g.col, g.w, ccid, (uint32_t)nc, rb, (uint32_t)cells, per_warp, dense);
     }
     DCD_LAUNCH_CHECK();
   }
+  *dense_out = dense;
+  *delta_out = delta;
+  return DCD_OK;
+}
+
+// What level 0's coarsening read (ent: the delta rule's row entries).
+void note_level0(dcd_ctx* c, bool delta, int64_t ent, int64_t m0, int64_t nc) {
+  c->n1.used = delta;
+  c->n1.entries = delta ? c->n1.distinct + ent : m0;
+  c->n1.h0_ready = c->n1.track;
+  tracef("level-0 coarse graph: %s, %lld entries read, %lld communities", delta ? "delta rule" : "every entry",
+         (long long)c->n1.entries, (long long)nc);
+}
+
+// The next level's vertex of every vertex (level 0 of a tracked graph: kept
+// for the next update).
+int coarse_ids(dcd_ctx* c, int64_t n, const int32_t* L, const int32_t* cid, bool level0, Buf<int32_t>& local,
+               int32_t** out) {
+  if (level0 && c->n1.track) {
+    DCD_TRY(c->h0_ccid.ensure(&c->mem, n > 0 ? n : 1));
+    *out = c->h0_ccid.get();
+  } else {
+    DCD_TRY(local.alloc(&c->mem, n > 0 ? n : 1));
+    *out = local.get();
+  }
+  if (n > 0) {
+    ::dcd::count_launch(), coarse_of<<<grid_for(n, 256), 256, 0, c->stream>>>(n, L, cid, *out);
+    DCD_LAUNCH_CHECK();
+  }
+  return DCD_OK;
+}
+
+// Sums of weights need 64 bits (2m of the largest graph bounds them).
+bool wide_sums(const dcd_ctx* c) {
+  int64_t m2max = 0;
+  for (int x = 0; x < c->G; x++) m2max = c->hgs[x].m2 > m2max ? c->hgs[x].m2 : m2max;
+  return m2max >= ((int64_t)1 << 31);
+}
+
+// Dense matrices for the coarse levels in one launch (levels.cu).
+struct DenseLevels {
+  DenseBlocks blocks;
+  Buf<int64_t> co, cb;
+  Buf<unsigned> h32;
+  Buf<unsigned long long> h64, ent;
+  Buf<int32_t> ccid;
+  LevelsIn in;
+  LevelsBufs bufs;
+  bool delta = false;
+};
+
+// Whether the levels after this one run in one launch: the communities with
+// entries (nz of each graph) fit dense matrices of at most kLevelNc rows.
+bool levels_fit(const dcd_ctx* c, const std::vector<int64_t>& nz, DenseLevels* d) {
+  if (c->cfg.pass_loop != 0) return false;  // the host enqueues every pass
+  int64_t mx = 0, cells = 0;
+  d->blocks.co.assign(c->G + 1, 0);
+  d->blocks.cb.assign(c->G + 1, 0);
+  for (int x = 0; x < c->G; x++) {
+    mx = nz[x] > mx ? nz[x] : mx;
+    if (mx > kLevelNc) return false;
+    cells += nz[x] * nz[x];
+    d->blocks.co[x + 1] = cells;
+    d->blocks.cb[x + 1] = d->blocks.cb[x] + nz[x];
+  }
+  d->blocks.cells = cells;
+  d->in.max_nz = mx;
+  d->in.cells = cells;
+  d->in.nz = d->blocks.cb[c->G];
+  return mx > 0 && cells <= kLevelCells;
+}
+
+template <typename W>
+int dense_levels_matrix(dcd_ctx* c, const Csr<W>& g, const int32_t* L, const int32_t* cid, bool level0,
+                        DenseLevels* d) {
+  cudaStream_t s = c->stream;
+  int32_t* ccid = nullptr;
+  DCD_TRY(coarse_ids(c, g.n, L, cid, level0, d->ccid, &ccid));
+  const DenseBlocks* blocks = nullptr;
+  if (c->G > 1) {
+    const int G = c->G;
+    DCD_TRY(d->co.alloc(&c->mem, G + 1));
+    DCD_TRY(d->cb.alloc(&c->mem, G + 1));
+    DCD_TRY(d->blocks.rowbase.alloc(&c->mem, d->in.nz));
+    DCD_TRY_CUDA(cudaMemcpyAsync(d->co.get(), d->blocks.co.data(), (G + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+    DCD_TRY_CUDA(cudaMemcpyAsync(d->cb.get(), d->blocks.cb.data(), (G + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+    ::dcd::count_launch(), fill_rowbase<<<G < 4096 ? G : 4096, 128, 0, s>>>(d->co.get(), d->cb.get(), G,
+                                                                            d->blocks.rowbase.get());
+    DCD_LAUNCH_CHECK();
+    d->in.co = d->co.get();
+    d->in.cb = d->cb.get();
+    blocks = &d->blocks;
+  }
+  d->in.wide = wide_sums(c);
+  if (d->in.wide) {
+    unsigned long long* H = nullptr;
+    DCD_TRY((dense_matrix<W, unsigned long long>(c, g, ccid, d->in.nz, blocks, level0, L, cid, d->h64, d->ent, &H,
+                                                 &d->delta)));
+    d->in.H = H;
+  } else {
+    unsigned* H = nullptr;
+    DCD_TRY((dense_matrix<W, unsigned>(c, g, ccid, d->in.nz, blocks, level0, L, cid, d->h32, d->ent, &H, &d->delta)));
+    d->in.H = H;
+  }
+  return DCD_OK;
+}
+
+// Dense coarsening (nc <= kDenseNc) to a CSR: matrix, count, scan, write.
+template <typename W, typename VT>
+int coarsen_dense(dcd_ctx* c, const Csr<W>& g, const int32_t* ccid, int64_t nc, CoarseGraph* out, bool level0,
+                  const int32_t* L, const int32_t* cid) {
+  cudaStream_t s = c->stream;
+  const int T = 256;
+  Buf<VT> dense_local;
+  Buf<int64_t> stmp;
+  Buf<unsigned long long> ent;
+  VT* dense = nullptr;
+  bool delta = false;
+  DCD_TRY((dense_matrix<W, VT>(c, g, ccid, nc, nullptr, level0, L, cid, dense_local, ent, &dense, &delta)));
+  DCD_TRY(stmp.alloc(&c->mem, scan_tmp_count(nc + 1) + 1));
   DCD_TRY(out->rp.alloc(&c->mem, nc + 1));
   DCD_TRY_CUDA(cudaMemsetAsync(out->rp.get(), 0, (nc + 1) * sizeof(int64_t), s));
   ::dcd::count_launch(), dense_count<VT><<<grid_for(nc * 32, T), T, 0, s>>>(dense, nc, out->rp.get());
@@ -2452,13 +2568,7 @@ int coarsen_dense(dcd_ctx* c, const Csr<W>& g, const int32_t* ccid, int64_t nc, 
   DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 1, ent.get(), sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   DCD_TRY_CUDA(cudaStreamSynchronize(s));
   const int64_t U = c->hscratch[0];
-  if (level0) {
-    c->n1.used = delta;
-    c->n1.entries = delta ? c->n1.distinct + c->hscratch[1] : m0;
-    c->n1.h0_ready = keep;
-    tracef("level-0 coarse graph: %s, %lld entries read, %lld communities", delta ? "delta rule" : "every entry",
-           (long long)c->n1.entries, (long long)nc);
-  }
+  if (level0) note_level0(c, delta, c->hscratch[1], g.nnz, nc);
   DCD_TRY(out->col.alloc(&c->mem, U));
   DCD_TRY(out->w.alloc(&c->mem, U));
   ::dcd::count_launch(), dense_write<VT><<<grid_for(nc * 32, T), T, 0, s>>>(dense, nc, out->rp.get(),
@@ -2480,20 +2590,8 @@ int coarsen(dcd_ctx* c, const Csr<W>& g, const int32_t* L, const int32_t* cid, i
   if (nc <= kDenseNc) {
     Buf<int32_t> ccid_local;
     int32_t* ccid = nullptr;
-    if (level0 && c->n1.track) {
-      DCD_TRY(c->h0_ccid.ensure(&c->mem, g.n > 0 ? g.n : 1));
-      ccid = c->h0_ccid.get();
-    } else {
-      DCD_TRY(ccid_local.alloc(&c->mem, g.n > 0 ? g.n : 1));
-      ccid = ccid_local.get();
-    }
-    if (g.n > 0) {
-      ::dcd::count_launch(), coarse_of<<<grid_for(g.n, T), T, 0, s>>>(g.n, L, cid, ccid);
-      DCD_LAUNCH_CHECK();
-    }
-    int64_t m2max = 0;
-    for (int x = 0; x < c->G; x++) m2max = c->hgs[x].m2 > m2max ? c->hgs[x].m2 : m2max;
-    if (m2max < ((int64_t)1 << 31)) return coarsen_dense<W, unsigned>(c, g, ccid, nc, out, level0, L, cid);
+    DCD_TRY(coarse_ids(c, g.n, L, cid, level0, ccid_local, &ccid));
+    if (!wide_sums(c)) return coarsen_dense<W, unsigned>(c, g, ccid, nc, out, level0, L, cid);
     return coarsen_dense<W, unsigned long long>(c, g, ccid, nc, out, level0, L, cid);
   }
   Buf<uint64_t> k0, k1, v0, v1;
@@ -2837,6 +2935,8 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
   const int32_t* gid = gid0;
   int64_t nvu = n0;  // vertices of the union at this level
   Buf<int32_t> n1_kidx, n1_klab;  // level-0 delta coarsening: K's index, extended
+  DenseLevels dl;
+  bool ran_dense = false, dense_first = false;
   int64_t iso = 0;   // communities without entries at the end of level 0
 
   for (;;) {
@@ -2915,6 +3015,29 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
       break;
     }
     DCD_TRY_CUDA(cudaMemcpyAsync(gs, c->hgs, G * sizeof(GraphState), cudaMemcpyHostToDevice, s));
+    // ---- few communities: every further level in one launch ----
+    std::vector<int64_t> nzg(G);
+    for (int x = 0; x < G; x++) nzg[x] = level == 1 ? c->hgs[x].nc - c->hgs[x].iso : c->hgs[x].nc;
+    if (levels_fit(c, nzg, &dl)) {
+      if (level == 1) DCD_TRY(dense_levels_matrix<int32_t>(c, *g_l0, L, cid.get(), G == 1, &dl));
+      else DCD_TRY(dense_levels_matrix<int64_t>(c, *g_lc, L, cid.get(), false, &dl));
+      DCD_TRY(kc[nx].alloc(&c->mem, nc));
+      DCD_TRY(Lc[nx].alloc(&c->mem, nc));
+      ::dcd::count_launch(), compose_ids<<<grid_for(n0, T), T, 0, s>>>(n0, nvu, nc, comp.get(), L, cid.get());
+      ::dcd::count_launch(), level_start<<<grid_for(nvu, T), T, 0, s>>>(nvu, nc, cid.get(), a.get(), kc[nx].get(),
+                                                                        Lc[nx].get());
+      DCD_LAUNCH_CHECK();
+      DCD_TRY_CUDA(cudaEventRecord(c->ev[6], s));
+      dl.in.kc = kc[nx].get();
+      dl.in.label = Lc[nx].get();
+      dl.in.level = (int32_t)level;
+      DCD_TRY(coarse_levels(c, dl.in, &dl.bufs));
+      ran_dense = true;
+      dense_first = level == 1;
+      L = Lc[nx].get();
+      nvu = nc;
+      break;
+    }
     // ---- compact: next level (all graphs together; finished graphs only
     // carry their labels along) ----
     if (level == 1) DCD_TRY(coarsen<int32_t>(c, *g_l0, L, cid.get(), nc, &cg[nx], G == 1));
@@ -2961,8 +3084,40 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
                                                                        out_labels, gid0, gs);
     DCD_LAUNCH_CHECK();
     DCD_TRY_CUDA(cudaEventRecord(c->ev[8], s));
+    std::vector<uint8_t> ran(G, 0);  // graphs whose levels the one launch finished
+    if (ran_dense) {
+      for (int x = 0; x < G; x++) ran[x] = !c->hgs[x].done;
+      static_assert(sizeof(LevelTotals) <= 32 * sizeof(int64_t), "pinned words 32 on");
+      DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 32, dl.bufs.tot, sizeof(LevelTotals), cudaMemcpyDeviceToHost, s));
+      DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 1, dl.ent.get(), sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    }
     DCD_TRY_CUDA(cudaMemcpyAsync(c->hgs, gs, G * sizeof(GraphState), cudaMemcpyDeviceToHost, s));
     DCD_TRY_CUDA(cudaStreamSynchronize(s));
+    if (ran_dense) {
+      const LevelTotals& t = *reinterpret_cast<const LevelTotals*>(c->hscratch + 32);
+      if (dense_first && G == 1) note_level0(c, dl.delta, c->hscratch[1], g0.nnz, dl.in.nz);
+      float tc = 0.f;
+      cudaEventElapsedTime(&tc, c->ev[5], c->ev[6]);
+      ms_coarsen += tc + (float)(t.t_compact_ns * 1e-6);
+      ms_lm += (float)(t.t_eval_ns * 1e-6);
+      ms_apply += (float)(t.t_apply_ns * 1e-6);
+      level += t.levels;
+      passes_total += t.passes;
+      verts_total += t.verts;
+      edges_total += t.edges;
+      for (int x = 0; x < 4; x++) {
+        verts_bin[x] += t.verts_bin[x];
+        edges_bin[x] += t.edges_bin[x];
+      }
+      for (int x = 0; x < G; x++) {
+        if (!ran[x]) continue;
+        tally.passes[x] += c->hgs[x].lv_passes;
+        tally.moves[x] += c->hgs[x].lv_moves;
+        tally.levels[x] = c->hgs[x].lv_levels;
+      }
+      tracef("coarse levels: %lld levels, %lld passes, evaluation %.3f ms, apply %.3f ms, compaction %.3f ms",
+             (long long)t.levels, (long long)t.passes, t.t_eval_ns * 1e-6, t.t_apply_ns * 1e-6, t.t_compact_ns * 1e-6);
+    }
   }
   if (G == 1) DCD_TRY(n1_keep(c, n0, out_labels, c->hgs[0].ncomm - iso));
   float tf = 0.f;

@@ -72,6 +72,9 @@ struct GraphState {
   int32_t passes;      // passes at this level
   int32_t done;        // the graph's levels are over
   int64_t iso;         // labels in use at the end of level 0 whose community has no entries (a_C = 0)
+  // the coarse levels that ran in one launch: passes, movers, levels done by their end
+  int64_t lv_moves;
+  int32_t lv_passes, lv_levels;
 };
 
 __device__ __forceinline__ int graph_of(const int32_t* gid, int64_t v) { return gid ? gid[v] : 0; }
@@ -385,6 +388,37 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g, int32_t* labels0, const uint8
                 Buf<int64_t>& k, int32_t* out_labels, dcd_step_stats* st, EntryLabels* nlab,
                 int32_t* level0_out = nullptr, dcd_step_stats* per_graph = nullptr, const int64_t* a0 = nullptr, const int32_t* size0 = nullptr,
                 const int32_t* pre0 = nullptr);
+
+// levels.cu: every level from `level` (>= 1) on in one launch, from dense
+// coarse matrices.  Writes the labels of the level's vertices and each graph's
+// GraphState (n_cur, in_cur, lv_*); no synchronisation.
+// A graph's levels stay in one launch up to kLevelNc communities: an update
+// whose levels start with 500, 1000, 1500, 2000, 3000 communities (sparse, 4-6
+// levels) takes 0.69, 1.02, 1.62, 2.38, 5.0 ms so and 1.78, 2.18, 2.25, 2.26,
+// 2.18 ms with a graph launch a level; the walk over D grows with the square.
+constexpr int64_t kLevelNc = 1536;
+constexpr int64_t kLevelCells = (int64_t)1 << 24;  // cells of all matrices, at most
+constexpr size_t kLevelSmem = 225 * 1024;
+struct LevelTotals {  // over the levels, as the step statistics count them
+  int64_t levels, passes, verts, edges, verts_bin[4], edges_bin[4];
+  unsigned long long t_eval_ns, t_apply_ns, t_compact_ns;
+};
+struct LevelsIn {
+  const int64_t *co = nullptr, *cb = nullptr;  // several graphs: first cells, first communities (G + 1)
+  int64_t nz = 0, max_nz = 0, cells = 0;       // communities of all, of the largest graph; cells of all
+  const void* H = nullptr;                     // matrices, 32-bit cells or wide
+  bool wide = false;
+  const int64_t* kc = nullptr;                 // weighted degrees of the communities
+  int32_t* label = nullptr;
+  int32_t level = 1;
+};
+struct LevelsBufs {  // lives until the launch has run
+  Buf<unsigned char> scratch;
+  Buf<unsigned> w32, e32;
+  Buf<unsigned long long> w64, e64;
+  LevelTotals* tot = nullptr;
+};
+int coarse_levels(dcd_ctx* c, const LevelsIn& in, LevelsBufs* b);
 
 // louvain.cu: multi-level smart local moving (dSLM) from level-0 labels and
 // level-0 active flags (NULL = all), k and 2m of G_t (one graph a context).
