@@ -36,15 +36,19 @@ __global__ void to_local(int64_t n, const int32_t* __restrict__ lab, const int32
     out[v] = lab[v] - (int32_t)off[gid[v]];
 }
 
+// One byte a vertex; a graph's vertices are split over gridDim.y CTAs (one CTA
+// a graph: 319 us at 64 graphs, the largest of 200 K vertices, a byte a thread
+// in flight).
 __global__ void per_graph_counts(int G, const int64_t* __restrict__ off, const int64_t* __restrict__ rp,
                                  const uint8_t* __restrict__ r, long long* __restrict__ nnz,
                                  unsigned long long* __restrict__ rsz) {
+  const int64_t st = (int64_t)gridDim.y * blockDim.x;
   for (int g = blockIdx.x; g < G; g += gridDim.x) {
     unsigned long long c = 0;
-    for (int64_t v = off[g] + threadIdx.x; v < off[g + 1]; v += blockDim.x) c += r[v] != 0;
+    for (int64_t v = off[g] + (int64_t)blockIdx.y * blockDim.x + threadIdx.x; v < off[g + 1]; v += st) c += r[v] != 0;
     c = warp_sum(c);
     if (lane_id() == 0 && c) atomicAdd(&rsz[g], c);
-    if (threadIdx.x == 0) nnz[g] = rp[off[g + 1]] - rp[off[g]];
+    if (blockIdx.y == 0 && threadIdx.x == 0) nnz[g] = rp[off[g + 1]] - rp[off[g]];
   }
 }
 
@@ -66,8 +70,9 @@ int group_finish(dcd_ctx* c, void* user) {
   DCD_TRY(nnz.alloc(&c->mem, G));
   DCD_TRY(rsz.alloc(&c->mem, G));
   DCD_TRY_CUDA(cudaMemsetAsync(rsz.get(), 0, G * sizeof(unsigned long long), s));
-  count_launch(), per_graph_counts<<<G < 4096 ? G : 4096, 256, 0, s>>>(G, c->goff_d.get(), c->rp[1 - c->cur].get(),
-                                                                      c->rset_nx.get(), nnz.get(), rsz.get());
+  const dim3 pg(G < 4096 ? G : 4096, G < 152 ? 32 : G < 2048 ? 4 : 1);
+  count_launch(), per_graph_counts<<<pg, 256, 0, s>>>(G, c->goff_d.get(), c->rp[1 - c->cur].get(), c->rset_nx.get(),
+                                                      nnz.get(), rsz.get());
   DCD_LAUNCH_CHECK();
   DCD_TRY_CUDA(cudaMemcpyAsync(o->hn, nnz.get(), G * sizeof(long long), cudaMemcpyDeviceToHost, s));
   DCD_TRY_CUDA(cudaMemcpyAsync(o->hr, rsz.get(), G * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));

@@ -6,10 +6,11 @@
 // compaction and five host round trips, about 0.2 ms a level whatever its size
 // (47 communities: 0.22 ms, of which 0.02 are evaluation and apply).  Here all
 // of them run in one launch, 10 us at that size: passes, stop rules, compaction
-// to the next matrix, level stop rule.  Updates of 2 K vertices went from 0.86 to
-// 0.64 ms, of 64 graphs (500 to 200 K vertices, 39 M entries in all) from 8.7 to 7.2.  A graph of the context gets a cluster of 1 to
-// 8 CTAs, which meet at the cluster barrier (a hardware barrier of CTAs that
-// are resident together), twice a pass.
+// to the next matrix, level stop rule.  Updates of 2 K vertices went from 0.86
+// to 0.64 ms, of 64 graphs (500 to 200 K vertices, 39 M entries in all) from 8.7
+// to 7.2.  A graph of the context gets a cluster of 1 to 8 CTAs, which meet at
+// the cluster barrier (a hardware barrier of CTAs that are resident together),
+// twice a pass.
 //
 // What bounds it is latency, so the work of a pass is laid out without
 // gathers: E(D, i) = the summed weight from vertex i into community D, the
@@ -393,7 +394,7 @@ template <typename VT>
 int launch_levels(dcd_ctx* c, LevelsArgs p, int G, int64_t cells, Buf<VT>& E) {
   using ST = typename std::conditional<sizeof(VT) == 4, long long, i128>::type;
   int CL = 1;
-  while (CL < kLvMaxCluster && CL * kLvColumns < p.cap && 2 * CL * G <= num_sms()) CL *= 2;
+  while (CL < kLvMaxCluster && CL * kLvColumns < p.cap) CL *= 2;
   const int slice = (p.cap + CL - 1) / CL;
   size_t sm = level_smem(p.cap, slice, sizeof(ST));
   const size_t smE = sm + (size_t)slice * p.cap * sizeof(VT);
