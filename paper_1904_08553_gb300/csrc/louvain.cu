@@ -23,6 +23,7 @@
 // communities, sort-by-key reduction for many; level 0 of an update can be
 // built from the previous update's coarse graph (delta coarsening, below).
 #include <cstdio>
+#include <memory>
 #include <type_traits>
 #include <vector>
 
@@ -650,12 +651,19 @@ __global__ void __launch_bounds__(256) hub_clear(HubTables t) {
 // does not hold one warp for its whole row.
 constexpr int kMoveChunk = 128;
 
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
 __global__ void lm_apply(const int32_t* __restrict__ list, int64_t cnt, const int32_t* __restrict__ prop,
                          int32_t* __restrict__ L, int2* __restrict__ LL, const int64_t* __restrict__ k,
                          const int64_t* __restrict__ rp, unsigned long long* __restrict__ a,
                          int32_t* __restrict__ size, int64_t* __restrict__ items, int32_t* __restrict__ item_cnt,
-                         unsigned long long* __restrict__ moved_deg, const int32_t* __restrict__ gid,
+                         DevScalars* __restrict__ d, const int32_t* __restrict__ gid,
                          GraphState* __restrict__ gs) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) d->stamp[1] = global_ns();  // the evaluation is over
   unsigned long long deg = 0;  // degrees of the movers
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int lane = lane_id();
@@ -675,9 +683,9 @@ __global__ void lm_apply(const int32_t* __restrict__ list, int64_t cnt, const in
       if (mv) {
         L[v] = p;
         kv = k[v];
-        const int64_t d = rp[v + 1] - rp[v];
-        deg += (unsigned long long)d;
-        nch = (int)((d + kMoveChunk - 1) / kMoveChunk);
+        const int64_t dv = rp[v + 1] - rp[v];
+        deg += (unsigned long long)dv;
+        nch = (int)((dv + kMoveChunk - 1) / kMoveChunk);
       } else {
         c = p = -1;
       }
@@ -711,7 +719,7 @@ __global__ void lm_apply(const int32_t* __restrict__ list, int64_t cnt, const in
     for (int j = 0; j < nch; j++) items[at + j] = (int64_t)v << 32 | (uint32_t)j;
   }
   deg = warp_sum(deg);
-  if (lane == 0 && deg) atomicAdd(moved_deg, deg);
+  if (lane == 0 && deg) atomicAdd((unsigned long long*)&d->moved_deg, deg);
 }
 
 // Entry labels (nlab_gather below) are kept from this many entries on: below,
@@ -787,51 +795,16 @@ __global__ void __launch_bounds__(256) lm_delta(LV<W> g, const int2* __restrict_
   }
 }
 
-// sum over labels of a^2 per graph, unsigned 128-bit: every contribution is
-// added with a carry into the high word, so the total is exact in any order.
-// One graph: a CTA reduction then one addition per CTA; several graphs: one
-// addition per community in use.
-__global__ void __launch_bounds__(256) sumsq_acc(const int64_t* __restrict__ a, int64_t n,
-                                                 const int32_t* __restrict__ gid, GraphState* __restrict__ gs) {
-  if (gid) {
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
-      const unsigned long long x = (unsigned long long)a[c];
-      if (x) {
-        GraphState& G = gs[gid[c]];
-        add128(&G.sq_lo, &G.sq_hi, (unsigned __int128)x * x);
-      }
-    }
-    return;
+// Start of a pass: its accumulators back to zero.
+__global__ void pass_begin(GraphState* __restrict__ gs, int G, DevScalars* __restrict__ d,
+                           int32_t* __restrict__ item_cnt) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    d->pass_id += 1;
+    d->any_running = 0;
+    d->moved_deg = 0;
+    d->stamp[0] = d->stamp[1] = global_ns();
+    if (item_cnt) *item_cnt = 0;
   }
-  __shared__ unsigned long long slo[8], shi[8];
-  unsigned __int128 s = 0;
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long x = (unsigned long long)a[c];
-    s += (unsigned __int128)x * x;
-  }
-  unsigned long long lo = (unsigned long long)s, hi = (unsigned long long)(s >> 64);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    unsigned long long lo2 = __shfl_xor_sync(0xffffffffu, lo, o), hi2 = __shfl_xor_sync(0xffffffffu, hi, o);
-    unsigned long long nlo = lo + lo2;
-    hi = hi + hi2 + (nlo < lo ? 1ull : 0ull);
-    lo = nlo;
-  }
-  if (lane_id() == 0) {
-    slo[threadIdx.x >> 5] = lo;
-    shi[threadIdx.x >> 5] = hi;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned __int128 t = 0;
-    for (int w = 0; w < 8; w++) t += ((unsigned __int128)shi[w] << 64) | slo[w];
-    add128(&gs[0].sq_lo, &gs[0].sq_hi, t);
-  }
-}
-
-// Per-pass accumulators back to zero (one thread per graph).
-__global__ void gs_reset_pass(GraphState* __restrict__ gs, int G, int32_t* __restrict__ pass_id) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) *pass_id += 1;
   for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
     gs[g].in_delta = 0;
     gs[g].sq_lo = gs[g].sq_hi = 0;
@@ -839,70 +812,134 @@ __global__ void gs_reset_pass(GraphState* __restrict__ gs, int G, int32_t* __res
   }
 }
 
-// The pass decision per graph (one thread per graph).  mode 0: level start
-// (N_start = N_cur = m2 in - sq; graphs whose levels are over do not run);
-// mode 1: after a pass.  any_running <- some graph goes on.
-__global__ void lm_decide(GraphState* __restrict__ gs, int G, int mode, int32_t max_iters, int64_t tau_inv,
-                          int32_t* __restrict__ any_running) {
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
-    GraphState& X = gs[g];
-    const unsigned __int128 sq = ((unsigned __int128)X.sq_hi << 64) | X.sq_lo;
-    if (mode == 0) {
-      const i128 N = (i128)X.m2 * (i128)X.in_cur - (i128)sq;
-      st128(&X.n_cur_lo, N);
-      st128(&X.n_start_lo, N);
-      X.running = X.done ? 0 : 1;
-      X.passes = 0;
-      X.moves = 0;
-      X.moves_level = 0;
-      if (X.running) atomicOr(any_running, 1);
-      continue;
+// The pass decision of one graph; true when its pass loop goes on.  start:
+// level start (N_start = N_cur = m2 in - sq; graphs whose levels are over do
+// not run); otherwise after a pass.
+__device__ __forceinline__ bool pass_decision(GraphState& X, bool start, int32_t max_iters, int64_t tau_inv) {
+  const unsigned __int128 sq = ((unsigned __int128)__ldcg(&X.sq_hi) << 64) | __ldcg(&X.sq_lo);
+  if (start) {
+    const i128 N = (i128)X.m2 * (i128)X.in_cur - (i128)sq;
+    st128(&X.n_cur_lo, N);
+    st128(&X.n_start_lo, N);
+    X.running = X.done ? 0 : 1;
+    X.passes = 0;
+    X.moves = 0;
+    X.moves_level = 0;
+    return X.running;
+  }
+  if (!X.running) return false;
+  X.passes++;
+  X.moves_level += X.moves;
+  if (X.moves == 0) {
+    X.running = 0;
+    return false;
+  }
+  const int64_t in_new = X.in_cur + X.in_delta;
+  const i128 N_new = (i128)X.m2 * (i128)in_new - (i128)sq;
+  const i128 N_old = ld128(&X.n_cur_lo);
+  X.in_cur = in_new;
+  st128(&X.n_cur_lo, N_new);
+  if (below_tau(N_new - N_old, N_old, tau_inv) || X.passes >= max_iters) X.running = 0;
+  return X.running;
+}
+
+// End of a pass on the device clock: its evaluation and apply times, the pass
+// count, the loop condition.
+__device__ __forceinline__ void pass_close(DevScalars* d, bool more, cudaGraphConditionalHandle h, int32_t cap,
+                                           int in_graph) {
+  const unsigned long long t = global_ns();
+  d->t_eval_ns += d->stamp[1] - d->stamp[0];
+  d->t_apply_ns += t - d->stamp[1];
+  d->level_passes += 1;
+  const bool capped = more && d->level_passes >= cap;
+  if (capped) d->loop_err = 1;
+  // outside a graph the host reads any_running and loop_err after the pass
+  if (in_graph) cudaGraphSetConditional(h, (more && !capped) ? 1u : 0u);
+}
+
+// What ends a pass (or starts a level): the sum over labels of a^2 per graph,
+// unsigned 128-bit, every contribution added with a carry into the high word,
+// so that the total is exact in any order (one graph: a CTA reduction, then one
+// addition per CTA; several graphs: one addition per community in use); then, in
+// the CTA that finishes last, the decision of every graph (any_running <- some
+// graph goes on) and, with close, the end of the pass.  One launch: as a
+// reset, two stamps, three memsets, a sum, a decision and an end, the fixed
+// part of a pass was nine nodes of the loop, now two (10 K vertices, two
+// passes: 0.105 -> 0.083 ms, and 0.062 -> 0.045 to instantiate the loop).
+enum PassEnd { kLevelStart, kPassOpen, kPassClose };
+__global__ void __launch_bounds__(256) pass_finish(const int64_t* __restrict__ a, int64_t n,
+                                                   const int32_t* __restrict__ gid, GraphState* __restrict__ gs, int G,
+                                                   int end, int32_t max_iters, int64_t tau_inv, DevScalars* d,
+                                                   cudaGraphConditionalHandle h, int32_t cap, int in_graph) {
+  __shared__ unsigned long long slo[8], shi[8];
+  __shared__ int last;
+  if (gid) {
+    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
+      const unsigned long long x = (unsigned long long)a[c];
+      if (x) {
+        GraphState& G1 = gs[gid[c]];
+        add128(&G1.sq_lo, &G1.sq_hi, (unsigned __int128)x * x);
+      }
     }
-    if (!X.running) continue;
-    X.passes++;
-    X.moves_level += X.moves;
-    if (X.moves == 0) {
-      X.running = 0;
-      continue;
+  } else if (n > 0) {
+    unsigned __int128 s = 0;
+    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
+      const unsigned long long x = (unsigned long long)a[c];
+      s += (unsigned __int128)x * x;
     }
-    const int64_t in_new = X.in_cur + X.in_delta;
-    const i128 N_new = (i128)X.m2 * (i128)in_new - (i128)sq;
-    const i128 N_old = ld128(&X.n_cur_lo);
-    X.in_cur = in_new;
-    st128(&X.n_cur_lo, N_new);
-    if (below_tau(N_new - N_old, N_old, tau_inv) || X.passes >= max_iters) X.running = 0;
-    if (X.running) atomicOr(any_running, 1);
+    unsigned long long lo = (unsigned long long)s, hi = (unsigned long long)(s >> 64);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      unsigned long long lo2 = __shfl_xor_sync(0xffffffffu, lo, o), hi2 = __shfl_xor_sync(0xffffffffu, hi, o);
+      unsigned long long nlo = lo + lo2;
+      hi = hi + hi2 + (nlo < lo ? 1ull : 0ull);
+      lo = nlo;
+    }
+    if (lane_id() == 0) {
+      slo[threadIdx.x >> 5] = lo;
+      shi[threadIdx.x >> 5] = hi;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      unsigned __int128 t = 0;
+      for (int w = 0; w < 8; w++) t += ((unsigned __int128)shi[w] << 64) | slo[w];
+      add128(&gs[0].sq_lo, &gs[0].sq_hi, t);
+    }
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&d->ticket, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  bool any = false;
+  for (int g = threadIdx.x; g < G; g += blockDim.x) any |= pass_decision(gs[g], end == kLevelStart, max_iters, tau_inv);
+  any = __syncthreads_or(any);
+  if (threadIdx.x == 0) {
+    d->ticket = 0;
+    d->any_running = any;
+    if (end == kPassClose) pass_close(d, any, h, cap, in_graph);
   }
 }
 
 // ---------------------------------------------------------------- device pass loop
 //
-// A level's passes run inside one CUDA graph: a 'while' conditional node
-// around the pass body.  The body's first and middle kernels stamp the
+// A level's passes after the first run inside one CUDA graph: a 'while'
+// conditional node around the pass body.  The body's first and middle kernels stamp the
 // global timer; its last kernel adds the pass's evaluation and apply times,
 // counts the pass, and keeps the loop going while some graph's pass loop goes
-// on (the stop rule of lm_decide).  The stop rule ends every level within
+// on (pass_decision).  The stop rule ends every level within
 // max_iters passes; the cap here is a second bound that can only be reached
 // if that rule were broken, and it is reported.
 
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
+// The loop of the passes after the first runs when that left one to run.
+__global__ void loop_enter(const DevScalars* d, cudaGraphConditionalHandle h) {
+  cudaGraphSetConditional(h, d->any_running != 0 && !d->loop_err ? 1u : 0u);
 }
 
-__global__ void pass_stamp(DevScalars* d, int k) { d->stamp[k] = global_ns(); }
-
+// Closes a pass after the entry labels were brought up to date.
 __global__ void pass_end(DevScalars* d, cudaGraphConditionalHandle h, int32_t cap, int in_graph) {
-  const unsigned long long t = global_ns();
-  d->t_eval_ns += d->stamp[1] - d->stamp[0];
-  d->t_apply_ns += t - d->stamp[1];
-  d->level_passes += 1;
-  const bool more = d->any_running != 0;
-  const bool capped = more && d->level_passes >= cap;
-  if (capped) d->loop_err = 1;
-  // outside a graph the host reads any_running and loop_err after the pass
-  if (in_graph) cudaGraphSetConditional(h, (more && !capped) ? 1u : 0u);
+  pass_close(d, d->any_running != 0, h, cap, in_graph);
 }
 
 // ---------------------------------------------------------------- entry labels
@@ -1035,7 +1072,9 @@ __global__ void mark_used(int64_t n, const int32_t* __restrict__ L, int32_t* __r
 // and follows the delta rule (0.5-0.9 ms), where the sort of every entry's key
 // took 4.8.  Packed for one scan: low word the former, high word the latter.
 __global__ void label_flags(int64_t n, const int32_t* __restrict__ size, const int64_t* __restrict__ a,
-                            int64_t* __restrict__ f) {
+                            int64_t* __restrict__ f, GraphState* __restrict__ gs, int G) {
+  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < G; g += (int64_t)gridDim.x * blockDim.x)
+    gs[g].nc = 0;  // counted by label_ids
   for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x <= n; x += (int64_t)gridDim.x * blockDim.x)
     f[x] = (x < n && size[x] > 0) ? (a[x] != 0 ? 1 : (int64_t)1 << 32) : 0;
 }
@@ -1275,7 +1314,9 @@ __global__ void __launch_bounds__(kEmitThreads) emit_dense(int64_t n, int64_t m,
                                                            const W* __restrict__ w,
                                                            const int32_t* __restrict__ ccid, uint32_t nc,
                                                            const uint32_t* __restrict__ rowbase, uint32_t cells,
-                                                           int64_t per_warp, VT* __restrict__ dense) {
+                                                           int64_t per_warp, VT* __restrict__ dense,
+                                                           const uint32_t* __restrict__ when) {
+  if (when && !*when) return;
   extern __shared__ __align__(16) unsigned char smem[];
   VT* local = reinterpret_cast<VT*>(smem);
   if (SMEM) {
@@ -1441,11 +1482,11 @@ __global__ void level_sums(int64_t nz, const int64_t* __restrict__ kc, int64_t* 
 
 // Vertex of the next level (of nz) of every original vertex; values from nv on
 // name the communities without entries, which stay behind the level's own.
-__global__ void compose_ids(int64_t n0, int64_t nv, int64_t nz, int32_t* __restrict__ comp,
+__global__ void compose_ids(int64_t n0, int64_t nv, int64_t nz, const int32_t* in, int32_t* out,
                             const int32_t* __restrict__ L, const int32_t* __restrict__ cid) {
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n0; v += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t x = comp[v];
-    comp[v] = x < nv ? cid[L[x]] : (int32_t)(x - nv + nz);
+    const int32_t x = in[v];
+    out[v] = x < nv ? cid[L[x]] : (int32_t)(x - nv + nz);
   }
 }
 
@@ -1462,12 +1503,20 @@ __device__ __forceinline__ int32_t level_label(const int32_t* __restrict__ L, in
   return x < nv ? L[x] : x;
 }
 
+__global__ void final_begin(int32_t* __restrict__ minid, int64_t n, GraphState* __restrict__ gs, int G) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n || v < G; v += (int64_t)gridDim.x * blockDim.x) {
+    if (v < n) minid[v] = INT32_MAX;
+    if (v < G) gs[v].ncomm = 0;
+  }
+}
+
+// comp (may be NULL: the level is level 0): the level's vertex of every vertex.
 __global__ void final_min(int64_t n0, int64_t nv, const int32_t* __restrict__ comp, const int32_t* __restrict__ L,
                           int32_t* __restrict__ minid) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t base = (blockIdx.x * (int64_t)blockDim.x) + (threadIdx.x & ~31); base < n0; base += stride) {
     const int64_t v = base + lane_id();
-    const int32_t c = v < n0 ? level_label(L, nv, comp[v]) : -1;
+    const int32_t c = v < n0 ? level_label(L, nv, comp ? comp[v] : (int32_t)v) : -1;
     const unsigned peers = __match_any_sync(0xffffffffu, c);
     const unsigned mn = __reduce_min_sync(peers, v < n0 ? (unsigned)v : 0xffffffffu);
     // labels of large communities repeat across the grid: read first, and
@@ -1488,7 +1537,7 @@ __global__ void final_labels(int64_t n0, int64_t nv, const int32_t* __restrict__
     int g = -1;
     bool head = false;
     if (v < n0) {
-      const int32_t x = minid[level_label(L, nv, comp[v])];
+      const int32_t x = minid[level_label(L, nv, comp ? comp[v] : (int32_t)v)];
       head = x == (int32_t)v;
       g = graph_of(gid, v);
       out[v] = x;
@@ -1764,10 +1813,42 @@ int entry_labels_impl(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L, Entry
   return DCD_OK;
 }
 
+// A level between the launch of its pass loop and the host's next look at the
+// device (the numbering of its labels needs nothing from the host, so both are
+// enqueued before one synchronisation).
+struct PendingLevel {
+  Bins bins;
+  Buf<int32_t> prop, item_cnt;
+  Buf<int2> LL;
+  Buf<int64_t> items;
+  int64_t sweep[kMaxBins] = {};
+  int64_t body_launches = 0;
+  bool pre = false;
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
+  cudaStream_t stream = nullptr;
+  PendingLevel() = default;
+  PendingLevel(const PendingLevel&) = delete;
+  PendingLevel& operator=(const PendingLevel&) = delete;
+  bool idle = false;  // the loop has run
+  void release() {
+    if (exec) {
+      if (!idle) cudaStreamSynchronize(stream);  // an error path may leave a launch of it in flight
+      cudaGraphExecDestroy(exec);
+    }
+    if (graph) cudaGraphDestroy(graph);
+    exec = nullptr;
+    graph = nullptr;
+  }
+  ~PendingLevel() { release(); }
+};
+
+// The level's pass loop, enqueued; the caller reads DevScalars and the graphs'
+// states back, synchronises and calls finish_level.
 template <typename W>
 int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<int64_t>& a, Buf<int32_t>& size,
-              const uint8_t* active, const int32_t* gid, int level, LevelRun* out, GraphTally* tally,
-              const int32_t* pre = nullptr, EntryLabels* nlab = nullptr) {
+              const uint8_t* active, const int32_t* gid, int level, PendingLevel* pl, const int32_t* pre = nullptr,
+              EntryLabels* nlab = nullptr) {
   cudaStream_t s = c->stream;
   DevScalars* d = c->dsc.get();
   GraphState* gs = c->gs.get();
@@ -1775,18 +1856,21 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
   const int64_t nv = g.n;
   const int T = 256;
 
-  // level start: N_start = N_cur per graph, running = not done
-  DCD_TRY_CUDA(cudaMemsetAsync(&d->any_running, 0, sizeof(int32_t), s));
-  ::dcd::count_launch(), lm_decide<<<cdiv(G, 128), 128, 0, s>>>(gs, G, 0, c->cfg.max_iters, c->cfg.tau_inv,
-                                                                 &d->any_running);
+  // level start: N_start = N_cur per graph, running = not done (level 0: with
+  // the sum of a^2; later levels carry it over)
+  ::dcd::count_launch(), pass_finish<<<level == 0 ? grid_for(nv, T, 4) : 1, T, 0, s>>>(
+      a.get(), level == 0 ? nv : 0, level == 0 ? gid : nullptr, gs, G, kLevelStart, c->cfg.max_iters, c->cfg.tau_inv,
+      d, cudaGraphConditionalHandle{}, 0, 0);
   DCD_LAUNCH_CHECK();
-  Bins bins;
+  Bins& bins = pl->bins;
   DCD_TRY(make_bins<W>(c, g, active, &bins, gid, pre));
   trace("level: binned");
   const int64_t total = bins.total;
-  Buf<int32_t> prop, item_cnt;
-  Buf<int2> LL;
-  Buf<int64_t> items;
+  Buf<int32_t>&prop = pl->prop, &item_cnt = pl->item_cnt;
+  Buf<int2>& LL = pl->LL;
+  Buf<int64_t>& items = pl->items;
+  pl->pre = pre != nullptr;
+  pl->stream = s;
   const int64_t item_cap = total + bins.act_deg / kMoveChunk;
   DCD_TRY(prop.alloc(&c->mem, total));
   DCD_TRY(LL.alloc(&c->mem, nv));
@@ -1816,70 +1900,71 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
   lvl.m2 = G == 1 ? lv.m2 : m2max;  // gain width chosen by the largest graph
   const int32_t* lst = bins.list.get();
   bool any = total > 0;
-  int64_t sweep[kMaxBins] = {};
+  int64_t* sweep = pl->sweep;
   // One pass: evaluate, apply, tracked N, stop rule, then the loop condition.
   // Every pass of a level enqueues the same work (the pass number lives on
   // the device), so the body is captured once, into the body of a 'while'
-  // conditional node, and the whole pass loop of the level is one graph
-  // launch.  With dcd_config.pass_loop = 1 the host enqueues the same body
+  // conditional node, and the passes after the first are one graph launch.  With dcd_config.pass_loop = 1 the host enqueues the same body
   // once per pass instead and reads the loop condition back after it.
   auto enqueue_pass = [&](cudaGraphConditionalHandle h, bool in_graph) -> int {
-    ::dcd::count_launch(), gs_reset_pass<<<cdiv(G, 128), 128, 0, s>>>(gs, G, &d->pass_id);
-    DCD_TRY_CUDA(cudaMemsetAsync(item_cnt.get(), 0, sizeof(int32_t), s));
-    DCD_TRY_CUDA(cudaMemsetAsync(&d->any_running, 0, sizeof(int32_t), s));
-    DCD_TRY_CUDA(cudaMemsetAsync(&d->moved_deg, 0, sizeof(int64_t), s));
-    ::dcd::count_launch(), pass_stamp<<<1, 1, 0, s>>>(d, 0);
+    const int32_t cap = c->cfg.max_iters + 2;
+    const int ig = in_graph ? 1 : 0;
+    ::dcd::count_launch(), pass_begin<<<cdiv(G, 256), 256, 0, s>>>(gs, G, d, item_cnt.get());
     if (any) DCD_TRY(launch_lm_nocfg<W>(c, lvl, bins, prop.get(), nullptr, 0, total >= kForkMin, sweep));
-    ::dcd::count_launch(), pass_stamp<<<1, 1, 0, s>>>(d, 1);
     if (total) {
       ::dcd::count_launch(), lm_apply<<<grid_for(total, T), T, 0, s>>>(
           lst, total, prop.get(), L, LL.get(), kbuf.get(), g.rp, (unsigned long long*)a.get(), size.get(), items.get(),
-          item_cnt.get(), (unsigned long long*)&d->moved_deg, gid, gs);
+          item_cnt.get(), d, gid, gs);
       ::dcd::count_launch(), lm_delta<W><<<wave_grid(lm_delta<W>, item_cap * 32, T), T, 0, s>>>(
           lv, LL.get(), g.nnz, items.get(), item_cnt.get(), lv.nlab ? nlab->buf.get() : nullptr, d, gs);
     }
-    ::dcd::count_launch(), sumsq_acc<<<sq_ctas, T, 0, s>>>(a.get(), nv, gid, gs);
-    ::dcd::count_launch(), lm_decide<<<cdiv(G, 128), 128, 0, s>>>(gs, G, 1, c->cfg.max_iters, c->cfg.tau_inv,
-                                                                   &d->any_running);
-    if (lv.nlab)  // returns at once unless the next pass runs and much has moved
+    ::dcd::count_launch(), pass_finish<<<sq_ctas, T, 0, s>>>(a.get(), nv, gid, gs, G, lv.nlab ? kPassOpen : kPassClose,
+                                                             c->cfg.max_iters, c->cfg.tau_inv, d, h, cap, ig);
+    if (lv.nlab) {  // the gather returns at once unless the next pass runs and much has moved
       ::dcd::count_launch(), nlab_gather<<<grid_for(g.nnz, T), T, 0, s>>>(g.col, L, g.nnz, nlab->buf.get(), d);
-    ::dcd::count_launch(), pass_end<<<1, 1, 0, s>>>(d, h, c->cfg.max_iters + 2, in_graph ? 1 : 0);
+      ::dcd::count_launch(), pass_end<<<1, 1, 0, s>>>(d, h, cap, ig);
+    }
     DCD_LAUNCH_CHECK();
     return DCD_OK;
   };
   if (any) DCD_TRY(prepare_lm<W>(lvl));
   resident_blocks(reinterpret_cast<const void*>(lm_delta<W>), T, 0);  // looked up outside the capture
   DCD_TRY(side_streams(c));
-  struct GraphGuard {
-    cudaGraph_t g = nullptr;
-    cudaGraphExec_t x = nullptr;
-    cudaStream_t s = nullptr;
-    ~GraphGuard() {
-      if (x) {
-        cudaStreamSynchronize(s);  // an error path may leave a launch of it in flight
-        cudaGraphExecDestroy(x);
-      }
-      if (g) cudaGraphDestroy(g);
-    }
-  } gg;
-  gg.s = s;
   {
-    int64_t body_launches = 0;
+    int64_t& body_launches = pl->body_launches;
     DCD_TRY_CUDA(cudaMemsetAsync(&d->level_passes, 0, sizeof(int32_t), s));
     DCD_TRY_CUDA(cudaMemsetAsync(&d->t_eval_ns, 0, 2 * sizeof(unsigned long long), s));
     if (c->cfg.pass_loop == 0) {
-      DCD_TRY_CUDA(cudaGraphCreate(&gg.g, 0));
+      // The first pass (a level runs at least one, even with nothing to
+      // evaluate, as the sequential definition does) is enqueued directly: the
+      // device runs it while the loop of the others is instantiated, which takes
+      // 50 to 140 us.  The loop is entered if the first pass says so.
+      {
+        const int64_t l0 = g_launches.load();
+        DCD_TRY(enqueue_pass(cudaGraphConditionalHandle{}, false));
+        g_launches -= g_launches.load() - l0;  // counted below, once per pass that ran
+      }
+      DCD_TRY_CUDA(cudaGraphCreate(&pl->graph, 0));
       cudaGraphConditionalHandle h;
-      // the condition starts at 1 on every launch: a level runs at least one
-      // pass, even with nothing to evaluate, as the sequential definition does
-      DCD_TRY_CUDA(cudaGraphConditionalHandleCreate(&h, gg.g, 1, cudaGraphCondAssignDefault));
+      DCD_TRY_CUDA(cudaGraphConditionalHandleCreate(&h, pl->graph, 0, cudaGraphCondAssignDefault));
+      cudaGraphNode_t enter;
+      {
+        DevScalars* dd = d;
+        void* args[] = {&dd, &h};
+        cudaKernelNodeParams kp{};
+        kp.func = reinterpret_cast<void*>(loop_enter);
+        kp.gridDim = dim3(1);
+        kp.blockDim = dim3(1);
+        kp.kernelParams = args;
+        DCD_TRY_CUDA(cudaGraphAddKernelNode(&enter, pl->graph, nullptr, 0, &kp));
+      }
       cudaGraphNodeParams np{};
       np.type = cudaGraphNodeTypeConditional;
       np.conditional.handle = h;
       np.conditional.type = cudaGraphCondTypeWhile;
       np.conditional.size = 1;
       cudaGraphNode_t node;
-      DCD_TRY_CUDA(cudaGraphAddNode(&node, gg.g, nullptr, nullptr, 0, &np));
+      DCD_TRY_CUDA(cudaGraphAddNode(&node, pl->graph, &enter, nullptr, 1, &np));
       cudaGraph_t body = np.conditional.phGraph_out[0];
       DCD_TRY_CUDA(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
       const int64_t l0 = g_launches.load();
@@ -1890,12 +1975,10 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
       g_launches -= body_launches;  // counted below, once per pass that ran
       if (rc != DCD_OK) return rc;
       DCD_TRY_CUDA(ec);
-      DCD_TRY_CUDA(cudaGraphInstantiate(&gg.x, gg.g, 0));
+      DCD_TRY_CUDA(cudaGraphInstantiate(&pl->exec, pl->graph, 0));
       trace("level: pass loop instantiated");
-      DCD_TRY_CUDA(cudaGraphLaunch(gg.x, s));
-      DCD_TRY_CUDA(cudaMemcpyAsync(c->hsc, d, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
-      DCD_TRY_CUDA(cudaMemcpyAsync(c->hgs, gs, G * sizeof(GraphState), cudaMemcpyDeviceToHost, s));
-      DCD_TRY_CUDA(cudaStreamSynchronize(s));
+      count_launch();  // loop_enter
+      DCD_TRY_CUDA(cudaGraphLaunch(pl->exec, s));
     } else {
       // the same pass, enqueued by the host once per pass; the stop rule is
       // read back after each (pass_end caps the loop as in the graph)
@@ -1905,12 +1988,10 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
         body_launches = g_launches.load() - l0;
         g_launches -= body_launches;
         DCD_TRY_CUDA(cudaMemcpyAsync(c->hsc, d, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
-        DCD_TRY_CUDA(cudaMemcpyAsync(c->hgs, gs, G * sizeof(GraphState), cudaMemcpyDeviceToHost, s));
         DCD_TRY_CUDA(cudaStreamSynchronize(s));
         if (c->hsc->loop_err || !c->hsc->any_running) break;
       }
     }
-    trace("level: pass loop ran");
     if (level == 0) {  // the level-0 bin record (dcd_get_level0_bins)
       c->l0_nb = bins.plan.nb;
       c->l0_side = any && total >= kForkMin;
@@ -1919,19 +2000,30 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
         c->l0_sweep[x] = x < bins.plan.nb ? sweep[x] : 0;
       }
     }
+  }
+  return DCD_OK;
+}
+
+// After the synchronisation: what the level did.
+int finish_level(dcd_ctx* c, PendingLevel& pl, int level, LevelRun* out, GraphTally* tally) {
+  const Bins& bins = pl.bins;
+  const int G = c->G;
+  pl.idle = true;
+  trace("level: pass loop ran, labels counted");
+  {
     if (c->hsc->loop_err) {
       note_cuda_error(cudaErrorUnknown, "local-move pass loop passed its cap", __FILE__, __LINE__);
       return DCD_ETIMEOUT;
     }
     const int64_t passes = c->hsc->level_passes;
-    g_launches += body_launches * passes;
+    g_launches += pl.body_launches * passes;
     out->passes = passes;
     out->ms_lm = (float)(c->hsc->t_eval_ns * 1e-6);
     out->ms_apply = (float)(c->hsc->t_apply_ns * 1e-6);
     out->edges = bins.act_deg * passes;
     out->verts = bins.n_active * passes;
-    out->edges_pre = pre ? bins.pre_deg : 0;
-    out->verts_pre = pre ? bins.pre_verts : 0;
+    out->edges_pre = pl.pre ? bins.pre_deg : 0;
+    out->verts_pre = pl.pre ? bins.pre_verts : 0;
     for (int x = 0; x < bins.plan.nb; x++) {
       const int k = lm_variant_class(bins.plan.var[x]);
       out->edges_bin[k] += bins.deg[x] * passes;
@@ -1953,7 +2045,6 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
     tally->passes[x] += c->hgs[x].passes;
     if (level == 0) tally->passes0[x] = c->hgs[x].passes;
   }
-  trace("level: passes done");
   return DCD_OK;
 }
 
@@ -1985,7 +2076,8 @@ int used_labels(dcd_ctx* c, const Csr<W>& g, const int32_t* L, Buf<int32_t>& cid
 }
 
 // The same for a Louvain level, whose community sizes and sums are tracked:
-// ids by label_ids, nz vertices of the next level; per-graph counts in hgs.
+// ids by label_ids, nz vertices of the next level; per-graph counts in hgs and
+// the device scalars in hsc (the level's pass loop among them).
 int level_labels(dcd_ctx* c, int64_t nv, const int32_t* size, const int64_t* a, Buf<int32_t>& cid, int64_t* nz,
                  const int32_t* gid, Buf<int32_t>* gid_next) {
   cudaStream_t s = c->stream;
@@ -1995,19 +2087,18 @@ int level_labels(dcd_ctx* c, int64_t nv, const int32_t* size, const int64_t* a, 
   DCD_TRY(f.alloc(&c->mem, nv + 1));
   DCD_TRY(tmp.alloc(&c->mem, scan_tmp_count(nv + 1)));
   if (gid_next) DCD_TRY(gid_next->alloc(&c->mem, nv));
-  ::dcd::count_launch(), gs_reset_nc<<<cdiv(c->G, 128), 128, 0, s>>>(c->gs.get(), c->G);
-  ::dcd::count_launch(), label_flags<<<grid_for(nv + 1, T), T, 0, s>>>(nv, size, a, f.get());
+  ::dcd::count_launch(), label_flags<<<grid_for(nv + 1, T), T, 0, s>>>(nv, size, a, f.get(), c->gs.get(), c->G);
   DCD_LAUNCH_CHECK();
   DCD_TRY(exclusive_scan<int64_t>(f.get(), f.get(), nv + 1, nullptr, tmp.get(), s));
   ::dcd::count_launch(), label_ids<<<grid_for(nv, T), T, 0, s>>>(nv, size, a, f.get(), gid, cid.get(), c->gs.get(),
                                                                  gid_next ? gid_next->get() : nullptr);
   DCD_LAUNCH_CHECK();
   DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch, f.get() + nv, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 1, &c->dsc.get()->n1_new, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  DCD_TRY_CUDA(cudaMemcpyAsync(c->hsc, c->dsc.get(), sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
   DCD_TRY_CUDA(cudaMemcpyAsync(c->hgs, c->gs.get(), c->G * sizeof(GraphState), cudaMemcpyDeviceToHost, s));
   DCD_TRY_CUDA(cudaStreamSynchronize(s));
   *nz = (int64_t)(int32_t)c->hscratch[0];
-  c->n1.fresh = (int64_t)(int32_t)c->hscratch[1];
+  c->n1.fresh = (int64_t)(int32_t)c->hsc->n1_new;
   return DCD_OK;
 }
 
@@ -2236,9 +2327,17 @@ __global__ void n1_final_of(int64_t n, int64_t nc0, const int32_t* __restrict__ 
     if (fs[i] >= 0 && F[i] != fs[i]) F[i] = fs[i];
 }
 
-// Rows of K: the distinct labels of F (at most nk), numbered as they come.
-__global__ void n1_index(int64_t nc0, const int32_t* __restrict__ F, int64_t nk, int32_t* __restrict__ kidx,
-                         int32_t* __restrict__ klab, int32_t* __restrict__ cnt) {
+// Rows of K: communities of the result with entries.
+__device__ __forceinline__ int64_t kept_rows(const GraphState* gs, int64_t iso, int64_t most) {
+  const int64_t nk = gs[0].ncomm - iso;
+  return nk < most ? nk : most;
+}
+
+// The distinct labels of F (at most nk), numbered as they come.
+__global__ void n1_index(int64_t nc0, const int32_t* __restrict__ F, const GraphState* __restrict__ gs, int64_t iso,
+                         int64_t most, int32_t* __restrict__ kidx, int32_t* __restrict__ klab,
+                         int32_t* __restrict__ cnt) {
+  const int64_t nk = kept_rows(gs, iso, most);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nc0; i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t l = F[i];
     if (kidx[l] != -1 || atomicCAS(&kidx[l], -1, -2) != -1) continue;
@@ -2252,7 +2351,9 @@ __global__ void n1_index(int64_t nc0, const int32_t* __restrict__ F, int64_t nk,
 
 template <typename VT>
 __global__ void n1_fold(const VT* __restrict__ H, int64_t nc0, const int32_t* __restrict__ F,
-                        const int32_t* __restrict__ kidx, int64_t nk, unsigned long long* __restrict__ K) {
+                        const int32_t* __restrict__ kidx, const GraphState* __restrict__ gs, int64_t iso, int64_t most,
+                        unsigned long long* __restrict__ K) {
+  const int64_t nk = kept_rows(gs, iso, most);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nc0 * nc0;
        i += (int64_t)gridDim.x * blockDim.x) {
     const VT x = H[i];
@@ -2261,43 +2362,34 @@ __global__ void n1_fold(const VT* __restrict__ H, int64_t nc0, const int32_t* __
   }
 }
 
-// Level 0's coarse matrix by the delta rule into H (nc x nc, zeroed).
-// *ok false (H unusable) when an index check failed: a label without a row
-// of K, which the rule excludes; the caller then rebuilds from every entry.
+// Level 0's coarse matrix by the delta rule into H (nc x nc, zeroed).  Three
+// words behind `entries` (zeroed): the row entries read; not zero (H unusable)
+// when an index check failed, a label without a row of K, which the rule
+// excludes: the caller then rebuilds from every entry; the work items.
 template <typename VT>
 int n1_build(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L0, const int32_t* cid, int64_t nc, VT* H,
-             unsigned long long* entries, bool* ok) {
+             unsigned long long* entries) {
   cudaStream_t s = c->stream;
   const int T = 256;
   const int64_t nk0 = c->kc_n, nk = nk0 + c->n1.fresh;
   const int32_t *kidx = c->n1.kidx, *klab = c->n1.klab;
   Buf<VT> D;
   Buf<int64_t> items;
-  Buf<int32_t> cnt;
-  Buf<uint32_t> bad;
+  uint32_t* bad = reinterpret_cast<uint32_t*>(entries + 1);
+  int32_t* cnt = reinterpret_cast<int32_t*>(entries + 2);
   DCD_TRY(D.alloc(&c->mem, nk * nk));
   DCD_TRY(items.alloc(&c->mem, g.n + g.nnz / kN1Chunk + 32));
-  DCD_TRY(cnt.alloc(&c->mem, 1));
-  DCD_TRY(bad.alloc(&c->mem, 1));
-  DCD_TRY_CUDA(cudaMemsetAsync(cnt.get(), 0, sizeof(int32_t), s));
-  DCD_TRY_CUDA(cudaMemsetAsync(bad.get(), 0, sizeof(uint32_t), s));
   ::dcd::count_launch(), n1_load<VT><<<grid_for(nk * nk, T), T, 0, s>>>(c->kc_mat.get(), nk0, nk, D.get());
   if (c->n1.P > 0)
     ::dcd::count_launch(), n1_pairs<VT><<<grid_for(c->n1.P, T), T, 0, s>>>(
-        c->n1.pkey, c->n1.pdelta, c->n1.P, c->n1.cprev, kidx, nk, D.get(), bad.get());
+        c->n1.pkey, c->n1.pdelta, c->n1.P, c->n1.cprev, kidx, nk, D.get(), bad);
   ::dcd::count_launch(), n1_movers_list<<<grid_for(g.n, T), T, 0, s>>>(g.n, L0, c->n1.cprev, g.rp, items.get(),
-                                                                        cnt.get(), entries);
+                                                                        cnt, entries);
   ::dcd::count_launch(), n1_movers<VT><<<wave_grid(n1_movers<VT>, g.n * 32, T), T, 0, s>>>(
-      items.get(), cnt.get(), g.rp, g.col, g.w, L0, c->n1.cprev, kidx, nk, D.get(), bad.get());
+      items.get(), cnt, g.rp, g.col, g.w, L0, c->n1.cprev, kidx, nk, D.get(), bad);
   ::dcd::count_launch(), n1_compact<VT><<<grid_for(nk * nk, T), T, 0, s>>>(D.get(), nk, klab, cid, L0, nc, H,
-                                                                            bad.get());
+                                                                            bad);
   DCD_LAUNCH_CHECK();
-  DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 2, bad.get(), sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-  DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 3, cnt.get(), sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  DCD_TRY_CUDA(cudaStreamSynchronize(s));
-  *ok = *reinterpret_cast<uint32_t*>(c->hscratch + 2) == 0;
-  tracef("level-0 delta rule: %lld pairs, %d row chunks of moved vertices, %lld x %lld kept cells", (long long)c->n1.P,
-         *reinterpret_cast<int32_t*>(c->hscratch + 3), (long long)nk, (long long)nk);
   return DCD_OK;
 }
 
@@ -2328,43 +2420,44 @@ int n1_extend(dcd_ctx* c, Buf<int32_t>& kidx, Buf<int32_t>& klab) {
   return DCD_OK;
 }
 
-// K of this update's final labels (into the *_nx buffers; taken at commit);
-// nk: the communities with entries.
+// K of this update's final labels (into the *_nx buffers; taken at commit, with
+// kc_n_nx = its rows, which the kernels take from the device: ncomm less the
+// iso communities without entries).  most: room for that many rows.
 template <typename VT>
-int n1_keep_t(dcd_ctx* c, int64_t n, const int32_t* fin, int64_t nk) {
+int n1_keep_t(dcd_ctx* c, int64_t n, const int32_t* fin, int64_t most, int64_t iso) {
   cudaStream_t s = c->stream;
   const int T = 256;
   const int64_t nc0 = c->n1.h0_nc;
-  if (nk > kDenseNc || nk < 0) return DCD_OK;  // cannot happen (nk <= nc0); kept out of K's size bound
+  if (most > kDenseNc || most < 0) return DCD_OK;  // cannot happen (most <= nc0); kept out of K's size bound
   Buf<int32_t> F, cnt;
   DCD_TRY(F.alloc(&c->mem, nc0 > 0 ? nc0 : 1));
   DCD_TRY(cnt.alloc(&c->mem, 1));
   DCD_TRY(c->kc_idx_nx.ensure(&c->mem, n));
-  DCD_TRY(c->kc_lab_nx.ensure(&c->mem, nk > 0 ? nk : 1));
-  DCD_TRY(c->kc_mat_nx.ensure(&c->mem, nk * nk > 0 ? nk * nk : 1));
+  DCD_TRY(c->kc_lab_nx.ensure(&c->mem, most > 0 ? most : 1));
+  DCD_TRY(c->kc_mat_nx.ensure(&c->mem, most * most > 0 ? most * most : 1));
   DCD_TRY_CUDA(cudaMemsetAsync(c->kc_idx_nx.get(), 0xff, n * sizeof(int32_t), s));
-  DCD_TRY_CUDA(cudaMemsetAsync(c->kc_mat_nx.get(), 0, nk * nk * sizeof(unsigned long long), s));
+  DCD_TRY_CUDA(cudaMemsetAsync(c->kc_mat_nx.get(), 0, most * most * sizeof(unsigned long long), s));
   DCD_TRY_CUDA(cudaMemsetAsync(cnt.get(), 0, sizeof(int32_t), s));
   if (nc0 > 0) {
     const int64_t blocks = cdiv(n, (int64_t)T);
     const int grid = (int)(blocks < 4 * c->sms ? blocks : 4 * c->sms);
     ::dcd::count_launch(), n1_final_of<<<grid > 0 ? grid : 1, T, nc0 * sizeof(int32_t), s>>>(
         n, nc0, c->h0_ccid.get(), fin, F.get());
-    ::dcd::count_launch(), n1_index<<<grid_for(nc0, T), T, 0, s>>>(nc0, F.get(), nk, c->kc_idx_nx.get(),
+    ::dcd::count_launch(), n1_index<<<grid_for(nc0, T), T, 0, s>>>(nc0, F.get(), c->gs.get(), iso, most, c->kc_idx_nx.get(),
                                                                    c->kc_lab_nx.get(), cnt.get());
     ::dcd::count_launch(), n1_fold<VT><<<grid_for(nc0 * nc0, T), T, 0, s>>>(
-        reinterpret_cast<const VT*>(c->h0.get()), nc0, F.get(), c->kc_idx_nx.get(), nk, c->kc_mat_nx.get());
+        reinterpret_cast<const VT*>(c->h0.get()), nc0, F.get(), c->kc_idx_nx.get(), c->gs.get(), iso, most,
+        c->kc_mat_nx.get());
     DCD_LAUNCH_CHECK();
   }
-  c->kc_n_nx = nk;
   c->kc_nx_ready = true;
   return DCD_OK;
 }
 
-int n1_keep(dcd_ctx* c, int64_t n, const int32_t* fin, int64_t nk) {
+int n1_keep(dcd_ctx* c, int64_t n, const int32_t* fin, int64_t most, int64_t iso) {
   c->kc_nx_ready = false;
   if (!c->n1.track || !c->n1.h0_ready) return DCD_OK;
-  return c->n1.h0_wide ? n1_keep_t<unsigned long long>(c, n, fin, nk) : n1_keep_t<unsigned>(c, n, fin, nk);
+  return c->n1.h0_wide ? n1_keep_t<unsigned long long>(c, n, fin, most, iso) : n1_keep_t<unsigned>(c, n, fin, most, iso);
 }
 
 // Block layout of the level-0 coarse graphs of several graphs: the matrix of
@@ -2385,9 +2478,18 @@ __global__ void fill_rowbase(const int64_t* __restrict__ co, const int64_t* __re
   }
 }
 
+template <typename VT>
+__global__ void zero_when(const uint32_t* __restrict__ when, VT* __restrict__ x, int64_t n) {
+  if (!*when) return;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    x[i] = VT(0);
+}
+
 // The dense coarse matrix (cells in all; blocks NULL: one nc x nc matrix) of the
 // sums of every entry, or of level 0 by the delta rule.  The level-0 matrix of
-// one graph is kept for the next update's delta rule.
+// one graph is kept for the next update's delta rule.  *delta_out: the delta
+// rule was tried; ent: the row entries it read, whether it failed (the matrix is
+// then the sums of every entry), its work items.
 template <typename W, typename VT>
 int dense_matrix(dcd_ctx* c, const Csr<W>& g, const int32_t* ccid, int64_t nc, const DenseBlocks* blocks, bool level0,
                  const int32_t* L, const int32_t* cid, Buf<VT>& dense_local, Buf<unsigned long long>& ent,
@@ -2405,22 +2507,24 @@ int dense_matrix(dcd_ctx* c, const Csr<W>& g, const int32_t* ccid, int64_t nc, c
     DCD_TRY(dense_local.alloc(&c->mem, cells));
     dense = dense_local.get();
   }
-  DCD_TRY(ent.alloc(&c->mem, 1));
+  DCD_TRY(ent.alloc(&c->mem, 3));
   DCD_TRY_CUDA(cudaMemsetAsync(dense, 0, cells * sizeof(VT), s));
-  DCD_TRY_CUDA(cudaMemsetAsync(ent.get(), 0, sizeof(unsigned long long), s));
+  DCD_TRY_CUDA(cudaMemsetAsync(ent.get(), 0, 3 * sizeof(unsigned long long), s));
   bool delta = false;
+  const uint32_t* when = nullptr;
   if constexpr (std::is_same<W, int32_t>::value) {
     if (level0 && !blocks && c->n1.usable && c->kc_valid && c->kc_n + c->n1.fresh <= kDenseNc) {
-      bool ok = false;
-      DCD_TRY(n1_build<VT>(c, g, L, cid, nc, dense, ent.get(), &ok));
-      delta = ok;
-      if (!ok) {  // rebuild from every entry
-        DCD_TRY_CUDA(cudaMemsetAsync(dense, 0, cells * sizeof(VT), s));
-        DCD_TRY_CUDA(cudaMemsetAsync(ent.get(), 0, sizeof(unsigned long long), s));
-      }
+      DCD_TRY(n1_build<VT>(c, g, L, cid, nc, dense, ent.get()));
+      delta = true;
+      // a label without a row: the matrix from every entry after all, decided on
+      // the device (two launches that return at once; asking the host instead
+      // took 15 us)
+      when = reinterpret_cast<const uint32_t*>(ent.get() + 1);
+      ::dcd::count_launch(), zero_when<VT><<<grid_for(cells, 256), 256, 0, s>>>(when, dense, cells);
+      DCD_LAUNCH_CHECK();
     }
   }
-  if (!delta && m0 > 0) {
+  if (m0 > 0) {
     const uint32_t* rb = blocks ? blocks->rowbase.get() : nullptr;
     // a CTA copy of the matrix when it fits in shared memory (two CTAs an SM)
     const size_t msm = (size_t)cells * sizeof(VT);
@@ -2430,45 +2534,31 @@ int dense_matrix(dcd_ctx* c, const Csr<W>& g, const int32_t* ccid, int64_t nc, c
       const int grid = wave_grid(emit_dense<W, VT, true>, cdiv(m0, 32) * 32, kEmitThreads, msm);
       const int64_t per_warp = cdiv(cdiv(m0, (int64_t)grid * (kEmitThreads / 32)), 32) * 32;
       ::dcd::count_launch(), emit_dense<W, VT, true><<<grid, kEmitThreads, msm, s>>>(
-          g.n, m0, g.rp, g.col, g.w, ccid, (uint32_t)nc, rb, (uint32_t)cells, per_warp, dense);
+          g.n, m0, g.rp, g.col, g.w, ccid, (uint32_t)nc, rb, (uint32_t)cells, per_warp, dense, when);
     } else {
       const int grid = wave_grid(emit_dense<W, VT, false>, cdiv(m0, 32) * 32, kEmitThreads);
       const int64_t per_warp = cdiv(cdiv(m0, (int64_t)grid * (kEmitThreads / 32)), 32) * 32;
       ::dcd::count_launch(), emit_dense<W, VT, false><<<grid, kEmitThreads, 0, s>>>(
-          g.n, m0, g.rp, g.col, g.w, ccid, (uint32_t)nc, rb, (uint32_t)cells, per_warp, dense);
+          g.n, m0, g.rp, g.col, g.w, ccid, (uint32_t)nc, rb, (uint32_t)cells, per_warp, dense, when);
     }
     DCD_LAUNCH_CHECK();
   }
   *dense_out = dense;
   *delta_out = delta;
+  if (keep) c->n1.h0_ready = true;
   return DCD_OK;
 }
 
-// What level 0's coarsening read (ent: the delta rule's row entries).
-void note_level0(dcd_ctx* c, bool delta, int64_t ent, int64_t m0, int64_t nc) {
+// What level 0's coarsening read (ent: dense_matrix's three words).
+void note_level0(dcd_ctx* c, bool tried, const int64_t* ent, int64_t m0, int64_t nc) {
+  const bool delta = tried && *reinterpret_cast<const uint32_t*>(ent + 1) == 0;
+  if (tried)
+    tracef("level-0 delta rule: %lld pairs, %d row chunks of moved vertices%s", (long long)c->n1.P,
+           *reinterpret_cast<const int32_t*>(ent + 2), delta ? "" : ", a label without a row");
   c->n1.used = delta;
-  c->n1.entries = delta ? c->n1.distinct + ent : m0;
-  c->n1.h0_ready = c->n1.track;
+  c->n1.entries = delta ? c->n1.distinct + ent[0] : m0;
   tracef("level-0 coarse graph: %s, %lld entries read, %lld communities", delta ? "delta rule" : "every entry",
          (long long)c->n1.entries, (long long)nc);
-}
-
-// The next level's vertex of every vertex (level 0 of a tracked graph: kept
-// for the next update).
-int coarse_ids(dcd_ctx* c, int64_t n, const int32_t* L, const int32_t* cid, bool level0, Buf<int32_t>& local,
-               int32_t** out) {
-  if (level0 && c->n1.track) {
-    DCD_TRY(c->h0_ccid.ensure(&c->mem, n > 0 ? n : 1));
-    *out = c->h0_ccid.get();
-  } else {
-    DCD_TRY(local.alloc(&c->mem, n > 0 ? n : 1));
-    *out = local.get();
-  }
-  if (n > 0) {
-    ::dcd::count_launch(), coarse_of<<<grid_for(n, 256), 256, 0, c->stream>>>(n, L, cid, *out);
-    DCD_LAUNCH_CHECK();
-  }
-  return DCD_OK;
 }
 
 // Sums of weights need 64 bits (2m of the largest graph bounds them).
@@ -2484,7 +2574,6 @@ struct DenseLevels {
   Buf<int64_t> co, cb;
   Buf<unsigned> h32;
   Buf<unsigned long long> h64, ent;
-  Buf<int32_t> ccid;
   LevelsIn in;
   LevelsBufs bufs;
   bool delta = false;
@@ -2512,11 +2601,9 @@ bool levels_fit(const dcd_ctx* c, const std::vector<int64_t>& nz, DenseLevels* d
 }
 
 template <typename W>
-int dense_levels_matrix(dcd_ctx* c, const Csr<W>& g, const int32_t* L, const int32_t* cid, bool level0,
-                        DenseLevels* d) {
+int dense_levels_matrix(dcd_ctx* c, const Csr<W>& g, const int32_t* ccid, bool level0, const int32_t* L,
+                        const int32_t* cid, DenseLevels* d) {
   cudaStream_t s = c->stream;
-  int32_t* ccid = nullptr;
-  DCD_TRY(coarse_ids(c, g.n, L, cid, level0, d->ccid, &ccid));
   const DenseBlocks* blocks = nullptr;
   if (c->G > 1) {
     const int G = c->G;
@@ -2565,10 +2652,10 @@ int coarsen_dense(dcd_ctx* c, const Csr<W>& g, const int32_t* ccid, int64_t nc, 
   DCD_LAUNCH_CHECK();
   DCD_TRY(exclusive_scan<int64_t>(out->rp.get(), out->rp.get(), nc + 1, nullptr, stmp.get(), s));
   DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch, out->rp.get() + nc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 1, ent.get(), sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 1, ent.get(), 3 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   DCD_TRY_CUDA(cudaStreamSynchronize(s));
   const int64_t U = c->hscratch[0];
-  if (level0) note_level0(c, delta, c->hscratch[1], g.nnz, nc);
+  if (level0) note_level0(c, delta, c->hscratch + 1, g.nnz, nc);
   DCD_TRY(out->col.alloc(&c->mem, U));
   DCD_TRY(out->w.alloc(&c->mem, U));
   ::dcd::count_launch(), dense_write<VT><<<grid_for(nc * 32, T), T, 0, s>>>(dense, nc, out->rp.get(),
@@ -2581,16 +2668,13 @@ int coarsen_dense(dcd_ctx* c, const Csr<W>& g, const int32_t* ccid, int64_t nc, 
 // level0: the coarsening of G_t's level-0 labels (the delta rule may apply,
 // and the matrix is kept for the next update).
 template <typename W>
-int coarsen(dcd_ctx* c, const Csr<W>& g, const int32_t* L, const int32_t* cid, int64_t nc, CoarseGraph* out,
-            bool level0 = false) {
+int coarsen(dcd_ctx* c, const Csr<W>& g, const int32_t* ccid, int64_t nc, CoarseGraph* out, bool level0,
+            const int32_t* L, const int32_t* cid) {
   cudaStream_t s = c->stream;
   const int T = 256;
   const int64_t m0 = g.nnz;
   if (level0) c->n1.entries = m0;
   if (nc <= kDenseNc) {
-    Buf<int32_t> ccid_local;
-    int32_t* ccid = nullptr;
-    DCD_TRY(coarse_ids(c, g.n, L, cid, level0, ccid_local, &ccid));
     if (!wide_sums(c)) return coarsen_dense<W, unsigned>(c, g, ccid, nc, out, level0, L, cid);
     return coarsen_dense<W, unsigned long long>(c, g, ccid, nc, out, level0, L, cid);
   }
@@ -2603,22 +2687,19 @@ int coarsen(dcd_ctx* c, const Csr<W>& g, const int32_t* L, const int32_t* cid, i
   DCD_TRY(cnt.alloc(&c->mem, 1));
   DCD_TRY_CUDA(cudaMemsetAsync(cnt.get(), 0, sizeof(unsigned long long), s));
   if (m0 > 0) {
-    Buf<int32_t> ccid;
-    DCD_TRY(ccid.alloc(&c->mem, g.n));
-    ::dcd::count_launch(), coarse_of<<<grid_for(g.n, T), T, 0, s>>>(g.n, L, cid, ccid.get());
     int64_t m2max = 0;
     for (int x = 0; x < c->G; x++) m2max = c->hgs[x].m2 > m2max ? c->hgs[x].m2 : m2max;
     const bool narrow = m2max < ((int64_t)1 << 31), small = nc < 65536;
     if (narrow && small)
-      DCD_TRY((launch_emit<W, uint32_t, unsigned>(c, g, m0, ccid.get(), nc, k0.get(), v0.get(), cnt.get())));
+      DCD_TRY((launch_emit<W, uint32_t, unsigned>(c, g, m0, ccid, nc, k0.get(), v0.get(), cnt.get())));
     else if (narrow)
-      DCD_TRY((launch_emit<W, unsigned long long, unsigned>(c, g, m0, ccid.get(), nc, k0.get(), v0.get(),
+      DCD_TRY((launch_emit<W, unsigned long long, unsigned>(c, g, m0, ccid, nc, k0.get(), v0.get(),
                                                              cnt.get())));
     else if (small)
-      DCD_TRY((launch_emit<W, uint32_t, unsigned long long>(c, g, m0, ccid.get(), nc, k0.get(), v0.get(),
+      DCD_TRY((launch_emit<W, uint32_t, unsigned long long>(c, g, m0, ccid, nc, k0.get(), v0.get(),
                                                              cnt.get())));
     else
-      DCD_TRY((launch_emit<W, unsigned long long, unsigned long long>(c, g, m0, ccid.get(), nc, k0.get(),
+      DCD_TRY((launch_emit<W, unsigned long long, unsigned long long>(c, g, m0, ccid, nc, k0.get(),
                                                                        v0.get(), cnt.get())));
     DCD_LAUNCH_CHECK();
   }
@@ -2903,10 +2984,9 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
   } else {
     DCD_TRY(community_sums(c, n0, labels0, k0.get(), a.get(), size.get()));
   }
-  ::dcd::count_launch(), fill_iota<<<grid_for(n0, T), T, 0, s>>>(comp.get(), n0);
-  ::dcd::count_launch(), gs_reset_pass<<<cdiv(G, 128), 128, 0, s>>>(gs, G, &c->dsc.get()->pass_id);
-  ::dcd::count_launch(), sumsq_acc<<<grid_for(n0, T, 4), T, 0, s>>>(a.get(), n0, gid0, gs);
+  ::dcd::count_launch(), pass_begin<<<cdiv(G, 256), 256, 0, s>>>(gs, G, c->dsc.get(), nullptr);
   DCD_LAUNCH_CHECK();
+  const int32_t* comp_cur = nullptr;  // the level's vertex of every vertex (NULL: itself)
 
   // per-graph host state of the level loop
   std::vector<int64_t> nv(G);
@@ -2939,16 +3019,27 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
   bool ran_dense = false, dense_first = false;
   int64_t iso = 0;   // communities without entries at the end of level 0
 
+  std::unique_ptr<PendingLevel> pending;
   for (;;) {
     LevelRun lr;
+    pending.reset(new PendingLevel);
+    PendingLevel& pl = *pending;
     if (level == 0) {
-      DCD_TRY(run_level<int32_t>(c, *g_l0, L, *kcur, a, size, active, gid, (int)level, &lr, &tally, pre0, nlab));
+      DCD_TRY(run_level<int32_t>(c, *g_l0, L, *kcur, a, size, active, gid, (int)level, &pl, pre0, nlab));
       nlab->ready = false;  // they follow the level's moves, not the labels the caller started from
       if (level0_out)
         DCD_TRY_CUDA(cudaMemcpyAsync(level0_out, L, n0 * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+      if (G == 1) DCD_TRY(n1_extend(c, n1_kidx, n1_klab));
     } else {
-      DCD_TRY(run_level<int64_t>(c, *g_lc, L, *kcur, a, size, nullptr, gid, (int)level, &lr, &tally));
+      DCD_TRY(run_level<int64_t>(c, *g_lc, L, *kcur, a, size, nullptr, gid, (int)level, &pl));
     }
+    DCD_TRY_CUDA(cudaEventRecord(c->ev[5], s));
+    Buf<int32_t> cid;
+    int64_t nc = 0;
+    const int nx = which ^ 1;
+    Buf<int32_t>* gnext = G > 1 ? &gidc[nx] : nullptr;
+    DCD_TRY(level_labels(c, nvu, size.get(), a.get(), cid, &nc, gid, gnext));
+    DCD_TRY(finish_level(c, pl, (int)level, &lr, &tally));
     if (first_level) {
       for (int x = 0; x < G; x++) N_start[x] = h128(c->hgs[x].n_start_lo, c->hgs[x].n_start_hi);
       first_level = false;
@@ -2977,14 +3068,6 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
     ms_lm += lr.ms_lm;
     ms_apply += lr.ms_apply;
 
-    DCD_TRY_CUDA(cudaEventRecord(c->ev[5], s));
-    Buf<int32_t> cid;
-    int64_t nc = 0;
-    const int nx = which ^ 1;
-    Buf<int32_t>* gnext = G > 1 ? &gidc[nx] : nullptr;
-    if (level == 0 && G == 1) DCD_TRY(n1_extend(c, n1_kidx, n1_klab));
-    DCD_TRY(level_labels(c, nvu, size.get(), a.get(), cid, &nc, gid, gnext));
-    trace("level: labels counted");
     level++;
     // level stop per graph: nothing merged, or (from the second level on) a
     // gain of at most |N_start| / tau_inv, or the level cap
@@ -3018,12 +3101,35 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
     // ---- few communities: every further level in one launch ----
     std::vector<int64_t> nzg(G);
     for (int x = 0; x < G; x++) nzg[x] = level == 1 ? c->hgs[x].nc - c->hgs[x].iso : c->hgs[x].nc;
+    // the next level's vertex of every vertex of this one
+    Buf<int32_t> ccid_buf;
+    const int32_t* ccid = nullptr;
+    {
+      int32_t* dst = comp.get();
+      const bool keep = level == 1 && c->n1.track && nc <= kDenseNc;  // for the next update's delta rule
+      if (keep) {
+        DCD_TRY(c->h0_ccid.ensure(&c->mem, n0 > 0 ? n0 : 1));
+        dst = c->h0_ccid.get();
+      } else if (level > 1) {
+        DCD_TRY(ccid_buf.alloc(&c->mem, nvu > 0 ? nvu : 1));
+        dst = ccid_buf.get();
+      }
+      if (nvu > 0) ::dcd::count_launch(), coarse_of<<<grid_for(nvu, T), T, 0, s>>>(nvu, L, cid.get(), dst);
+      ccid = dst;
+      if (level == 1) {
+        comp_cur = ccid;
+      } else {
+        ::dcd::count_launch(), compose_ids<<<grid_for(n0, T), T, 0, s>>>(n0, nvu, nc, comp_cur, comp.get(), L,
+                                                                         cid.get());
+        comp_cur = comp.get();
+      }
+      DCD_LAUNCH_CHECK();
+    }
     if (levels_fit(c, nzg, &dl)) {
-      if (level == 1) DCD_TRY(dense_levels_matrix<int32_t>(c, *g_l0, L, cid.get(), G == 1, &dl));
-      else DCD_TRY(dense_levels_matrix<int64_t>(c, *g_lc, L, cid.get(), false, &dl));
+      if (level == 1) DCD_TRY(dense_levels_matrix<int32_t>(c, *g_l0, ccid, G == 1, L, cid.get(), &dl));
+      else DCD_TRY(dense_levels_matrix<int64_t>(c, *g_lc, ccid, false, L, cid.get(), &dl));
       DCD_TRY(kc[nx].alloc(&c->mem, nc));
       DCD_TRY(Lc[nx].alloc(&c->mem, nc));
-      ::dcd::count_launch(), compose_ids<<<grid_for(n0, T), T, 0, s>>>(n0, nvu, nc, comp.get(), L, cid.get());
       ::dcd::count_launch(), level_start<<<grid_for(nvu, T), T, 0, s>>>(nvu, nc, cid.get(), a.get(), kc[nx].get(),
                                                                         Lc[nx].get());
       DCD_LAUNCH_CHECK();
@@ -3040,11 +3146,10 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
     }
     // ---- compact: next level (all graphs together; finished graphs only
     // carry their labels along) ----
-    if (level == 1) DCD_TRY(coarsen<int32_t>(c, *g_l0, L, cid.get(), nc, &cg[nx], G == 1));
-    else DCD_TRY(coarsen<int64_t>(c, *g_lc, L, cid.get(), nc, &cg[nx]));
+    if (level == 1) DCD_TRY(coarsen<int32_t>(c, *g_l0, ccid, nc, &cg[nx], G == 1, L, cid.get()));
+    else DCD_TRY(coarsen<int64_t>(c, *g_lc, ccid, nc, &cg[nx], false, L, cid.get()));
     DCD_TRY(kc[nx].alloc(&c->mem, nc));
     DCD_TRY(Lc[nx].alloc(&c->mem, nc));
-    ::dcd::count_launch(), compose_ids<<<grid_for(n0, T), T, 0, s>>>(n0, nvu, nc, comp.get(), L, cid.get());
     // next level starts from singletons; in and sum a^2 carry over
     ::dcd::count_launch(), level_start<<<grid_for(nvu, T), T, 0, s>>>(nvu, nc, cid.get(), a.get(), kc[nx].get(),
                                                                       Lc[nx].get());
@@ -3077,25 +3182,29 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
   {
     Buf<int32_t> minid;
     DCD_TRY(minid.alloc(&c->mem, nvu + iso));
-    ::dcd::count_launch(), fill_i32<<<grid_for(nvu + iso, T), T, 0, s>>>(minid.get(), nvu + iso, INT32_MAX);
-    ::dcd::count_launch(), final_min<<<grid_for(n0, T), T, 0, s>>>(n0, nvu, comp.get(), L, minid.get());
-    ::dcd::count_launch(), gs_reset_nc<<<cdiv(G, 128), 128, 0, s>>>(gs, G);
-    ::dcd::count_launch(), final_labels<<<grid_for(n0, T), T, 0, s>>>(n0, nvu, comp.get(), L, minid.get(),
+    const int64_t most = nvu + iso > G ? nvu + iso : G;
+    ::dcd::count_launch(), final_begin<<<grid_for(most, T), T, 0, s>>>(minid.get(), nvu + iso, gs, G);
+    ::dcd::count_launch(), final_min<<<grid_for(n0, T), T, 0, s>>>(n0, nvu, comp_cur, L, minid.get());
+    ::dcd::count_launch(), final_labels<<<grid_for(n0, T), T, 0, s>>>(n0, nvu, comp_cur, L, minid.get(),
                                                                        out_labels, gid0, gs);
     DCD_LAUNCH_CHECK();
     DCD_TRY_CUDA(cudaEventRecord(c->ev[8], s));
+    // the coarse graph of the result, for the next update (with few
+    // communities before their number is read back: sized by the level's)
+    if (G == 1 && ran_dense) DCD_TRY(n1_keep(c, n0, out_labels, c->n1.h0_nc, iso));
     std::vector<uint8_t> ran(G, 0);  // graphs whose levels the one launch finished
     if (ran_dense) {
       for (int x = 0; x < G; x++) ran[x] = !c->hgs[x].done;
       static_assert(sizeof(LevelTotals) <= 32 * sizeof(int64_t), "pinned words 32 on");
       DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 32, dl.bufs.tot, sizeof(LevelTotals), cudaMemcpyDeviceToHost, s));
-      DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 1, dl.ent.get(), sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+      DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 1, dl.ent.get(), 3 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     }
     DCD_TRY_CUDA(cudaMemcpyAsync(c->hgs, gs, G * sizeof(GraphState), cudaMemcpyDeviceToHost, s));
+    pending.reset();  // while the device works
     DCD_TRY_CUDA(cudaStreamSynchronize(s));
     if (ran_dense) {
       const LevelTotals& t = *reinterpret_cast<const LevelTotals*>(c->hscratch + 32);
-      if (dense_first && G == 1) note_level0(c, dl.delta, c->hscratch[1], g0.nnz, dl.in.nz);
+      if (dense_first && G == 1) note_level0(c, dl.delta, c->hscratch + 1, g0.nnz, dl.in.nz);
       float tc = 0.f;
       cudaEventElapsedTime(&tc, c->ev[5], c->ev[6]);
       ms_coarsen += tc + (float)(t.t_compact_ns * 1e-6);
@@ -3119,7 +3228,10 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
              (long long)t.levels, (long long)t.passes, t.t_eval_ns * 1e-6, t.t_apply_ns * 1e-6, t.t_compact_ns * 1e-6);
     }
   }
-  if (G == 1) DCD_TRY(n1_keep(c, n0, out_labels, c->hgs[0].ncomm - iso));
+  if (G == 1) {
+    if (!ran_dense) DCD_TRY(n1_keep(c, n0, out_labels, c->hgs[0].ncomm - iso, iso));
+    c->kc_n_nx = c->hgs[0].ncomm - iso;
+  }
   float tf = 0.f;
   cudaEventElapsedTime(&tf, c->ev[7], c->ev[8]);
   auto fill = [&](dcd_step_stats* o, int x) {
@@ -3741,12 +3853,15 @@ int run_slm(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint8_t*
     Buf<int32_t> cid;
     int64_t nc = 0;
     const int nx = which ^ 1;
-    if (level == 1) {
-      DCD_TRY(used_labels<int32_t>(c, g0, sub.get(), cid, &nc, nullptr, nullptr));
-      DCD_TRY(coarsen<int32_t>(c, g0, sub.get(), cid.get(), nc, &cg[nx]));
-    } else {
-      DCD_TRY(used_labels<int64_t>(c, *gc, sub.get(), cid, &nc, nullptr, nullptr));
-      DCD_TRY(coarsen<int64_t>(c, *gc, sub.get(), cid.get(), nc, &cg[nx]));
+    if (level == 1) DCD_TRY(used_labels<int32_t>(c, g0, sub.get(), cid, &nc, nullptr, nullptr));
+    else DCD_TRY(used_labels<int64_t>(c, *gc, sub.get(), cid, &nc, nullptr, nullptr));
+    {
+      Buf<int32_t> ccid;
+      DCD_TRY(ccid.alloc(&c->mem, nv));
+      ::dcd::count_launch(), coarse_of<<<grid_for(nv, T), T, 0, s>>>(nv, sub.get(), cid.get(), ccid.get());
+      DCD_LAUNCH_CHECK();
+      if (level == 1) DCD_TRY(coarsen<int32_t>(c, g0, ccid.get(), nc, &cg[nx], false, sub.get(), cid.get()));
+      else DCD_TRY(coarsen<int64_t>(c, *gc, ccid.get(), nc, &cg[nx], false, sub.get(), cid.get()));
     }
     DCD_TRY(kc[nx].alloc(&c->mem, nc));
     DCD_TRY(Lc[nx].alloc(&c->mem, nc));

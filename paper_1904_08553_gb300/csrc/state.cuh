@@ -21,7 +21,7 @@ struct Csr {
 struct DevScalars {
   int64_t pad_[9];
   int32_t any_running;  // some graph's pass loop goes on
-  int32_t stop_unused;
+  int32_t ticket;       // CTAs of pass_finish that are done
   int32_t nc;        // labels in use (coarsening)
   int32_t pad0;
   int64_t uniq;      // distinct coarse entries (coarsening)
