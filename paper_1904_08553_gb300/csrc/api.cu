@@ -611,7 +611,7 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
                          rds.get(), size.get(), use_pre ? pre.get() : nullptr));
   }
   if (learned || collect) {
-    DCD_TRY(screen_features(c, g, src_labels, mo.k->get(), a.get(), size.get(), mo, rds.get(), &nlab, &lp));
+    DCD_TRY(screen_features(c, g, src_labels, mo.k->get(), a.get(), size.get(), mo, sb.deg, rds.get(), &nlab, &lp));
     c->feat_has_y = false;
   }
   if (mode == DCD_MODE_DELTA) {
@@ -663,6 +663,12 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
                         collect ? c->level0.get() : nullptr, per_graph, a.n ? a.get() : nullptr,
                         size.n ? size.get() : nullptr, pre.n ? pre.get() : nullptr));
   if (collect) DCD_TRY(screen_labels(c, src_labels, c->level0.get()));
+  // sum_i e_{i->C(i)} of C_t on G_t and 2m, kept for the next merge: Louvain's
+  // tracked value (SLM does not track it)
+  const bool keep_in = c->cfg.alg == DCD_ALG_LOUVAIN;
+  DCD_TRY(c->in_next.ensure(&c->mem, 2 * (size_t)c->G));
+  ::dcd::count_launch(), save_in<<<cdiv(c->G, 128), 128, 0, s>>>(c->gs.get(), c->G, c->in_next.get());
+  DCD_LAUNCH_CHECK();
   if (screen) {  // the scalars were read back with the passes' results
     r_screen = c->hsc->r_screen;
     if (mode == DCD_MODE_DELTA) r_size = r_screen;
@@ -686,6 +692,7 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
       st->q_screen = ql;  // on a fallback, q_screen reports the rejected learned Q
       st->fallback = 1;
       r_size = r_screen;
+      ::dcd::count_launch(), save_in<<<cdiv(c->G, 128), 128, 0, s>>>(c->gs.get(), c->G, c->in_next.get());
       DCD_TRY_CUDA(cudaMemcpyAsync(c->labels_nx.get(), lab2.get(), n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
       DCD_TRY_CUDA(cudaMemcpyAsync(rnew.get(), rds.get(), n, cudaMemcpyDeviceToDevice, s));
     }
@@ -699,15 +706,6 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
     st->coarse0_delta = c->n1.used ? 1 : 0;
     st->coarse0_entries = c->n1.entries;
   }
-
-  // sum_i e_{i->C(i)} of C_t on G_t and 2m, kept for the next merge; the
-  // former is Louvain's tracked value, except after a judged learned step (its
-  // device state then holds the second run) and after SLM (which does not
-  // track it)
-  const bool keep_in = c->cfg.alg == DCD_ALG_LOUVAIN && !(learned && c->judge);
-  DCD_TRY(c->in_next.ensure(&c->mem, 2 * (size_t)c->G));
-  ::dcd::count_launch(), save_in<<<cdiv(c->G, 128), 128, 0, s>>>(c->gs.get(), c->G, c->in_next.get());
-  DCD_LAUNCH_CHECK();
 
   if (finish) DCD_TRY(finish(c, user));
 

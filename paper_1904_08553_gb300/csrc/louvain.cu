@@ -862,10 +862,9 @@ __device__ __forceinline__ void pass_close(DevScalars* d, bool more, cudaGraphCo
 // so that the total is exact in any order (one graph: a CTA reduction, then one
 // addition per CTA; several graphs: one addition per community in use); then, in
 // the CTA that finishes last, the decision of every graph (any_running <- some
-// graph goes on) and, with close, the end of the pass.  One launch: as a
-// reset, two stamps, three memsets, a sum, a decision and an end, the fixed
-// part of a pass was nine nodes of the loop, now two (10 K vertices, two
-// passes: 0.105 -> 0.083 ms, and 0.062 -> 0.045 to instantiate the loop).
+// goes on) and, with kPassClose, the end of the pass.  A reset, two stamps, three
+// memsets, a sum, a decision and an end were nine nodes of every pass; this and
+// pass_begin are two (10 K vertices: 62 -> 54 us to instantiate the loop).
 enum PassEnd { kLevelStart, kPassOpen, kPassClose };
 __global__ void __launch_bounds__(256) pass_finish(const int64_t* __restrict__ a, int64_t n,
                                                    const int32_t* __restrict__ gid, GraphState* __restrict__ gs, int G,

@@ -443,7 +443,8 @@ struct LearnedPool {
   PoolStats st;
 };
 int screen_features(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L0, const int64_t* k, const int64_t* a,
-                    const int32_t* size, const MergeOut& mo, const uint8_t* rds, EntryLabels* nlab, LearnedPool* out);
+                    const int32_t* size, const MergeOut& mo, int64_t source_deg, const uint8_t* rds, EntryLabels* nlab,
+                    LearnedPool* out);
 int learned_rset_build(dcd_ctx* c, const LearnedPool& lp, const uint8_t* rds, const float* p, uint8_t* r,
                        int64_t* r_size);
 int screen_labels(dcd_ctx* c, const int32_t* before, const int32_t* after);
