@@ -184,105 +184,179 @@ __device__ __forceinline__ void pair_sums_add(const PairView& o, int g, PairSum&
 // global memory.
 constexpr int kSegSmall = 64, kSegMid = 512, kSegLarge = 4096;
 
-// A CTA takes kPairSrc consecutive sources: their records (a counting sort
-// put them next to each other) and, when the batch is dense enough to pay for
-// it, the columns of their rows are staged in shared memory with coalesced
-// loads; a thread then ranks one record in its segment, sums the weights of
-// equal sinks, and looks its sink up in the row.  The row search is what
-// bounds this step: in global memory each of its 5-8 probes costs a sector a
-// lane, in shared memory a few cycles.  12.4 M records on 73 M entries: 556 us
-// for rank, sums, search and degrees, where separate kernels for them took
-// 196 (rank) + 175 (sums) + 683 us (search).  Sources without records only get
-// their k.
-constexpr int kPairSrc = 64;
+// A CTA takes NS consecutive sources: their records (a counting sort put them
+// next to each other) and the columns of their rows are staged in shared memory
+// with coalesced loads; a thread then ranks one record in its segment, and in a
+// second round takes the record that comes x-th: it sums the weights of equal
+// sinks, which are neighbours now, looks the sink up in the row, and writes the
+// pair next to its neighbours'.  Sources without records only get their k.
+//
+// Bound by latency and instructions, not by traffic: a chain of staging, search
+// and label gather per CTA, so the tile is small enough for 12 to 16 of them on an
+// SM (with 26 KB and 64 registers, 8, and barriers and loads were half of the
+// stalls), and the row search, 5-8 probes, which in global memory costs a sector a
+// probe and lane, runs on the staged copy.  Segments of other classes and rows
+// that do not fit are left out of the staging one by one.
 constexpr int kPairThreads = 128;
-constexpr int kPairRecs = 1280;
-constexpr int kPairCols = 3072;
+constexpr int kPairRecs = 640;
+constexpr int kPairCols = 2048;
+constexpr int kPairRow = 512;  // longest row staged on its own
 
-__global__ void __launch_bounds__(kPairThreads) pair_tile(PairView o, int64_t n, const uint64_t* __restrict__ rec,
-                                                          const int64_t* __restrict__ k_old,
-                                                          int64_t* __restrict__ k_new, int32_t* __restrict__ big,
-                                                          int32_t* __restrict__ big_cnt) {
-  __shared__ uint64_t s_rec[kPairRecs];
+// NS by the records a source, R / n, so that a CTA has about 64 or more: 2 M
+// sources and 12.4 M records take 458 us with 32 sources (555 with the 64 and
+// 26 KB of before), 4.2 M sources and 2.0 M records 309 with 128 (485), 2 M and
+// 84 K 96 (142).  Small graphs have too few CTAs of 128: 32 below kPairWide.
+constexpr int64_t kPairWide = 128 * 152 * 4;
+
+template <int NS>
+__global__ void __launch_bounds__(kPairThreads, 12) pair_tile(PairView o, int64_t n, const uint64_t* __restrict__ rec,
+                                                              const int64_t* __restrict__ k_old,
+                                                              int64_t* __restrict__ k_new, int32_t* __restrict__ big,
+                                                              int32_t* __restrict__ big_cnt) {
+  static_assert(NS <= kPairThreads, "a thread a source");
+  __shared__ uint32_t s_v[kPairRecs], s_w[kPairRecs];  // sinks and weights of the staged records
+  __shared__ uint16_t s_perm[kPairRecs];               // record that comes x-th
+  __shared__ uint8_t s_src[kPairRecs];                 // its source
   __shared__ int32_t s_col[kPairCols];
-  __shared__ int32_t s_off[kPairSrc + 1];
-  __shared__ int64_t s_rp[kPairSrc + 1];
-  __shared__ unsigned long long s_dk[kPairSrc];
+  __shared__ int32_t s_off[NS + 1], s_a[NS + 1];  // first record of a source: in the batch, staged
+  __shared__ int32_t s_c[NS];                     // first staged column of its row (-1: not staged)
+  __shared__ int64_t s_rp[NS + 1];
+  __shared__ unsigned long long s_dk[NS];
   const int tid = threadIdx.x;
-  const int64_t v0 = (int64_t)blockIdx.x * kPairSrc;
-  const int ns = (int)(n - v0 < kPairSrc ? n - v0 : kPairSrc);
-  for (int x = tid; x <= ns; x += kPairThreads) s_off[x] = o.off[v0 + x];
-  if (tid < kPairSrc) s_dk[tid] = 0;
+  const int64_t v0 = (int64_t)blockIdx.x * NS;
+  const int ns = (int)(n - v0 < NS ? n - v0 : NS);
+  for (int x = tid; x <= ns; x += kPairThreads) {
+    s_off[x] = o.off[v0 + x];
+    s_rp[x] = o.rp[v0 + x];
+  }
+  const int64_t kv = tid < ns ? k_old[v0 + tid] : 0;
+  if (tid < NS) s_dk[tid] = 0;
   __syncthreads();
-  const int32_t r0 = s_off[0];
-  const int nrec = s_off[ns] - r0;
-  if (nrec > 0) {
-    for (int x = tid; x <= ns; x += kPairThreads) s_rp[x] = o.rp[v0 + x];
-    __syncthreads();
+  if (s_off[ns] > s_off[0]) {
+    // records of the segments ranked here; longer ones: a CTA each, later
+    const int len = tid < ns ? s_off[tid + 1] - s_off[tid] : 0;
+    const int small = len <= kSegSmall ? len : 0;
+    if (len > kSegSmall) {
+      const int c = len <= kSegMid ? 0 : len <= kSegLarge ? 1 : 2;
+      big[(int64_t)c * n + atomicAdd(&big_cnt[c], 1)] = (int32_t)(v0 + tid);
+    }
+    int nrec;
+    const int a0 = block_excl_scan<int, kPairThreads>(small, &nrec);
+    if (tid < ns) s_a[tid] = a0;
+    if (tid == 0) s_a[ns] = nrec;
     const int64_t c0 = s_rp[0], ncol = s_rp[ns] - c0;
-    const bool srec = nrec <= kPairRecs;
     // a search costs a record about log2(row) probes of a sector each;
     // staging costs an eighth of a sector an entry
-    const bool scol = ncol <= kPairCols && ncol <= 32 * (int64_t)nrec;
-    if (srec)
-      for (int x = tid; x < nrec; x += kPairThreads) s_rec[x] = rec[r0 + x];
-    if (scol)
+    const bool flat = ncol <= kPairCols && ncol <= 32 * (int64_t)nrec;
+    if (flat) {
+      if (tid < ns) s_c[tid] = (int)(s_rp[tid] - c0);
       for (int x = tid; x < (int)ncol; x += kPairThreads) s_col[x] = ld_stream(o.col + c0 + x);
-    if (tid < ns) {  // longer segments: a CTA each, later
-      const int len = s_off[tid + 1] - s_off[tid];
-      if (len > kSegSmall) {
-        const int c = len <= kSegMid ? 0 : len <= kSegLarge ? 1 : 2;
-        big[(int64_t)c * n + atomicAdd(&big_cnt[c], 1)] = (int32_t)(v0 + tid);
-      }
+    } else {
+      const int64_t row = tid < ns ? s_rp[tid + 1] - s_rp[tid] : 0;
+      const int take = row <= kPairRow && row <= 32 * (int64_t)small ? (int)row : 0;
+      int all;
+      const int at = block_excl_scan<int, kPairThreads>(take, &all);
+      if (tid < ns) s_c[tid] = take > 0 && at + take <= kPairCols ? at : -1;
     }
     __syncthreads();
+    if (!flat)
+      for (int x = tid >> 5; x < ns; x += kPairThreads / 32) {
+        const int at = s_c[x];
+        if (at < 0) continue;
+        const int64_t b = s_rp[x];
+        const int row = (int)(s_rp[x + 1] - b);
+        for (int y = lane_id(); y < row; y += 32) s_col[at + y] = ld_stream(o.col + b + y);
+      }
+    auto source_of = [&](int x) {  // last source whose staged records start at or before x
+      int lo = 0, hi = ns - 1;
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (s_a[mid] <= x) lo = mid; else hi = mid - 1;
+      }
+      return lo;
+    };
     const int g0 = graph_of(o.gid, v0);
     const bool uni = !o.gid || g0 == o.gid[v0 + ns - 1];
     PairSum acc;
-    for (int x = tid; x < nrec; x += kPairThreads) {
-      int lo = 0, hi = ns - 1;  // last source whose segment starts at or before x
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (s_off[mid] - r0 <= x) lo = mid; else hi = mid - 1;
-      }
-      const int a = s_off[lo] - r0, b = s_off[lo + 1] - r0;
-      if (b - a > kSegSmall) continue;
-      const uint64_t me = srec ? s_rec[x] : rec[r0 + x];
-      const uint32_t v = (uint32_t)(me >> 32);
-      int rank = 0;
-      int64_t W = 0;
-      bool isdel = false, head = true;
-      for (int j = a; j < b; j++) {
-        const uint64_t kj = srec ? s_rec[j] : rec[r0 + j];
-        const bool before = kj < me || (kj == me && j < x);
-        rank += before ? 1 : 0;
-        if ((uint32_t)(kj >> 32) == v) {
-          W += (int64_t)(uint32_t)kj;
-          isdel |= (uint32_t)kj == 0;
-          head &= before || j == x;
-        }
-      }
+    auto put = [&](int lo, int64_t p, uint32_t v, int64_t W, bool isdel, bool head) {
       int64_t e;
       bool present;
-      if (scol) {
-        const int q1 = (int)(s_rp[lo + 1] - c0);
-        const int q = lower_bound_col<int>(s_col, (int)(s_rp[lo] - c0), q1, (int32_t)v);
+      const int cs = s_c[lo];
+      const int64_t e0 = s_rp[lo], e1 = s_rp[lo + 1];
+      if (cs >= 0) {
+        const int q1 = cs + (int)(e1 - e0);
+        const int q = lower_bound_col<int>(s_col, cs, q1, (int32_t)v);
         present = q < q1 && s_col[q] == (int32_t)v;
-        e = c0 + q;
+        e = e0 + (q - cs);
       } else {
-        const int64_t e1 = s_rp[lo + 1];
-        e = lower_bound_col<int64_t>(o.col, s_rp[lo], e1, (int32_t)v);
+        e = lower_bound_col<int64_t>(o.col, e0, e1, (int32_t)v);
         present = e < e1 && o.col[e] == (int32_t)v;
       }
       const int32_t u = (int32_t)(v0 + lo);
-      const int32_t d = put_pair(o, (int64_t)r0 + a + rank, u, (int32_t)v, W, W > 0, isdel, head, e, present, acc);
+      const int32_t d = put_pair(o, p, u, (int32_t)v, W, W > 0, isdel, head, e, present, acc);
       if (d) atomicAdd(&s_dk[lo], (unsigned long long)(long long)d);
       if (!uni) pair_sums_add(o, graph_of(o.gid, u), acc);
+    };
+    if (nrec <= kPairRecs) {
+      for (int x = tid; x < nrec; x += kPairThreads) {
+        const int lo = source_of(x);
+        const uint64_t me = rec[s_off[lo] + (x - s_a[lo])];
+        s_src[x] = (uint8_t)lo;
+        s_v[x] = (uint32_t)(me >> 32);
+        s_w[x] = (uint32_t)me;
+      }
+      __syncthreads();
+      for (int x = tid; x < nrec; x += kPairThreads) {
+        const int lo = s_src[x], a = s_a[lo], b = s_a[lo + 1];
+        const uint32_t v = s_v[x];
+        int rank = a;  // equal sinks keep their order
+        for (int j = a; j < x; j++) rank += s_v[j] <= v ? 1 : 0;
+        for (int j = x + 1; j < b; j++) rank += s_v[j] < v ? 1 : 0;
+        s_perm[rank] = (uint16_t)x;
+      }
+      __syncthreads();
+      for (int x = tid; x < nrec; x += kPairThreads) {
+        const int lo = s_src[x], a = s_a[lo], b = s_a[lo + 1];
+        const uint32_t v = s_v[s_perm[x]];
+        const bool head = x + 1 == b || s_v[s_perm[x + 1]] != v;
+        int64_t W = 0;
+        bool isdel = false;
+        if (head)
+          for (int j = x; j >= a; j--) {
+            const int y = s_perm[j];
+            if (s_v[y] != v) break;
+            W += (int64_t)s_w[y];
+            isdel |= s_w[y] == 0;
+          }
+        put(lo, (int64_t)s_off[lo] + (x - a), v, W, isdel, head);
+      }
+    } else {
+      __syncthreads();  // the staged columns
+      for (int x = tid; x < nrec; x += kPairThreads) {
+        const int lo = source_of(x), m = s_a[lo + 1] - s_a[lo], y = x - s_a[lo];
+        const uint64_t* seg = rec + s_off[lo];
+        const uint64_t me = seg[y];
+        const uint32_t v = (uint32_t)(me >> 32);
+        int rank = 0;
+        int64_t W = 0;
+        bool isdel = false, head = true;
+        for (int j = 0; j < m; j++) {
+          const uint64_t kj = seg[j];
+          const bool before = (uint32_t)(kj >> 32) < v || ((uint32_t)(kj >> 32) == v && j < y);
+          rank += before ? 1 : 0;
+          if ((uint32_t)(kj >> 32) == v) {
+            W += (int64_t)(uint32_t)kj;
+            isdel |= (uint32_t)kj == 0;
+            head &= before || j == y;
+          }
+        }
+        put(lo, (int64_t)s_off[lo] + rank, v, head ? W : 0, isdel, head);
+      }
     }
     __syncthreads();
     pair_sums_out<kPairThreads>(o, g0, acc);
   }
-  if (tid < ns) k_new[v0 + tid] = k_old[v0 + tid] + (int64_t)s_dk[tid];
+  if (tid < ns) k_new[v0 + tid] = kv + (int64_t)s_dk[tid];
 }
 
 // One pair of a long segment whose sorted neighbourhood the caller knows; the
@@ -303,47 +377,11 @@ __device__ __forceinline__ void segment_out(const PairView& o, int32_t u, const 
   pair_sums_out<NT>(o, graph_of(o.gid, u), acc);
 }
 
-// Segments of kSegSmall + 1 .. kSegMid records: a CTA each, ranked in shared
-// memory (every thread reads the same word at the same time).
-constexpr int kMidThreads = 128;
-__global__ void __launch_bounds__(kMidThreads) pair_mid(PairView o, const uint64_t* __restrict__ rec,
-                                                        const int32_t* __restrict__ list,
-                                                        const int32_t* __restrict__ cnt, int64_t* __restrict__ k_new) {
-  __shared__ uint64_t s[kSegMid];
-  const int nl = *cnt, tid = threadIdx.x;
-  for (int i = blockIdx.x; i < nl; i += gridDim.x) {
-    const int32_t u = list[i];
-    const int32_t a = o.off[u];
-    const int len = o.off[u + 1] - a;
-    for (int x = tid; x < len; x += kMidThreads) s[x] = rec[a + x];
-    __syncthreads();
-    PairSum acc;
-    for (int x = tid; x < len; x += kMidThreads) {
-      const uint64_t me = s[x];
-      const uint32_t v = (uint32_t)(me >> 32);
-      int rank = 0;
-      int64_t W = 0;
-      bool isdel = false, head = true;
-      for (int j = 0; j < len; j++) {
-        const uint64_t kj = s[j];
-        const bool before = kj < me || (kj == me && j < x);
-        rank += before ? 1 : 0;
-        if ((uint32_t)(kj >> 32) == v) {
-          W += (int64_t)(uint32_t)kj;
-          isdel |= (uint32_t)kj == 0;
-          head &= before || j == x;
-        }
-      }
-      put_searched(o, (int64_t)a + rank, u, v, W, isdel, head, acc);
-    }
-    segment_out<kMidThreads>(o, u, acc, k_new);
-  }
-}
-
-// The pairs of a sorted segment s[0 .. len) of source u at place a.
+// The pairs of a sorted segment s[0 .. len) of source u at place a; s_col: the
+// row of u in shared memory (may be NULL).
 template <typename P>
 __device__ __forceinline__ void put_sorted(const PairView& o, int32_t u, int64_t a, int len, const P* s, int tid,
-                                           int NT, PairSum& acc) {
+                                           int NT, PairSum& acc, const int32_t* s_col = nullptr) {
   for (int x = tid; x < len; x += NT) {
     const uint32_t v = (uint32_t)(s[x] >> 32);
     const bool head = x + 1 == len || (uint32_t)(s[x + 1] >> 32) != v;
@@ -354,7 +392,62 @@ __device__ __forceinline__ void put_sorted(const PairView& o, int32_t u, int64_t
         W += (int64_t)(uint32_t)s[j];
         isdel |= (uint32_t)s[j] == 0;
       }
-    put_searched(o, a + x, u, v, W, isdel, head, acc);
+    if (s_col) {
+      const int n = (int)(o.rp[u + 1] - o.rp[u]);
+      const int q = lower_bound_col<int>(s_col, 0, n, (int32_t)v);
+      put_pair(o, a + x, u, (int32_t)v, W, W > 0, isdel, head, o.rp[u] + q, q < n && s_col[q] == (int32_t)v, acc);
+    } else {
+      put_searched(o, a + x, u, v, W, isdel, head, acc);
+    }
+  }
+}
+
+// In place, P a power of two, by every thread of the CTA.
+template <int NT>
+__device__ __forceinline__ void bitonic_sort(uint64_t* s, int P) {
+  for (int k = 2; k <= P; k <<= 1)
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      for (int q = threadIdx.x; q < P / 2; q += NT) {
+        const int x = ((q & ~(j - 1)) << 1) | (q & (j - 1)), y = x | j;  // the q-th pair at distance j
+        const uint64_t kx = s[x], ky = s[y];
+        if ((kx > ky) == ((x & k) == 0)) {
+          s[x] = ky;
+          s[y] = kx;
+        }
+      }
+      __syncthreads();
+    }
+}
+
+// Segments of kSegSmall + 1 .. kSegMid records: a CTA each, sorted in shared
+// memory by a bitonic network (a rank by comparing all pairs takes len^2 / 128
+// steps a thread: 373 us for this kernel in a batch of 12.4 M records, with the
+// rows searched in global memory and the results written out of order; 126
+// so).  The row is staged when it fits: it is at least as long as most segments.
+constexpr int kMidThreads = 128;
+constexpr int kMidCols = 3072;
+__global__ void __launch_bounds__(kMidThreads) pair_mid(PairView o, const uint64_t* __restrict__ rec,
+                                                        const int32_t* __restrict__ list,
+                                                        const int32_t* __restrict__ cnt, int64_t* __restrict__ k_new) {
+  __shared__ uint64_t s[kSegMid];
+  __shared__ int32_t s_col[kMidCols];
+  const int nl = *cnt, tid = threadIdx.x;
+  for (int i = blockIdx.x; i < nl; i += gridDim.x) {
+    const int32_t u = list[i];
+    const int32_t a = o.off[u];
+    const int len = o.off[u + 1] - a;
+    const int64_t c0 = o.rp[u], ncol = o.rp[u + 1] - c0;
+    int P = 1;
+    while (P < len) P <<= 1;
+    const bool scol = ncol <= kMidCols && ncol <= 32 * (int64_t)len;  // as in pair_tile
+    if (scol)
+      for (int x = tid; x < (int)ncol; x += kMidThreads) s_col[x] = ld_stream(o.col + c0 + x);
+    for (int x = tid; x < P; x += kMidThreads) s[x] = x < len ? rec[a + x] : ~0ull;
+    __syncthreads();
+    bitonic_sort<kMidThreads>(s, P);
+    PairSum acc;
+    put_sorted(o, u, a, len, s, tid, kMidThreads, acc, scol ? s_col : nullptr);
+    segment_out<kMidThreads>(o, u, acc, k_new);
   }
 }
 
@@ -375,18 +468,7 @@ __global__ void __launch_bounds__(kLargeThreads) pair_large(PairView o, const ui
     while (P < len) P <<= 1;
     for (int x = tid; x < P; x += kLargeThreads) s[x] = x < len ? rec[a + x] : ~0ull;
     __syncthreads();
-    for (int k = 2; k <= P; k <<= 1)
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int q = tid; q < P / 2; q += kLargeThreads) {
-          const int x = ((q & ~(j - 1)) << 1) | (q & (j - 1)), y = x | j;  // the q-th pair at distance j
-          const uint64_t kx = s[x], ky = s[y];
-          if ((kx > ky) == ((x & k) == 0)) {
-            s[x] = ky;
-            s[y] = kx;
-          }
-        }
-        __syncthreads();
-      }
+    bitonic_sort<kLargeThreads>(s, P);
     PairSum acc;
     put_sorted(o, u, a, len, s, tid, kLargeThreads, acc);
     segment_out<kLargeThreads>(o, u, acc, k_new);
@@ -736,7 +818,10 @@ int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut*
   PairView o{off, rp_o, col_o, w_o, from_prev ? labels0 : nullptr, gid, out->pkey.get(), out->pw.get(),
              out->pflag.get(), out->pdelta.get(), epos.get(), S.get(), c->gs.get(), &d->npairs, &d->err};
   if (R > 0) {
-    ::dcd::count_launch(), pair_tile<<<(unsigned)cdiv(n, kPairSrc), kPairThreads, 0, s>>>(
+    // sources a CTA: about 64 records for its 128 threads (pair_tile)
+    const int ns = R >= 2 * n || n < kPairWide ? 32 : 2 * R >= n ? 64 : 128;
+    auto* tile = ns == 32 ? pair_tile<32> : ns == 64 ? pair_tile<64> : pair_tile<128>;
+    ::dcd::count_launch(), tile<<<(unsigned)cdiv(n, ns), kPairThreads, 0, s>>>(
         o, n, rec.get(), c->kdeg[cur].get(), out->k->get(), big.get(), big_cnt);
     // a segment holds at most one record per batch record: the classes the
     // batch is too small for are not launched

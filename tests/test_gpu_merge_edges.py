@@ -112,3 +112,33 @@ def test_bad_device_record_leaves_the_graph():
         assert e.value.code == dcd.DCD_EINVAL
         for x, y in zip(before, ctx.graph()):
             assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("records", [400, 60_000, 200_000])
+def test_sources_per_tile(records):
+    """A large graph with batches of few, about one, and several records a
+    source: tiles of 128, 64 and 32 sources, some of them with more records than a
+    tile stages (runs of sources with 60 each) or with rows too long to stage."""
+    from paper_1904_08553_gb300 import dcd
+
+    n = 90_000
+    rng = np.random.default_rng(records)
+    edges = {}
+    with dcd.Context(n, mode=dcd.MODE_BASE) as ctx:
+        for t in range(3):
+            u, v = rng.integers(0, n, records), rng.integers(0, n, records)
+            if t == 0:  # long rows
+                u[: records // 4] = rng.integers(0, 3, records // 4) * 40
+            if t == 1:  # crowded tiles
+                m = min(records // 2, 130 * 58)
+                u[:m] = 5000 + np.arange(m) // 58
+                v[:m] = rng.integers(0, 4, m) + 60_000 + 9 * (np.arange(m) // 58)
+            ok = u != v
+            ins = np.stack([u, v, rng.integers(1, 9, records)], 1)[ok]
+            dels = np.zeros((0, 2), np.int64)
+            if t:
+                dels = np.array(list(edges))[rng.integers(0, len(edges), records // 3)]
+            ctx.apply_batch(ins.astype(np.int32), dels.astype(np.int32))
+            ctx.update(labels_out=None)
+            model_step(edges, ins, dels)
+            check(ctx, edges, n)
