@@ -643,12 +643,17 @@ __global__ void __launch_bounds__(256) hub_clear(HubTables t) {
 // ---------------------------------------------------------------- apply + N
 
 // Moves of one pass (proposals of graphs whose pass loop has stopped are
-// dropped).  Community sums change by warp-aggregated atomics (one per distinct
-// community of the warp); per-graph mover counts feed the stop rule.  LL[v] =
+// dropped).  Community sums change by way of a table in shared memory, added to
+// global memory once per CTA: with few communities, the atomics of every warp
+// meet in the same few words otherwise (R-MAT 22, 2 M active vertices and 700
+// communities with entries: 320 us a pass with one atomic per warp and
+// community, 35 so).  A warp whose labels find no place in the table (from
+// singletons there are as many communities as vertices) goes on with one atomic
+// per warp and community.  Per-graph mover counts feed the stop rule.  LL[v] =
 // (label before, label after) is written for every active vertex, so that the
 // row pass below needs one gather per neighbour; the movers' rows become work
 // items of at most kMoveChunk entries (v << 32 | chunk), so that a moved hub
-// does not hold one warp for its whole row.
+// does not hold one warp for its whole row, reserved once per CTA and step.
 constexpr int kMoveChunk = 128;
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -657,20 +662,64 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-__global__ void lm_apply(const int32_t* __restrict__ list, int64_t cnt, const int32_t* __restrict__ prop,
-                         int32_t* __restrict__ L, int2* __restrict__ LL, const int64_t* __restrict__ k,
-                         const int64_t* __restrict__ rp, unsigned long long* __restrict__ a,
-                         int32_t* __restrict__ size, int64_t* __restrict__ items, int32_t* __restrict__ item_cnt,
-                         DevScalars* __restrict__ d, const int32_t* __restrict__ gid,
-                         GraphState* __restrict__ gs) {
+constexpr int kApplyThreads = 512;
+constexpr int kApplySlots = 1024;
+constexpr int kApplyProbes = 4;
+
+// x more degree and one more (dir = 1) or less (-1) vertex for community c; false:
+// no place in the table.  VT = 32 bits: 2m < 2^31 bounds the CTA's net change.
+template <typename VT>
+__device__ __forceinline__ bool apply_add(int32_t* tk, VT* tv, int32_t* tc, int32_t c, int64_t x, int dir) {
+  uint32_t sl = hash_label(c, kApplySlots - 1);
+  for (int probe = 0; probe < kApplyProbes; probe++) {
+    int32_t key = tk[sl];
+    if (key == -1) {
+      key = atomicCAS(&tk[sl], -1, c);
+      if (key == -1) key = c;
+    }
+    if (key == c) {
+      atomicAdd(&tv[sl], (VT)(dir > 0 ? x : -x));
+      atomicAdd(&tc[sl], dir);
+      return true;
+    }
+    sl = (sl + 1) & (kApplySlots - 1);
+  }
+  return false;
+}
+
+template <typename VT>
+__global__ void __launch_bounds__(kApplyThreads) lm_apply(
+    const int32_t* __restrict__ list, int64_t cnt, const int32_t* __restrict__ prop, int32_t* __restrict__ L,
+    int2* __restrict__ LL, const int64_t* __restrict__ k, const int64_t* __restrict__ rp,
+    unsigned long long* __restrict__ a, int32_t* __restrict__ size, int64_t* __restrict__ items,
+    int32_t* __restrict__ item_cnt, DevScalars* __restrict__ d, const int32_t* __restrict__ gid,
+    GraphState* __restrict__ gs) {
+  using SV = typename std::conditional<sizeof(VT) == 4, int32_t, long long>::type;
+  __shared__ int32_t tk[kApplySlots], tc[kApplySlots];
+  __shared__ VT tv[kApplySlots];
+  __shared__ int32_t s_at;
+  __shared__ unsigned long long s_deg;
+  __shared__ int s_moves;
   if (blockIdx.x == 0 && threadIdx.x == 0) d->stamp[1] = global_ns();  // the evaluation is over
+  for (int x = threadIdx.x; x < kApplySlots; x += kApplyThreads) {
+    tk[x] = -1;
+    tc[x] = 0;
+    tv[x] = 0;
+  }
+  if (threadIdx.x == 0) {
+    s_deg = 0;
+    s_moves = 0;
+  }
+  __syncthreads();
   unsigned long long deg = 0;  // degrees of the movers
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  int moved = 0;               // movers (one graph)
+  bool table = true;           // uniform over the warp
+  const int64_t stride = (int64_t)gridDim.x * kApplyThreads;
   const int lane = lane_id();
-  for (int64_t base = (blockIdx.x * (int64_t)blockDim.x) + (threadIdx.x & ~31); base < cnt; base += stride) {
-    const int64_t i = base + lane;
+  for (int64_t base0 = blockIdx.x * (int64_t)kApplyThreads; base0 < cnt; base0 += stride) {
+    const int64_t i = base0 + threadIdx.x;
     bool mv = false;
-    int32_t v = 0, c = -1, p = -1, gv = -1;
+    int32_t v = 0, c = -1, p = -1, gv = 0;
     int64_t kv = 0;
     int nch = 0;
     if (i < cnt) {
@@ -686,40 +735,66 @@ __global__ void lm_apply(const int32_t* __restrict__ list, int64_t cnt, const in
         const int64_t dv = rp[v + 1] - rp[v];
         deg += (unsigned long long)dv;
         nch = (int)((dv + kMoveChunk - 1) / kMoveChunk);
-      } else {
-        c = p = -1;
+        moved++;
       }
     }
-    if (!__any_sync(0xffffffffu, mv)) continue;
-    {  // leaving c
-      const unsigned peers = __match_any_sync(0xffffffffu, c);
-      const int64_t sk = group_sum_exact(peers, kv);
-      if (mv && (int)(__ffs(peers) - 1) == lane) {
-        atomicAdd(&a[c], 0ull - (unsigned long long)sk);
-        atomicSub(&size[c], __popc(peers));
+    if (__any_sync(0xffffffffu, mv)) {
+      bool out = mv, in = mv;  // still to be added
+      if (table) {
+        if (mv) {
+          out = !apply_add(tk, tv, tc, c, kv, -1);
+          in = !apply_add(tk, tv, tc, p, kv, 1);
+        }
+        table = __popc(__ballot_sync(0xffffffffu, out || in)) < 16;
+      }
+      if (__any_sync(0xffffffffu, out)) {  // leaving c
+        const unsigned peers = __match_any_sync(0xffffffffu, out ? c : -1);
+        const int64_t sk = group_sum_exact(peers, out ? kv : 0);
+        if (out && (int)(__ffs(peers) - 1) == lane) {
+          atomicAdd(&a[c], 0ull - (unsigned long long)sk);
+          atomicSub(&size[c], __popc(peers));
+        }
+      }
+      if (__any_sync(0xffffffffu, in)) {  // joining p
+        const unsigned peers = __match_any_sync(0xffffffffu, in ? p : -1);
+        const int64_t sk = group_sum_exact(peers, in ? kv : 0);
+        if (in && (int)(__ffs(peers) - 1) == lane) {
+          atomicAdd(&a[p], (unsigned long long)sk);
+          atomicAdd(&size[p], __popc(peers));
+        }
+      }
+      if (gid) {  // movers per graph
+        const unsigned peers = __match_any_sync(0xffffffffu, mv ? gv : -1);
+        if (mv && (int)(__ffs(peers) - 1) == lane) atomicAdd(&gs[gv].moves, __popc(peers));
       }
     }
-    {  // joining p
-      const unsigned peers = __match_any_sync(0xffffffffu, p);
-      const int64_t sk = group_sum_exact(peers, kv);
-      if (mv && (int)(__ffs(peers) - 1) == lane) {
-        atomicAdd(&a[p], (unsigned long long)sk);
-        atomicAdd(&size[p], __popc(peers));
-      }
+    int total;
+    const int excl = block_excl_scan<int, kApplyThreads>(nch, &total);
+    if (total > 0) {  // uniform over the CTA
+      if (threadIdx.x == 0) s_at = atomicAdd(item_cnt, total);
+      __syncthreads();
+      const int32_t at = s_at + excl;
+      for (int x = 0; x < nch; x++) items[at + x] = (int64_t)v << 32 | (uint32_t)x;
+      __syncthreads();
     }
-    {  // movers per graph
-      const unsigned peers = __match_any_sync(0xffffffffu, mv ? gv : -1);
-      if (mv && (int)(__ffs(peers) - 1) == lane) atomicAdd(&gs[gv].moves, __popc(peers));
-    }
-    const int incl = warp_incl_scan(nch);
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    int32_t at = 0;
-    if (lane == 0) at = atomicAdd(item_cnt, total);
-    at = __shfl_sync(0xffffffffu, at, 0) + incl - nch;
-    for (int j = 0; j < nch; j++) items[at + j] = (int64_t)v << 32 | (uint32_t)j;
   }
   deg = warp_sum(deg);
-  if (lane == 0 && deg) atomicAdd((unsigned long long*)&d->moved_deg, deg);
+  moved = (int)__reduce_add_sync(0xffffffffu, (unsigned)moved);
+  if (lane == 0 && deg) atomicAdd(&s_deg, deg);
+  if (lane == 0 && moved) atomicAdd(&s_moves, moved);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_moves) {
+    if (s_deg) atomicAdd((unsigned long long*)&d->moved_deg, s_deg);
+    if (!gid) atomicAdd(&gs[0].moves, s_moves);
+  }
+  if (s_moves == 0) return;
+  for (int x = threadIdx.x; x < kApplySlots; x += kApplyThreads) {
+    const int32_t c = tk[x];
+    if (c < 0) continue;
+    const SV y = (SV)tv[x];
+    if (y) atomicAdd(&a[c], (unsigned long long)(long long)y);
+    if (tc[x]) atomicAdd(&size[c], tc[x]);
+  }
 }
 
 // Entry labels (nlab_gather below) are kept from this many entries on: below,
@@ -1531,6 +1606,7 @@ __global__ void final_labels(int64_t n0, int64_t nv, const int32_t* __restrict__
                              const int32_t* __restrict__ minid, int32_t* __restrict__ out,
                              const int32_t* __restrict__ gid, GraphState* __restrict__ gs) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  unsigned long long heads = 0;  // one graph: counted once per warp at the end
   for (int64_t base = (blockIdx.x * (int64_t)blockDim.x) + (threadIdx.x & ~31); base < n0; base += stride) {
     const int64_t v = base + lane_id();
     int g = -1;
@@ -1541,10 +1617,15 @@ __global__ void final_labels(int64_t n0, int64_t nv, const int32_t* __restrict__
       g = graph_of(gid, v);
       out[v] = x;
     }
+    if (!gid) {
+      heads += __popc(__ballot_sync(0xffffffffu, head));
+      continue;
+    }
     const unsigned peers = __match_any_sync(0xffffffffu, head ? g : -1);
     if (head && (int)(__ffs(peers) - 1) == (int)lane_id())
       atomicAdd((unsigned long long*)&gs[g].ncomm, (unsigned long long)__popc(peers));
   }
+  if (heads && lane_id() == 0) atomicAdd((unsigned long long*)&gs[0].ncomm, heads);
 }
 
 // ---------------------------------------------------------------- host side
@@ -1911,7 +1992,8 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
     ::dcd::count_launch(), pass_begin<<<cdiv(G, 256), 256, 0, s>>>(gs, G, d, item_cnt.get());
     if (any) DCD_TRY(launch_lm_nocfg<W>(c, lvl, bins, prop.get(), nullptr, 0, total >= kForkMin, sweep));
     if (total) {
-      ::dcd::count_launch(), lm_apply<<<grid_for(total, T), T, 0, s>>>(
+      auto* apply = lvl.m2 < ((int64_t)1 << 31) ? lm_apply<unsigned> : lm_apply<unsigned long long>;
+      ::dcd::count_launch(), apply<<<grid_for(total, kApplyThreads, 4), kApplyThreads, 0, s>>>(
           lst, total, prop.get(), L, LL.get(), kbuf.get(), g.rp, (unsigned long long*)a.get(), size.get(), items.get(),
           item_cnt.get(), d, gid, gs);
       ::dcd::count_launch(), lm_delta<W><<<wave_grid(lm_delta<W>, item_cap * 32, T), T, 0, s>>>(
@@ -2215,33 +2297,34 @@ __global__ void n1_pairs(const uint64_t* __restrict__ pkey, const int32_t* __res
 // does not hold one warp for its whole row.
 constexpr int kN1Chunk = 256;
 
-__global__ void n1_movers_list(int64_t n, const int32_t* __restrict__ L0, const int32_t* __restrict__ cprev,
-                               const int64_t* __restrict__ rp, int64_t* __restrict__ items,
-                               int32_t* __restrict__ cnt, unsigned long long* __restrict__ entries) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int lane = lane_id();
-  for (int64_t b0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31u); b0 < n; b0 += stride) {
-    const int64_t v = b0 + lane;
+constexpr int kN1Threads = 512;
+__global__ void __launch_bounds__(kN1Threads) n1_movers_list(int64_t n, const int32_t* __restrict__ L0,
+                                                             const int32_t* __restrict__ cprev,
+                                                             const int64_t* __restrict__ rp,
+                                                             int64_t* __restrict__ items, int32_t* __restrict__ cnt,
+                                                             unsigned long long* __restrict__ entries) {
+  __shared__ int32_t s_at;
+  const int64_t stride = (int64_t)gridDim.x * kN1Threads;
+  unsigned long long sum = 0;
+  for (int64_t b0 = blockIdx.x * (int64_t)kN1Threads; b0 < n; b0 += stride) {
+    const int64_t v = b0 + threadIdx.x;
     const bool mv = v < n && L0[v] != cprev[v];
-    if (!__any_sync(0xffffffffu, mv)) continue;
     const int64_t d = mv ? rp[v + 1] - rp[v] : 0;
+    sum += (unsigned long long)d;
     const int nch = (int)((d + kN1Chunk - 1) / kN1Chunk);
-    int incl = nch;  // inclusive prefix of the chunk counts over the warp
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    const unsigned long long dsum = peer_sum(0xffffffffu, (long long)d, 0ull);
-    int32_t base = 0;
-    if (lane == 0 && total > 0) {
-      base = atomicAdd(cnt, total);
-      atomicAdd(entries, dsum);
-    }
-    base = __shfl_sync(0xffffffffu, base, 0);
-    for (int j = 0; j < nch; j++) items[base + incl - nch + j] = (int64_t)v << 32 | (uint32_t)j;
+    if (!__syncthreads_or(nch)) continue;
+    int total;
+    const int excl = block_excl_scan<int, kN1Threads>(nch, &total);
+    // one reservation per CTA and step (one per warp: 107 us for 2 M vertices,
+    // all on this one word)
+    if (threadIdx.x == 0) s_at = atomicAdd(cnt, total);
+    __syncthreads();
+    const int32_t at = s_at + excl;
+    for (int j = 0; j < nch; j++) items[at + j] = (int64_t)v << 32 | (uint32_t)j;
+    __syncthreads();
   }
+  sum = warp_sum(sum);
+  if (lane_id() == 0 && sum) atomicAdd(entries, sum);
 }
 
 // A warp per item (a chunk of a moved vertex v's row): entry (v, u, w)
@@ -2382,7 +2465,7 @@ int n1_build(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L0, const int32_t
   if (c->n1.P > 0)
     ::dcd::count_launch(), n1_pairs<VT><<<grid_for(c->n1.P, T), T, 0, s>>>(
         c->n1.pkey, c->n1.pdelta, c->n1.P, c->n1.cprev, kidx, nk, D.get(), bad);
-  ::dcd::count_launch(), n1_movers_list<<<grid_for(g.n, T), T, 0, s>>>(g.n, L0, c->n1.cprev, g.rp, items.get(),
+  ::dcd::count_launch(), n1_movers_list<<<grid_for(g.n, kN1Threads, 4), kN1Threads, 0, s>>>(g.n, L0, c->n1.cprev, g.rp, items.get(),
                                                                         cnt, entries);
   ::dcd::count_launch(), n1_movers<VT><<<wave_grid(n1_movers<VT>, g.n * 32, T), T, 0, s>>>(
       items.get(), cnt, g.rp, g.col, g.w, L0, c->n1.cprev, kidx, nk, D.get(), bad);
