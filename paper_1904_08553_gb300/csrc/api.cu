@@ -551,7 +551,13 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
   DCD_TRY_CUDA(cudaMemcpyAsync(L0.get(), src_labels, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
 
   MergeOut mo;
-  DCD_TRY(merge_batch(c, src_labels, mode == DCD_MODE_STATIC, &mo));
+  // the entry labels are made by the merge when level 0 will evaluate every
+  // vertex, or when the last update needed them
+  EntryLabels nlab;
+  const bool all_active = c->cfg.alg == DCD_ALG_LOUVAIN && (mode == DCD_MODE_STATIC || mode == DCD_MODE_BASE);
+  const bool merge_labels = c->nnz + 2 * c->n_ins >= kNlabMin && (all_active || c->nlab_used);
+  c->nlab_used = false;
+  DCD_TRY(merge_batch(c, src_labels, mode == DCD_MODE_STATIC, &mo, merge_labels ? &nlab : nullptr));
   const int nxt = 1 - c->cur;
   const bool learned = mode == DCD_MODE_LEARNED;
   const bool collect = c->collect && !first;
@@ -585,7 +591,6 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
   Buf<int64_t> a;
   Buf<int32_t> size;
   LearnedPool lp;
-  EntryLabels nlab;
   // the first level-0 pass of a Delta-screening update reads the state the
   // screening reads (C_{t-1}, its sums on G_t): the screening hands over its
   // proposals for the sources whose rows it sums (one Louvain graph)

@@ -797,10 +797,6 @@ __global__ void __launch_bounds__(kApplyThreads) lm_apply(
   }
 }
 
-// Entry labels (nlab_gather below) are kept from this many entries on: below,
-// a pass over the graph stays in L2 and takes about as long as the gather's own
-// launches.
-constexpr int64_t kNlabMin = (int64_t)1 << 21;
 // The search of a mirror entry (two row bounds, 5-7 probes, one store) costs
 // about as many sectors as this many entries gathered.
 constexpr int kNlabSearch = 8;
@@ -1969,8 +1965,9 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
   if (nlab && nlab->ready) lv.nlab = nlab->buf.get();
   if constexpr (std::is_same<W, int32_t>::value) {
     // labels in entry order: worth one gather when a pass evaluates a fair part of the entries
-    if (nlab && !nlab->ready && g.nnz >= kNlabMin && 4 * bins.act_deg >= g.nnz) {
-      DCD_TRY(entry_labels_impl(c, g, L, nlab));
+    if (nlab && g.nnz >= kNlabMin && 4 * bins.act_deg >= g.nnz) {
+      c->nlab_used = true;
+      if (!nlab->ready) DCD_TRY(entry_labels_impl(c, g, L, nlab));
       lv.nlab = nlab->buf.get();
     }
   }
@@ -2881,8 +2878,9 @@ unsigned hub_grid(dcd_ctx* c, const HubBufs& b) {
 }
 
 int entry_labels(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L, int64_t entries, EntryLabels* out) {
-  if (out->ready || g.nnz < kNlabMin || 4 * entries < g.nnz) return DCD_OK;
-  return entry_labels_impl(c, g, L, out);
+  if (g.nnz < kNlabMin || 4 * entries < g.nnz) return DCD_OK;
+  c->nlab_used = true;
+  return out->ready ? DCD_OK : entry_labels_impl(c, g, L, out);
 }
 
 int pool_stats(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L, const int64_t* k, const int64_t* a,

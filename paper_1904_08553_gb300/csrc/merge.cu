@@ -636,11 +636,20 @@ __global__ void merge_split(const int64_t* __restrict__ epos, const int32_t* __r
 // 233 us (5.5 TB/s), 73 M entries and 12.4 M pairs 375 us.  With the per-entry
 // searches (row of an entry, its place among the pairs) and row sums that ran
 // here before, it was issue-bound: 1059 and 1534 us.
+//
+// NL: also the entry labels (label of every entry's column under lab; NULL: the
+// column itself) of the new graph, for an update that will need them.  80 M
+// entries and 84 K pairs: 480 us, where the copy alone takes 233 and the gather
+// alone 316; both count against the rate of L2 sectors (one a gathered label,
+// 5/8 of one for the streams of an entry), so what is saved is the second read of
+// the columns and a launch.
+template <bool NL>
 __global__ void __launch_bounds__(kMergeThreads) merge_tile(
     int64_t nnz, const int32_t* __restrict__ col_o, const int32_t* __restrict__ w_o,
     const int32_t* __restrict__ sq, const int64_t* __restrict__ epos, const uint64_t* __restrict__ pkey,
     const int32_t* __restrict__ pdelta, const uint8_t* __restrict__ pflag, const int32_t* __restrict__ S,
-    int32_t* __restrict__ col_n, int32_t* __restrict__ w_n) {
+    int32_t* __restrict__ col_n, int32_t* __restrict__ w_n, const int32_t* __restrict__ lab,
+    int32_t* __restrict__ nlab) {
   __shared__ int32_t s_sh[kMergeTile + kMergeThreads];  // shift marks, then shifts (padded: one word a thread's run)
   __shared__ int32_t s_adj[kMergeTile];                 // weight change of an entry; INT32_MIN: removed
   auto at = [](int i) { return i + i / kMergeItems; };
@@ -661,6 +670,12 @@ __global__ void __launch_bounds__(kMergeThreads) merge_tile(
       w[x] = ld_stream(w_o + e0 + j);
     }
   }
+  int32_t l[kMergeItems];
+  if constexpr (NL) {
+#pragma unroll
+    for (int x = 0; x < kMergeItems; x++)
+      if (x * kMergeThreads + tid < ne) l[x] = lab ? lab[c[x]] : c[x];
+  }
   // the last pair before the tile may stand for the tile's first entry
   const bool lead = q0 > 0 && ne > 0 && epos[q0 - 1] == e0 && (pflag[q0 - 1] & kPairPresent);
   if (np == 0 && !lead) {
@@ -670,6 +685,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_tile(
       if (j < ne) {
         st_stream(col_n + e0 + shift0 + j, c[x]);
         st_stream(w_n + e0 + shift0 + j, w[x]);
+        if constexpr (NL) st_stream(nlab + e0 + shift0 + j, l[x]);
       }
     }
     return;
@@ -689,8 +705,10 @@ __global__ void __launch_bounds__(kMergeThreads) merge_tile(
       const int32_t d = pdelta[q];
       if (f & kPairAdded) {
         const int64_t pos = ep + S[q];
-        st_stream(col_n + pos, (int32_t)(pkey[q] & 0xffffffffu));
+        const int32_t v = (int32_t)(pkey[q] & 0xffffffffu);
+        st_stream(col_n + pos, v);
         st_stream(w_n + pos, d);
+        if constexpr (NL) st_stream(nlab + pos, lab ? lab[v] : v);
         if (rel < ne) atomicAdd(&s_sh[at(rel)], 1);
       } else if (rel < ne) {
         if (f & kPairRemoved) {
@@ -725,6 +743,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_tile(
         const int64_t pos = e0 + j + s_sh[at(j)];
         st_stream(col_n + pos, c[x]);
         st_stream(w_n + pos, w[x] + d);
+        if constexpr (NL) st_stream(nlab + pos, l[x]);
       }
     }
   }
@@ -747,7 +766,7 @@ int validate_batch(dcd_ctx* c, const dcd_edge* ins, int64_t n_ins, const dcd_edg
   return DCD_OK;
 }
 
-int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut* out) {
+int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut* out, EntryLabels* nlab) {
   cudaStream_t s = c->stream;
   const int64_t n = c->n;
   const int64_t n_ins = c->n_ins, n_del = c->n_del, nr = n_ins + n_del;
@@ -857,10 +876,12 @@ int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut*
     DCD_TRY(split.alloc(&c->mem, nt + 1));
     ::dcd::count_launch(), merge_split<<<grid_for(nt + 1, T), T, 0, s>>>(epos.get(), off + n, nt, split.get());
     DCD_LAUNCH_CHECK();
-    ::dcd::count_launch(), merge_tile<<<(unsigned)nt, kMergeThreads, 0, s>>>(
+    if (nlab) DCD_TRY(nlab->buf.alloc(&c->mem, cap));
+    ::dcd::count_launch(), (nlab ? merge_tile<true> : merge_tile<false>)<<<(unsigned)nt, kMergeThreads, 0, s>>>(
         c->nnz, col_o, w_o, split.get(), epos.get(), out->pkey.get(), out->pdelta.get(), out->pflag.get(), S.get(),
-        c->col[nxt].get(), c->w[nxt].get());
+        c->col[nxt].get(), c->w[nxt].get(), static_start ? nullptr : labels0, nlab ? nlab->buf.get() : nullptr);
     DCD_LAUNCH_CHECK();
+    if (nlab) nlab->ready = true;
   }
   if (!static_start && !c->in_valid && c->cfg.alg == DCD_ALG_LOUVAIN) {
     ::dcd::count_launch(), in_weight<<<grid_for(n * 32, T), T, 0, s>>>(n, rp_n, c->col[nxt].get(), c->w[nxt].get(),

@@ -221,6 +221,10 @@ struct dcd_ctx {
   bool k_valid = false;
   dcd::Buf<int64_t> kdeg[2];
   bool in_valid = false;
+  // the last update's level 0 or screening read enough rows to gather the entry
+  // labels: the next merge makes them on the way (a guess: a wrong one costs the
+  // labels' writes, or a gather of their own)
+  bool nlab_used = false;
   dcd::Buf<int64_t> in_prev, in_next;
   // Per-step delta coarsening of level 0 (dense coarse graphs only): K is
   // the coarse graph of G_t under C_t (the last committed labels) as a dense
@@ -338,6 +342,10 @@ struct SideBySide {
 using UpdateFinish = int (*)(dcd_ctx* c, void* user);
 int update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, UpdateFinish finish, void* user);
 
+// Entry labels are kept from this many entries on: below, a pass over the graph
+// stays in L2 and takes about as long as the gather's own launches.
+constexpr int64_t kNlabMin = (int64_t)1 << 21;
+
 // The label of every entry's column (level 0), from one gather per update;
 // ready: it holds the labels the update starts from.
 struct EntryLabels {
@@ -359,7 +367,8 @@ struct MergeOut {
   Buf<int32_t> pdelta;     // per pair: its weight in G_t minus its weight in G_{t-1}
   int64_t npairs = 0;      // pairs, null ones among them
 };
-int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut* out);
+// nlab (may be NULL): the entry labels of G_t under the start labels, made on the way.
+int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut* out, EntryLabels* nlab);
 
 // The batch's sources (vertices with pairs) by degree in G_t.
 struct SourceBins {
