@@ -19,6 +19,15 @@ __device__ __forceinline__ ST gain(int64_t m2, int64_t kv, int64_t eD, int64_t e
   return (ST)m2 * (ST)(eD - eC) - (ST)kv * (ST)(aD - aC + kv);
 }
 
+// No community can gain S > 0 for v: of S, e_{v->D} is at most k_v - e_{v->C\v}
+// and a_D at least 0, so S <= m2 (k_v - 2 e_{v->C\v}) + k_v (a_C - k_v).  Exact (64
+// bits hold both products and, each below 2^62, their sum), and known before the
+// row is summed by community: true for most vertices once the labels settle.
+template <typename ST>
+__device__ __forceinline__ bool stays(int64_t m2, int64_t kv, int64_t eC, int64_t aC) {
+  return (ST)m2 * (ST)(kv - 2 * eC) + (ST)kv * (ST)(aC - kv) <= 0;
+}
+
 template <typename ST>
 __device__ __forceinline__ ST gain_lowest();
 template <>

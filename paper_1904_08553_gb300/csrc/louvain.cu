@@ -147,7 +147,7 @@ __device__ __forceinline__ void put_best(const LV<W>& g, int64_t i, int64_t eC, 
 }
 
 template <typename W, typename ST, int S, int Q, int CAP>
-__global__ void __launch_bounds__(256) lm_vert(LV<W> g, const int32_t* __restrict__ list, int64_t cnt, int per,
+__global__ void __launch_bounds__(256, 5) lm_vert(LV<W> g, const int32_t* __restrict__ list, int64_t cnt, int per,
                                                int32_t* __restrict__ prop) {
   static_assert(S == 4 || S == 8, "segments of 4 or 8 lanes");
   using VT = typename TblVal<ST>::type;
@@ -256,19 +256,20 @@ __global__ void __launch_bounds__(256) lm_vert(LV<W> g, const int32_t* __restric
     }
     __syncwarp();
     if (own && n_l >= 0 && (n_l > 0 || g.f_eC)) {
-      // the list folded by community, in place
       Ent* const my = ent + lane;
-      int nd = 0;
       VT tot = 0;
+      for (int j = 0; j < n_l; j++) tot += my[j * 32].w;
+      const int64_t eC = k_l - (int64_t)tot, m2v = g.m2_of(v_l);
+      if (!g.f_eC && stays<ST>(m2v, k_l, eC, aC_l)) n_l = 0;
+      // the list folded by community, in place
+      int nd = 0;
       for (int j = 0; j < n_l; j++) {
         const Ent x = my[j * 32];
-        tot += x.w;
         int i = 0;
         while (i < nd && my[i * 32].lab != x.lab) i++;
         if (i < nd) my[i * 32].w += x.w;
         else my[nd++ * 32] = x;
       }
-      const int64_t eC = k_l - (int64_t)tot, m2v = g.m2_of(v_l);
       ST Sb = gain_lowest<ST>();
       int32_t D = INT_MAX;
       int64_t eD = 0;
@@ -345,13 +346,23 @@ __global__ void __launch_bounds__(256) lm_seg(LV<W> g, const int32_t* __restrict
     VT eCl = 0;
     int nd = 0;
 #pragma unroll
+    for (int q = 0; q < Q; q++) eCl += lab[q] == C ? (VT)wt[q] : VT(0);
+    const int64_t eC = seg_total<S>(eCl);
+    const int64_t kv = g.k[v], aC = g.a[C], m2v = g.m2_of(v);
+    const bool open = g.f_eC || !stays<ST>(m2v, kv, eC, aC);
+    if (!__any_sync(0xffffffffu, open && d > 0)) {  // nothing to sum
+      if (sl == 0 && has) {
+        prop[i] = pv >= 0 ? pv : C;
+        if (g.f_eC) put_features(g, i, eC, keys, vals, mask, gain_lowest<ST>(), INT_MAX);
+      }
+      continue;
+    }
+#pragma unroll
     for (int q = 0; q < Q; q++) {
       if (q * S < dmax) {
-        const bool isC = lab[q] == C;
-        eCl += isC ? (VT)wt[q] : VT(0);
         bool claimed = false;
         uint32_t s = 0;
-        if (lab[q] >= 0 && !isC) {
+        if (lab[q] >= 0 && lab[q] != C && open) {
           s = probe_claim(keys, mask, lab[q], claimed);
           atomicAdd(&vals[s], (VT)wt[q]);
         }
@@ -361,8 +372,6 @@ __global__ void __launch_bounds__(256) lm_seg(LV<W> g, const int32_t* __restrict
       }
     }
     __syncwarp();
-    const int64_t eC = seg_total<S>(eCl);
-    const int64_t kv = g.k[v], aC = g.a[C], m2v = g.m2_of(v);
     ST Sb = gain_lowest<ST>();
     int32_t D = INT_MAX;
     for (int j = sl; j < nd; j += S) {
@@ -445,13 +454,25 @@ __global__ void __launch_bounds__(T) lm_cta(LV<W> g, const int32_t* __restrict__
     }
     VT eCl = 0;
 #pragma unroll
+    for (int q = 0; q < Q; q++) eCl += lab[q] == C ? (VT)wt[q] : VT(0);
+    const int64_t ew = seg_total<32>(eCl);
+    if (lane == 0) redC[wid] = (VT)ew;
+    const int64_t kv = g.k[v], aC = g.a[C], m2v = g.m2_of(v);
+    __syncthreads();
+    int64_t eC = 0;
+#pragma unroll
+    for (int x = 0; x < NW; x++) eC += (int64_t)redC[x];
+    if (pv >= 0 || (!g.f_eC && stays<ST>(m2v, kv, eC, aC))) {  // uniform: nothing to sum
+      if (tid == 0) prop[i] = pv >= 0 ? pv : C;
+      __syncthreads();
+      continue;
+    }
+#pragma unroll
     for (int q = 0; q < Q; q++) {
       if (q * T < d) {
-        const bool isC = lab[q] == C;
-        eCl += isC ? (VT)wt[q] : VT(0);
         bool claimed = false;
         uint32_t s = 0;
-        if (lab[q] >= 0 && !isC) {
+        if (lab[q] >= 0 && lab[q] != C) {
           s = probe_claim(keys, mask, lab[q], claimed);
           atomicAdd(&vals[s], (VT)wt[q]);
         }
@@ -462,14 +483,8 @@ __global__ void __launch_bounds__(T) lm_cta(LV<W> g, const int32_t* __restrict__
         if (claimed) slots[at + __popc(bal & lanemask_lt())] = (uint16_t)s;
       }
     }
-    const int64_t ew = seg_total<32>(eCl);
-    if (lane == 0) redC[wid] = (VT)ew;
     __syncthreads();
     const int nd = s_nd;
-    int64_t eC = 0;
-#pragma unroll
-    for (int x = 0; x < NW; x++) eC += (int64_t)redC[x];
-    const int64_t kv = g.k[v], aC = g.a[C], m2v = g.m2_of(v);
     ST Sb = gain_lowest<ST>();
     int32_t D = INT_MAX;
     for (int j = tid; j < nd; j += T) {
@@ -492,7 +507,7 @@ __global__ void __launch_bounds__(T) lm_cta(LV<W> g, const int32_t* __restrict__
       D = lane < NW ? redD[lane] : INT_MAX;
       warp_argmax(Sb, D);
       if (lane == 0) {
-        prop[i] = pv >= 0 ? pv : proposal(Sb, D, C, g.size);
+        prop[i] = proposal(Sb, D, C, g.size);
         if (g.f_eC) put_features(g, i, eC, keys, vals, mask, Sb, D);
       }
     }
