@@ -149,6 +149,15 @@ __device__ __forceinline__ void best_sink(const SV& g, int32_t C, int64_t p0, in
   }
 }
 
+// The same for a source that gains nowhere (stays, agg.cuh): 0 stands for its
+// gains.  Phase B compares a pair's reverse gain with one above 0, for which all
+// values up to 0 are alike.
+template <typename ST>
+__device__ __forceinline__ void no_sink(const SV& g, int64_t p0, int64_t p1, int tid, int NT) {
+  for (int64_t q = p0 + tid; q < p1; q += NT)
+    if (g.pflag[q] & kPairIns) st_pair_gain(g, q, ST(0));
+}
+
 // ---- phase A ----
 //
 // The kernels follow the local move's for the same row lengths (louvain.cu says
@@ -282,19 +291,21 @@ __global__ void __launch_bounds__(256) scr_vert(SV g, int64_t off, int64_t cnt, 
     }
     __syncwarp();
     if (own && n_l >= 0 && (f_l & 2)) {
-      // the lane's list folded by community, in place
       Ent* const my = ent + lane;
-      int nd = 0;
       VT tot = 0;
+      for (int j = 0; j < n_l; j++) tot += my[j * 32].w;
+      const int64_t eC = k_l - (int64_t)tot, m2 = g.m2_of(u_l);
+      const bool open = !stays<ST>(m2, k_l, eC, aC_l);
+      if (!open) n_l = 0;
+      // the lane's list folded by community, in place
+      int nd = 0;
       for (int j = 0; j < n_l; j++) {
         const Ent x = my[j * 32];
-        tot += x.w;
         int i = 0;
         while (i < nd && my[i * 32].lab != x.lab) i++;
         if (i < nd) my[i * 32].w += x.w;
         else my[nd++ * 32] = x;
       }
-      const int64_t eC = k_l - (int64_t)tot, m2 = g.m2_of(u_l);
       if (g.pre) {
         ST Sb = gain_lowest<ST>();
         int32_t D = INT_MAX;
@@ -308,16 +319,20 @@ __global__ void __launch_bounds__(256) scr_vert(SV g, int64_t off, int64_t cnt, 
         }
         if (Sb > 0) D_l = D;
       }
-      ST Sj;
-      int32_t Dj, Jj;
-      best_sink<ST>(g, C_l, p0, p1, 0, 1, m2, k_l, eC, aC_l,
-                    [&](int32_t D) {
-                      for (int i = 0; i < nd; i++)
-                        if (my[i * 32].lab == D) return (int64_t)my[i * 32].w;
-                      return (int64_t)0;
-                    },
-                    Sj, Dj, Jj);
-      if (Sj > 0) J_l = Jj;
+      if (open) {
+        ST Sj;
+        int32_t Dj, Jj;
+        best_sink<ST>(g, C_l, p0, p1, 0, 1, m2, k_l, eC, aC_l,
+                      [&](int32_t D) {
+                        for (int i = 0; i < nd; i++)
+                          if (my[i * 32].lab == D) return (int64_t)my[i * 32].w;
+                        return (int64_t)0;
+                      },
+                      Sj, Dj, Jj);
+        if (Sj > 0) J_l = Jj;
+      } else {
+        no_sink<ST>(g, p0, p1, 0, 1);
+      }
     }
     if (own) {
       g.jstar[off + wb + lane] = J_l;
@@ -381,13 +396,16 @@ __global__ void __launch_bounds__(256) scr_seg(SV g, int64_t off, int64_t cnt) {
       VT eCl = 0;
       int nd = 0;
 #pragma unroll
+      for (int q = 0; q < Q; q++) eCl += lab[q] == C ? (VT)wt[q] : VT(0);
+      const int64_t eC = seg_total<S>(eCl);
+      const int64_t ku = g.k[u], aC = g.a[C], m2 = g.m2_of(u);
+      const bool open = !stays<ST>(m2, ku, eC, aC);
+#pragma unroll
       for (int q = 0; q < Q; q++) {
-        if (q * S < dmax) {
-          const bool isC = lab[q] == C;
-          eCl += isC ? (VT)wt[q] : VT(0);
+        if (q * S < dmax && __any_sync(0xffffffffu, open)) {
           bool claimed = false;
           uint32_t s = 0;
-          if (lab[q] >= 0 && !isC) {
+          if (lab[q] >= 0 && lab[q] != C && open) {
             s = probe_claim(keys, mask, lab[q], claimed);
             atomicAdd(&vals[s], (VT)wt[q]);
           }
@@ -397,8 +415,6 @@ __global__ void __launch_bounds__(256) scr_seg(SV g, int64_t off, int64_t cnt) {
         }
       }
       __syncwarp();
-      const int64_t eC = seg_total<S>(eCl);
-      const int64_t ku = g.k[u], aC = g.a[C], m2 = g.m2_of(u);
       if (g.pre) {  // the local move's choice over the table's communities
         ST Sb = gain_lowest<ST>();
         int32_t D = INT_MAX;
@@ -416,7 +432,8 @@ __global__ void __launch_bounds__(256) scr_seg(SV g, int64_t off, int64_t cnt) {
       }
       ST Sj;
       int32_t Dj, Jj;
-      best_sink<ST>(g, C, p0, ins ? p1 : p0, sl, S, m2, ku, eC, aC,
+      if (!open) no_sink<ST>(g, p0, p1, sl, S);
+      best_sink<ST>(g, C, p0, ins && open ? p1 : p0, sl, S, m2, ku, eC, aC,
                     [&](int32_t D) { return tbl_get(keys, vals, mask, D); }, Sj, Dj, Jj);
       seg_argmax3<S>(Sj, Dj, Jj);
       if (Sj > 0) J = Jj;
@@ -488,13 +505,30 @@ __global__ void __launch_bounds__(T) scr_cta(SV g, int64_t off, int64_t cnt) {
     }
     VT eCl = 0;
 #pragma unroll
+    for (int q = 0; q < Q; q++) eCl += lab[q] == C ? (VT)wt[q] : VT(0);
+    const int64_t ew = seg_total<32>(eCl);
+    if (lane == 0) redC[wid] = (VT)ew;
+    const int64_t ku = g.k[u], aC = g.a[C], m2 = g.m2_of(u);
+    __syncthreads();
+    int64_t eC = 0;
+#pragma unroll
+    for (int x = 0; x < NW; x++) eC += (int64_t)redC[x];
+    if (stays<ST>(m2, ku, eC, aC)) {  // uniform
+      no_sink<ST>(g, p0, p1, tid, T);
+      if (tid == 0) {
+        g.jstar[off + i] = -1;
+        g.intra[off + i] = intra ? 1 : 0;
+        if (g.pre) g.pre[u] = C;
+      }
+      __syncthreads();
+      continue;
+    }
+#pragma unroll
     for (int q = 0; q < Q; q++) {
       if (q * T < d) {
-        const bool isC = lab[q] == C;
-        eCl += isC ? (VT)wt[q] : VT(0);
         bool claimed = false;
         uint32_t s = 0;
-        if (lab[q] >= 0 && !isC) {
+        if (lab[q] >= 0 && lab[q] != C) {
           s = probe_claim(keys, mask, lab[q], claimed);
           atomicAdd(&vals[s], (VT)wt[q]);
         }
@@ -505,14 +539,8 @@ __global__ void __launch_bounds__(T) scr_cta(SV g, int64_t off, int64_t cnt) {
         if (claimed) slots[at + __popc(bal & lanemask_lt())] = (uint16_t)s;
       }
     }
-    const int64_t ew = seg_total<32>(eCl);
-    if (lane == 0) redC[wid] = (VT)ew;
     __syncthreads();
     const int nd = s_nd;
-    int64_t eC = 0;
-#pragma unroll
-    for (int x = 0; x < NW; x++) eC += (int64_t)redC[x];
-    const int64_t ku = g.k[u], aC = g.a[C], m2 = g.m2_of(u);
     if (g.pre) {  // the local move's choice over the table's communities
       ST Sb = gain_lowest<ST>();
       int32_t D = INT_MAX;
@@ -631,15 +659,17 @@ constexpr int kGammaChunk = 256;  // entries of a row a work item marks
 // summing row j* again took 0.6 ms (R-MAT 22: 1.6 ms), 25 launches and two
 // host round trips.  The sources whose neighbourhood is marked set listed[] and
 // become work items (u << 32 | chunk).
+constexpr int kDecideThreads = 256;
 template <typename ST>
-__global__ void __launch_bounds__(256) scr_decide(SV g, int64_t nsrc, uint8_t* __restrict__ listed,
+__global__ void __launch_bounds__(kDecideThreads) scr_decide(SV g, int64_t nsrc, uint8_t* __restrict__ listed,
                                                   int64_t* __restrict__ items, int32_t* __restrict__ item_cnt,
                                                   unsigned long long* __restrict__ gamma_deg) {
+  __shared__ int32_t s_at;
   const int lane = lane_id();
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t stride = (int64_t)gridDim.x * kDecideThreads;
   unsigned long long deg = 0;
-  for (int64_t base = (blockIdx.x * (int64_t)blockDim.x) + (threadIdx.x & ~31); base < nsrc; base += stride) {
-    const int64_t i = base + lane;
+  for (int64_t base = blockIdx.x * (int64_t)kDecideThreads; base < nsrc; base += stride) {
+    const int64_t i = base + threadIdx.x;
     int nch = 0;
     int32_t u = 0;
     if (i < nsrc) {
@@ -662,13 +692,14 @@ __global__ void __launch_bounds__(256) scr_decide(SV g, int64_t nsrc, uint8_t* _
         nch = (int)((d + kGammaChunk - 1) / kGammaChunk);
       }
     }
-    if (!__any_sync(0xffffffffu, nch > 0)) continue;
-    const int incl = warp_incl_scan(nch);
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    int32_t at = 0;
-    if (lane == 0) at = atomicAdd(item_cnt, total);
-    at = __shfl_sync(0xffffffffu, at, 0) + incl - nch;
+    if (!__syncthreads_or(nch)) continue;
+    int total;
+    const int excl = block_excl_scan<int, kDecideThreads>(nch, &total);
+    if (threadIdx.x == 0) s_at = atomicAdd(item_cnt, total);  // once a CTA and step: all on one word
+    __syncthreads();
+    const int32_t at = s_at + excl;
     for (int x = 0; x < nch; x++) items[at + x] = (int64_t)u << 32 | (uint32_t)x;
+    __syncthreads();
   }
   deg = warp_sum(deg);
   if (lane == 0 && deg) atomicAdd(gamma_deg, deg);
