@@ -289,7 +289,11 @@ __device__ __forceinline__ void add128(unsigned long long* lo, unsigned long lon
 }
 
 __device__ __forceinline__ bool below_tau(i128 gain, i128 base, int64_t tau_inv) {
+  // gain <= floor(|base| / tau_inv), without the 128-bit division where the
+  // product fits (tau_inv < 2^31)
   const i128 y = base < 0 ? -base : base;
+  if (gain <= 0) return true;
+  if (gain < ((i128)1 << 95)) return gain * (i128)tau_inv <= y;
   return gain <= y / (i128)tau_inv;
 }
 

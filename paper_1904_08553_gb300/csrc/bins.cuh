@@ -111,21 +111,24 @@ __global__ void __launch_bounds__(256) bin_count(const int64_t* __restrict__ rp,
 // (a reservation per warp and bin took 195 us for 2 M vertices, this 20) and a
 // bin's list stays close to vertex order.
 constexpr int kBinThreads = 256;
+// Vertices a thread: few small blocks leave a small graph to a handful of SMs
+// (10 K vertices: 12 us with 8 a thread, 4 with 1).
 constexpr int kBinItems = 8;
-template <typename Want>
+constexpr int64_t kBinSmall = (int64_t)1 << 18;
+template <typename Want, int ITEMS>
 __global__ void __launch_bounds__(kBinThreads) bin_scatter(const int64_t* __restrict__ rp, int64_t n, Want want,
                                                            const DevScalars* __restrict__ d,
                                                            int32_t* __restrict__ cursor, int32_t* __restrict__ list,
                                                            BinPlan plan) {
   __shared__ int32_t s_cnt[kMaxBins], s_base[kMaxBins];
   const int tid = threadIdx.x;
-  const int64_t block = (int64_t)kBinThreads * kBinItems;
+  const int64_t block = (int64_t)kBinThreads * ITEMS;
   for (int64_t v0 = blockIdx.x * block; v0 < n; v0 += gridDim.x * block) {
     if (tid < kMaxBins) s_cnt[tid] = 0;
     __syncthreads();
-    int bin[kBinItems], rank[kBinItems];
+    int bin[ITEMS], rank[ITEMS];
 #pragma unroll
-    for (int i = 0; i < kBinItems; i++) {
+    for (int i = 0; i < ITEMS; i++) {
       const int64_t v = v0 + i * kBinThreads + tid;
       bin[i] = -1;
       if (v < n && want(v)) {
@@ -134,7 +137,7 @@ __global__ void __launch_bounds__(kBinThreads) bin_scatter(const int64_t* __rest
       }
     }
 #pragma unroll
-    for (int i = 0; i < kBinItems; i++) {
+    for (int i = 0; i < ITEMS; i++) {
       const unsigned peers = __match_any_sync(0xffffffffu, bin[i]);
       int at = 0;
       const int lead = __ffs(peers) - 1;
@@ -144,17 +147,27 @@ __global__ void __launch_bounds__(kBinThreads) bin_scatter(const int64_t* __rest
     __syncthreads();
     if (tid < plan.nb) {
       int64_t o = 0;
-      for (int b = 0; b < tid; b++) o += d->bcnt[b];
+#pragma unroll
+      for (int b = 0; b < kMaxBins - 1; b++) o += b < tid ? d->bcnt[b] : 0;
       s_base[tid] = (int32_t)o + (s_cnt[tid] ? atomicAdd(&cursor[tid], s_cnt[tid]) : 0);
     }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < kBinItems; i++)
+    for (int i = 0; i < ITEMS; i++)
       if (bin[i] >= 0) list[s_base[bin[i]] + rank[i]] = (int32_t)(v0 + i * kBinThreads + tid);
     __syncthreads();
   }
 }
 
-inline int bin_scatter_grid(int64_t n) { return grid_for(cdiv(n, kBinItems), kBinThreads); }
+template <typename Want>
+void launch_bin_scatter(cudaStream_t s, const int64_t* rp, int64_t n, const Want& want, const DevScalars* d,
+                        int32_t* cursor, int32_t* list, const BinPlan& plan) {
+  if (n < kBinSmall)
+    count_launch(), bin_scatter<Want, 1><<<grid_for(n, kBinThreads), kBinThreads, 0, s>>>(rp, n, want, d, cursor, list,
+                                                                                          plan);
+  else
+    count_launch(), bin_scatter<Want, kBinItems><<<grid_for(cdiv(n, kBinItems), kBinThreads), kBinThreads, 0, s>>>(
+        rp, n, want, d, cursor, list, plan);
+}
 
 }  // namespace dcd

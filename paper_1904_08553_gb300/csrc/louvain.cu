@@ -1704,8 +1704,7 @@ int make_bins(dcd_ctx* c, const Csr<W>& g, const uint8_t* active, Bins* b, const
   DCD_TRY(cursor.alloc(&c->mem, kMaxBins));
   DCD_TRY_CUDA(cudaMemsetAsync(cursor.get(), 0, kMaxBins * sizeof(int32_t), s));
   if (b->total > 0) {
-    ::dcd::count_launch(), bin_scatter<<<bin_scatter_grid(nv), kBinThreads, 0, s>>>(
-        g.rp, nv, WantActive{active, gid, c->gs.get()}, d, cursor.get(), b->list.get(), plan);
+    launch_bin_scatter(s, g.rp, nv, WantActive{active, gid, c->gs.get()}, d, cursor.get(), b->list.get(), plan);
     DCD_LAUNCH_CHECK();
   }
   // tables of the hub bin: a region per hub, sized by its degree
@@ -3832,8 +3831,7 @@ struct SlmLevel {
     DCD_TRY(cursor.alloc(&c->mem, kMaxBins));
     DCD_TRY_CUDA(cudaMemsetAsync(cursor.get(), 0, kMaxBins * sizeof(int32_t), s));
     if (total)
-      ::dcd::count_launch(), bin_scatter<<<bin_scatter_grid(n), kBinThreads, 0, s>>>(
-          g.rp, n, WantActive{active, nullptr, nullptr}, d, cursor.get(), list.get(), plan);
+      launch_bin_scatter(s, g.rp, n, WantActive{active, nullptr, nullptr}, d, cursor.get(), list.get(), plan);
     // CTA tables in global memory for the long rows
     using VT = typename TblVal<ST>::type;
     const uint32_t tcap = cnt1 ? table_cap(maxd1) : 64;

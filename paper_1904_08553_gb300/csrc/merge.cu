@@ -618,14 +618,25 @@ __global__ void new_rows(const int64_t* __restrict__ rp_o, const int32_t* __rest
 __global__ void merge_split(const int64_t* __restrict__ epos, const int32_t* __restrict__ npair, int64_t nt,
                             int32_t* __restrict__ sq) {
   const int64_t P = *npair;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t <= nt; t += (int64_t)gridDim.x * blockDim.x) {
+  const int lane = lane_id();
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  // a warp a tile: 32 probes a step, so that the chain is log32 of the pairs
+  for (int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; t <= nt; t += nw) {
     const int64_t d = t * kMergeTile;
     int64_t lo = 0, hi = P < d ? P : d;  // first q with q + epos[q] >= d
     while (lo < hi) {
-      const int64_t mid = (lo + hi) >> 1;
-      if (mid + epos[mid] < d) lo = mid + 1; else hi = mid;
+      const int64_t step = (hi - lo + 31) / 32, q = lo + lane * step;
+      const unsigned below = __ballot_sync(0xffffffffu, q < hi && q + epos[q] < d);  // a prefix of the lanes
+      const int k = __popc(below);
+      if (k == 0) {
+        hi = lo;
+      } else {
+        const int64_t last = lo + (k - 1) * step;  // below d
+        lo = last + 1;
+        hi = last + step < hi ? last + step : hi;
+      }
     }
-    sq[t] = (int32_t)lo;
+    if (lane == 0) sq[t] = (int32_t)lo;
   }
 }
 
@@ -874,7 +885,7 @@ int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut*
   if (nt > 0) {
     Buf<int32_t> split;
     DCD_TRY(split.alloc(&c->mem, nt + 1));
-    ::dcd::count_launch(), merge_split<<<grid_for(nt + 1, T), T, 0, s>>>(epos.get(), off + n, nt, split.get());
+    ::dcd::count_launch(), merge_split<<<grid_for((nt + 1) * 32, T), T, 0, s>>>(epos.get(), off + n, nt, split.get());
     DCD_LAUNCH_CHECK();
     if (nlab) DCD_TRY(nlab->buf.alloc(&c->mem, cap));
     ::dcd::count_launch(), (nlab ? merge_tile<true> : merge_tile<false>)<<<(unsigned)nt, kMergeThreads, 0, s>>>(

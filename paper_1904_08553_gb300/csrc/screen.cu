@@ -942,8 +942,7 @@ int screen_batch(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* labels0, cons
     DCD_TRY(src.alloc(&c->mem, nsrc));
     DCD_TRY(cursor.alloc(&c->mem, kMaxBins));
     DCD_TRY_CUDA(cudaMemsetAsync(cursor.get(), 0, kMaxBins * sizeof(int32_t), s));
-    count_launch(), bin_scatter<<<bin_scatter_grid(n), kBinThreads, 0, s>>>(g.rp, n, WantSource{mo.pair_ptr.get()}, d,
-                                                                           cursor.get(), src.get(), sb.plan);
+    launch_bin_scatter(s, g.rp, n, WantSource{mo.pair_ptr.get()}, d, cursor.get(), src.get(), sb.plan);
     DCD_LAUNCH_CHECK();
     int64_t m2max = 0;
     for (int x = 0; x < c->G; x++) m2max = c->hgs[x].m2 > m2max ? c->hgs[x].m2 : m2max;
