@@ -12,16 +12,22 @@
 // the change of sum_i e_{i->C(i)}, a full reduction gives sum_C a_C^2.
 //
 // Kernels (degree-binned; a bin is a list of active vertex ids, see BinPlan):
-//   lm_seg       rows of at most 16 .. 256 entries: a segment of 8, 16 or 32
-//                lanes per vertex, each segment with its own table in shared
-//                memory
+//   lm_vert      rows of at most 32 entries: 4 or 8 lanes read a row, a lane
+//                chooses from the list of its foreign entries
+//   lm_seg       rows of 33 .. 256 entries: a segment of 16 or 32 lanes per
+//                vertex, each segment with its own table in shared memory
 //   lm_cta       rows of at most 512 .. 4096 entries: a CTA per vertex with a
 //                shared table
 //   hub_*        longer rows: split into chunks over many CTAs, per-hub tables
 //                in global memory
+// A row is summed by community only when a bound leaves v a gain (stays, agg.cuh).
+// On large graphs level 0 reads neighbours' labels in entry order (entry labels,
+// below) instead of gathering them.
 // Compaction (graph of the next level): dense nc x nc sums for few
 // communities, sort-by-key reduction for many; level 0 of an update can be
 // built from the previous update's coarse graph (delta coarsening, below).
+// With at most kLevelNc communities a graph, every level from the dense matrix
+// on runs in one launch (levels.cu); the kernels here take the others.
 #include <cstdio>
 #include <memory>
 #include <type_traits>
@@ -825,10 +831,12 @@ template <typename W>
 __global__ void __launch_bounds__(256) lm_delta(LV<W> g, const int2* __restrict__ LL, int64_t nnz,
                                                 const int64_t* __restrict__ items,
                                                 const int32_t* __restrict__ item_cnt, int32_t* __restrict__ nlab,
-                                                const DevScalars* __restrict__ d, GraphState* __restrict__ gs) {
+                                                int resum, const DevScalars* __restrict__ d,
+                                                GraphState* __restrict__ gs) {
   constexpr int U = kMoveChunk / 32;
   const int64_t cnt = *item_cnt;
   const bool search = nlab && d->moved_deg * kNlabSearch < nnz;
+  if (resum && !search) return;  // nlab_resum reads every row
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int lane = lane_id();
   long long acc = 0;
@@ -1268,6 +1276,55 @@ struct RowWalk {
 // level 0 of a step that starts from the previous step's communities -- then
 // writes a few hundred pairs per warp instead of one per chunk, and the sort
 // that follows has little to do.
+// After a pass of one graph that moved vertices with many entries: the entry
+// labels by a gather of every entry (as nlab_gather), and sum_i e_{i->C(i)} from
+// the same read, so that the movers' rows need not be read by themselves (19 M
+// entries: 100 us for lm_delta's 85-100 and the gather's 78).
+__global__ void __launch_bounds__(256) nlab_resum(int64_t n, int64_t m, const int64_t* __restrict__ rp,
+                                                  const int32_t* __restrict__ col, const int32_t* __restrict__ w,
+                                                  const int32_t* __restrict__ L, int32_t* __restrict__ nlab,
+                                                  int64_t per_warp, const DevScalars* __restrict__ d,
+                                                  GraphState* __restrict__ gs) {
+  if (d->moved_deg * kNlabSearch < m) return;
+  constexpr int U = 4;
+  const int lane = lane_id();
+  const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int64_t W0 = gw * per_warp, W1 = W0 + per_warp < m ? W0 + per_warp : m;
+  unsigned long long acc = 0;
+  if (W0 < W1) {
+    RowWalk rw;
+    rw.start(rp, n, W0);
+    for (int64_t c0 = W0; c0 < W1; c0 += 32 * U) {
+      int32_t y[U], x[U], own[U];
+#pragma unroll
+      for (int q = 0; q < U; q++) {
+        const int64_t e = c0 + q * 32 + lane;
+        y[q] = e < W1 ? ld_stream(col + e) : 0;
+        x[q] = e < W1 ? ld_stream(w + e) : 0;
+      }
+#pragma unroll
+      for (int q = 0; q < U; q++) {
+        const int64_t c = c0 + q * 32;
+        y[q] = L[y[q]];
+        own[q] = -1;
+        if (c < W1) own[q] = L[rw.row(rp, n, c, c + lane < W1)];  // uniform
+      }
+#pragma unroll
+      for (int q = 0; q < U; q++) {
+        const int64_t e = c0 + q * 32 + lane;
+        if (e < W1) {
+          st_stream(nlab + e, y[q]);
+          if (y[q] == own[q]) acc += (unsigned long long)x[q];
+        }
+      }
+    }
+  }
+  acc = warp_sum(acc);
+  if (lane == 0 && acc) atomicAdd((unsigned long long*)&gs[0].in_delta, acc);
+  if (blockIdx.x == 0 && threadIdx.x == 0)  // the pass's change
+    atomicAdd((unsigned long long*)&gs[0].in_delta, 0ull - (unsigned long long)gs[0].in_cur);
+}
+
 constexpr int kEmitThreads = 256;
 
 // Warp table slots: 512 when key and sum are 32-bit (4 KB a warp), 256
@@ -1992,6 +2049,11 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
   const int32_t* lst = bins.list.get();
   bool any = total > 0;
   int64_t* sweep = pl->sweep;
+  // nlab_resum finds the rows of 32 entries among 32 row ends: it wants rows of some
+  // length and few empty ones (R-MAT 22, half of the vertices without entries: 567
+  // us, where lm_delta and the gather take 480): known when nearly every vertex is
+  // active with entries
+  const bool resum = lv.nlab && !gid && g.nnz >= 16 * nv && 32 * (nv - total) <= nv;
   // One pass: evaluate, apply, tracked N, stop rule, then the loop condition.
   // Every pass of a level enqueues the same work (the pass number lives on
   // the device), so the body is captured once, into the body of a 'while'
@@ -2008,11 +2070,20 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
           lst, total, prop.get(), L, LL.get(), kbuf.get(), g.rp, (unsigned long long*)a.get(), size.get(), items.get(),
           item_cnt.get(), d, gid, gs);
       ::dcd::count_launch(), lm_delta<W><<<wave_grid(lm_delta<W>, item_cap * 32, T), T, 0, s>>>(
-          lv, LL.get(), g.nnz, items.get(), item_cnt.get(), lv.nlab ? nlab->buf.get() : nullptr, d, gs);
+          lv, LL.get(), g.nnz, items.get(), item_cnt.get(), lv.nlab ? nlab->buf.get() : nullptr, resum, d, gs);
     }
-    ::dcd::count_launch(), pass_finish<<<sq_ctas, T, 0, s>>>(a.get(), nv, gid, gs, G, lv.nlab ? kPassOpen : kPassClose,
+    if (resum) {  // returns at once unless much has moved
+      if constexpr (std::is_same<W, int32_t>::value) {
+        const int grid = wave_grid(nlab_resum, cdiv(g.nnz, 128) * 32, T);
+        const int64_t per_warp = cdiv(cdiv(g.nnz, (int64_t)grid * (T / 32)), 128) * 128;
+        ::dcd::count_launch(), nlab_resum<<<grid, T, 0, s>>>(g.n, g.nnz, g.rp, g.col, g.w, L, nlab->buf.get(), per_warp,
+                                                             d, gs);
+      }
+    }
+    ::dcd::count_launch(), pass_finish<<<sq_ctas, T, 0, s>>>(a.get(), nv, gid, gs, G,
+                                                             lv.nlab && !resum ? kPassOpen : kPassClose,
                                                              c->cfg.max_iters, c->cfg.tau_inv, d, h, cap, ig);
-    if (lv.nlab) {  // the gather returns at once unless the next pass runs and much has moved
+    if (lv.nlab && !resum) {  // the gather returns at once unless the next pass runs and much has moved
       ::dcd::count_launch(), nlab_gather<<<grid_for(g.nnz, T), T, 0, s>>>(g.col, L, g.nnz, nlab->buf.get(), d);
       ::dcd::count_launch(), pass_end<<<1, 1, 0, s>>>(d, h, cap, ig);
     }
@@ -2021,6 +2092,7 @@ int run_level(dcd_ctx* c, const Csr<W>& g, int32_t* L, Buf<int64_t>& kbuf, Buf<i
   };
   if (any) DCD_TRY(prepare_lm<W>(lvl));
   resident_blocks(reinterpret_cast<const void*>(lm_delta<W>), T, 0);  // looked up outside the capture
+  resident_blocks(reinterpret_cast<const void*>(nlab_resum), T, 0);
   DCD_TRY(side_streams(c));
   {
     int64_t& body_launches = pl->body_launches;

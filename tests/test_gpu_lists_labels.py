@@ -70,3 +70,30 @@ def test_entry_labels(dcd, orc, synth, mode, host_loop):  # noqa: F811
             assert_step_equal(st, rst, lab, rlab, q, rq, ctx.rset(), ref.rset())
             nnz.append(st.nnz)
         assert nnz[1] >= 1 << 21
+
+
+@pytest.mark.parametrize("empty,wmax", [(0, 1), (40, 4000), (20, 1)])
+def test_entry_labels_resummed(dcd, orc, empty, wmax):  # noqa: F811
+    """Passes that move most vertices, with no empty rows, with some among the
+    others (few enough to sum the labels' agreement along with their gather), and
+    with too many; ragged sizes, 64- and 128-bit gains."""
+    n = 70_013
+    rng = np.random.default_rng(empty + wmax)
+    live = np.arange(n) if not empty else np.nonzero(np.arange(n) % empty)[0]
+    m = 19 * n
+    u = live[rng.integers(0, len(live), m)]
+    v = live[np.minimum(np.searchsorted(live, u) // 60 * 60 + rng.integers(0, 60, m), len(live) - 1)]
+    far = rng.random(m) < 0.2
+    v[far] = live[rng.integers(0, len(live), int(far.sum()))]
+    ok = u != v
+    ins = np.stack([u, v, rng.integers(1, wmax + 1, m)], 1)[ok].astype(np.int32)
+    none = np.zeros((0, 2), np.int32)
+    ref = orc.Context(n)
+    with dcd.Context(n, mode=dcd.MODE_STATIC) as ctx:
+        for a, b in [(ins, none), (ins[:50], ins[100:160, :2])]:
+            ctx.apply_batch(a, b)
+            ref.apply_batch(a, b)
+            lab, q, st = ctx.update()
+            rlab, rq, rst = ref.update(orc.STATIC)
+            assert_step_equal(st, rst, lab, rlab, q, rq, ctx.rset(), ref.rset())
+        assert st.nnz >= 1 << 21 and (wmax == 1 or st.m2 >= 1 << 31)
