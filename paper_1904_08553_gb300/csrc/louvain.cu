@@ -140,7 +140,8 @@ __device__ __forceinline__ void put_features(const LV<W>& g, int64_t i, int64_t 
 // Once the labels come in entry order (below), short rows are bound by issue and
 // by the latency of shared-memory and shuffle chains: 0.88 M rows of 17..32
 // entries take 118 us here and 200 us with a hash table a row (0.38 of its
-// instructions).  Rows of 33..64 entries are the other way round (146 against
+// instructions); 91 us with the bound (stays) before the fold and five CTAs an SM
+// (6: 14 % slower, 4: 5 %).  Rows of 33..64 entries are the other way round (146 against
 // 107 us: the lists of 32 vertices leave room for fewer warps), so they keep
 // the table.  A vertex with more than CAP foreign entries is chosen in phase 2
 // by its segment together (list_best), before the next step.
@@ -1040,9 +1041,10 @@ __global__ void pass_end(DevScalars* d, cudaGraphConditionalHandle h, int32_t ca
 // The gather of a neighbour's label costs a 32-byte sector per entry, pass
 // after pass, and bounds the evaluation (73 M entries: 1.09 ms with it, 0.55
 // without).  Level 0 of a large graph therefore keeps the labels in entry order:
-// one gather of its own when the level starts (entry-linear, 0.29 ms, 250 G
-// sectors/s), then after every pass the entries that point to a moved vertex,
-// by lm_delta when few have moved, by this gather again otherwise.  A level 0 of
+// written by the merge or by one gather when the level starts (entry-linear, 0.29
+// ms, 250 G sectors/s), then after every pass the entries that point to a moved
+// vertex, by lm_delta when few have moved, by a gather of all otherwise (this
+// one or nlab_resum).  A level 0 of
 // three evaluated passes over 73 M entries: 3.30 ms with gathers in every pass,
 // 0.29 + 1.55 + 0.09 ms so; of 13-17 passes over 19 M entries (from
 // singletons): 4.9 -> 2.6 ms.

@@ -655,7 +655,7 @@ __device__ __forceinline__ int64_t find_pair(const SV& g, int32_t u, int32_t v) 
 constexpr int kGammaChunk = 256;  // entries of a row a work item marks
 
 // A source per lane: gain1 >= gain2 decides; jstar holds only sinks of
-// gain1 > 0.  87 us for 2 M sources, where sorting the sources by j* and
+// gain1 > 0.  82 us for 2 M sources, where sorting the sources by j* and
 // summing row j* again took 0.6 ms (R-MAT 22: 1.6 ms), 25 launches and two
 // host round trips.  The sources whose neighbourhood is marked set listed[] and
 // become work items (u << 32 | chunk).
