@@ -5,19 +5,20 @@
 // accumulators.  A warp owns 16 rows: layer-1 and layer-2 accumulator tiles
 // are turned into the next product's A fragments in registers (bias, ReLU,
 // BF16 pack).  Training adds the backward pass in the same kernel: the
-// activation gradients stay in registers, the weight gradients of a CTA's rows
-// are formed 64 rows at a time with mma from shared-memory tiles and stay in
-// registers until its rows are done, and the CTAs' partial gradients are
-// reduced in a fixed order (deterministic), then Adam updates the FP32 master
-// weights and refreshes the BF16 copies.  A training run is one cooperative
-// kernel over all its mini-batches: a step is a few microseconds of work, so
-// four launches a step were most of its time.
+// activation gradients stay in registers, the weight gradients of a tile of 64
+// rows are formed with mma from shared-memory tiles, and the tiles' partial
+// gradients are added in tile order, whatever CTA formed them: the sums depend
+// on the rows alone, not on the grid (a run of a hundred steps multiplies the
+// last bit of a sum: a BF16 copy flips, and Adam divides a gradient by its own
+// size).  Then Adam updates the FP32 master weights and refreshes the BF16
+// copies.  A training run is one cooperative kernel over all its mini-batches: a
+// step is a few microseconds of work, so four launches a step were most of its
+// time.
 #include <cuda_bf16.h>
 
 #include <cmath>
 #include <cstring>
 #include <new>
-#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -228,25 +229,6 @@ __device__ __forceinline__ void load_grad_weights(GradSmem& s, const Weights& W)
   load_rows(s.w2, SH, W.w2, 64, 64);
 }
 
-// Gradient sums of a CTA, over its 64-row tiles: warp w holds dW2 rows 16 w ..
-// 16 w + 15 and dW1 columns likewise; thread j < 64 db1[j] and dW3[j], thread
-// 64 + j db2[j], thread 0 db3 and thread 1 the loss.
-struct GradAcc {
-  float w2[8][4];
-  float w1[2][4];
-  float b, w3;
-  float b3;
-  double loss;
-};
-__device__ __forceinline__ void grad_zero(GradAcc& a) {
-#pragma unroll
-  for (int j = 0; j < 8; j++) a.w2[j][0] = a.w2[j][1] = a.w2[j][2] = a.w2[j][3] = 0.f;
-#pragma unroll
-  for (int j = 0; j < 2; j++) a.w1[j][0] = a.w1[j][1] = a.w1[j][2] = a.w1[j][3] = 0.f;
-  a.b = a.w3 = a.b3 = 0.f;
-  a.loss = 0;
-}
-
 // A thread's inputs of the 64-row tile at tile0 (of rows [0, n)).
 struct TileIn {
   uint32_t xa[4];
@@ -260,10 +242,12 @@ __device__ __forceinline__ void load_tile(const float* __restrict__ X, const flo
   in.yb = rb < n ? Y[rb] : 0.f;
 }
 
-// The tile at tile0 of [0, n) into the sums (128 threads; the weights are in s,
-// and the caller has synchronised).
+// The gradient sums of the tile at tile0 of [0, n) to its partial vector (128
+// threads; the weights are in s, and the caller has synchronised).  Warp w forms
+// dW2 rows 16 w .. 16 w + 15 and dW1 columns likewise; thread j < 64 db1[j] and
+// dW3[j], thread 64 + j db2[j], thread 0 db3 and thread 1 the loss.
 __device__ __forceinline__ void grad_tile(GradSmem& s, const TileIn& in, int64_t tile0, int64_t n, float inv_n,
-                                          GradAcc& acc) {
+                                          float* __restrict__ out, double* __restrict__ lout) {
   const int lane = lane_id(), g = lane >> 2, t = lane & 3, wid = threadIdx.x >> 5;
   const int64_t r0 = tile0 + wid * 16;
   Fwd f;
@@ -351,6 +335,11 @@ __device__ __forceinline__ void grad_tile(GradSmem& s, const TileIn& in, int64_t
   __syncthreads();
   // dW2[i][j] = sum_r h1[r][i] dh2[r][j], dW1[i][j] = sum_r x[r][i] dh1[r][j]:
   // both operands lie with K (the rows r) along the stored rows
+  float a2[8][4], a1[2][4];
+#pragma unroll
+  for (int j = 0; j < 8; j++) a2[j][0] = a2[j][1] = a2[j][2] = a2[j][3] = 0.f;
+#pragma unroll
+  for (int j = 0; j < 2; j++) a1[j][0] = a1[j][1] = a1[j][2] = a1[j][3] = 0.f;
   const int tr = lane & 7, tq = lane >> 3;
 #pragma unroll
   for (int kk = 0; kk < 4; kk++) {
@@ -364,14 +353,28 @@ __device__ __forceinline__ void grad_tile(GradSmem& s, const TileIn& in, int64_t
       // B tiles: (k0, n0), (k8, n0), (k0, n8), (k8, n8)
       uint32_t b[4];
       ldsm_t(b, s.dh2 + (16 * kk + (tq & 1) * 8 + tr) * SH + 16 * jp + (tq >> 1) * 8);
-      mma16816(acc.w2[2 * jp], a, b[0], b[1]);
-      mma16816(acc.w2[2 * jp + 1], a, b[2], b[3]);
+      mma16816(a2[2 * jp], a, b[0], b[1]);
+      mma16816(a2[2 * jp + 1], a, b[2], b[3]);
     }
     uint32_t ax[4], bx[4];
     ldsm_t(ax, s.x + ar * SX + ac);
     ldsm_t(bx, s.dh1 + (16 * kk + (tq & 1) * 8 + tr) * SH + 16 * wid + (tq >> 1) * 8);
-    mma16816(acc.w1[0], ax, bx[0], bx[1]);
-    mma16816(acc.w1[1], ax, bx[2], bx[3]);
+    mma16816(a1[0], ax, bx[0], bx[1]);
+    mma16816(a1[1], ax, bx[2], bx[3]);
+  }
+  const int i0 = 16 * wid + g;
+#pragma unroll
+  for (int j = 0; j < 8; j++) {
+    const int c = 8 * j + 2 * t;
+    __stcg(reinterpret_cast<float2*>(out + OFF_W2 + i0 * 64 + c), make_float2(a2[j][0], a2[j][1]));
+    __stcg(reinterpret_cast<float2*>(out + OFF_W2 + (i0 + 8) * 64 + c), make_float2(a2[j][2], a2[j][3]));
+  }
+#pragma unroll
+  for (int jj = 0; jj < 2; jj++) {
+    const int c = 16 * wid + 8 * jj + 2 * t;
+    __stcg(reinterpret_cast<float2*>(out + OFF_W1 + g * NH + c), make_float2(a1[jj][0], a1[jj][1]));
+    if (g + 8 < NF)
+      __stcg(reinterpret_cast<float2*>(out + OFF_W1 + (g + 8) * NH + c), make_float2(a1[jj][2], a1[jj][3]));
   }
   // biases, W3, loss (fixed-order sums)
   {
@@ -380,113 +383,106 @@ __device__ __forceinline__ void grad_tile(GradSmem& s, const TileIn& in, int64_t
     float v = 0.f;
 #pragma unroll 16
     for (int r = 0; r < kRowsPerCta; r++) v += __bfloat162float(m[r * SH + j]);
-    acc.b += v;
-    if (threadIdx.x < 64) acc.w3 += s.wpart[0][j] + s.wpart[1][j] + s.wpart[2][j] + s.wpart[3][j];
+    if (threadIdx.x < 64) {
+      __stcg(out + OFF_B1 + j, v);
+      __stcg(out + OFF_W3 + j, s.wpart[0][j] + s.wpart[1][j] + s.wpart[2][j] + s.wpart[3][j]);
+    } else {
+      __stcg(out + OFF_B2 + j, v);
+    }
   }
-  if (threadIdx.x == 0) acc.b3 += s.wpart[0][64] + s.wpart[1][64] + s.wpart[2][64] + s.wpart[3][64];
+  if (threadIdx.x == 0) __stcg(out + OFF_B3, s.wpart[0][64] + s.wpart[1][64] + s.wpart[2][64] + s.wpart[3][64]);
   if (threadIdx.x == 1)
-    acc.loss += (double)s.wpart[0][65] + s.wpart[1][65] + s.wpart[2][65] + s.wpart[3][65];
+    __stcg(lout, (double)s.wpart[0][65] + s.wpart[1][65] + s.wpart[2][65] + s.wpart[3][65]);
 }
 
-// A CTA's sums to its partial vector.
-__device__ __forceinline__ void grad_store(const GradAcc& acc, float* __restrict__ out, double* __restrict__ lout) {
-  const int lane = lane_id(), g = lane >> 2, t = lane & 3, wid = threadIdx.x >> 5;
-  const int i0 = 16 * wid + g;
-#pragma unroll
-  for (int j = 0; j < 8; j++) {
-    const int c = 8 * j + 2 * t;
-    __stcg(reinterpret_cast<float2*>(out + OFF_W2 + i0 * 64 + c), make_float2(acc.w2[j][0], acc.w2[j][1]));
-    __stcg(reinterpret_cast<float2*>(out + OFF_W2 + (i0 + 8) * 64 + c), make_float2(acc.w2[j][2], acc.w2[j][3]));
-  }
-#pragma unroll
-  for (int jj = 0; jj < 2; jj++) {
-    const int c = 16 * wid + 8 * jj + 2 * t;
-    __stcg(reinterpret_cast<float2*>(out + OFF_W1 + g * NH + c), make_float2(acc.w1[jj][0], acc.w1[jj][1]));
-    if (g + 8 < NF)
-      __stcg(reinterpret_cast<float2*>(out + OFF_W1 + (g + 8) * NH + c), make_float2(acc.w1[jj][2], acc.w1[jj][3]));
-  }
-  const int j = threadIdx.x & 63;
-  if (threadIdx.x < 64) {
-    __stcg(out + OFF_B1 + j, acc.b);
-    __stcg(out + OFF_W3 + j, acc.w3);
-  } else {
-    __stcg(out + OFF_B2 + j, acc.b);
-  }
-  if (threadIdx.x == 0) __stcg(out + OFF_B3, acc.b3);
-  if (threadIdx.x == 1) __stcg(lout, acc.loss);
-}
+constexpr int kPartStride = 5060;  // floats a partial vector takes (float4 loads stay aligned)
 
-constexpr int kPartStride = 5060;  // floats a partial vector takes (float2 stores stay aligned)
-
-// Gradient partials of rows [0, n), 64-row tiles dealt to the CTAs in turn.
+// Gradient partials of the tiles [t0, t1) of rows [0, n), dealt to the CTAs in
+// turn; part[x] is tile t0 + x.
 __global__ void __launch_bounds__(128) mlp_grad_cta(Weights W, const float* __restrict__ X,
-                                                    const float* __restrict__ Y, int64_t n, float inv_n,
-                                                    float* __restrict__ part, double* __restrict__ lpart) {
+                                                    const float* __restrict__ Y, int64_t n, float inv_n, int64_t t0,
+                                                    int64_t t1, float* __restrict__ part, double* __restrict__ lpart) {
   extern __shared__ __align__(16) unsigned char smem[];
   GradSmem& s = *reinterpret_cast<GradSmem*>(smem);
   load_grad_weights(s, W);
   __syncthreads();
-  GradAcc acc;
-  grad_zero(acc);
-  for (int64_t r = (int64_t)blockIdx.x * kRowsPerCta; r < n; r += (int64_t)gridDim.x * kRowsPerCta) {
+  for (int64_t x = blockIdx.x; x < t1 - t0; x += gridDim.x) {
+    const int64_t r = (t0 + x) * kRowsPerCta;
     TileIn in;
     load_tile(X, Y, r, n, in);
-    grad_tile(s, in, r, n, inv_n, acc);
+    grad_tile(s, in, r, n, inv_n, part + x * kPartStride, lpart + x);
   }
-  grad_store(acc, part + (int64_t)blockIdx.x * kPartStride, lpart + blockIdx.x);
 }
 
-// Sums over the CTAs' partials: warp w of four takes CTAs w, w + 4, ... in
-// turn, then the four in turn: a fixed order.  A lane takes two parameters
-// (k, k + 1), so a CTA does kSumBlock of them, with up to 32 loads a thread in
-// flight.  128 threads; every warp's lanes get the sums.
+// carry + part[0][k] + part[1][k] + ... for the kSumBlock parameters k of block
+// b, in this order: thread j < 64 gets parameter 64 b + j.  128 threads, all
+// calling.  The order makes the sum a chain of additions, so only the loads are
+// spread: the partials of kSumTiles tiles come 16 bytes a thread, all in flight,
+// into shared memory, from where 64 threads add them (4 cycles each; 128 tiles:
+// 0.3 us), while the loads of the next kSumTiles run.
 constexpr int kSumBlock = 64;
 constexpr int kSumBlocks = (NP + kSumBlock - 1) / kSumBlock;
-__device__ __forceinline__ float2 grad_sum(const float* __restrict__ part, int ncta, int k, float2 (*red)[32]) {
-  const int lane = lane_id(), wid = threadIdx.x >> 5;
-  float2 v = make_float2(0.f, 0.f);
-  if (k < NP) {  // (a partial vector has room behind its last parameter)
-    auto ld = [&](int c) { return __ldcg(reinterpret_cast<const float2*>(part + (int64_t)c * kPartStride + k)); };
-    int c = wid;
-    auto run = [&](auto u) {
-      constexpr int U = decltype(u)::value;
-      for (; c + 4 * (U - 1) < ncta; c += 4 * U) {
-        float2 x[U];
+constexpr int kSumTiles = 160;
+constexpr int kSumLoads = kSumTiles / 8;  // 16 threads a tile
+using SumStage = float[kSumTiles][kSumBlock];
+__device__ __forceinline__ float grad_sum(const float* __restrict__ part, int tiles, int b, float carry,
+                                          SumStage& stage) {
+  const int tid = threadIdx.x, row = tid >> 4, col = (tid & 15) * 4;
+  const bool in = b * kSumBlock + col < kPartStride;  // the last block is short
+  const float* src = part + b * kSumBlock + col;
+  float4 x[kSumLoads];
+  auto load = [&](int c0) {
 #pragma unroll
-        for (int i = 0; i < U; i++) x[i] = ld(c + 4 * i);
+    for (int i = 0; i < kSumLoads; i++) {
+      const int c = c0 + i * 8 + row;
+      x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (in && c < tiles) x[i] = __ldcg(reinterpret_cast<const float4*>(src + (int64_t)c * kPartStride));
+    }
+  };
+  float s = carry;
+  load(0);
+  for (int c0 = 0; c0 < tiles; c0 += kSumTiles) {
+    const int m = tiles - c0 < kSumTiles ? tiles - c0 : kSumTiles;
 #pragma unroll
-        for (int i = 0; i < U; i++) {
-          v.x += x[i].x;
-          v.y += x[i].y;
-        }
+    for (int i = 0; i < kSumLoads; i++)
+      if (i * 8 + row < m) *reinterpret_cast<float4*>(&stage[i * 8 + row][col]) = x[i];
+    __syncthreads();
+    if (c0 + kSumTiles < tiles) load(c0 + kSumTiles);
+    if (tid < kSumBlock) {
+      int c = 0;
+      for (; c + 16 <= m; c += 16) {
+        float v[16];
+#pragma unroll
+        for (int i = 0; i < 16; i++) v[i] = stage[c + i][tid];
+#pragma unroll
+        for (int i = 0; i < 16; i++) s += v[i];
       }
-    };
-    run(std::integral_constant<int, 32>{});
-    run(std::integral_constant<int, 8>{});
-    run(std::integral_constant<int, 1>{});
+      for (; c < m; c++) s += stage[c][tid];
+    }
+    __syncthreads();
   }
-  red[wid][lane] = v;
-  __syncthreads();
-  v = make_float2(red[0][lane].x + red[1][lane].x + red[2][lane].x + red[3][lane].x,
-                  red[0][lane].y + red[1][lane].y + red[2][lane].y + red[3][lane].y);
-  __syncthreads();
-  return v;
+  return s;
 }
 
-__global__ void __launch_bounds__(128) grad_reduce(const float* __restrict__ part, int ncta, float* __restrict__ grad,
-                                                   const double* __restrict__ lpart, double* __restrict__ loss,
-                                                   double inv_n) {
-  __shared__ float2 red[4][32];
-  const int k = blockIdx.x * kSumBlock + 2 * (int)lane_id();
-  const float2 v = grad_sum(part, ncta, k, red);
-  if (threadIdx.x < 32) {
-    if (k < NP) grad[k] = v.x;
-    if (k + 1 < NP) grad[k + 1] = v.y;
-  }
+// The losses of the tiles, in tile order.
+__device__ __forceinline__ double loss_sum(const double* __restrict__ lpart, int tiles, double l) {
+  for (int c = 0; c < tiles; c++) l += __ldcg(lpart + c);
+  return l;
+}
+
+// first: the tiles are the first of the rows; else grad and loss hold the sums
+// of those before.  inv_n (not zero on the last call): the loss becomes a mean.
+__global__ void __launch_bounds__(128) grad_reduce(const float* __restrict__ part, int tiles, int first,
+                                                   float* __restrict__ grad, const double* __restrict__ lpart,
+                                                   double* __restrict__ loss, double inv_n) {
+  __shared__ __align__(16) SumStage stage;
+  const int k = blockIdx.x * kSumBlock + threadIdx.x;
+  const bool mine = threadIdx.x < kSumBlock && k < NP;
+  const float v = grad_sum(part, tiles, blockIdx.x, mine && !first ? grad[k] : 0.f, stage);
+  if (mine) grad[k] = v;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    double l = 0;
-    for (int c = 0; c < ncta; c++) l += lpart[c];
-    *loss = l * inv_n;
+    const double l = loss_sum(lpart, tiles, first ? 0.0 : *loss);
+    *loss = inv_n != 0 ? l * inv_n : l;
   }
 }
 
@@ -545,35 +541,40 @@ __device__ __forceinline__ bool grid_wait(unsigned* bar, unsigned target, int* e
 }
 
 // Steps [s0, s1) of a training run: step s takes mini-batch s % per_epoch.  A
-// step is: gradient partials of the first `rows` CTAs' tiles | wait | the CTAs'
-// shares of the parameters summed and updated | wait.  corr: Adam's bias
-// corrections (two floats a step).  Bound by the latency of its two waits and
-// of the passes through L2 between them (weights in, partials out and in), so
-// what does not depend on the other CTAs is loaded before each wait: the
-// parameters and moments to update, the next step's rows.  A step of 8192 rows
-// takes 10.5 us; as four kernels (partials 18, sums 19, Adam 4, BF16 copies 3 us)
-// it took 41.
+// step is: gradient partials of the tiles, dealt to the first `rows` CTAs | wait
+// | the CTAs' shares of the parameters summed and updated | wait.  A batch of more
+// tiles than there is room for partials takes them in chunks, the sums so far in
+// grad.  corr: Adam's bias corrections (two floats a step).  Bound by the latency
+// of its two waits and of the passes through L2 between them (weights in,
+// partials out and in), so what does not depend on the other CTAs is loaded
+// before each wait: the parameters and moments to update, the next step's rows.
+// 32 steps of 8192 rows take 412 us (401 with sums split over four warps, which
+// depend on the split); as four kernels a step (partials 18, sums 19, Adam 4, BF16
+// copies 3 us) 1308.
 struct TrainArgs {
   const float* X;
   const float* Y;
   int64_t n, batch, per_epoch;
   int64_t s0, s1;
-  int rows;  // CTAs that take rows; the others only parameters
+  int64_t chunk;  // tiles there is room for
+  int rows;       // CTAs that take tiles; the others only parameters
   float lr, b1, b2, eps;
   const float* corr;
   float* part;
   double* lpart;
+  float* grad;
   double* loss;
   unsigned* bar;  // zero
   int* err;
 };
+constexpr size_t kTrainSmem = sizeof(GradSmem) + sizeof(SumStage);
 __global__ void __launch_bounds__(128) mlp_train_steps(Weights W, Master M, TrainArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   GradSmem& s = *reinterpret_cast<GradSmem*>(smem);
-  __shared__ float2 red[4][32];
+  SumStage& stage = *reinterpret_cast<SumStage*>(smem + sizeof(GradSmem));
   const int G = gridDim.x, rows = a.rows;
-  const int64_t mine = (int64_t)blockIdx.x * kRowsPerCta;
   const bool works = (int)blockIdx.x < rows;
+  const int j = threadIdx.x < kSumBlock ? (int)threadIdx.x : NP;  // (NP: no parameter)
   auto batch_of = [&](int64_t st, int64_t& r0, int64_t& nb) {
     r0 = (st % a.per_epoch) * a.batch;
     nb = r0 + a.batch <= a.n ? a.batch : a.n - r0;
@@ -582,42 +583,45 @@ __global__ void __launch_bounds__(128) mlp_train_steps(Weights W, Master M, Trai
   int64_t r0, nb;
   batch_of(a.s0, r0, nb);
   TileIn in;
+  const int64_t mine = (int64_t)blockIdx.x * kRowsPerCta;
   if (works) load_tile(a.X + r0 * NF, a.Y + r0, mine, nb, in);
   for (int64_t st = a.s0; st < a.s1; st++) {
+    const float inv_n = 1.f / (float)nb;
+    const int64_t tiles = (nb + kRowsPerCta - 1) / kRowsPerCta;
+    const float c1 = a.corr[2 * (st - a.s0)], c2 = a.corr[2 * (st - a.s0) + 1];
     if (works) {
       load_grad_weights(s, W);
       __syncthreads();
-      GradAcc acc;
-      grad_zero(acc);
-      const float inv_n = 1.f / (float)nb;
-      for (int64_t r = mine; r < nb; r += (int64_t)rows * kRowsPerCta) {
-        if (r != mine) load_tile(a.X + r0 * NF, a.Y + r0, r, nb, in);
-        grad_tile(s, in, r, nb, inv_n, acc);
-      }
-      grad_store(acc, a.part + (int64_t)blockIdx.x * kPartStride, a.lpart + blockIdx.x);
     }
-    const float c1 = a.corr[2 * (st - a.s0)], c2 = a.corr[2 * (st - a.s0) + 1];
-    int k = (int)blockIdx.x * kSumBlock + 2 * (int)lane_id();
-    Moments o0 = load_moments(M, k), o1 = load_moments(M, k + 1);
-    if (!grid_wait(a.bar, target += G, a.err)) return;
-    for (int b = blockIdx.x; b < kSumBlocks; b += G) {
-      if (b != (int)blockIdx.x) {
-        k = b * kSumBlock + 2 * (int)lane_id();
-        o0 = load_moments(M, k);
-        o1 = load_moments(M, k + 1);
+    double l = 0;  // CTA 0's first thread
+    for (int64_t t0 = 0; t0 < tiles; t0 += a.chunk) {
+      const int m = (int)(tiles - t0 < a.chunk ? tiles - t0 : a.chunk);
+      const bool last = t0 + m == tiles;
+      if (works)
+        for (int x = blockIdx.x; x < m; x += rows) {
+          const int64_t r = (t0 + x) * kRowsPerCta;
+          if (r != mine) load_tile(a.X + r0 * NF, a.Y + r0, r, nb, in);
+          grad_tile(s, in, r, nb, inv_n, a.part + (int64_t)x * kPartStride, a.lpart + x);
+        }
+      int k = (int)blockIdx.x * kSumBlock + j;
+      Moments o = load_moments(M, k);
+      if (!grid_wait(a.bar, target += G, a.err)) return;
+      for (int b = blockIdx.x; b < kSumBlocks; b += G) {
+        if (b != (int)blockIdx.x) {
+          k = b * kSumBlock + j;
+          o = load_moments(M, k);
+        }
+        const float gk = grad_sum(a.part, m, b, t0 > 0 && k < NP ? a.grad[k] : 0.f, stage);
+        if (k >= NP) continue;
+        if (last) adam_one(M, k, o, gk, a.lr, a.b1, a.b2, a.eps, c1, c2);
+        else a.grad[k] = gk;
       }
-      const float2 gk = grad_sum(a.part, rows, k, red);
-      if (threadIdx.x < 32) {
-        if (k < NP) adam_one(M, k, o0, gk.x, a.lr, a.b1, a.b2, a.eps, c1, c2);
-        if (k + 1 < NP) adam_one(M, k + 1, o1, gk.y, a.lr, a.b1, a.b2, a.eps, c1, c2);
-      }
+      if (st + 1 == a.s1 && blockIdx.x == 0 && threadIdx.x == 0) l = loss_sum(a.lpart, m, l);
+      if (last) break;
+      if (!grid_wait(a.bar, target += G, a.err)) return;
     }
     if (st + 1 == a.s1) {
-      if (blockIdx.x == 0 && threadIdx.x == 0) {
-        double l = 0;
-        for (int c = 0; c < rows; c++) l += __ldcg(a.lpart + c);
-        *a.loss = l / (double)nb;
-      }
+      if (blockIdx.x == 0 && threadIdx.x == 0) *a.loss = l * (1.0 / (double)nb);
       break;
     }
     batch_of(st + 1, r0, nb);
@@ -642,8 +646,10 @@ struct dcd_mlp {
   __nv_bfloat16* w2 = nullptr;
   __nv_bfloat16* w2t = nullptr;
   __nv_bfloat16* w3 = nullptr;
-  float* part = nullptr;
+  float* part = nullptr;     // partials of part_tiles tiles, in block or in more
   double* lpart = nullptr;
+  int64_t part_tiles = 0;
+  unsigned char* more = nullptr;  // allocation for batches of more tiles than block has room for
   unsigned* sync = nullptr;  // [0] the training kernel's barrier, [1] its error word
   float* corr = nullptr;     // Adam's bias corrections of kTrainSteps steps
   int64_t adam_t = 0;
@@ -660,31 +666,50 @@ int refresh(dcd_mlp* m) {
   return DCD_OK;
 }
 
-// CTAs of the gradient kernels: a 64-row tile each, one CTA an SM at most (the
-// partial vectors are written and read back, 20 KB each).
-int64_t grad_ctas(int64_t n) {
-  const int64_t tiles = cdiv(n, kRowsPerCta);
-  return tiles < num_sms() ? tiles : num_sms();
+// CTAs that take tiles: one an SM at most.
+int64_t grad_ctas(int64_t tiles) { return tiles < num_sms() ? tiles : num_sms(); }
+
+// Tiles whose partials (20 KB each) are held at once: what dcd_mlp_create has
+// room for (kPartFew an SM; batches to 19,456 rows), for larger batches up to kPartMost
+// an SM (25 MB, within L2); a batch of more takes them in chunks.  Growth that
+// fails leaves smaller chunks.
+constexpr int64_t kPartFew = 2, kPartMost = 8;
+void part_room(dcd_mlp* m, int64_t tiles) {
+  const int64_t want = tiles < kPartMost * num_sms() ? tiles : kPartMost * num_sms();
+  if (want <= m->part_tiles) return;
+  const int64_t room = kPartMost * num_sms();
+  unsigned char* q = nullptr;
+  if (fault_hit(kFaultAlloc) || cudaMalloc(&q, (size_t)room * (kPartStride * sizeof(float) + sizeof(double))) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  m->more = q;  // (growth happens once: block's own room is the only smaller one)
+  m->lpart = reinterpret_cast<double*>(q);
+  m->part = reinterpret_cast<float*>(q + (size_t)room * sizeof(double));
+  m->part_tiles = room;
 }
 
 constexpr int64_t kTrainSteps = 4096;  // steps a launch of the training kernel takes at most
 
 int grad_attrs() {
   DCD_TRY_CUDA(cudaFuncSetAttribute(mlp_grad_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem)));
-  DCD_TRY_CUDA(
-      cudaFuncSetAttribute(mlp_train_steps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem)));
+  DCD_TRY_CUDA(cudaFuncSetAttribute(mlp_train_steps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrainSmem));
   return DCD_OK;
 }
 
 // Mean BCE gradient of rows [0, n) into m->grad and m->loss.
 int grad_pass(dcd_mlp* m, const float* X, const float* Y, int64_t n) {
-  const int64_t ctas = grad_ctas(n);
+  const int64_t tiles = cdiv(n, kRowsPerCta);
+  part_room(m, tiles);
   DCD_TRY(grad_attrs());
-  count_launch(), mlp_grad_cta<<<(unsigned)ctas, 128, sizeof(GradSmem), m->stream>>>(
-      weights_of(m), X, Y, n, 1.f / (float)n, m->part, m->lpart);
-  count_launch(), grad_reduce<<<kSumBlocks, 128, 0, m->stream>>>(m->part, (int)ctas, m->grad, m->lpart, m->loss,
-                                                                      1.0 / (double)n);
-  DCD_LAUNCH_CHECK();
+  for (int64_t t0 = 0; t0 < tiles; t0 += m->part_tiles) {
+    const int64_t t1 = t0 + m->part_tiles < tiles ? t0 + m->part_tiles : tiles;
+    count_launch(), mlp_grad_cta<<<(unsigned)grad_ctas(t1 - t0), 128, sizeof(GradSmem), m->stream>>>(
+        weights_of(m), X, Y, n, 1.f / (float)n, t0, t1, m->part, m->lpart);
+    count_launch(), grad_reduce<<<kSumBlocks, 128, 0, m->stream>>>(m->part, (int)(t1 - t0), t0 == 0, m->grad, m->lpart,
+                                                                   m->loss, t1 == tiles ? 1.0 / (double)n : 0.0);
+    DCD_LAUNCH_CHECK();
+  }
   return DCD_OK;
 }
 
@@ -730,8 +755,8 @@ int dcd_mlp_create(uint64_t seed, void* cuda_stream, dcd_mlp** out) {
                  og = part(NP * sizeof(float)), ol = part(sizeof(double)), o1 = part(64 * 16 * sizeof(__nv_bfloat16)),
                  o2 = part(64 * 64 * sizeof(__nv_bfloat16)), o2t = part(64 * 64 * sizeof(__nv_bfloat16)),
                  o3 = part(64 * sizeof(__nv_bfloat16)),
-                 op = part((size_t)num_sms() * kPartStride * sizeof(float)),
-                 olp = part((size_t)num_sms() * sizeof(double)), os = part(2 * sizeof(unsigned)),
+                 op = part((size_t)(kPartFew * num_sms()) * kPartStride * sizeof(float)),
+                 olp = part((size_t)(kPartFew * num_sms()) * sizeof(double)), os = part(2 * sizeof(unsigned)),
                  oc = part(2 * kTrainSteps * sizeof(float));
     if (cudaMalloc(&m->block, at) != cudaSuccess) {
       cudaGetLastError();
@@ -749,6 +774,7 @@ int dcd_mlp_create(uint64_t seed, void* cuda_stream, dcd_mlp** out) {
     m->w3 = reinterpret_cast<__nv_bfloat16*>(m->block + o3);
     m->part = reinterpret_cast<float*>(m->block + op);
     m->lpart = reinterpret_cast<double*>(m->block + olp);
+    m->part_tiles = kPartFew * num_sms();
     m->sync = reinterpret_cast<unsigned*>(m->block + os);
     m->corr = reinterpret_cast<float*>(m->block + oc);
     // He-uniform initialisation from SplitMix64; biases zero
@@ -771,6 +797,7 @@ int dcd_mlp_create(uint64_t seed, void* cuda_stream, dcd_mlp** out) {
 int dcd_mlp_destroy(dcd_mlp* m) {
   if (!m) return DCD_OK;
   cudaStreamSynchronize(m->stream);
+  if (m->more) cudaFree(m->more);
   if (m->block) cudaFree(m->block);
   delete m;
   return DCD_OK;
@@ -832,14 +859,18 @@ int dcd_mlp_train(dcd_mlp* m, const float* d_X, const float* d_y, int64_t n, int
   a.b2 = b2;
   a.eps = eps;
   a.corr = m->corr;
+  const int64_t tiles = cdiv(batch < n ? batch : n, kRowsPerCta);
+  part_room(m, tiles);
+  a.chunk = m->part_tiles;
   a.part = m->part;
   a.lpart = m->lpart;
+  a.grad = m->grad;
   a.loss = m->loss;
   a.bar = m->sync;
   a.err = reinterpret_cast<int*>(m->sync + 1);
   Weights W = weights_of(m);
   Master M{m->P, m->m, m->v, m->w1t, m->w2, m->w2t, m->w3};
-  a.rows = (int)grad_ctas(batch < n ? batch : n);
+  a.rows = (int)grad_ctas(tiles < a.chunk ? tiles : a.chunk);
   // every parameter block a CTA of its own, co-resident (one CTA an SM)
   const unsigned ctas = (unsigned)(a.rows >= kSumBlocks ? a.rows : kSumBlocks < num_sms() ? kSumBlocks : num_sms());
   std::vector<float> corr;
@@ -859,7 +890,7 @@ int dcd_mlp_train(dcd_mlp* m, const float* d_X, const float* d_y, int64_t n, int
     void* args[] = {&W, &M, &a};
     count_launch();
     DCD_TRY_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(mlp_train_steps), dim3(ctas), dim3(128), args,
-                                             sizeof(GradSmem), m->stream));
+                                             kTrainSmem, m->stream));
     DCD_TRY_CUDA(cudaMemcpyAsync(&last, m->loss, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
     DCD_TRY_CUDA(cudaMemcpyAsync(&err, m->sync + 1, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
     DCD_TRY_CUDA(cudaStreamSynchronize(m->stream));
