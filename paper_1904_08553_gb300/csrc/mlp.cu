@@ -499,8 +499,11 @@ __device__ __forceinline__ Moments load_moments(const Master& M, int k) {
 }
 __device__ __forceinline__ void adam_one(const Master& M, int k, const Moments& o, float gk, float lr, float b1,
                                          float b2, float eps, float c1, float c2) {
-  const float mk = b1 * o.m + (1.f - b1) * gk;
-  const float vk = b2 * o.v + (1.f - b2) * gk * gk;
+  // the roundings are spelled out: which product of a sum is fused is otherwise
+  // the compiler's choice, which may change with the code around it, and these
+  // bits decide where a run ends
+  const float mk = __fmaf_rn(1.f - b1, gk, __fmul_rn(b1, o.m));
+  const float vk = __fmaf_rn(__fmul_rn(1.f - b2, gk), gk, __fmul_rn(b2, o.v));
   M.m[k] = mk;
   M.v[k] = vk;
   const float p = o.p - lr * (mk / c1) / (sqrtf(vk / c2) + eps);
