@@ -344,7 +344,10 @@ int dcd_mlp_forward(dcd_mlp* mlp, const float* d_X, int64_t n, float* d_p);
  * (host, DCD_MLP_PARAMS floats; may be NULL); no update. */
 int dcd_mlp_grad(dcd_mlp* mlp, const float* d_X, const float* d_y, int64_t n, float* grad_out, double* loss_out);
 /* epochs passes of Adam over rows [0, n) in consecutive minibatches of
- * `batch` rows (the caller shuffles); *loss_out = last minibatch loss. */
+ * `batch` rows (the caller shuffles); *loss_out = last minibatch loss.  The
+ * steps run in kernels whose CTAs wait for one another, with a limit (about ten
+ * seconds).  Errors: DCD_EINVAL, DCD_ECUDA, DCD_ETIMEOUT (a wait passed its
+ * limit); on error the network, its optimiser state included, is as it was. */
 int dcd_mlp_train(dcd_mlp* mlp, const float* d_X, const float* d_y, int64_t n, int64_t batch, int32_t epochs,
                   float lr, double* loss_out);
 
@@ -437,7 +440,10 @@ int dcd_modularity_noalloc(int64_t n, const int64_t* d_row_ptr, const int32_t* d
  * "cuda:N" the N-th checked CUDA runtime call (DCD_ECUDA, with
  * dcd_last_cuda_error naming the call); "alloc:N,cuda:M" arms both.  The
  * failing call is not made -- the library takes the error path a real
- * failure of that call would take -- and each armed kind fires once.  NULL
+ * failure of that call would take -- and each armed kind fires once.
+ * "wait:N" lets the wait between the CTAs of the N-th training launch
+ * (dcd_mlp_train) run out: it waits, with a limit of milliseconds, for more
+ * CTAs than there are, and the call returns DCD_ETIMEOUT.  NULL
  * or "" disarms.  The environment variable DCD_FAULT, read when the library
  * loads, takes the same spec.  Process-wide; counts from every thread and
  * context.  Errors: DCD_EINVAL (a malformed spec: the armed state is kept). */

@@ -520,16 +520,18 @@ __device__ __forceinline__ void adam_one(const Master& M, int k, const Moments& 
   }
 }
 
-// All CTAs of the (cooperative) grid; false when the wait ran out (it cannot:
-// they are co-resident), after which every CTA leaves.
-__device__ __forceinline__ bool grid_wait(unsigned* bar, unsigned target, int* err) {
+// All CTAs of the (cooperative) grid; false when the wait ran out (they are
+// co-resident and a step's work is evenly dealt, so only a wait made to, or a CTA
+// that is seconds behind, does), after which every CTA leaves.
+constexpr int64_t kWaitPolls = (int64_t)1 << 24;  // about ten seconds
+__device__ __forceinline__ bool grid_wait(unsigned* bar, unsigned target, int64_t polls, int* err) {
   __shared__ int bad;
   __syncthreads();
   if (threadIdx.x == 0) {
     bad = 0;
     __threadfence();
     atomicAdd(bar, 1u);
-    long long left = 1ll << 24;
+    int64_t left = polls;
     unsigned x;
     do {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(bar) : "memory");
@@ -567,9 +569,13 @@ struct TrainArgs {
   double* lpart;
   float* grad;
   double* loss;
+  float* saved;   // not NULL: P, m and v as they are before the first step (kSavedStride floats each)
   unsigned* bar;  // zero
+  unsigned more;  // CTAs waited for that do not exist
+  int64_t polls;
   int* err;
 };
+constexpr int kSavedStride = (NP * 4 + 255) / 256 * 256 / 4;
 constexpr size_t kTrainSmem = sizeof(GradSmem) + sizeof(SumStage);
 __global__ void __launch_bounds__(128) mlp_train_steps(Weights W, Master M, TrainArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -582,7 +588,16 @@ __global__ void __launch_bounds__(128) mlp_train_steps(Weights W, Master M, Trai
     r0 = (st % a.per_epoch) * a.batch;
     nb = r0 + a.batch <= a.n ? a.batch : a.n - r0;
   };
-  unsigned target = 0;
+  if (a.saved)  // before the first wait: what a CTA that leaves there has not touched yet is saved too
+    for (int b = blockIdx.x; b < kSumBlocks; b += G) {
+      const int k = b * kSumBlock + j;
+      const Moments o = load_moments(M, k);
+      if (k >= NP) continue;
+      a.saved[k] = o.p;
+      a.saved[kSavedStride + k] = o.m;
+      a.saved[2 * kSavedStride + k] = o.v;
+    }
+  unsigned target = a.more;
   int64_t r0, nb;
   batch_of(a.s0, r0, nb);
   TileIn in;
@@ -608,7 +623,7 @@ __global__ void __launch_bounds__(128) mlp_train_steps(Weights W, Master M, Trai
         }
       int k = (int)blockIdx.x * kSumBlock + j;
       Moments o = load_moments(M, k);
-      if (!grid_wait(a.bar, target += G, a.err)) return;
+      if (!grid_wait(a.bar, target += G, a.polls, a.err)) return;
       for (int b = blockIdx.x; b < kSumBlocks; b += G) {
         if (b != (int)blockIdx.x) {
           k = b * kSumBlock + j;
@@ -621,7 +636,7 @@ __global__ void __launch_bounds__(128) mlp_train_steps(Weights W, Master M, Trai
       }
       if (st + 1 == a.s1 && blockIdx.x == 0 && threadIdx.x == 0) l = loss_sum(a.lpart, m, l);
       if (last) break;
-      if (!grid_wait(a.bar, target += G, a.err)) return;
+      if (!grid_wait(a.bar, target += G, a.polls, a.err)) return;
     }
     if (st + 1 == a.s1) {
       if (blockIdx.x == 0 && threadIdx.x == 0) *a.loss = l * (1.0 / (double)nb);
@@ -629,7 +644,7 @@ __global__ void __launch_bounds__(128) mlp_train_steps(Weights W, Master M, Trai
     }
     batch_of(st + 1, r0, nb);
     if (works) load_tile(a.X + r0 * NF, a.Y + r0, mine, nb, in);
-    if (!grid_wait(a.bar, target += G, a.err)) return;
+    if (!grid_wait(a.bar, target += G, a.polls, a.err)) return;
   }
 }
 
@@ -655,6 +670,7 @@ struct dcd_mlp {
   unsigned char* more = nullptr;  // allocation for batches of more tiles than block has room for
   unsigned* sync = nullptr;  // [0] the training kernel's barrier, [1] its error word
   float* corr = nullptr;     // Adam's bias corrections of kTrainSteps steps
+  float* saved = nullptr;    // P, m, v before the training run (they lie behind each other in block, as here)
   int64_t adam_t = 0;
 };
 
@@ -760,7 +776,7 @@ int dcd_mlp_create(uint64_t seed, void* cuda_stream, dcd_mlp** out) {
                  o3 = part(64 * sizeof(__nv_bfloat16)),
                  op = part((size_t)(kPartFew * num_sms()) * kPartStride * sizeof(float)),
                  olp = part((size_t)(kPartFew * num_sms()) * sizeof(double)), os = part(2 * sizeof(unsigned)),
-                 oc = part(2 * kTrainSteps * sizeof(float));
+                 oc = part(2 * kTrainSteps * sizeof(float)), ov0 = part(3 * kSavedStride * sizeof(float));
     if (cudaMalloc(&m->block, at) != cudaSuccess) {
       cudaGetLastError();
       rc = DCD_ENOMEM;
@@ -780,6 +796,7 @@ int dcd_mlp_create(uint64_t seed, void* cuda_stream, dcd_mlp** out) {
     m->part_tiles = kPartFew * num_sms();
     m->sync = reinterpret_cast<unsigned*>(m->block + os);
     m->corr = reinterpret_cast<float*>(m->block + oc);
+    m->saved = reinterpret_cast<float*>(m->block + ov0);
     // He-uniform initialisation from SplitMix64; biases zero
     std::vector<float> P(NP, 0.f);
     uint64_t s = seed;
@@ -845,9 +862,12 @@ int dcd_mlp_grad(dcd_mlp* m, const float* d_X, const float* d_y, int64_t n, floa
   return DCD_OK;
 }
 
-int dcd_mlp_train(dcd_mlp* m, const float* d_X, const float* d_y, int64_t n, int64_t batch, int32_t epochs,
-                  float lr, double* loss_out) {
-  if (!m || n <= 0 || batch <= 0 || epochs <= 0 || !d_X || !d_y || !(lr > 0.f)) return DCD_EINVAL;
+}  // extern "C"
+
+namespace {
+// The run of dcd_mlp_train.  *saved: m->saved holds the state from before it.
+int train_run(dcd_mlp* m, const float* d_X, const float* d_y, int64_t n, int64_t batch, int32_t epochs, float lr,
+              double* last, bool* saved) {
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   DCD_TRY(grad_attrs());
   const int64_t per_epoch = cdiv(n, batch), steps = per_epoch * epochs;
@@ -877,7 +897,6 @@ int dcd_mlp_train(dcd_mlp* m, const float* d_X, const float* d_y, int64_t n, int
   // every parameter block a CTA of its own, co-resident (one CTA an SM)
   const unsigned ctas = (unsigned)(a.rows >= kSumBlocks ? a.rows : kSumBlocks < num_sms() ? kSumBlocks : num_sms());
   std::vector<float> corr;
-  double last = 0;
   int err = 0;
   for (int64_t s0 = 0; s0 < steps; s0 += kTrainSteps) {
     a.s0 = s0;
@@ -890,14 +909,46 @@ int dcd_mlp_train(dcd_mlp* m, const float* d_X, const float* d_y, int64_t n, int
     }
     DCD_TRY_CUDA(cudaMemcpyAsync(m->corr, corr.data(), corr.size() * sizeof(float), cudaMemcpyHostToDevice, m->stream));
     DCD_TRY_CUDA(cudaMemsetAsync(m->sync, 0, 2 * sizeof(unsigned), m->stream));
+    const bool stuck = fault_hit(kFaultWait);
+    a.more = stuck ? 1 : 0;
+    a.polls = stuck ? 4096 : kWaitPolls;
+    a.saved = s0 == 0 ? m->saved : nullptr;
     void* args[] = {&W, &M, &a};
     count_launch();
     DCD_TRY_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(mlp_train_steps), dim3(ctas), dim3(128), args,
                                              kTrainSmem, m->stream));
-    DCD_TRY_CUDA(cudaMemcpyAsync(&last, m->loss, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
+    *saved = true;
+    DCD_TRY_CUDA(cudaMemcpyAsync(last, m->loss, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
     DCD_TRY_CUDA(cudaMemcpyAsync(&err, m->sync + 1, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
     DCD_TRY_CUDA(cudaStreamSynchronize(m->stream));
     if (err) return DCD_ETIMEOUT;
+  }
+  return DCD_OK;
+}
+
+// The network as it was before a run that failed.
+void train_undo(dcd_mlp* m, int64_t adam_t, bool saved) {
+  m->adam_t = adam_t;
+  if (saved) {
+    cudaMemcpyAsync(m->P, m->saved, 3 * kSavedStride * sizeof(float), cudaMemcpyDeviceToDevice, m->stream);
+    count_launch(), prepare<<<16, 256, 0, m->stream>>>(m->P, m->w1t, m->w2, m->w2t, m->w3);
+  }
+  cudaStreamSynchronize(m->stream);
+}
+}  // namespace
+
+extern "C" {
+
+int dcd_mlp_train(dcd_mlp* m, const float* d_X, const float* d_y, int64_t n, int64_t batch, int32_t epochs,
+                  float lr, double* loss_out) {
+  if (!m || n <= 0 || batch <= 0 || epochs <= 0 || !d_X || !d_y || !(lr > 0.f)) return DCD_EINVAL;
+  const int64_t adam_t = m->adam_t;
+  double last = 0;
+  bool saved = false;
+  const int rc = train_run(m, d_X, d_y, n, batch, epochs, lr, &last, &saved);
+  if (rc != DCD_OK) {
+    train_undo(m, adam_t, saved);
+    return rc;
   }
   if (loss_out) *loss_out = last;
   return DCD_OK;
