@@ -443,7 +443,9 @@ int dcd_modularity_noalloc(int64_t n, const int64_t* d_row_ptr, const int32_t* d
  * failure of that call would take -- and each armed kind fires once.
  * "wait:N" lets the wait between the CTAs of the N-th training launch
  * (dcd_mlp_train) run out: it waits, with a limit of milliseconds, for more
- * CTAs than there are, and the call returns DCD_ETIMEOUT.  NULL
+ * CTAs than there are, and the call returns DCD_ETIMEOUT.  "grid:N" refuses,
+ * until it is disarmed, training launches of more than N CTAs as too large to
+ * run at once (as a part of a GPU does); the library then launches fewer.  NULL
  * or "" disarms.  The environment variable DCD_FAULT, read when the library
  * loads, takes the same spec.  Process-wide; counts from every thread and
  * context.  Errors: DCD_EINVAL (a malformed spec: the armed state is kept). */

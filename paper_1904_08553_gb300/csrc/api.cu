@@ -25,7 +25,7 @@ bool fault_fire(int kind) {
 }
 
 namespace {
-// "alloc:N,cuda:M,wait:K" (any of them, or empty = disarmed); N, M, K >= 1
+// "alloc:N,cuda:M,wait:K,grid:J" (any of them, or empty = disarmed), all >= 1
 int parse_fault(const char* spec, int64_t left[kFaultKinds]) {
   for (int k = 0; k < kFaultKinds; k++) left[k] = 0;
   if (!spec) return DCD_OK;
@@ -37,6 +37,7 @@ int parse_fault(const char* spec, int64_t left[kFaultKinds]) {
     const int kind = (len == 5 && !strncmp(p, "alloc", 5)) ? kFaultAlloc
                      : (len == 4 && !strncmp(p, "cuda", 4)) ? kFaultCuda
                      : (len == 4 && !strncmp(p, "wait", 4)) ? kFaultWait
+                     : (len == 4 && !strncmp(p, "grid", 4)) ? kFaultGrid
                                                              : -1;
     if (kind < 0) return DCD_EINVAL;
     char* end = nullptr;

@@ -32,8 +32,9 @@ void note_cuda_error(cudaError_t e, const char* what, const char* file, int line
 // for tests of the error paths: an armed kind counts its events -- device
 // allocations, checked CUDA calls, training launches (whose grid-wide wait then
 // runs out) -- and the N-th one reports failure instead of being made.  Disarmed,
-// the cost is one relaxed load per event.
-enum FaultKind : int { kFaultAlloc = 0, kFaultCuda, kFaultWait, kFaultKinds };
+// the cost is one relaxed load per event.  kFaultGrid counts nothing: it is the
+// most CTAs a training launch may have.
+enum FaultKind : int { kFaultAlloc = 0, kFaultCuda, kFaultWait, kFaultGrid, kFaultKinds };
 extern std::atomic<int64_t> g_fault_left[kFaultKinds];
 bool fault_fire(int kind);
 inline bool fault_hit(int kind) {

@@ -895,7 +895,7 @@ int train_run(dcd_mlp* m, const float* d_X, const float* d_y, int64_t n, int64_t
   Master M{m->P, m->m, m->v, m->w1t, m->w2, m->w2t, m->w3};
   a.rows = (int)grad_ctas(tiles < a.chunk ? tiles : a.chunk);
   // every parameter block a CTA of its own, co-resident (one CTA an SM)
-  const unsigned ctas = (unsigned)(a.rows >= kSumBlocks ? a.rows : kSumBlocks < num_sms() ? kSumBlocks : num_sms());
+  unsigned ctas = (unsigned)(a.rows >= kSumBlocks ? a.rows : kSumBlocks < num_sms() ? kSumBlocks : num_sms());
   std::vector<float> corr;
   int err = 0;
   for (int64_t s0 = 0; s0 < steps; s0 += kTrainSteps) {
@@ -913,10 +913,25 @@ int train_run(dcd_mlp* m, const float* d_X, const float* d_y, int64_t n, int64_t
     a.more = stuck ? 1 : 0;
     a.polls = stuck ? 4096 : kWaitPolls;
     a.saved = s0 == 0 ? m->saved : nullptr;
-    void* args[] = {&W, &M, &a};
+    // a stream that has fewer SMs than the device reports (a partition of it) refuses
+    // the grid: any smaller one gives the same results
+    auto launch = [&] {
+      for (;;) {
+        void* args[] = {&W, &M, &a};
+        const int64_t most = g_fault_left[kFaultGrid].load(std::memory_order_relaxed);
+        const cudaError_t e =
+            most > 0 && (int64_t)ctas > most
+                ? cudaErrorCooperativeLaunchTooLarge
+                : cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(mlp_train_steps), dim3(ctas), dim3(128),
+                                              args, kTrainSmem, m->stream);
+        if (e != cudaErrorCooperativeLaunchTooLarge || ctas == 1) return e;
+        cudaGetLastError();
+        ctas /= 2;
+        if (a.rows > (int)ctas) a.rows = (int)ctas;
+      }
+    };
     count_launch();
-    DCD_TRY_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(mlp_train_steps), dim3(ctas), dim3(128), args,
-                                             kTrainSmem, m->stream));
+    DCD_TRY_CUDA(launch());
     *saved = true;
     DCD_TRY_CUDA(cudaMemcpyAsync(last, m->loss, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
     DCD_TRY_CUDA(cudaMemcpyAsync(&err, m->sync + 1, sizeof(int), cudaMemcpyDeviceToHost, m->stream));

@@ -300,7 +300,7 @@ def dcd_get_screen_data(h, X_out=None, y_out=None, vertex_out=None, cap: int = 0
 
 
 def dcd_set_fault(spec: str | None) -> None:
-    """Arm host-side fault injection ("alloc:N", "cuda:N", "wait:N", comma-separated; None or "" disarms)."""
+    """Arm host-side fault injection ("alloc:N", "cuda:N", "wait:N", "grid:N", comma-separated; None or "" disarms)."""
     _check(lib().dcd_set_fault(None if spec is None else spec.encode()), "dcd_set_fault")
 
 

@@ -84,3 +84,23 @@ def test_launches_share_one_run():
     for a, b in ((0, 2000), (2000, 4096), (4096, N)):
         two.train(dX[a:b].contiguous(), dy[a:b].contiguous(), b - a, batch=1, epochs=1, lr=1e-3)
     assert np.array_equal(one.params, two.params)
+
+
+@pytest.mark.parametrize("n,batch,most", [(3000, 1000, 79), (30_000, 10_000, 100), (30_000, 10_000, 1), (64, 64, 3)])
+def test_a_grid_too_large_for_the_device_is_made_smaller(n, batch, most):
+    """On a part of the GPU fewer CTAs run at once: the launch is refused, and half as many, down to
+    one, end in the same parameters."""
+    from paper_1904_08553_gb300 import dcd
+
+    rng = np.random.default_rng(n)
+    X = rng.standard_normal((n, 12)).astype(np.float32)
+    y = (X[:, 2] > X[:, 5]).astype(np.float32)
+    dX, dy = torch.from_numpy(X).cuda(), torch.from_numpy(y).cuda()
+    net, ref = dcd.Mlp(seed=4), dcd.Mlp(seed=4)
+    ref.train(dX, dy, n, batch=batch, epochs=2, lr=1e-3)
+    try:
+        dcd.dcd_set_fault(f"grid:{most}")
+        assert net.train(dX, dy, n, batch=batch, epochs=2, lr=1e-3) > 0
+    finally:
+        dcd.dcd_set_fault(None)
+    assert np.array_equal(net.params, ref.params)
