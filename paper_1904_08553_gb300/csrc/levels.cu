@@ -406,7 +406,9 @@ int launch_levels(dcd_ctx* c, LevelsArgs p, int G, int64_t cells, Buf<VT>& E) {
     DCD_TRY(E.alloc(&c->mem, cells));
     p.E = E.get();
   }
-  DCD_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  // the attribute belongs to the process: always the same value, so that another
+  // thread's context cannot lower it between this and the launch
+  DCD_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLevelSmem));
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(G * CL));
   cfg.blockDim = dim3(kLvThreads);
