@@ -3390,6 +3390,7 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
 
   // ---- compose + canonical labels (smallest member id) ----
   DCD_TRY_CUDA(cudaEventRecord(c->ev[7], s));
+  bool kept = false;
   {
     Buf<int32_t> minid;
     DCD_TRY(minid.alloc(&c->mem, nvu + iso));
@@ -3400,9 +3401,11 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
                                                                        out_labels, gid0, gs);
     DCD_LAUNCH_CHECK();
     DCD_TRY_CUDA(cudaEventRecord(c->ev[8], s));
-    // the coarse graph of the result, for the next update (with few
-    // communities before their number is read back: sized by the level's)
-    if (G == 1 && ran_dense) DCD_TRY(n1_keep(c, n0, out_labels, c->n1.h0_nc, iso));
+    // the coarse graph of the result, for the next update: with few communities
+    // before their number is read back, sized by the level's (to 24 MB); else by
+    // the number (level 0's up to 4096 would keep 168 MB in each of two buffers)
+    kept = G == 1 && ran_dense && c->n1.h0_nc <= kLevelNc;
+    if (kept) DCD_TRY(n1_keep(c, n0, out_labels, c->n1.h0_nc, iso));
     std::vector<uint8_t> ran(G, 0);  // graphs whose levels the one launch finished
     if (ran_dense) {
       for (int x = 0; x < G; x++) ran[x] = !c->hgs[x].done;
@@ -3440,7 +3443,7 @@ int run_louvain(dcd_ctx* c, const Csr<int32_t>& g0, int32_t* labels0, const uint
     }
   }
   if (G == 1) {
-    if (!ran_dense) DCD_TRY(n1_keep(c, n0, out_labels, c->hgs[0].ncomm - iso, iso));
+    if (!kept) DCD_TRY(n1_keep(c, n0, out_labels, c->hgs[0].ncomm - iso, iso));
     c->kc_n_nx = c->hgs[0].ncomm - iso;
   }
   float tf = 0.f;
