@@ -2736,8 +2736,10 @@ int dense_matrix(dcd_ctx* c, const Csr<W>& g, const int32_t* ccid, int64_t nc, c
   }
   if (m0 > 0) {
     const uint32_t* rb = blocks ? blocks->rowbase.get() : nullptr;
-    // a CTA copy of the matrix when it fits in shared memory (two CTAs an SM)
-    const size_t msm = (size_t)cells * sizeof(VT);
+    // a CTA copy of the matrix when it fits in shared memory (two CTAs an SM); in
+    // steps of 8 KB, so that the occupancy lookups it is the key of stay a dozen
+    // whatever sizes a stream of updates brings
+    const size_t msm = ((size_t)cells * sizeof(VT) + 8191) / 8192 * 8192;
     if (msm <= kDenseSmem) {
       DCD_TRY_CUDA(cudaFuncSetAttribute(emit_dense<W, VT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)kDenseSmem));
