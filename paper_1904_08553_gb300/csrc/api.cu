@@ -565,14 +565,21 @@ int dcd::update_impl(dcd_ctx* c, dcd_step_stats* st, dcd_step_stats* per_graph, 
   const bool collect = c->collect && !first;
   const bool screen = mode == DCD_MODE_DELTA || learned || collect;
   SourceBins sb;
-  if (screen) DCD_TRY(source_counts(c, c->rp[nxt].get(), mo.pair_ptr.get(), &sb));
-  DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 8, c->rp[nxt].get() + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  DCD_TRY_CUDA(cudaMemcpyAsync(c->hsc, d, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
-  DCD_TRY_CUDA(cudaMemcpyAsync(c->hgs, c->gs.get(), c->G * sizeof(GraphState), cudaMemcpyDeviceToHost, s));
-  DCD_TRY_CUDA(cudaEventRecord(c->ev[1], s));
-  DCD_TRY_CUDA(cudaStreamSynchronize(s));
+  for (bool again = false;;) {
+    if (screen) DCD_TRY(source_counts(c, c->rp[nxt].get(), mo.pair_ptr.get(), &sb));
+    DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch + 8, c->rp[nxt].get() + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    DCD_TRY_CUDA(cudaMemcpyAsync(c->hsc, d, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
+    DCD_TRY_CUDA(cudaMemcpyAsync(c->hgs, c->gs.get(), c->G * sizeof(GraphState), cudaMemcpyDeviceToHost, s));
+    DCD_TRY_CUDA(cudaEventRecord(c->ev[1], s));
+    DCD_TRY_CUDA(cudaStreamSynchronize(s));
+    if (c->hsc->err & kErrBadRecord) return DCD_EINVAL;
+    if (again || c->hsc->n_long == 0) break;
+    // sources with more records than a CTA sorts
+    DCD_TRY(merge_long(c, src_labels, mode == DCD_MODE_STATIC, c->hsc->n_long, &mo, merge_labels ? &nlab : nullptr));
+    again = true;
+  }
+  mo.done();
   trace("update: merge done");
-  if (c->hsc->err & kErrBadRecord) return DCD_EINVAL;
   if (c->hsc->err & kErrOverflow) return DCD_EOVERFLOW;
   for (int x = 0; x < c->G; x++)
     if (c->hgs[x].m2 < 0 || c->hgs[x].m2 >= ((int64_t)1 << 62)) return DCD_EOVERFLOW;

@@ -179,10 +179,12 @@ __device__ __forceinline__ void pair_sums_add(const PairView& o, int g, PairSum&
 }
 
 // Segments of at most kSegSmall records are ranked by pair_tile; of at most
-// kSegMid by a CTA each in shared memory (rank); of at most kSegLarge by a
-// CTA each with a bitonic network; longer ones by a CTA's radix sort in
-// global memory.
-constexpr int kSegSmall = 64, kSegMid = 512, kSegLarge = 4096;
+// kSegMid and kSegLarge by a CTA each with a bitonic network in shared memory; of
+// at most kSegHuge by a CTA's radix sort in global memory.  Longer ones (a batch centred on one vertex, or one that repeats an edge) are
+// only counted on the way (DevScalars::n_long): the rows are then not merged, and
+// when the host has read the count, merge_long sorts them over the whole device
+// and merges.  The usual batch has none and pays nothing for them.
+constexpr int kSegSmall = 64, kSegMid = 512, kSegLarge = 4096, kSegHuge = 32768;
 
 // A CTA takes NS consecutive sources: their records (a counting sort put them
 // next to each other) and the columns of their rows are staged in shared memory
@@ -212,7 +214,8 @@ template <int NS>
 __global__ void __launch_bounds__(kPairThreads, 12) pair_tile(PairView o, int64_t n, const uint64_t* __restrict__ rec,
                                                               const int64_t* __restrict__ k_old,
                                                               int64_t* __restrict__ k_new, int32_t* __restrict__ big,
-                                                              int32_t* __restrict__ big_cnt) {
+                                                              int32_t* __restrict__ big_cnt,
+                                                              int32_t* __restrict__ n_long) {
   static_assert(NS <= kPairThreads, "a thread a source");
   __shared__ uint32_t s_v[kPairRecs], s_w[kPairRecs];  // sinks and weights of the staged records
   __shared__ uint16_t s_perm[kPairRecs];               // record that comes x-th
@@ -238,7 +241,9 @@ __global__ void __launch_bounds__(kPairThreads, 12) pair_tile(PairView o, int64_
     const int small = len <= kSegSmall ? len : 0;
     if (len > kSegSmall) {
       const int c = len <= kSegMid ? 0 : len <= kSegLarge ? 1 : 2;
-      big[(int64_t)c * n + atomicAdd(&big_cnt[c], 1)] = (int32_t)(v0 + tid);
+      // (merge_long's sources at the end of the third list)
+      const int64_t at = len <= kSegHuge ? (int64_t)c * n + atomicAdd(&big_cnt[c], 1) : 3 * n - 1 - atomicAdd(n_long, 1);
+      big[at] = (int32_t)(v0 + tid);
     }
     int nrec;
     const int a0 = block_excl_scan<int, kPairThreads>(small, &nrec);
@@ -378,20 +383,52 @@ __device__ __forceinline__ void segment_out(const PairView& o, int32_t u, const 
 }
 
 // The pairs of a sorted segment s[0 .. len) of source u at place a; s_col: the
-// row of u in shared memory (may be NULL).
+// row of u in shared memory (may be NULL).  A record a thread, whole warps: the
+// last of a run of equal sinks walks back over it, and what is left of a run of
+// more than kRunWalk is summed by the warp (an edge repeated 20,000 times in a
+// batch: RUN_FIGURES).
+constexpr int kRunWalk = 32;
 template <typename P>
 __device__ __forceinline__ void put_sorted(const PairView& o, int32_t u, int64_t a, int len, const P* s, int tid,
                                            int NT, PairSum& acc, const int32_t* s_col = nullptr) {
-  for (int x = tid; x < len; x += NT) {
-    const uint32_t v = (uint32_t)(s[x] >> 32);
-    const bool head = x + 1 == len || (uint32_t)(s[x + 1] >> 32) != v;
+  const int lane = lane_id();
+  for (int x0 = tid & ~31; x0 < len; x0 += NT) {
+    const int x = x0 + lane;
+    const uint32_t v = x < len ? (uint32_t)(s[x] >> 32) : 0u;
+    const bool head = x < len && (x + 1 == len || (uint32_t)(s[x + 1] >> 32) != v);
     int64_t W = 0;
     bool isdel = false;
-    if (head)
-      for (int j = x; j >= 0 && (uint32_t)(s[j] >> 32) == v; j--) {
+    int left = 0;  // records of the run before those walked over end here
+    if (head) {
+      int j = x;
+      for (; j >= 0 && x - j < kRunWalk && (uint32_t)(s[j] >> 32) == v; j--) {
         W += (int64_t)(uint32_t)s[j];
         isdel |= (uint32_t)s[j] == 0;
       }
+      if (x - j == kRunWalk && j >= 0 && (uint32_t)(s[j] >> 32) == v) left = j + 1;
+    }
+    for (unsigned more = __ballot_sync(0xffffffffu, left > 0); more; more &= more - 1) {
+      const int who = __ffs(more) - 1, end = __shfl_sync(0xffffffffu, left, who);
+      const uint32_t vw = __shfl_sync(0xffffffffu, v, who);
+      int lo = 0, hi = end;  // first record of the run
+      while (lo < hi) {
+        const int m = (lo + hi) >> 1;
+        if ((uint32_t)(s[m] >> 32) < vw) lo = m + 1; else hi = m;
+      }
+      unsigned long long sum = 0;
+      bool del = false;
+      for (int j = lo + lane; j < end; j += 32) {
+        sum += (unsigned long long)(uint32_t)s[j];
+        del |= (uint32_t)s[j] == 0;
+      }
+      sum = warp_sum(sum);
+      del = __any_sync(0xffffffffu, del);
+      if (lane == who) {
+        W += (int64_t)sum;
+        isdel |= del;
+      }
+    }
+    if (x >= len) continue;
     if (s_col) {
       const int n = (int)(o.rp[u + 1] - o.rp[u]);
       const int q = lower_bound_col<int>(s_col, 0, n, (int32_t)v);
@@ -540,6 +577,112 @@ __global__ void __launch_bounds__(kHugeThreads) pair_huge(PairView o, uint64_t* 
   }
 }
 
+// ---- segments above kSegHuge (merge_long) ----
+//
+// Their records are copied to one array, keyed by (place in the list of these
+// sources, sink), sorted by the device-wide radix sort, and a record a thread
+// becomes a pair: the last of a run of equal sinks takes the run's weights as a
+// difference of their prefix sums, so neither a long segment nor a long run of one
+// pair is ever one thread's or one CTA's work.
+// 1 M records on one source: the merge takes 1.2 ms so and 9.7 with a CTA's radix
+// sort in global memory (0.26 when they are spread); 1 M records of one pair 1.1 and
+// 87.  A CTA's sort is the faster one to
+// about 30 K records (20 K: 0.33 against 0.39 ms; 65 K: 0.76 and 0.47).
+
+__global__ void long_sizes(const int32_t* __restrict__ list, int64_t n_long, const int32_t* __restrict__ off,
+                           int64_t* __restrict__ len) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= n_long; i += (int64_t)gridDim.x * blockDim.x)
+    len[i] = i < n_long ? off[list[i] + 1] - off[list[i]] : 0;
+}
+
+__global__ void long_keys(const int32_t* __restrict__ list, int64_t n_long, const int64_t* __restrict__ first,
+                          const int32_t* __restrict__ off, const uint64_t* __restrict__ rec, int64_t T,
+                          uint64_t* __restrict__ key, uint32_t* __restrict__ val) {
+  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < T; x += (int64_t)gridDim.x * blockDim.x) {
+    int64_t lo = 0, hi = n_long - 1;  // last segment that starts at or before x
+    while (lo < hi) {
+      const int64_t mid = (lo + hi + 1) >> 1;
+      if (first[mid] <= x) lo = mid; else hi = mid - 1;
+    }
+    const uint64_t r = rec[off[list[lo]] + (x - first[lo])];
+    key[x] = (uint64_t)lo << 32 | r >> 32;
+    val[x] = (uint32_t)r;
+  }
+}
+
+// Weights and deletes of the sorted records, to be scanned.
+__global__ void long_terms(const uint32_t* __restrict__ val, int64_t T, int64_t* __restrict__ ws,
+                           int32_t* __restrict__ ds) {
+  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x <= T; x += (int64_t)gridDim.x * blockDim.x) {
+    ws[x] = x < T ? (int64_t)val[x] : 0;
+    ds[x] = x < T && val[x] == 0 ? 1 : 0;
+  }
+}
+
+// The pairs, a warp per kLongChunk sorted records; the sums of a chunk within one
+// segment are added once.
+constexpr int kLongChunk = 1024;
+__global__ void __launch_bounds__(256) long_pairs(PairView o, const int32_t* __restrict__ list,
+                                                  const int64_t* __restrict__ first, const uint64_t* __restrict__ key,
+                                                  const int64_t* __restrict__ ws, const int32_t* __restrict__ ds,
+                                                  int64_t T, int64_t* __restrict__ k_new) {
+  const int lane = lane_id();
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t c0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * kLongChunk; c0 < T; c0 += nw * kLongChunk) {
+    const int64_t c1 = c0 + kLongChunk < T ? c0 + kLongChunk : T;
+    PairSum acc;
+    auto add = [&](int32_t u, unsigned long long m2, unsigned long long in, unsigned heads) {
+      GraphState& gs = o.gs[graph_of(o.gid, u)];
+      if (m2) {
+        atomicAdd((unsigned long long*)&k_new[u], m2);
+        atomicAdd((unsigned long long*)&gs.m2, m2);
+      }
+      if (in) atomicAdd((unsigned long long*)&gs.in_cur, in);
+      if (heads) atomicAdd((unsigned long long*)o.npairs, (unsigned long long)heads);
+    };
+    const bool one = key[c0] >> 32 == key[c1 - 1] >> 32;  // the chunk lies in one segment
+    for (int64_t x0 = c0; x0 < c1; x0 += 32) {
+      const int64_t x = x0 + lane;
+      if (x < c1) {
+        const uint64_t kx = key[x];
+        const int64_t i = (int64_t)(kx >> 32);
+        const int32_t u = list[i];
+        const uint32_t v = (uint32_t)kx;
+        const bool head = x + 1 == T || key[x + 1] != kx;
+        int64_t W = 0;
+        bool isdel = false;
+        if (head) {
+          int64_t lo = first[i], hi = x;  // first record of the run
+          while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (key[mid] < kx) lo = mid + 1; else hi = mid;
+          }
+          W = ws[x + 1] - ws[lo];
+          isdel = ds[x + 1] != ds[lo];
+        }
+        put_searched(o, o.off[u] + (x - first[i]), u, v, W, isdel, head, acc);
+        if (!one) {
+          add(u, (unsigned long long)acc.m2, (unsigned long long)acc.in, (unsigned)acc.heads);
+          acc = PairSum();
+        }
+      }
+    }
+    if (one) {
+      const unsigned long long m2 = warp_sum((unsigned long long)acc.m2), in = warp_sum((unsigned long long)acc.in);
+      const unsigned heads = __reduce_add_sync(0xffffffffu, (unsigned)acc.heads);
+      if (lane == 0) add(list[key[c0] >> 32], m2, in, heads);
+    }
+  }
+}
+
+// The entries every pair adds or removes, again (the scan took them).
+__global__ void pair_net(const uint8_t* __restrict__ pflag, int64_t R, int32_t* __restrict__ net) {
+  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p <= R; p += (int64_t)gridDim.x * blockDim.x) {
+    const uint8_t f = p < R ? pflag[p] : 0;
+    net[p] = f & kPairAdded ? 1 : f & kPairRemoved ? -1 : 0;
+  }
+}
+
 // sum_i e_{i->C(i)} and 2m of G_{t-1} per graph (kept by the previous update:
 // prev[g], prev[G + g]); with_in: the former is tracked through the merge.
 __global__ void seed_sums(GraphState* __restrict__ gs, int G, const int64_t* __restrict__ prev, int with_in) {
@@ -569,7 +712,9 @@ __global__ void row_degrees(int64_t n, const int64_t* __restrict__ rp, const int
 // labels set by the caller, a loaded checkpoint).
 __global__ void in_weight(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
                           const int32_t* __restrict__ w, const int32_t* __restrict__ L,
-                          const int32_t* __restrict__ gid, GraphState* __restrict__ gs) {
+                          const int32_t* __restrict__ gid, GraphState* __restrict__ gs,
+                          const int32_t* __restrict__ n_long) {
+  if (*n_long) return;  // the rows are not merged yet
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int cur = 0;
   unsigned long long acc = 0;
@@ -614,16 +759,17 @@ __global__ void new_rows(const int64_t* __restrict__ rp_o, const int32_t* __rest
 
 // Pairs before merged item t * kMergeTile.  *npair: the pairs there are (fewer
 // than the batch's records when bad records took no place; the update then
-// fails, but stays within its buffers).
+// fails, but stays within its buffers).  While segments are left to merge_long
+// (*n_long), their pairs hold nothing yet: -1, and merge_tile leaves.
 __global__ void merge_split(const int64_t* __restrict__ epos, const int32_t* __restrict__ npair, int64_t nt,
-                            int32_t* __restrict__ sq) {
-  const int64_t P = *npair;
+                            int32_t* __restrict__ sq, const int32_t* __restrict__ n_long) {
+  const int64_t P = *n_long ? -1 : *npair;
   const int lane = lane_id();
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   // a warp a tile: 32 probes a step, so that the chain is log32 of the pairs
   for (int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; t <= nt; t += nw) {
     const int64_t d = t * kMergeTile;
-    int64_t lo = 0, hi = P < d ? P : d;  // first q with q + epos[q] >= d
+    int64_t lo = P < 0 ? -1 : 0, hi = P < d ? P : d;  // first q with q + epos[q] >= d
     while (lo < hi) {
       const int64_t step = (hi - lo + 31) / 32, q = lo + lane * step;
       const unsigned below = __ballot_sync(0xffffffffu, q < hi && q + epos[q] < d);  // a prefix of the lanes
@@ -667,6 +813,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_tile(
   const int tid = threadIdx.x;
   const int64_t t = blockIdx.x;
   const int32_t q0 = sq[t], q1 = sq[t + 1];
+  if (q0 < 0) return;
   const int64_t e0 = t * kMergeTile - q0;
   const int64_t e1x = (t + 1) * kMergeTile - q1;
   const int64_t e1 = e1x < nnz ? e1x : nnz;
@@ -777,6 +924,66 @@ int validate_batch(dcd_ctx* c, const dcd_edge* ins, int64_t n_ins, const dcd_edg
   return DCD_OK;
 }
 
+namespace {
+
+PairView pair_view(dcd_ctx* c, const int32_t* labels0, const MergeOut& m) {
+  const int cur = c->cur;
+  DevScalars* d = c->dsc.get();
+  return PairView{m.pair_ptr.get(), c->rp[cur].get(), c->col[cur].get(), c->w[cur].get(),
+                  m.track_in ? labels0 : nullptr, c->G > 1 ? c->gid.get() : nullptr, m.pkey.get(), m.pw.get(),
+                  m.pflag.get(), m.pdelta.get(), m.epos.get(), m.S.get(), c->gs.get(), &d->npairs, &d->err};
+}
+
+// G_t's rows from G_{t-1}'s and the pairs (nothing but the row starts while segments are left to merge_long).
+int merge_rows(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut* out, EntryLabels* nlab) {
+  cudaStream_t s = c->stream;
+  const int64_t n = c->n, R = out->npairs, n_ins = c->n_ins;
+  DevScalars* d = c->dsc.get();
+  const int T = 256;
+  const int cur = c->cur, nxt = 1 - c->cur;
+  const int64_t* rp_o = c->rp[cur].get();
+  const int32_t* col_o = c->col[cur].get();
+  const int32_t* w_o = c->w[cur].get();
+  const int32_t* gid = c->G > 1 ? c->gid.get() : nullptr;
+  const int32_t* off = out->pair_ptr.get();
+  Buf<int64_t>& epos = out->epos;
+  Buf<int32_t>& S = out->S;
+  Buf<int32_t> stmp;
+  DCD_TRY(stmp.alloc(&c->mem, scan_tmp_count(R + 1)));
+  DCD_TRY(exclusive_scan<int32_t>(S.get(), S.get(), R + 1, nullptr, stmp.get(), s));
+
+  // ---- new row pointers, merge ----
+  const int64_t cap = c->nnz + 2 * n_ins;
+  DCD_TRY(c->rp[nxt].ensure(&c->mem, n + 1));
+  DCD_TRY(c->col[nxt].ensure(&c->mem, cap));
+  DCD_TRY(c->w[nxt].ensure(&c->mem, cap));
+  int64_t* rp_n = c->rp[nxt].get();
+  ::dcd::count_launch(), new_rows<<<grid_for(n + 1, T), T, 0, s>>>(rp_o, off, S.get(), n, rp_n);
+  DCD_LAUNCH_CHECK();
+  const int64_t nt = cdiv(c->nnz + R, (int64_t)kMergeTile);
+  if (nt > 0) {
+    Buf<int32_t> split;
+    DCD_TRY(split.alloc(&c->mem, nt + 1));
+    ::dcd::count_launch(), merge_split<<<grid_for((nt + 1) * 32, T), T, 0, s>>>(epos.get(), off + n, nt, split.get(),
+                                                                              &d->n_long);
+    DCD_LAUNCH_CHECK();
+    if (nlab && nlab->buf.n < (size_t)cap) DCD_TRY(nlab->buf.alloc(&c->mem, cap));
+    ::dcd::count_launch(), (nlab ? merge_tile<true> : merge_tile<false>)<<<(unsigned)nt, kMergeThreads, 0, s>>>(
+        c->nnz, col_o, w_o, split.get(), epos.get(), out->pkey.get(), out->pdelta.get(), out->pflag.get(), S.get(),
+        c->col[nxt].get(), c->w[nxt].get(), static_start ? nullptr : labels0, nlab ? nlab->buf.get() : nullptr);
+    DCD_LAUNCH_CHECK();
+    if (nlab) nlab->ready = true;
+  }
+  if (!static_start && !c->in_valid && c->cfg.alg == DCD_ALG_LOUVAIN) {
+    ::dcd::count_launch(), in_weight<<<grid_for(n * 32, T), T, 0, s>>>(n, rp_n, c->col[nxt].get(), c->w[nxt].get(),
+                                                                        labels0, gid, c->gs.get(), &d->n_long);
+    DCD_LAUNCH_CHECK();
+  }
+  return DCD_OK;
+}
+
+}  // namespace
+
 int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut* out, EntryLabels* nlab) {
   cudaStream_t s = c->stream;
   const int64_t n = c->n;
@@ -815,19 +1022,20 @@ int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut*
 
   // ---- records by source ----
   Buf<int2> rank;
-  Buf<uint64_t> rec, rec2;
-  Buf<int32_t> stmp, big;
+  Buf<uint64_t> rec2;
+  Buf<int32_t> stmp;
+  Buf<uint64_t>& rec = out->rec;
+  Buf<int32_t>& big = out->big;
   out->npairs = R;
   DCD_TRY(out->pair_ptr.alloc(&c->mem, n + 4));  // + 3: the counts of the long segments' lists
   DCD_TRY(out->pkey.alloc(&c->mem, R));
   DCD_TRY(out->pw.alloc(&c->mem, R));
   DCD_TRY(out->pflag.alloc(&c->mem, R));
   DCD_TRY(out->pdelta.alloc(&c->mem, R));
-  DCD_TRY(stmp.alloc(&c->mem, scan_tmp_count(n + 1) + scan_tmp_count(R + 1)));
-  Buf<int64_t> epos;
-  Buf<int32_t> S;
-  DCD_TRY(epos.alloc(&c->mem, R));
-  DCD_TRY(S.alloc(&c->mem, R + 1));
+  DCD_TRY(stmp.alloc(&c->mem, scan_tmp_count(n + 1)));
+  DCD_TRY(out->epos.alloc(&c->mem, R));
+  DCD_TRY(out->S.alloc(&c->mem, R + 1));
+  Buf<int32_t>& S = out->S;
   int32_t* off = out->pair_ptr.get();
   int32_t* big_cnt = off + n + 1;
   DCD_TRY_CUDA(cudaMemsetAsync(off, 0, (n + 4) * sizeof(int32_t), s));
@@ -845,14 +1053,14 @@ int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut*
                                                                       rank.get(), rec.get());
     DCD_LAUNCH_CHECK();
   }
-  PairView o{off, rp_o, col_o, w_o, from_prev ? labels0 : nullptr, gid, out->pkey.get(), out->pw.get(),
-             out->pflag.get(), out->pdelta.get(), epos.get(), S.get(), c->gs.get(), &d->npairs, &d->err};
+  out->track_in = from_prev;
+  const PairView o = pair_view(c, labels0, *out);
   if (R > 0) {
     // sources a CTA: about 64 records for its 128 threads (pair_tile)
     const int ns = R >= 2 * n || n < kPairWide ? 32 : 2 * R >= n ? 64 : 128;
     auto* tile = ns == 32 ? pair_tile<32> : ns == 64 ? pair_tile<64> : pair_tile<128>;
     ::dcd::count_launch(), tile<<<(unsigned)cdiv(n, ns), kPairThreads, 0, s>>>(
-        o, n, rec.get(), c->kdeg[cur].get(), out->k->get(), big.get(), big_cnt);
+        o, n, rec.get(), c->kdeg[cur].get(), out->k->get(), big.get(), big_cnt, &d->n_long);
     // a segment holds at most one record per batch record: the classes the
     // batch is too small for are not launched
     if (nr > kSegSmall)
@@ -871,35 +1079,57 @@ int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut*
   ::dcd::count_launch(), seed_sums<<<cdiv(c->G, 128), 128, 0, s>>>(c->gs.get(), c->G, c->in_prev.get(),
                                                                     from_prev ? 1 : 0);
   DCD_LAUNCH_CHECK();
-  DCD_TRY(exclusive_scan<int32_t>(S.get(), S.get(), R + 1, nullptr, stmp.get(), s));
+  return merge_rows(c, labels0, static_start, out, nlab);
+}
 
-  // ---- new row pointers, merge ----
-  const int64_t cap = c->nnz + 2 * n_ins;
-  DCD_TRY(c->rp[nxt].ensure(&c->mem, n + 1));
-  DCD_TRY(c->col[nxt].ensure(&c->mem, cap));
-  DCD_TRY(c->w[nxt].ensure(&c->mem, cap));
-  int64_t* rp_n = c->rp[nxt].get();
-  ::dcd::count_launch(), new_rows<<<grid_for(n + 1, T), T, 0, s>>>(rp_o, off, S.get(), n, rp_n);
+int merge_long(dcd_ctx* c, const int32_t* labels0, bool static_start, int64_t n_long, MergeOut* out,
+               EntryLabels* nlab) {
+  cudaStream_t s = c->stream;
+  const int64_t n = c->n, R = out->npairs;
+  DevScalars* d = c->dsc.get();
+  const int T = 256;
+  const int32_t* off = out->pair_ptr.get();
+  const int32_t* list = out->big.get() + 3 * n - n_long;
+  Buf<int64_t> first, ws;
+  Buf<int64_t> ltmp;
+  DCD_TRY(first.alloc(&c->mem, n_long + 1));
+  DCD_TRY(ltmp.alloc(&c->mem, scan_tmp_count(n_long + 1)));
+  ::dcd::count_launch(), long_sizes<<<grid_for(n_long + 1, T), T, 0, s>>>(list, n_long, off, first.get());
   DCD_LAUNCH_CHECK();
-  const int64_t nt = cdiv(c->nnz + R, (int64_t)kMergeTile);
-  if (nt > 0) {
-    Buf<int32_t> split;
-    DCD_TRY(split.alloc(&c->mem, nt + 1));
-    ::dcd::count_launch(), merge_split<<<grid_for((nt + 1) * 32, T), T, 0, s>>>(epos.get(), off + n, nt, split.get());
-    DCD_LAUNCH_CHECK();
-    if (nlab) DCD_TRY(nlab->buf.alloc(&c->mem, cap));
-    ::dcd::count_launch(), (nlab ? merge_tile<true> : merge_tile<false>)<<<(unsigned)nt, kMergeThreads, 0, s>>>(
-        c->nnz, col_o, w_o, split.get(), epos.get(), out->pkey.get(), out->pdelta.get(), out->pflag.get(), S.get(),
-        c->col[nxt].get(), c->w[nxt].get(), static_start ? nullptr : labels0, nlab ? nlab->buf.get() : nullptr);
-    DCD_LAUNCH_CHECK();
-    if (nlab) nlab->ready = true;
-  }
-  if (!static_start && !c->in_valid && c->cfg.alg == DCD_ALG_LOUVAIN) {
-    ::dcd::count_launch(), in_weight<<<grid_for(n * 32, T), T, 0, s>>>(n, rp_n, c->col[nxt].get(), c->w[nxt].get(),
-                                                                        labels0, gid, c->gs.get());
-    DCD_LAUNCH_CHECK();
-  }
-  return DCD_OK;
+  DCD_TRY(exclusive_scan<int64_t>(first.get(), first.get(), n_long + 1, nullptr, ltmp.get(), s));
+  DCD_TRY_CUDA(cudaMemcpyAsync(c->hscratch, first.get() + n_long, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  DCD_TRY_CUDA(cudaStreamSynchronize(s));
+  const int64_t recs = c->hscratch[0];
+  Buf<uint64_t> k0, k1;
+  Buf<uint32_t> v0, v1, stmp;
+  Buf<int64_t> wtmp;
+  Buf<int32_t> ds;
+  DCD_TRY(k0.alloc(&c->mem, recs));
+  DCD_TRY(k1.alloc(&c->mem, recs));
+  DCD_TRY(v0.alloc(&c->mem, recs));
+  DCD_TRY(v1.alloc(&c->mem, recs));
+  DCD_TRY(stmp.alloc(&c->mem, sort_tmp_words(recs) + scan_tmp_count(recs + 1)));
+  ::dcd::count_launch(), long_keys<<<grid_for(recs, T), T, 0, s>>>(list, n_long, first.get(), off, out->rec.get(), recs,
+                                                                   k0.get(), v0.get());
+  DCD_LAUNCH_CHECK();
+  const int ranges[4] = {0, bits_for(n - 1), 32, 32 + bits_for(n_long - 1)};
+  bool in1 = false;
+  DCD_TRY(sort_pairs<uint32_t>(k0.get(), v0.get(), k1.get(), v1.get(), recs, ranges, 2, stmp.get(), &in1, s));
+  DCD_TRY(ws.alloc(&c->mem, recs + 1));
+  DCD_TRY(ds.alloc(&c->mem, recs + 1));
+  DCD_TRY(wtmp.alloc(&c->mem, scan_tmp_count(recs + 1)));
+  ::dcd::count_launch(), long_terms<<<grid_for(recs + 1, T), T, 0, s>>>(in1 ? v1.get() : v0.get(), recs, ws.get(),
+                                                                        ds.get());
+  DCD_LAUNCH_CHECK();
+  DCD_TRY(exclusive_scan<int64_t>(ws.get(), ws.get(), recs + 1, nullptr, wtmp.get(), s));
+  DCD_TRY(exclusive_scan<int32_t>(ds.get(), ds.get(), recs + 1, nullptr, reinterpret_cast<int32_t*>(stmp.get()), s));
+  ::dcd::count_launch(), long_pairs<<<grid_for(cdiv(recs, kLongChunk) * 32, T), T, 0, s>>>(
+      pair_view(c, labels0, *out), list, first.get(), in1 ? k1.get() : k0.get(), ws.get(), ds.get(), recs,
+      out->k->get());
+  ::dcd::count_launch(), pair_net<<<grid_for(R + 1, T), T, 0, s>>>(out->pflag.get(), R, out->S.get());
+  DCD_LAUNCH_CHECK();
+  DCD_TRY_CUDA(cudaMemsetAsync(&d->n_long, 0, sizeof(int32_t), s));
+  return merge_rows(c, labels0, static_start, out, nlab);
 }
 
 }  // namespace dcd

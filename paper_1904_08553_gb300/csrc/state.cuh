@@ -51,6 +51,8 @@ struct DevScalars {
   int64_t rest_cnt;
   int64_t n1_new;  // communities K gets a row for in this update
   int64_t moved_deg;  // degrees of the last pass's movers (level 0, entry labels kept)
+  int32_t n_long;     // merge: sources with more records than a CTA sorts (merge_long)
+  int32_t pad4;
 };
 
 // Per-graph state of one update.  A context holds G graphs on disjoint vertex
@@ -366,9 +368,25 @@ struct MergeOut {
   Buf<int32_t> pair_ptr;   // n + 1: pairs of source u are [pair_ptr[u], pair_ptr[u+1])
   Buf<int32_t> pdelta;     // per pair: its weight in G_t minus its weight in G_{t-1}
   int64_t npairs = 0;      // pairs, null ones among them
+  // what merge_long goes on from
+  bool track_in = false;  // sum_i e_{i->C(i)} follows the pairs
+  Buf<uint64_t> rec;      // the records by source
+  Buf<int32_t> big;       // three lists of n: sources by the length of their segments
+  Buf<int64_t> epos;
+  Buf<int32_t> S;
+  void done() {
+    rec.reset();
+    big.reset();
+    epos.reset();
+    S.reset();
+  }
 };
 // nlab (may be NULL): the entry labels of G_t under the start labels, made on the way.
+// When the device scalar n_long is not zero after it, the rows are not merged:
+// merge_long, with that number, takes the sources it left and merges them.
 int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut* out, EntryLabels* nlab);
+int merge_long(dcd_ctx* c, const int32_t* labels0, bool static_start, int64_t n_long, MergeOut* out,
+               EntryLabels* nlab);
 
 // The batch's sources (vertices with pairs) by degree in G_t.
 struct SourceBins {
