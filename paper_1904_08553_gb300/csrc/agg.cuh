@@ -126,13 +126,7 @@ __device__ __forceinline__ void seg_argmax(ST& S, int32_t& D) {
 
 // Exact sum of non-negative weights over the lanes of `peers` (a match_any
 // group), from 16-bit slices reduced with redux.sync: no slice sum can carry
-// out of 32 bits, so the result is exact for any int32/int64 weight.
-__device__ __forceinline__ int64_t group_sum_exact(unsigned peers, int32_t w) {
-  unsigned lo = (unsigned)w & 0xffffu, hi = (unsigned)w >> 16;
-  unsigned slo = __reduce_add_sync(peers, lo);
-  unsigned shi = __reduce_add_sync(peers, hi);
-  return (int64_t)slo + ((int64_t)shi << 16);
-}
+// out of 32 bits, so the result is exact for any int64 weight.
 __device__ __forceinline__ int64_t group_sum_exact(unsigned peers, int64_t w) {
   unsigned long long x = (unsigned long long)w;
   int64_t s = 0;
@@ -144,76 +138,8 @@ __device__ __forceinline__ int64_t group_sum_exact(unsigned peers, int64_t w) {
   return s;
 }
 
-// Sum of weights over the lanes of `peers` as the gain arithmetic needs it:
-// with 64-bit gains 2m < 2^31, so every sum of a vertex's weights is below
-// 2^31 and one 32-bit reduction is exact; with 128-bit gains the sum is
-// taken exactly from 16-bit slices.
-template <typename ST, typename W>
-__device__ __forceinline__ int64_t group_sum(unsigned peers, W w);
-template <>
-__device__ __forceinline__ int64_t group_sum<long long, int32_t>(unsigned peers, int32_t w) {
-  return (int64_t)__reduce_add_sync(peers, (unsigned)w);
-}
-template <>
-__device__ __forceinline__ int64_t group_sum<long long, int64_t>(unsigned peers, int64_t w) {
-  return (int64_t)__reduce_add_sync(peers, (unsigned)w);
-}
-template <>
-__device__ __forceinline__ int64_t group_sum<i128, int32_t>(unsigned peers, int32_t w) {
-  return group_sum_exact(peers, w);
-}
-template <>
-__device__ __forceinline__ int64_t group_sum<i128, int64_t>(unsigned peers, int64_t w) {
-  return group_sum_exact(peers, w);
-}
-
 // ---- open-addressing table: key -1 = empty; capacity a power of two that is
 // at least twice the number of distinct keys, so probing always ends. ----
-__device__ __forceinline__ void tbl_add(int32_t* keys, unsigned long long* vals, uint32_t mask, int32_t lab,
-                                        unsigned long long x) {
-  uint32_t s = hash_label(lab, mask);
-  for (;;) {
-    int32_t k = keys[s];
-    if (k == lab) {
-      atomicAdd(&vals[s], x);
-      return;
-    }
-    if (k == -1) {
-      int32_t old = atomicCAS(&keys[s], -1, lab);
-      if (old == -1 || old == lab) {
-        atomicAdd(&vals[s], x);
-        return;
-      }
-    }
-    s = (s + 1) & mask;
-  }
-}
-
-// tbl_add that also appends each newly claimed slot to slots[] (counter *ns),
-// so the distinct keys can be visited, and the table emptied again, without a
-// scan over the whole capacity.
-template <typename VT>
-__device__ __forceinline__ void tbl_add_list(int32_t* keys, VT* vals, uint16_t* slots, int32_t* ns, uint32_t mask,
-                                             int32_t lab, VT x) {
-  uint32_t s = hash_label(lab, mask);
-  for (;;) {
-    int32_t k = keys[s];
-    if (k == lab) {
-      atomicAdd(&vals[s], x);
-      return;
-    }
-    if (k == -1) {
-      const int32_t old = atomicCAS(&keys[s], -1, lab);
-      if (old == -1) slots[atomicAdd(ns, 1)] = (uint16_t)s;
-      if (old == -1 || old == lab) {
-        atomicAdd(&vals[s], x);
-        return;
-      }
-    }
-    s = (s + 1) & mask;
-  }
-}
-
 template <typename VT>
 __device__ __forceinline__ int64_t tbl_get(const int32_t* keys, const VT* vals, uint32_t mask, int32_t lab) {
   uint32_t s = hash_label(lab, mask);
@@ -261,10 +187,13 @@ __device__ __forceinline__ uint32_t probe_claim(int32_t* keys, uint32_t mask, in
 // weights is below 2m < 2^31), 64-bit sums with 128-bit gains.
 template <int S>
 __device__ __forceinline__ int64_t seg_total(unsigned x) {
-  if constexpr (S == 32) return (int64_t)__reduce_add_sync(0xffffffffu, x);
+  if constexpr (S == 32) {
+    return (int64_t)__reduce_add_sync(0xffffffffu, x);
+  } else {
 #pragma unroll
-  for (int o = S / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return (int64_t)x;
+    for (int o = S / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return (int64_t)x;
+  }
 }
 template <int S>
 __device__ __forceinline__ int64_t seg_total(unsigned long long x) {

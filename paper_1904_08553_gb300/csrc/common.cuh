@@ -89,7 +89,6 @@ inline int wave_grid(K* kernel, int64_t items, int threads, size_t smem = 0) {
 enum : uint32_t {
   kErrBadRecord = 1u,   // invalid batch record
   kErrOverflow = 2u,    // weight above INT32_MAX or 2m too large
-  kErrTableFull = 4u,   // aggregation table overflow (cannot happen when sized by degree)
 };
 
 // ---- device memory of a context ----

@@ -894,7 +894,6 @@ __global__ void __launch_bounds__(256) lm_delta(LV<W> g, const int2* __restrict_
 __global__ void pass_begin(GraphState* __restrict__ gs, int G, DevScalars* __restrict__ d,
                            int32_t* __restrict__ item_cnt) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    d->pass_id += 1;
     d->any_running = 0;
     d->moved_deg = 0;
     d->stamp[0] = d->stamp[1] = global_ns();
@@ -1268,16 +1267,6 @@ struct RowWalk {
   }
 };
 
-// Coarse entries of one level (sort path): every entry (u, y, w) becomes the
-// key cid(L(u)) * nc + cid(L(y)) with weight w.  Equal keys are summed twice
-// before they are written: within a warp's 32-entry chunk (match_any + redux),
-// then across the warp's whole range of entries in a warp-private hash table
-// in shared memory (the chunk's leaders hold distinct keys, so their updates
-// of the table never contend).  A warp writes its table out when it passes
-// half full, and at the end.  A level that collapses into few communities --
-// level 0 of a step that starts from the previous step's communities -- then
-// writes a few hundred pairs per warp instead of one per chunk, and the sort
-// that follows has little to do.
 // After a pass of one graph that moved vertices with many entries: the entry
 // labels by a gather of every entry (as nlab_gather), and sum_i e_{i->C(i)} from
 // the same read, so that the movers' rows need not be read by themselves (19 M
@@ -1327,6 +1316,16 @@ __global__ void __launch_bounds__(256) nlab_resum(int64_t n, int64_t m, const in
     atomicAdd((unsigned long long*)&gs[0].in_delta, 0ull - (unsigned long long)gs[0].in_cur);
 }
 
+// Coarse entries of one level (sort path): every entry (u, y, w) becomes the
+// key cid(L(u)) * nc + cid(L(y)) with weight w.  Equal keys are summed twice
+// before they are written: within a warp's 32-entry chunk (match_any + redux),
+// then across the warp's whole range of entries in a warp-private hash table
+// in shared memory (the chunk's leaders hold distinct keys, so their updates
+// of the table never contend).  A warp writes its table out when it passes
+// half full, and at the end.  A level that collapses into few communities --
+// level 0 of a step that starts from the previous step's communities -- then
+// writes a few hundred pairs per warp instead of one per chunk, and the sort
+// that follows has little to do.
 constexpr int kEmitThreads = 256;
 
 // Warp table slots: 512 when key and sum are 32-bit (4 KB a warp), 256

@@ -19,15 +19,10 @@ struct Csr {
 
 // Per-step scalars kept on the device (one struct, copied back in one go).
 struct DevScalars {
-  int64_t pad_[9];
   int32_t any_running;  // some graph's pass loop goes on
   int32_t ticket;       // CTAs of pass_finish that are done
-  int32_t nc;        // labels in use (coarsening)
-  int32_t pad0;
-  int64_t uniq;      // distinct coarse entries (coarsening)
   int64_t act_deg;   // sum of the active vertices' degrees
   int64_t ncomm;     // communities at the end
-  int64_t nsrc;      // screening: distinct sources
   int64_t npairs;    // distinct (src, dst) pairs of the batch
   int64_t r_size;    // |R_t|
   uint32_t err;      // kErr* bits
@@ -35,7 +30,7 @@ struct DevScalars {
   int64_t bcnt[12];  // active vertices in each degree bin
   int64_t bdeg[12];  // sum of their degrees
   int64_t bmax[12];  // largest degree in the bin
-  int32_t pass_id;   // local-move passes started in this update (moved-in-pass marks)
+  int32_t pad0;
   int32_t level_passes;  // passes of the level running on the device
   unsigned long long stamp[2];  // globaltimer at the start of a pass and after its evaluation
   unsigned long long t_eval_ns, t_apply_ns;  // a level's evaluation and apply time, summed over its passes
