@@ -53,9 +53,10 @@ __global__ void to_local(int64_t n, const int32_t* __restrict__ lab, const int32
     out[v] = lab[v] - (int32_t)off[gid[v]];
 }
 
-// One byte a vertex; a graph's vertices are split over gridDim.y CTAs (one CTA
-// a graph: 319 us at 64 graphs, the largest of 200 K vertices, a byte a thread
-// in flight).
+// One byte a vertex; a graph's vertices are split over gridDim.y CTAs: as many as
+// make about 16 CTAs an SM in all, 32 at most (a graph of 200 K vertices is then 25
+// strides).  64 graphs, the largest of 200 K vertices: below 5 us, 319 with one CTA
+// a graph, a byte a thread in flight.
 __global__ void per_graph_counts(int G, const int64_t* __restrict__ off, const int64_t* __restrict__ rp,
                                  const uint8_t* __restrict__ r, long long* __restrict__ nnz,
                                  unsigned long long* __restrict__ rsz) {
@@ -107,7 +108,8 @@ int group_finish(dcd_ctx* c, void* user) {
   DCD_TRY(nnz.alloc(&c->mem, G));
   DCD_TRY(rsz.alloc(&c->mem, G));
   DCD_TRY_CUDA(cudaMemsetAsync(rsz.get(), 0, G * sizeof(unsigned long long), s));
-  const dim3 pg(G < 4096 ? G : 4096, G < 152 ? 32 : G < 2048 ? 4 : 1);
+  const int64_t split = 16 * (int64_t)num_sms() / G;
+  const dim3 pg(G < 4096 ? G : 4096, split < 1 ? 1 : split > 32 ? 32 : (unsigned)split);
   count_launch(), per_graph_counts<<<pg, 256, 0, s>>>(G, c->goff_d.get(), c->rp[1 - c->cur].get(), c->rset_nx.get(),
                                                       nnz.get(), rsz.get());
   DCD_LAUNCH_CHECK();

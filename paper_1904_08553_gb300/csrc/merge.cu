@@ -207,8 +207,9 @@ constexpr int kPairRow = 512;  // longest row staged on its own
 // NS by the records a source, R / n, so that a CTA has about 64 or more: 2 M
 // sources and 12.4 M records take 458 us with 32 sources (555 with the 64 and
 // 26 KB of before), 4.2 M sources and 2.0 M records 309 with 128 (485), 2 M and
-// 84 K 96 (142).  Small graphs have too few CTAs of 128: 32 below kPairWide.
-constexpr int64_t kPairWide = 128 * 152 * 4;
+// 84 K 96 (142).  A graph of fewer sources than four CTAs of 128 an SM has too few
+// CTAs of 128 or 64: 32.
+inline int64_t pair_wide() { return (int64_t)128 * 4 * num_sms(); }
 
 template <int NS>
 __global__ void __launch_bounds__(kPairThreads, 12) pair_tile(PairView o, int64_t n, const uint64_t* __restrict__ rec,
@@ -1057,7 +1058,7 @@ int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut*
   const PairView o = pair_view(c, labels0, *out);
   if (R > 0) {
     // sources a CTA: about 64 records for its 128 threads (pair_tile)
-    const int ns = R >= 2 * n || n < kPairWide ? 32 : 2 * R >= n ? 64 : 128;
+    const int ns = R >= 2 * n || n < pair_wide() ? 32 : 2 * R >= n ? 64 : 128;
     auto* tile = ns == 32 ? pair_tile<32> : ns == 64 ? pair_tile<64> : pair_tile<128>;
     ::dcd::count_launch(), tile<<<(unsigned)cdiv(n, ns), kPairThreads, 0, s>>>(
         o, n, rec.get(), c->kdeg[cur].get(), out->k->get(), big.get(), big_cnt, &d->n_long);
