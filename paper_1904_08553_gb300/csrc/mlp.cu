@@ -550,9 +550,9 @@ __device__ __forceinline__ bool grid_wait(unsigned* bar, unsigned target, int64_
 // of its two waits and of the passes through L2 between them (weights in,
 // partials out and in), so what does not depend on the other CTAs is loaded
 // before each wait: the parameters and moments to update, the next step's rows.
-// 32 steps of 8192 rows take 412 us (401 with sums split over four warps, which
+// 32 steps of 8192 rows take 402 us (386 with sums split over four warps, which
 // depend on the split); as four kernels a step (partials 18, sums 19, Adam 4, BF16
-// copies 3 us) 1308.
+// copies 3 us) 1300.
 struct TrainArgs {
   const float* X;
   const float* Y;
