@@ -35,14 +35,16 @@ LFR_N = 2_000_000
 LFR_EVENTS = 63_000_000
 LFR_STEPS = 12
 METRIC = "ms per time-step update"
-BYTES_PER_ENTRY = 12   # int32 col + int32 weight + int32 neighbour label, per directed entry visited
+# int32 neighbour label (entry labels) + int32 weight, per directed entry visited; graphs below 2^21 entries have no
+# entry labels and gather the label by column, 12 bytes, which are counted as 8 all the same
+BYTES_PER_ENTRY = 8
 BYTES_PER_VERTEX = 40  # row_ptr pair, k, label, a_C, |C|, proposal, list entry per active vertex
-# DRAM bytes per algorithmic byte of the local-move kernels: 525.9 MB of
-# dram__bytes_read.sum + dram__bytes_write.sum over 433.7 MB algorithmic, from
+# DRAM bytes per algorithmic byte of the local-move kernels: 506.9 MB of
+# dram__bytes_read.sum + dram__bytes_write.sum over 302.5 MB algorithmic, from
 # the ncu capture of one evaluation of every vertex of the n = 1,000,000
 # stream at t = 7 (the caches cold, as ncu leaves them before each pass)
-LM_TRAFFIC_RATIO = 525.9 / 433.7
-LM_KERNELS = ["lm_seg<8,2> (degree <= 16)", "lm_seg<16,2> (<= 32)", "lm_seg<16,4> (<= 64)",
+LM_TRAFFIC_RATIO = 506.9 / 302.5
+LM_KERNELS = ["lm_vert<4,4> (degree <= 16)", "lm_vert<8,4> (<= 32)", "lm_seg<16,4> (<= 64)",
               "lm_seg<32,4> (<= 128)", "lm_seg<32,8> (<= 256)", "lm_cta<128,4> (<= 512)",
               "lm_cta<256,4> (<= 1024)", "lm_cta<512,4> (<= 2048)", "lm_cta<512,8> (<= 4096)",
               "hub_agg + hub_gain + hub_pick + hub_clear (> 4096)"]
@@ -403,7 +405,7 @@ def gpu_arm(args):
     # per degree-bin kernel class: its share of the algorithmic bytes (the
     # bins of a pass run side by side inside one graph launch, so their times
     # are not separated)
-    names = ["lm_seg (degree <= 32)", "lm_seg (33..256)", "lm_cta (257..4096)",
+    names = ["lm_vert (degree <= 32)", "lm_seg (33..256)", "lm_cta (257..4096)",
              "hub_agg + hub_gain + hub_pick (> 4096)"]
     bins = []
     for b in range(4):
@@ -447,12 +449,13 @@ def gpu_arm(args):
             "levels": float(np.mean([s.levels for s in stats])),
         },
         "roofline": {
-            "kernel": "level-0 local-move evaluation: the degree-bin kernels of a pass (lm_seg, lm_cta, hub_*) over "
-                      "R_t on G_t, run side by side",
+            "kernel": "level-0 local-move evaluation: the degree-bin kernels of a pass (lm_vert, lm_seg, lm_cta, "
+                      "hub_*) over R_t on G_t, run side by side; the entry labels they read are made by the merge or "
+                      "a gather outside this time",
             "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": (achieved / peak) if achieved else None,
             "traffic": LM_TRAFFIC_RATIO * lm0_bytes / max(passes0, 1),
-            "traffic_note": ("DRAM bytes of one level-0 evaluation: its algorithmic bytes x 1.21, the "
+            "traffic_note": ("DRAM bytes of one level-0 evaluation: its algorithmic bytes x 1.68, the "
                              "DRAM-to-algorithmic ratio of an ncu capture of the same kernels at n = 1,000,000 "
                              "(cold L2, an upper bound for a pass of the timed loop)"),
             "peak_kind": peak_kind,
