@@ -130,7 +130,8 @@ typedef struct {
                             C_{t-1}, plus the batch's weight changes, plus the rows
                             of the vertices that level 0 moved.  Taken for a single
                             Louvain graph whose level-0 and previous communities
-                            number at most 4096, after a non-static update        */
+                            with entries number at most 4096, in an update that
+                            starts from the previous communities                  */
   int64_t coarse0_entries; /* entries that built level 0's coarse graph: nnz of G_t,
                               or batch pairs + rows of the moved vertices          */
   int64_t edges_level0_screen; /* of edges_level0, entries of the first level-0 pass
