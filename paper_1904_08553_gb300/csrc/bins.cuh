@@ -18,15 +18,24 @@ struct WantActive {
   __device__ __forceinline__ bool operator()(int64_t v) const {
     return (!active || active[v]) && (!gid || gs[gid[v]].running);
   }
+  __device__ __forceinline__ int64_t size(int64_t, int64_t deg) const { return deg; }
 };
-// ... or the sources of the batch's pairs.
+// ... or the sources of the batch's pairs, whose kernels walk over the pairs as
+// well as the row: a vertex that lost its edges, or whose edges the batch repeats,
+// has many pairs and a short row, and takes the kernel its pairs want (to the
+// largest one with a table in shared memory; the hub kernels are for long rows).
 struct WantSource {
   static constexpr bool kEmptyRows = true;  // a source may have lost its last edge: its deletes still mark
   const int32_t* pair_ptr;
   __device__ __forceinline__ bool operator()(int64_t v) const { return pair_ptr[v + 1] > pair_ptr[v]; }
+  __device__ __forceinline__ int64_t size(int64_t v, int64_t deg) const {
+    const int64_t p = pair_ptr[v + 1] - pair_ptr[v], most = lm_variant_max(kLmCta4k);
+    const int64_t q = p < most ? p : most;
+    return deg > q ? deg : q;
+  }
 };
 
-// Wanted vertices per degree bin, their degree sums and largest degree
+// Wanted vertices per bin (of the size Want gives them), their degree sums and largest degree
 // (DevScalars bcnt, bdeg, bmax; all of them, rows without entries included:
 // ncomm and act_deg).  Lane b of a warp keeps bin b's figures in registers: a
 // ballot and two reductions per bin and 32 vertices, no shared-memory traffic
@@ -53,7 +62,7 @@ __global__ void __launch_bounds__(256) bin_count(const int64_t* __restrict__ rp,
     const unsigned deg = ok ? (unsigned)(rp[v + 1] - rp[v]) : 0u;  // columns are int32: a row has fewer than 2^31
     deg_sum += deg;
     act += ok ? 1 : 0;
-    const int bin = (deg > 0 || (Want::kEmptyRows && ok)) ? bin_of(plan, deg) : -1;
+    const int bin = ok && (deg > 0 || Want::kEmptyRows) ? bin_of(plan, want.size(v, deg)) : -1;
     // a first-pass proposal from the screening, which the table kernels take
     // (the hub kernels evaluate their rows all the same)
     if (pre && deg > 0 && pre[v] >= 0 && plan.var[bin] != kLmHub) {
@@ -133,7 +142,7 @@ __global__ void __launch_bounds__(kBinThreads) bin_scatter(const int64_t* __rest
       bin[i] = -1;
       if (v < n && want(v)) {
         const int64_t deg = rp[v + 1] - rp[v];
-        if (deg > 0 || Want::kEmptyRows) bin[i] = bin_of(plan, deg);
+        if (deg > 0 || Want::kEmptyRows) bin[i] = bin_of(plan, want.size(v, deg));
       }
     }
 #pragma unroll

@@ -163,8 +163,11 @@ __device__ __forceinline__ void no_sink(const SV& g, int64_t p0, int64_t p1, int
 // The kernels follow the local move's for the same row lengths (louvain.cu says
 // why each is built as it is); what they add is a pass over the source's
 // pairs before the row (deletes; a source without inserts needs no row) and
-// one over its inserts after.  Bound like them by the latency of dependent
-// loads; on the LFR 2M step (2 M sources, 74 M entries, 12.4 M pairs) the bins
+// one over its inserts after.  A source's kernel is chosen by its row or its
+// pairs, whichever is longer: a vertex that loses 60,000 edges has no row left, and
+// one lane walked over its pairs for 9 ms (0.15 so, 0.08 when as many are spread).
+// Bound like them by the latency of dependent loads; on the LFR 2M step (2 M
+// sources, 74 M entries, 12.4 M pairs) the bins
 // run side by side in about 0.6 ms.  With four classes of sources (a warp with
 // lane compares to 32 entries, a warp table to 256, a CTA with an 8192-slot
 // table to 4096: two CTAs an SM for a row of 300) it took 1.9 ms, on R-MAT 22

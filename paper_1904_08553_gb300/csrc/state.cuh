@@ -383,7 +383,7 @@ int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut*
 int merge_long(dcd_ctx* c, const int32_t* labels0, bool static_start, int64_t n_long, MergeOut* out,
                EntryLabels* nlab);
 
-// The batch's sources (vertices with pairs) by degree in G_t.
+// The batch's sources (vertices with pairs) by degree in G_t or pairs (WantSource).
 struct SourceBins {
   BinPlan plan;
   int64_t cnt[kMaxBins] = {};
