@@ -1210,63 +1210,6 @@ __global__ void label_ids(int64_t n, const int32_t* __restrict__ size, const int
   }
 }
 
-// Row of entry e for the entry-linear walks below: a warp walks a range of
-// consecutive entries, finds the row of its first entry by binary search,
-// then advances 32 entries at a time with the row ends of the next 32 rows
-// in its lanes.
-struct RowWalk {
-  int64_t r;     // row of the chunk's first entry
-  int64_t rb;    // lane i holds the end of row rb + i (valid while chunks stay below `last`)
-  int64_t bk, last;
-  __device__ __forceinline__ void load(const int64_t* __restrict__ rp, int64_t n, int64_t r0) {
-    rb = r0;
-    bk = (r0 + 1 + lane_id() <= n) ? rp[r0 + 1 + lane_id()] : INT64_MAX;
-    last = __shfl_sync(0xffffffffu, bk, 31);
-  }
-  __device__ __forceinline__ void start(const int64_t* __restrict__ rp, int64_t n, int64_t E0) {
-    int64_t x = 0;
-    if (lane_id() == 0) {  // last row whose start is <= E0
-      int64_t lo = 0, hi = n - 1;
-      while (lo < hi) {
-        const int64_t mid = (lo + hi + 1) >> 1;
-        if (rp[mid] <= E0) lo = mid; else hi = mid - 1;
-      }
-      x = lo;
-    }
-    r = __shfl_sync(0xffffffffu, x, 0);
-    load(rp, n, r);
-  }
-  // row of entry c0 + lane (entries past the segment get the last row); the
-  // ends of 32 rows stay in the lanes across chunks and are reloaded only when
-  // a chunk runs past them
-  __device__ __forceinline__ int64_t row(const int64_t* __restrict__ rp, int64_t n, int64_t c0, bool valid) {
-    const int lane = lane_id();
-    const int64_t e = c0 + lane;
-    if (last <= c0 + 31) load(rp, n, r);
-    int64_t rw;
-    if (last <= c0 + 31) {
-      // more than 31 rows end inside this chunk (empty rows): search per lane
-      int64_t lo = r, hi = n - 1, x = valid ? e : c0;
-      while (lo < hi) {
-        const int64_t mid = (lo + hi + 1) >> 1;
-        if (rp[mid] <= x) lo = mid; else hi = mid - 1;
-      }
-      rw = lo;
-    } else {
-      int cntv = 0;
-      const int64_t x = valid ? e : c0;
-#pragma unroll
-      for (int step = 16; step > 0; step >>= 1) {
-        const int64_t v = __shfl_sync(0xffffffffu, bk, cntv + step - 1);
-        if (v <= x) cntv += step;
-      }
-      rw = rb + cntv;
-    }
-    r = __shfl_sync(0xffffffffu, rw, 31);
-    return rw;
-  }
-};
-
 // After a pass of one graph that moved vertices with many entries: the entry
 // labels by a gather of every entry (as nlab_gather), and sum_i e_{i->C(i)} from
 // the same read, so that the movers' rows need not be read by themselves (19 M

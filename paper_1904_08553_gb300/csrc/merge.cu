@@ -14,6 +14,7 @@
 // stands for all; so the pairs of source u are [off[u], off[u+1]) with no
 // compaction, and nothing has to be counted on the host before the merge.
 #include "prims.cuh"
+#include "rows.cuh"
 #include "state.cuh"
 
 namespace dcd {
@@ -693,49 +694,87 @@ __global__ void seed_sums(GraphState* __restrict__ gs, int G, const int64_t* __r
   }
 }
 
-// k of a graph whose degrees no update of this context has computed (a
-// loaded checkpoint), and its 2m into *m2.
-__global__ void row_degrees(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ w,
-                            int64_t* __restrict__ k, unsigned long long* __restrict__ m2) {
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  long long tot = 0;
-  for (int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; v < n; v += nw) {
-    long long x = 0;
-    for (int64_t e = rp[v] + lane_id(); e < rp[v + 1]; e += 32) x += w[e];
-    x = warp_sum(x);
-    if (lane_id() == 0) k[v] = x;
+// Sums over every entry of a graph, entry-linear: a warp takes a range of entries
+// whatever rows they belong to (a warp a row, as these once were, takes 4 ms for a
+// row of 400,000 entries).
+//
+// k of a graph whose degrees no update of this context has computed (a loaded
+// checkpoint), zeroed before, and its 2m into *m2.
+__global__ void __launch_bounds__(256) row_degrees(int64_t n, int64_t m, const int64_t* __restrict__ rp,
+                                                   const int32_t* __restrict__ w, int64_t per_warp,
+                                                   unsigned long long* __restrict__ k,
+                                                   unsigned long long* __restrict__ m2) {
+  const int lane = lane_id();
+  const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int64_t W0 = gw * per_warp, W1 = W0 + per_warp < m ? W0 + per_warp : m;
+  if (W0 >= W1) return;
+  RowWalk rw;
+  rw.start(rp, n, W0);
+  unsigned long long acc = 0, tot = 0;  // of row cur, a lane's share
+  int64_t cur = -1;
+  auto flush = [&]() {
+    acc = warp_sum(acc);
+    if (lane == 0 && acc) atomicAdd(&k[cur], acc);
+    acc = 0;
+  };
+  for (int64_t c0 = W0; c0 < W1; c0 += 32) {
+    const bool valid = c0 + lane < W1;
+    const int64_t r = rw.row(rp, n, c0, valid);
+    const unsigned long long x = valid ? (unsigned long long)ld_stream(w + c0 + lane) : 0ull;
     tot += x;
+    const int64_t r0 = __shfl_sync(0xffffffffu, r, 0);
+    const bool one = __all_sync(0xffffffffu, !valid || r == r0);
+    if (cur >= 0 && !(one && r0 == cur)) flush();
+    if (one) {
+      cur = r0;
+      acc += x;
+    } else {  // several rows: a run each
+      const unsigned peers = __match_any_sync(0xffffffffu, (unsigned long long)(valid ? r : -1));
+      const int64_t sum = group_sum_exact(peers, (int64_t)x);
+      if (valid && (int)(__ffs(peers) - 1) == lane) atomicAdd(&k[r], (unsigned long long)sum);
+      cur = -1;
+    }
   }
-  if (lane_id() == 0 && tot) atomicAdd(m2, (unsigned long long)tot);
+  if (cur >= 0) flush();
+  tot = warp_sum(tot);
+  if (lane == 0 && tot) atomicAdd(m2, tot);
 }
 
-// sum_i e_{i->C(i)} under labels L over every entry (when no update kept it:
-// labels set by the caller, a loaded checkpoint).
-__global__ void in_weight(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                          const int32_t* __restrict__ w, const int32_t* __restrict__ L,
-                          const int32_t* __restrict__ gid, GraphState* __restrict__ gs,
-                          const int32_t* __restrict__ n_long) {
+// sum_i e_{i->C(i)} under labels L (when no update kept it: labels set by the
+// caller, a loaded checkpoint; one graph).  *nnz: the entries.
+__global__ void __launch_bounds__(256) in_weight(int64_t n, const int64_t* __restrict__ rp,
+                                                 const int32_t* __restrict__ col, const int32_t* __restrict__ w,
+                                                 const int32_t* __restrict__ L, GraphState* __restrict__ gs,
+                                                 const int32_t* __restrict__ n_long) {
   if (*n_long) return;  // the rows are not merged yet
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  int cur = 0;
+  constexpr int U = 4;
+  const int lane = lane_id();
+  const int64_t m = rp[n], warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int64_t per_warp = (((m + warps - 1) / warps) + 32 * U - 1) / (32 * U) * (32 * U);
+  const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int64_t W0 = gw * per_warp, W1 = W0 + per_warp < m ? W0 + per_warp : m;
+  if (W0 >= W1) return;
+  RowWalk rw;
+  rw.start(rp, n, W0);
   unsigned long long acc = 0;
-  for (int64_t u = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; u < n; u += nw) {
-    const int g = graph_of(gid, u);
-    if (g != cur) {
-      acc = warp_sum(acc);
-      if (lane_id() == 0 && acc) atomicAdd((unsigned long long*)&gs[cur].in_cur, acc);
-      acc = 0;
-      cur = g;
+  for (int64_t c0 = W0; c0 < W1; c0 += 32 * U) {
+    int32_t y[U], x[U];
+#pragma unroll
+    for (int q = 0; q < U; q++) {
+      const int64_t e = c0 + q * 32 + lane;
+      y[q] = e < W1 ? ld_stream(col + e) : -1;
+      x[q] = e < W1 ? ld_stream(w + e) : 0;
     }
-    const int32_t Lu = L[u];
-    const int64_t e1 = rp[u + 1];
-    for (int64_t e = rp[u] + lane_id(); e < e1; e += 32) {
-      const int32_t x = ld_stream(w + e);
-      if (L[ld_stream(col + e)] == Lu) acc += (unsigned long long)x;
+#pragma unroll
+    for (int q = 0; q < U; q++) y[q] = y[q] >= 0 ? L[y[q]] : -1;
+#pragma unroll
+    for (int q = 0; q < U; q++) {
+      const int64_t c = c0 + q * 32;
+      if (c < W1 && L[rw.row(rp, n, c, c + lane < W1)] == y[q]) acc += (unsigned long long)x[q];  // (c < W1: uniform)
     }
   }
   acc = warp_sum(acc);
-  if (lane_id() == 0 && acc) atomicAdd((unsigned long long*)&gs[cur].in_cur, acc);
+  if (lane == 0 && acc) atomicAdd((unsigned long long*)&gs[0].in_cur, acc);
 }
 
 // ---- tiled merge ----
@@ -976,8 +1015,9 @@ int merge_rows(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut* 
     if (nlab) nlab->ready = true;
   }
   if (!static_start && !c->in_valid && c->cfg.alg == DCD_ALG_LOUVAIN) {
-    ::dcd::count_launch(), in_weight<<<grid_for(n * 32, T), T, 0, s>>>(n, rp_n, c->col[nxt].get(), c->w[nxt].get(),
-                                                                        labels0, gid, c->gs.get(), &d->n_long);
+    ::dcd::count_launch(), in_weight<<<wave_grid(in_weight, cap, T), T, 0, s>>>(n, rp_n, c->col[nxt].get(),
+                                                                                c->w[nxt].get(), labels0, c->gs.get(),
+                                                                                &d->n_long);
     DCD_LAUNCH_CHECK();
   }
   return DCD_OK;
@@ -1003,12 +1043,14 @@ int merge_batch(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut*
     DCD_TRY(c->kdeg[cur].ensure(&c->mem, n));
     DCD_TRY(c->in_prev.ensure(&c->mem, 2 * (size_t)c->G));
     DCD_TRY_CUDA(cudaMemsetAsync(c->in_prev.get(), 0, 2 * c->G * sizeof(int64_t), s));
+    DCD_TRY_CUDA(cudaMemsetAsync(c->kdeg[cur].get(), 0, n * sizeof(int64_t), s));
     if (c->nnz > 0) {  // a loaded checkpoint: one graph
-      ::dcd::count_launch(), row_degrees<<<grid_for(n * 32, T), T, 0, s>>>(
-          n, rp_o, w_o, c->kdeg[cur].get(), reinterpret_cast<unsigned long long*>(c->in_prev.get() + c->G));
+      const int grid = wave_grid(row_degrees, c->nnz, T);
+      const int64_t per_warp = cdiv(cdiv(c->nnz, (int64_t)grid * (T / 32)), 32) * 32;
+      ::dcd::count_launch(), row_degrees<<<grid, T, 0, s>>>(
+          n, c->nnz, rp_o, w_o, per_warp, reinterpret_cast<unsigned long long*>(c->kdeg[cur].get()),
+          reinterpret_cast<unsigned long long*>(c->in_prev.get() + c->G));
       DCD_LAUNCH_CHECK();
-    } else {
-      DCD_TRY_CUDA(cudaMemsetAsync(c->kdeg[cur].get(), 0, n * sizeof(int64_t), s));
     }
     c->k_valid = true;
   }
