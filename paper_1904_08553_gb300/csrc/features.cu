@@ -14,6 +14,7 @@
 // C_{t-1}.
 #include "agg.cuh"
 #include "prims.cuh"
+#include "pull.cuh"
 #include "state.cuh"
 
 namespace dcd {
@@ -36,37 +37,43 @@ __global__ void pool_mark(int64_t n, const int64_t* __restrict__ rp, const int32
 }
 
 // Pull: the vertices that the first two terms leave out look for a neighbour
-// with a pair, a warp a row, and stop at the first.  Reads at most the rows of
-// the vertices without pairs, where push reads (and writes a byte for) those with
+// with a pair, a warp a row (the rest of a long row: pull_rest), and stop at the
+// first.  Reads at most the rows of the vertices without pairs, where push reads (and writes a byte for) those with
 // pairs: taken when these hold half of the entries (kPoolPull).  1 M vertices, 21 M
 // entries, nearly all of them in rows with pairs: 414 us by push, below 5 so.
 constexpr int kPoolPull = 2;
+struct HasPair {
+  const int32_t* pair_ptr;
+  __device__ __forceinline__ bool operator()(int32_t x) const { return pair_ptr[x + 1] != pair_ptr[x]; }
+};
 __global__ void pool_pull(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
                           const int32_t* __restrict__ pair_ptr, const uint8_t* __restrict__ rds,
-                          uint8_t* __restrict__ pool) {
+                          uint8_t* __restrict__ pool, PullRest rest) {
+  const HasPair marked{pair_ptr};
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int lane = lane_id();
   for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
     const int64_t v = base + lane;
     bool in = v < n && (rds[v] || pair_ptr[v + 1] != pair_ptr[v]);
     unsigned left = __ballot_sync(0xffffffffu, v < n && !in);
+    int64_t deg = 0;  // of an undecided vertex
     while (left) {
       const int src = __ffs(left) - 1;
       left &= left - 1;
-      const int64_t u = base + src, end = rp[u + 1];
+      const int64_t u = base + src, b = rp[u], d = rp[u + 1] - b;
+      const int64_t end = b + (d < kPullFirst ? d : kPullFirst);
       bool hit = false;
-      for (int64_t e0 = rp[u]; e0 < end && !hit; e0 += 32) {
+      for (int64_t e0 = b; e0 < end && !hit; e0 += 32) {
         const int64_t e = e0 + lane;
-        bool h = false;
-        if (e < end) {
-          const int32_t x = col[e];
-          h = pair_ptr[x + 1] != pair_ptr[x];
-        }
-        hit = __any_sync(0xffffffffu, h);
+        hit = __any_sync(0xffffffffu, e < end && marked(col[e]));
       }
-      if (lane == src) in = hit;
+      if (lane == src) {
+        in = hit;
+        deg = d;
+      }
     }
     if (v < n) pool[v] = in ? 1 : 0;
+    pull_defer(rest, v < n && !in && deg > kPullFirst, v, deg);
   }
 }
 
@@ -183,7 +190,14 @@ int screen_features(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* L0, const 
   Buf<uint8_t> pool;
   DCD_TRY(pool.alloc(&c->mem, n));
   if (kPoolPull * source_deg >= g.nnz) {
-    count_launch(), pool_pull<<<grid_for(n, T), T, 0, s>>>(n, g.rp, g.col, mo.pair_ptr.get(), rds, pool.get());
+    PullBufs bufs;
+    PullRest rest{};
+    int32_t* cnt = c->dsc.get()->rest_cnt;  // the screening is done with it
+    DCD_TRY(bufs.alloc(&c->mem, n, g.nnz, cnt, &rest));
+    DCD_TRY_CUDA(cudaMemsetAsync(cnt, 0, 2 * sizeof(int32_t), s));
+    count_launch(), pool_pull<<<grid_for(n, T), T, 0, s>>>(n, g.rp, g.col, mo.pair_ptr.get(), rds, pool.get(), rest);
+    count_launch(), pull_rest<<<4 * c->sms, kPullThreads, 0, s>>>(g.rp, g.col, rest, HasPair{mo.pair_ptr.get()},
+                                                                  pool.get(), nullptr);
   } else {
     DCD_TRY_CUDA(cudaMemsetAsync(pool.get(), 0, n, s));
     count_launch(), pool_mark<<<grid_for(n * 32, T, 16), T, 0, s>>>(n, g.rp, g.col, mo.pair_ptr.get(), rds,

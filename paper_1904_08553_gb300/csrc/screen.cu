@@ -29,6 +29,7 @@
 #include "bins.cuh"
 #include "hub.cuh"
 #include "prims.cuh"
+#include "pull.cuh"
 #include "rows.cuh"
 #include "state.cuh"
 
@@ -743,16 +744,17 @@ __global__ void __launch_bounds__(256) scr_push(SV g, int64_t nnz, const int64_t
 }
 
 // R_t.  Pull: the vertices of a warp that are not in R_t yet are taken 8 lanes
-// each, up to kPullFirst entries; who is still undecided is listed for
-// rset_rest.
-constexpr int kPullFirst = 64;
+// each, up to kPullFirst entries; who is still undecided is left to pull_rest.
+struct Listed {
+  const uint8_t* listed;
+  __device__ __forceinline__ bool operator()(int32_t x) const { return listed[x] != 0; }
+};
 __global__ void __launch_bounds__(256) build_rset(int64_t n, int64_t nnz, const int64_t* __restrict__ rp,
                                                   const int32_t* __restrict__ col, const uint8_t* __restrict__ mark,
                                                   const uint8_t* __restrict__ cflag, const uint8_t* __restrict__ listed,
                                                   const unsigned long long* __restrict__ gamma_deg,
                                                   const int32_t* __restrict__ L, uint8_t* __restrict__ r,
-                                                  int32_t* __restrict__ rest, int32_t* __restrict__ rest_cnt,
-                                                  unsigned long long* __restrict__ count) {
+                                                  PullRest rest, unsigned long long* __restrict__ count) {
   const bool pull = listed && pulls(*gamma_deg, nnz);
   unsigned long long c = 0;
   const int lane = lane_id(), grp = lane >> 3, gl = lane & 7;
@@ -796,14 +798,7 @@ __global__ void __launch_bounds__(256) build_rset(int64_t n, int64_t nnz, const 
         }
         todo = left;
       }
-      const bool more = !x && d > kPullFirst;
-      const unsigned bal = __ballot_sync(0xffffffffu, more);
-      if (bal) {
-        int at = 0;
-        if (lane == 0) at = atomicAdd(rest_cnt, __popc(bal));
-        at = __shfl_sync(0xffffffffu, at, 0);
-        if (more) rest[at + __popc(bal & lanemask_lt())] = (int32_t)v;
-      }
+      pull_defer(rest, !x && d > kPullFirst, v, d);
     }
     if (v < n) {
       r[v] = x;
@@ -812,27 +807,6 @@ __global__ void __launch_bounds__(256) build_rset(int64_t n, int64_t nnz, const 
   }
   c = warp_sum(c);
   if (lane == 0 && c) atomicAdd(count, c);
-}
-
-// The undecided ones: a CTA per vertex, from entry kPullFirst on.
-__global__ void __launch_bounds__(256) rset_rest(const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                                                 const uint8_t* __restrict__ listed, const int32_t* __restrict__ rest,
-                                                 const int32_t* __restrict__ rest_cnt, uint8_t* __restrict__ r,
-                                                 unsigned long long* __restrict__ count) {
-  const int n = *rest_cnt;
-  for (int i = blockIdx.x; i < n; i += gridDim.x) {
-    const int32_t v = rest[i];
-    const int64_t e1 = rp[v + 1];
-    bool hit = false;
-    for (int64_t e = rp[v] + kPullFirst; e < e1 && !hit; e += 256) {
-      const int64_t x = e + threadIdx.x;
-      hit = __syncthreads_or(x < e1 && listed[col[x]]) != 0;
-    }
-    if (hit && threadIdx.x == 0) {
-      r[v] = 1;
-      atomicAdd(count, 1ull);
-    }
-  }
 }
 
 // ---- host side ----
@@ -933,9 +907,10 @@ int screen_batch(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* labels0, cons
   DCD_TRY_CUDA(cudaMemsetAsync(&d->r_screen, 0, 4 * sizeof(int64_t), s));  // r_screen, gamma_deg, gamma_items, rest
   unsigned long long* gamma_deg = reinterpret_cast<unsigned long long*>(&d->gamma_deg);
   int32_t* item_cnt = reinterpret_cast<int32_t*>(&d->gamma_items);
-  int32_t* rest_cnt = reinterpret_cast<int32_t*>(&d->rest_cnt);
-  Buf<int32_t> rest;
-  DCD_TRY(rest.alloc(&c->mem, n));
+  const bool may_pull = sb.total > 0 && 4 * sb.deg >= g.nnz;  // else pull cannot be taken
+  PullBufs rest_bufs;
+  PullRest rest{};
+  if (may_pull) DCD_TRY(rest_bufs.alloc(&c->mem, n, g.nnz, d->rest_cnt, &rest));
   if (sb.total > 0) {
     const int64_t nsrc = sb.total, item_cap = nsrc + sb.deg / kGammaChunk;
     Buf<int32_t> src, cursor, jstar;
@@ -972,10 +947,10 @@ int screen_batch(dcd_ctx* c, const Csr<int32_t>& g, const int32_t* labels0, cons
   }
   unsigned long long* count = reinterpret_cast<unsigned long long*>(&d->r_screen);
   count_launch(), build_rset<<<grid_for(n, T), T, 0, s>>>(n, g.nnz, g.rp, g.col, mark, cflag,
-                                                          sb.total > 0 ? listed : nullptr, gamma_deg, labels0, rset,
-                                                          rest.get(), rest_cnt, count);
-  if (sb.total > 0 && 4 * sb.deg >= g.nnz)  // else pull cannot have been taken
-    count_launch(), rset_rest<<<4 * c->sms, 256, 0, s>>>(g.rp, g.col, listed, rest.get(), rest_cnt, rset, count);
+                                                          may_pull ? listed : nullptr, gamma_deg, labels0, rset,
+                                                          rest, count);
+  if (may_pull)
+    count_launch(), pull_rest<<<4 * c->sms, kPullThreads, 0, s>>>(g.rp, g.col, rest, Listed{listed}, rset, count);
   DCD_LAUNCH_CHECK();
   return DCD_OK;
 }

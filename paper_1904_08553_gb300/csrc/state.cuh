@@ -43,7 +43,7 @@ struct DevScalars {
   int64_t r_screen;
   int64_t gamma_deg;
   int64_t gamma_items;
-  int64_t rest_cnt;
+  int32_t rest_cnt[2];
   int64_t n1_new;  // communities K gets a row for in this update
   int64_t moved_deg;  // degrees of the last pass's movers (level 0, entry labels kept)
   int32_t n_long;     // merge: sources with more records than a CTA sorts (merge_long)
