@@ -181,10 +181,11 @@ __device__ __forceinline__ void pair_sums_add(const PairView& o, int g, PairSum&
 
 // Segments of at most kSegSmall records are ranked by pair_tile; of at most
 // kSegMid and kSegLarge by a CTA each with a bitonic network in shared memory; of
-// at most kSegHuge by a CTA's radix sort in global memory.  Longer ones (a batch centred on one vertex, or one that repeats an edge) are
-// only counted on the way (DevScalars::n_long): the rows are then not merged, and
-// when the host has read the count, merge_long sorts them over the whole device
-// and merges.  The usual batch has none and pays nothing for them.
+// at most kSegHuge by a CTA's radix sort in global memory.  Longer ones (a batch
+// centred on one vertex, or one that repeats an edge) are only counted on the way
+// (DevScalars::n_long): what is merged then is of no use, and when the host has
+// read the count, merge_long sorts them over the whole device and merges again.
+// The usual batch has none and pays nothing for them.
 constexpr int kSegSmall = 64, kSegMid = 512, kSegLarge = 4096, kSegHuge = 32768;
 
 // A CTA takes NS consecutive sources: their records (a counting sort put them
@@ -800,16 +801,18 @@ __global__ void new_rows(const int64_t* __restrict__ rp_o, const int32_t* __rest
 // Pairs before merged item t * kMergeTile.  *npair: the pairs there are (fewer
 // than the batch's records when bad records took no place; the update then
 // fails, but stays within its buffers).  While segments are left to merge_long
-// (*n_long), their pairs hold nothing yet: -1, and merge_tile leaves.
+// (*n_long), their pairs hold nothing yet: no pairs, and merge_tile copies the old
+// entries, which the next merge overwrites (a test in merge_tile for an early return
+// cost it 37 us of 660 at 73 M entries and 12.4 M pairs).
 __global__ void merge_split(const int64_t* __restrict__ epos, const int32_t* __restrict__ npair, int64_t nt,
                             int32_t* __restrict__ sq, const int32_t* __restrict__ n_long) {
-  const int64_t P = *n_long ? -1 : *npair;
+  const int64_t P = *n_long ? 0 : *npair;
   const int lane = lane_id();
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   // a warp a tile: 32 probes a step, so that the chain is log32 of the pairs
   for (int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; t <= nt; t += nw) {
     const int64_t d = t * kMergeTile;
-    int64_t lo = P < 0 ? -1 : 0, hi = P < d ? P : d;  // first q with q + epos[q] >= d
+    int64_t lo = 0, hi = P < d ? P : d;  // first q with q + epos[q] >= d
     while (lo < hi) {
       const int64_t step = (hi - lo + 31) / 32, q = lo + lane * step;
       const unsigned below = __ballot_sync(0xffffffffu, q < hi && q + epos[q] < d);  // a prefix of the lanes
@@ -853,7 +856,6 @@ __global__ void __launch_bounds__(kMergeThreads) merge_tile(
   const int tid = threadIdx.x;
   const int64_t t = blockIdx.x;
   const int32_t q0 = sq[t], q1 = sq[t + 1];
-  if (q0 < 0) return;
   const int64_t e0 = t * kMergeTile - q0;
   const int64_t e1x = (t + 1) * kMergeTile - q1;
   const int64_t e1 = e1x < nnz ? e1x : nnz;
@@ -974,7 +976,7 @@ PairView pair_view(dcd_ctx* c, const int32_t* labels0, const MergeOut& m) {
                   m.pflag.get(), m.pdelta.get(), m.epos.get(), m.S.get(), c->gs.get(), &d->npairs, &d->err};
 }
 
-// G_t's rows from G_{t-1}'s and the pairs (nothing but the row starts while segments are left to merge_long).
+// G_t's rows from G_{t-1}'s and the pairs (of no use yet while segments are left to merge_long).
 int merge_rows(dcd_ctx* c, const int32_t* labels0, bool static_start, MergeOut* out, EntryLabels* nlab) {
   cudaStream_t s = c->stream;
   const int64_t n = c->n, R = out->npairs, n_ins = c->n_ins;
